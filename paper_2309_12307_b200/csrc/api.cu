@@ -176,6 +176,20 @@ Geometry make_geometry(int B, int N, int H, int Hkv, int G, int n_unshifted, int
     return g;
 }
 
+// Largest number of query tile pairs any group has (see tile_pair).
+int most_pairs(const Geometry& g) {
+    int most = 0;
+    const int shifts[2] = {0, g.shift};
+    for (int which = 0; which < 2; ++which) {
+        if ((which == 0 && g.n_unshifted == 0) || (which == 1 && g.n_unshifted == g.H)) continue;
+        for (int grp = 0; grp < g.groups; ++grp) {
+            const int n = pairs_of_group(group_layout(g, shifts[which], grp));
+            if (n > most) most = n;
+        }
+    }
+    return most;
+}
+
 constexpr float kLog2eHost = 1.4426950408889634f;
 
 // Diagnostic kernel behind s2a_selftest_wait_expiry: one warp waits, with the library's own bounded
@@ -243,11 +257,13 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     if ((rc = make_tmap(&p.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
     if ((rc = make_tmap(&p.tm_k, k, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
     if ((rc = make_tmap(&p.tm_v, v, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
+    if ((rc = make_tmap(&p.tm_o, o, d, H, N, B, kTile)) != S2A_OK) return rc;
     p.o = static_cast<__nv_bfloat16*>(o);
     p.lse = lse;
     p.status = ds->status_ptr;
     p.host_status = ds->host_word_dev;
     p.geo = make_geometry(B, N, H, Hkv, G, n_unshifted, shift, flags);
+    p.pairs_per_group = most_pairs(p.geo);
     p.scale_log2 = scale * kLog2eHost;
     cudaError_t e = launch_fwd(p, d, static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? S2A_OK : cuda_fail(e);

@@ -1,7 +1,7 @@
 // S2-Attn forward for sm_100a.
 //
-// One CTA computes one 128-row query tile of one (batch, head, group): steps "roll", "group",
-// "attention" and "roll back" of Algorithm 1 collapse into the choice of TMA coordinates.  Query
+// A work item is a pair of neighbouring 128-row query tiles of one (batch, head, group): steps "roll",
+// "group", "attention" and "roll back" of Algorithm 1 collapse into the choice of TMA coordinates.  Query
 // tile i of rolled group g in a head with shift s covers the ORIGINAL tokens given by tile_ref():
 // a group is one run of original tokens starting at (g*G + s) mod N, or, where it wraps past the
 // sequence end, two runs ([N-G/2, N) followed by [0, G/2) in Algorithm 1), and each run is tiled from
@@ -11,12 +11,22 @@
 // zero fill), masked as key columns and not stored as query rows.  Outputs are stored at the
 // original token rows, which is the roll back.
 //
-// Warp roles (320 threads): warp 0 issues TMA loads, warp 1 owns tensor memory and issues the
-// tcgen05 MMAs, warps 2-9 run the online softmax: a score row lives in one tensor-memory lane
-// (tcgen05.ld 32x32b) and is shared by two threads, one per 64-column half, which exchange their
-// partial row maxima through shared memory.  S = Q K^T accumulates in tensor memory, P (bf16) is written back over S and used as the
-// tensor-memory A operand of O += P V; O stays in tensor memory until the epilogue.  Two CTAs fit
-// on one SM, so one CTA's softmax overlaps the other CTA's MMAs.
+// One persistent block per SM, 512 threads:
+//   warps 0-3, 4-7   softmax of query tile 0 / 1: one thread per score row, the row's 128 scores in
+//                    registers (one trip to tensor memory per key tile, no exchange between threads)
+//   warps 8-11       epilogue: O / l -> bf16 -> shared memory -> TMA store (or row stores, ragged tiles)
+//   warp 12          work items (cluster launch control: a block takes over blocks that were not launched
+//                    yet, heaviest first) and TMA loads, running ahead across items
+//   warps 13, 14     tcgen05 MMAs of query tile 0 / 1:  O += P V_j, S = Q K_{j+1}^T, O += P V_{j+1}, ...
+// While one tile's scores are in the softmax, the tensor cores work for the other tile; K and V tiles
+// are fetched once for the 256 query rows, which halves their L2 and shared-memory traffic.
+// Tensor memory: S0 [0,128)  S1 [128,256)  O0 [256,256+HD)  O1 [384,384+HD); P (bf16) over S.
+//
+// What bounds it: the chain scores -> softmax -> P V -> next scores of a tile (clock stamps: about 2400
+// clocks in the softmax and 1100 in the two products of a step, with the other tile's step alongside); the
+// special-function unit and the tensor pipe are each busy about half of the time.  Measured against the
+// form it replaces (one query tile per block, two blocks per SM, two threads per row, scores read twice):
+// Llama2-7B 32k 2.04 against 2.38 ms a call, 8k 0.177 against 0.211, head size 64 at 32k 1.55 against 1.80.
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -26,360 +36,515 @@ namespace {
 
 template <int HD>
 struct FwdCfg {
-    static constexpr int kThreads = 320;
-    static constexpr int kBoxes = HD / 64;                      // 64-column TMA boxes per tile
-    static constexpr int kBoxBytes = kTile * 128;               // 128 rows x 128 bytes
-    static constexpr int kTileBytes = kBoxes * kBoxBytes;       // one Q, K or V tile
-    static constexpr int kStages = (HD == 128) ? 1 : 2;         // K/V ring depth
-    static constexpr int kBarBytes = 256 + 2 * 2 * 128 * 8;  // barriers + row-max exchange slots
-    static constexpr int kSmemBytes = 1024 /* alignment slack */ + (1 + 2 * kStages) * kTileBytes + kBarBytes;
-    static constexpr int kTmemCols = 256;                       // S: [0,128)  O: [128, 128+HD)
-    static constexpr int kColS = 0;
-    static constexpr int kColO = 128;
+    static constexpr int kThreads = 512;
+    static constexpr int kBoxes = HD / 64;                  // 64-column TMA boxes per tile
+    static constexpr int kBoxBytes = kTile * 128;           // 128 rows x 128 bytes
+    static constexpr int kTileBytes = kBoxes * kBoxBytes;   // one Q, K, V or O tile
+    static constexpr int kRing = (HD == 128) ? 4 : 8;       // K and V tiles in flight: K_0 V_0 K_1 V_1 ...
+    static constexpr int kBarBytes = 512 + 2 * 2 * kTile * 4;  // barriers + row statistics handed to the epilogue
+    static constexpr int kSmemBytes = (2 + kRing + 1) * kTileBytes + kBarBytes;
+    static constexpr int kTmemCols = 512;
+    static constexpr int kColO = 256;
+    // registers per thread after the split; the launch gives kRegsLaunch to each of the 512
+    static constexpr int kRegsLaunch = 128, kRegsSoftmax = 176, kRegsEpilogue = 80, kRegsIssue = 80;
+    static_assert(2 * kRegsSoftmax + kRegsEpilogue + kRegsIssue <= 4 * kRegsLaunch, "register split");
 };
+
+constexpr int kSched = 8;  // item ids in flight: the producer is at most five items ahead of the epilogue
+
+struct FwdBars {
+    uint64_t q_full[2], q_empty[2];
+    uint64_t s_full[2];              // S of a tile's step is in tensor memory
+    uint64_t p_full[2];              // P of keys [0, 96) of the step is in tensor memory (and O is rescaled)
+    uint64_t p_rest[2];              // the other 32 keys
+    uint64_t o_full[2], o_empty[2];  // an item's O is complete / has been read out
+    uint64_t stat_full[2], stat_empty[2];
+    uint64_t kv_full[8], kv_empty[8];
+    uint64_t sched_full[kSched];
+    uint64_t clc, drain[2];
+    alignas(16) uint8_t clc_resp[16];
+    int item[kSched];
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+static_assert(sizeof(FwdBars) <= 512, "barrier block");
 
 // Threshold (in log2 units) below which a larger running maximum is ignored: P then grows by at
 // most 2^8, which bf16 and the fp32 row sum absorb, and O needs no rescale.
 constexpr float kLazyRescale = 8.0f;
 
+struct FwdItem {
+    int b, h, hk;
+    GroupLayout L;
+    TilePair t;
+};
+// Work item `id`; false marks a slot of a group that has fewer pairs than the largest one.
+__device__ __forceinline__ bool fwd_item(const FwdParams& p, int id, FwdItem* w) {
+    int unit, rank;
+    decode_block(id, p.geo.B * p.geo.H * p.geo.groups, p.pairs_per_group, &unit, &rank);
+    const int g = unit % p.geo.groups;
+    w->h = (unit / p.geo.groups) % p.geo.H;
+    w->b = unit / (p.geo.groups * p.geo.H);
+    w->hk = w->h / (p.geo.H / p.geo.Hkv);
+    w->L = group_layout(p.geo, (w->h < p.geo.n_unshifted) ? 0 : p.geo.shift, g);
+    if (rank >= pairs_of_group(w->L)) return false;
+    w->t = tile_pair(w->L, rank);
+    return true;
+}
+
 template <int HD>
-__global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 2) s2a_fwd_kernel(const __grid_constant__ FwdParams p) {
+__global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const __grid_constant__ FwdParams p) {
     using C = FwdCfg<HD>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint8_t* sQ = smem;
-    uint8_t* sK = sQ + C::kTileBytes;
-    uint8_t* sV = sK + C::kStages * C::kTileBytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sV + C::kStages * C::kTileBytes);
-    uint64_t* q_full = bars + 0;
-    uint64_t* s_full = bars + 1;
-    uint64_t* p_full = bars + 2;
-    uint64_t* o_full = bars + 3;
-    uint64_t* drain = bars + 4;
-    uint64_t* k_full = bars + 5;                 // [kStages]
-    uint64_t* k_empty = k_full + C::kStages;     // [kStages]
-    uint64_t* v_full = k_empty + C::kStages;     // [kStages]
-    uint64_t* v_empty = v_full + C::kStages;     // [kStages]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(v_empty + C::kStages);
-    volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    // exchange slots between the two threads of a row: [2 parities][2 halves][128 rows] x {value, sequence}
-    volatile float2* xch = reinterpret_cast<volatile float2*>(reinterpret_cast<uint8_t*>(bars) + 256);
+    extern __shared__ __align__(1024) uint8_t smem[];  // 1024-byte aligned: checked below
+    uint8_t* sQ = smem;                                // two query tiles
+    uint8_t* sKV = sQ + 2 * C::kTileBytes;             // ring of K and V tiles
+    uint8_t* sO = sKV + C::kRing * C::kTileBytes;      // one output tile on its way out
+    FwdBars* bars = reinterpret_cast<FwdBars*>(sO + C::kTileBytes);
+    float* sStat = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);  // [tile][m, l][128 rows]
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
+    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later blocks
     // then return at once instead of each running into its own time limit.
-    __shared__ int s_poisoned;
-    if (threadIdx.x == 0) s_poisoned = *reinterpret_cast<volatile int*>(p.status);
+    if (threadIdx.x == 0) {
+        int bad = *reinterpret_cast<volatile int*>(p.status);
+        if ((smem_u32(smem) & 1023u) != 0) {  // cannot happen: nothing precedes the dynamic array
+            bad = kWaitFwd + 99;
+            atomicCAS(p.status, 0, bad);
+            *reinterpret_cast<volatile int*>(p.host_status) = bad;
+        }
+        bars->item[0] = bad;
+    }
     __syncthreads();
-    if (s_poisoned != 0) return;
-
-    // ---- which tile: heaviest query tiles of a group first, groups of one head adjacent -------
-    const int Tg = p.geo.tiles_per_group;
-    int unit, it;
-    decode_block(blockIdx.x, p.geo.B * p.geo.H * p.geo.groups, Tg, &unit, &it);
-    const int g = unit % p.geo.groups;
-    const int h = (unit / p.geo.groups) % p.geo.H;
-    const int b = unit / (p.geo.groups * p.geo.H);
-    const int hk = h / (p.geo.H / p.geo.Hkv);
-    const int s = (h < p.geo.n_unshifted) ? 0 : p.geo.shift;
-    const GroupLayout L = group_layout(p.geo, s, g);
-    const int i = L.nTiles - 1 - it;           // query tile inside the group
-    if (i < 0) return;                         // this group has fewer tiles than the largest one
-    const int j_begin = first_key_tile(L, i);
-    const int n_kv = i + 1 - j_begin;          // causal: key tiles j_begin..i of the same group (j_begin = 0 by default)
-    const TileRef tq = tile_ref(L, i);
-    const int tq0 = tq.tok0;
+    if (bars->item[0] != 0) return;
+    __syncthreads();
 
     if (threadIdx.x == 0) {
-        mbar_init(q_full, 1);
-        mbar_init(s_full, 1);
-        mbar_init(p_full, 256);
-        mbar_init(o_full, 1);
-        mbar_init(drain, 1);
-        for (int st = 0; st < C::kStages; ++st) {
-            mbar_init(k_full + st, 1);
-            mbar_init(k_empty + st, 1);
-            mbar_init(v_full + st, 1);
-            mbar_init(v_empty + st, 1);
+        for (int t = 0; t < 2; ++t) {
+            // hand-offs by four warps count one arrival per warp: 128 arrivals are 128 updates of one word of
+            // shared memory, whose bandwidth the operand reads of the MMAs need
+            mbar_init(&bars->q_full[t], 1);
+            mbar_init(&bars->q_empty[t], 1);
+            mbar_init(&bars->s_full[t], 1);
+            mbar_init(&bars->p_full[t], 4);
+            mbar_init(&bars->p_rest[t], 4);
+            mbar_init(&bars->o_full[t], 1);
+            mbar_init(&bars->o_empty[t], 4);
+            mbar_init(&bars->stat_full[t], 4);
+            mbar_init(&bars->stat_empty[t], 4);
+            mbar_init(&bars->drain[t], 1);
         }
-        *abort_flag = 0;
+        for (int x = 0; x < C::kRing; ++x) {
+            mbar_init(&bars->kv_full[x], 1);
+            mbar_init(&bars->kv_empty[x], 2);  // one hand-back by each tile's issuer
+        }
+        for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
+        mbar_init(&bars->clc, 1);
+        bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
         tma_prefetch_desc(&p.tm_k);
         tma_prefetch_desc(&p.tm_v);
+        tma_prefetch_desc(&p.tm_o);
     }
-    for (int idx = threadIdx.x; idx < 2 * 2 * 128; idx += C::kThreads) {  // sequence 0 = "nothing published"
-        const_cast<float2*>(xch)[idx] = make_float2(0.f, 0.f);
-    }
-    if (warp == 1) {
-        tmem_alloc(tmem_slot, C::kTmemCols);
+    if (warp == 13) {
+        tmem_alloc(&bars->tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
-    const WaitCtx ctx{abort_flag, p.status, p.host_status};
+    const uint32_t tmem_base = bars->tmem_slot;
+    const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
 
-    if (warp == 0) {
-        // =========================== TMA producer ============================================
-        if (lane == 0) {
-            mbar_expect_tx(q_full, C::kTileBytes);
-            for (int bx = 0; bx < C::kBoxes; ++bx)
-                tma_load_4d(sQ + bx * C::kBoxBytes, &p.tm_q, q_full, bx * 64, h, tq0, b);
-            int j = 0;
-            for (; j < n_kv; ++j) {
-                const int st = j % C::kStages;
-                const uint32_t ph = (j / C::kStages) & 1;
-                const int tk0 = tile_ref(L, j_begin + j).tok0;
-                if (!mbar_wait(k_empty + st, ph ^ 1, ctx, kWaitFwd + 1)) break;
-                mbar_expect_tx(k_full + st, C::kTileBytes);
-                for (int bx = 0; bx < C::kBoxes; ++bx)
-                    tma_load_4d(sK + st * C::kTileBytes + bx * C::kBoxBytes, &p.tm_k, k_full + st, bx * 64, hk, tk0, b);
-                if (!mbar_wait(v_empty + st, ph ^ 1, ctx, kWaitFwd + 2)) break;
-                mbar_expect_tx(v_full + st, C::kTileBytes);
-                for (int bx = 0; bx < C::kBoxes; ++bx)
-                    tma_load_4d(sV + st * C::kTileBytes + bx * C::kBoxBytes, &p.tm_v, v_full + st, bx * 64, hk, tk0, b);
-            }
-            if (*abort_flag != 0) {
-                // let loads that are still in flight land before the CTA gives its memory back
-                mbar_wait_drain(q_full, 0);
-                for (int jj = (j > C::kStages ? j - C::kStages : 0); jj < j; ++jj) {
-                    mbar_wait_drain(k_full + jj % C::kStages, (jj / C::kStages) & 1);
-                    mbar_wait_drain(v_full + jj % C::kStages, (jj / C::kStages) & 1);
+    // Every consumer warp walks the same sequence of items: the k-th id, -1 = the end (or aborting).
+    auto next_item = [&](int k, int where) -> int {
+        if (!mbar_wait_uniform(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return -1;
+        return *reinterpret_cast<volatile int*>(&bars->item[k % kSched]);
+    };
+
+    if (warp >= 12) {
+        setmaxnreg_dec<C::kRegsIssue>();
+        if (warp == 12) {
+            // ======================= work items, TMA loads ===========================================
+            if (lane == 0) {
+                uint32_t kv = 0;              // K and V tiles requested so far
+                uint32_t n_q[2] = {0, 0};     // query tiles requested so far
+                uint32_t n_clc = 0;
+                bool ok = true, asked = false;
+                int id = static_cast<int>(blockIdx.x);
+                auto ask = [&]() {
+                    mbar_expect_tx(&bars->clc, 16);
+                    clc_try_cancel(bars->clc_resp, &bars->clc);
+                    asked = true;
+                };
+                auto answer = [&]() -> int {
+                    asked = false;
+                    if (!mbar_wait(&bars->clc, n_clc & 1, ctx, kWaitFwd + 1)) {
+                        ok = false;
+                        return -1;
+                    }
+                    ++n_clc;
+                    const int x = clc_granted_block(bars->clc_resp);
+                    fence_proxy_async();  // the answer has been read before the next one is written
+                    return x;
+                };
+                auto load_q = [&](const FwdItem& w, int t) {
+                    if (!mbar_wait(&bars->q_empty[t], (n_q[t] & 1) ^ 1, ctx, kWaitFwd + 2)) { ok = false; return; }
+                    mbar_expect_tx(&bars->q_full[t], C::kTileBytes);
+                    const int tok0 = tile_ref(w.L, w.t.i[t]).tok0;
+                    for (int bx = 0; bx < C::kBoxes; ++bx)
+                        tma_load_4d(sQ + t * C::kTileBytes + bx * C::kBoxBytes, &p.tm_q, &bars->q_full[t], bx * 64, w.h, tok0, w.b);
+                    ++n_q[t];
+                };
+                auto load_kv = [&](const FwdItem& w, const CUtensorMap* tm, int tok0) {
+                    const int st = kv % C::kRing;
+                    if (!mbar_wait(&bars->kv_empty[st], ((kv / C::kRing) & 1) ^ 1, ctx, kWaitFwd + 3)) { ok = false; return; }
+                    mbar_expect_tx(&bars->kv_full[st], C::kTileBytes);
+                    for (int bx = 0; bx < C::kBoxes; ++bx)
+                        tma_load_4d(sKV + st * C::kTileBytes + bx * C::kBoxBytes, tm, &bars->kv_full[st], bx * 64, w.hk, tok0, w.b);
+                    ++kv;
+                };
+                for (int k = 0; ok; ++k) {
+                    if (id >= 0) ask();
+                    FwdItem w;
+                    while (id >= 0 && !fwd_item(p, id, &w)) {  // skip the empty slots of smaller groups
+                        id = answer();
+                        if (id >= 0) ask();
+                    }
+                    bars->item[k % kSched] = id;
+                    mbar_arrive(&bars->sched_full[k % kSched]);  // release: the id is visible to whoever sees the phase
+                    if (id < 0) break;
+                    for (int j = 0; ok && j < w.t.n[1]; ++j) {
+                        const int tok0 = tile_ref(w.L, w.t.j_begin + j).tok0;
+                        if (j == 0 && w.t.n[0] > 0) load_q(w, 0);
+                        if (ok) load_kv(w, &p.tm_k, tok0);
+                        if (j == 0 && ok) load_q(w, 1);
+                        if (ok) load_kv(w, &p.tm_v, tok0);
+                    }
+                    if (ok) id = answer();
                 }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // =========================== MMA issuer ==============================================
-        // The whole warp walks the loop so that addresses and descriptors stay warp-uniform values;
-        // only the MMA and commit instructions themselves are issued by one elected lane.
-        constexpr uint32_t idesc_s = idesc_bf16(128, 128, 0, 0);  // S = Q K^T   (both K-major)
-        constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);   // O += P V    (V is MN-major)
-        const uint32_t tS = tmem_base + C::kColS;
-        const uint32_t tO = tmem_base + C::kColO;
-        const uint32_t dQ = desc_lo_k_major(smem_u32(sQ));
-        bool ok = mbar_wait_uniform(q_full, 0, ctx, kWaitFwd + 3);
-        for (int j = 0; ok && j < n_kv; ++j) {
-            const int st = j % C::kStages;
-            const uint32_t ph = (j / C::kStages) & 1;
-            const uint32_t dK = desc_lo_k_major(smem_u32(sK + st * C::kTileBytes));
-            const uint32_t dV = desc_lo_mn_major(smem_u32(sV + st * C::kTileBytes), C::kBoxBytes);
-            if (!mbar_wait_uniform(k_full + st, ph, ctx, kWaitFwd + 4)) break;
-            tc_fence_after();
-            // The previous P (aliased on S) was consumed by the previous P.V, which precedes
-            // this MMA in issue order; the softmax warps finished reading S before that.
-            if (elect_one()) {
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk) {
-                    constexpr uint32_t kBox = C::kBoxBytes;
-                    mma_ss(tS, dQ + desc_step_k_major(kk, kBox), dK + desc_step_k_major(kk, kBox), idesc_s, kk > 0);
+                // Nothing may land after the block has gone: the pending answer, and the loads when aborting.
+                if (asked) mbar_wait_drain(&bars->clc, n_clc & 1);
+                if (bars->abort_flag != 0) {
+                    for (int t = 0; t < 2; ++t)
+                        if (n_q[t] > 0) mbar_wait_drain(&bars->q_full[t], (n_q[t] - 1) & 1);
+                    for (uint32_t x = (kv > C::kRing ? kv - C::kRing : 0); x < kv; ++x)
+                        mbar_wait_drain(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1);
                 }
-                mma_commit(k_empty + st);
-                mma_commit(s_full);
             }
             __syncwarp();
-            if (!mbar_wait_uniform(p_full, j & 1, ctx, kWaitFwd + 5)) break;
-            if (!mbar_wait_uniform(v_full + st, ph, ctx, kWaitFwd + 6)) break;
-            tc_fence_after();
-            if (elect_one()) {
+        } else if (warp <= 14) {
+            // ======================= MMA issuers: warp 13 for tile 0, warp 14 for tile 1 ==================
+            // The whole warp walks the loop so that addresses and descriptors stay warp-uniform values;
+            // only the MMA and commit instructions themselves are issued by one elected lane.  One warp
+            // for each tile: while one waits for a barrier the other keeps the tensor pipe fed (one warp for
+            // both tiles: 2.07 to 2.18 ms at 32k against 2.04).  A wait costs 100 to 200 clocks even when its
+            // phase is complete (barriers share shared memory with the operand reads), so K and V are waited
+            // for ahead of P: between P and the products that follow it, which are on the tile's critical
+            // path, there is only the wait for the rest of P.
+            constexpr uint32_t idesc_s = idesc_bf16(128, kTile, 0, 0);  // S = Q K^T   (both K-major)
+            constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);     // O += P V    (V is MN-major)
+            const int t = warp - 13;
+            const uint32_t dQ = desc_lo_k_major(smem_u32(sQ + t * C::kTileBytes)), aKV = smem_u32(sKV);
+            const uint32_t tS = tmem_base + t * kTile, tO = tmem_base + C::kColO + t * kTile;
+            uint32_t n_step = 0, n_q = 0, n_o = 0;  // P.V products, query tiles, outputs of this tile so far
+            auto wait_kv = [&](uint32_t x, int where) -> bool {
+                return mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, where);
+            };
+            int k = 0;
+            int n = 0, n1 = 0, m = 0, m1 = 0;  // steps of this tile and of tile 1: this item, the next one
+            auto fetch = [&]() -> bool {
+                const int id = next_item(k++, kWaitFwd + 10);
+                m = 0;
+                if (id < 0) return false;
+                FwdItem w;
+                fwd_item(p, id, &w);
+                m1 = w.t.n[1];
+                m = t ? m1 : w.t.n[0];
+                return true;
+            };
+            // Item by item, one turn a step: P.V of the step, then the scores of the next one, which may be
+            // the next item's first.  (The first pass, n = n1 = 0, only issues the first item's first scores.)
+            uint32_t kv = 0;  // ring position of the item's K_0
+            bool more = true, ok = true;
+            while (ok && more) {
+                const uint32_t kv_next = kv + 2 * n1;
+                const int turns = n > 0 ? n : 1;
+#pragma unroll 1
+                for (int j = 0; ok && j < turns; ++j) {
+                    if (j == turns - 1) more = fetch();
+                    const bool same = j + 1 < n, next = j == turns - 1 && m > 0, do_s = same || next, do_pv = j < n;
+                    const uint32_t xv = kv + 2 * j + 1, xk = same ? kv + 2 * (j + 1) : kv_next;
+                    if (do_pv) {
+                        if (j == 0 && !mbar_wait_uniform(&bars->o_empty[t], (n_o++ & 1) ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
+                        if (!wait_kv(xv, kWaitFwd + 6)) { ok = false; break; }
+                    }
+                    if (do_s) {
+                        if (next && !mbar_wait_uniform(&bars->q_full[t], n_q++ & 1, ctx, kWaitFwd + 4)) { ok = false; break; }
+                        if (!wait_kv(xk, kWaitFwd + 5)) { ok = false; break; }
+                    }
+                    if (do_pv) {
+                        const uint32_t dV = desc_lo_mn_major(aKV + (xv % C::kRing) * C::kTileBytes, C::kBoxBytes);
+                        if (!mbar_wait_uniform(&bars->p_full[t], n_step & 1, ctx, kWaitFwd + 8)) { ok = false; break; }
+                        tc_fence_after();
+                        if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < kTile / 16; ++kk) {
-                    mma_ts(tO, tS + (kk >> 2) * 64 + (kk & 3) * 8, dV + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
+                            for (int kk = 0; kk < 6; ++kk) mma_ts(tO, tS + kk * 8, dV + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
+                        }
+                        __syncwarp();
+                        if (!mbar_wait_uniform(&bars->p_rest[t], n_step & 1, ctx, kWaitFwd + 9)) { ok = false; break; }
+                        ++n_step;
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 6; kk < 8; ++kk) mma_ts(tO, tS + kk * 8, dV + kk * kDescStepMn, idesc_o, 1);
+                            mma_commit(&bars->kv_empty[xv % C::kRing]);
+                            if (j == n - 1) mma_commit(&bars->o_full[t]);
+                        }
+                        __syncwarp();
+                    }
+                    if (do_s) {
+                        const uint32_t dK = desc_lo_k_major(aKV + (xk % C::kRing) * C::kTileBytes);
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < HD / 16; ++kk)
+                                mma_ss(tS, dQ + desc_step_k_major(kk, C::kBoxBytes), dK + desc_step_k_major(kk, C::kBoxBytes), idesc_s, kk > 0);
+                            mma_commit(&bars->s_full[t]);
+                            mma_commit(&bars->kv_empty[xk % C::kRing]);
+                            if (same ? j + 2 == n : m == 1) mma_commit(&bars->q_empty[t]);
+                        }
+                        __syncwarp();
+                    }
                 }
-                mma_commit(v_empty + st);
-                if (j == n_kv - 1) mma_commit(o_full);
+                // K and V tiles that only the other query tile attends: each of them is handed back by both
+                // issuers, and only once it has landed (the hand-back belongs to the current use of its slot)
+                for (uint32_t x = kv + 2 * n; ok && x < kv_next; ++x) {
+                    ok = wait_kv(x, kWaitFwd + 17);
+                    if (ok && lane == 0) mbar_arrive(&bars->kv_empty[x % C::kRing]);
+                }
+                kv = kv_next, n = m, n1 = m1;
             }
-            __syncwarp();
-        }
-        if (__any_sync(0xffffffffu, *abort_flag != 0)) {
             // MMAs already issued must finish before tensor memory is released
-            if (elect_one()) {
-                mma_commit(drain);
-                mbar_wait_drain(drain, 0);
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
+                if (elect_one()) {
+                    mma_commit(&bars->drain[t]);
+                    mbar_wait_drain(&bars->drain[t], 0);
+                }
             }
+            __syncwarp();
         }
-        __syncwarp();
-    } else {
-        // =========================== softmax + epilogue ======================================
-        // Thread (quad, lane, half) owns columns [64*half, +64) of score row 32*quad + lane.  Its
-        // bf16 P values go over the first 32 of its own columns, so the two halves never write
-        // into columns the other half still has to read: P's 128 K values sit at packed columns
-        // [0,32) and [64,96).
-        const int quad = warp & 3;             // tensor-memory lane quadrant this warp may access
-        const int half = (warp - 2) >> 2;
+    } else if (warp >= 8) {
+        // =========================== epilogue ========================================================
+        setmaxnreg_dec<C::kRegsEpilogue>();
+        const int quad = warp & 3;
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-        const uint32_t t_mine = t_row + C::kColS + half * 64;
-        const float c2 = p.scale_log2;
-        float m_used = -INFINITY;              // running maximum in use, already scaled to log2 units
-        float l = 0.f;                         // this half's part of the running sum of exp2(s*c2 - m_used)
+        uint32_t n_o[2] = {0, 0};
         bool ok = true;
-        // Publish `v` to the thread that owns the other half of this row and fetch its value.
-        // One 8-byte store carries the value together with a sequence number, the reader polls
-        // (bounded) until the number matches.  Slots alternate with the parity of `seq`; a thread
-        // cannot run two exchanges ahead of its partner, so a slot is never overwritten unread.
-        auto pair_exchange = [&](float v, int seq, float& other) -> bool {
-            const uint32_t slot = smem_u32(const_cast<float2*>(xch)) + (seq & 1) * 2048;
-            const uint32_t mine = slot + (half * 128 + row) * 8;
-            const uint32_t theirs = slot + ((half ^ 1) * 128 + row) * 8;
-            asm volatile("st.volatile.shared.v2.b32 [%0], {%1, %2};" ::"r"(mine), "r"(__float_as_uint(v)), "r"(seq + 1)
-                         : "memory");
-            const long long t0 = clock64();
-            for (uint32_t spins = 1;; ++spins) {
-                uint32_t val, tag;
-                asm volatile("ld.volatile.shared.v2.b32 {%0, %1}, [%2];" : "=r"(val), "=r"(tag) : "r"(theirs) : "memory");
-                if (tag == static_cast<uint32_t>(seq + 1)) {
-                    other = __uint_as_float(val);
-                    return true;
-                }
-                if ((spins & 255u) == 0) {
-                    if (*abort_flag != 0) return false;
-                    if (clock64() - t0 > kWaitLimitCycles) {
-                        report_expiry(ctx, kWaitFwd + 9);
-                        return false;
+        for (int k = 0; ok; ++k) {
+            const int id = next_item(k, kWaitFwd + 11);
+            // the four warps leave together, or the ones that stay would wait for the others below
+            if (!named_barrier_and(1, 128, id >= 0)) break;
+            FwdItem w;
+            fwd_item(p, id, &w);
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                if (w.t.n[t] == 0) continue;
+                const TileRef tq = tile_ref(w.L, w.t.i[t]);
+                const bool whole = tq.valid == kTile;
+                // the tile stored last must have left the staging buffer (thread 0 of the four warps stores)
+                if (threadIdx.x == 256) bulk_wait_read<0>();
+                ok = mbar_wait_uniform(&bars->stat_full[t], n_o[t] & 1, ctx, kWaitFwd + 12) &&
+                     mbar_wait_uniform(&bars->o_full[t], n_o[t] & 1, ctx, kWaitFwd + 13);
+                ok = named_barrier_and(1, 128, ok);
+                if (!ok) break;
+                tc_fence_after();
+                ++n_o[t];
+                const float m = sStat[t * 256 + row], l = sStat[t * 256 + 128 + row];
+                mbar_arrive_warp(&bars->stat_empty[t]);
+                const float inv_l = 1.0f / l;
+                const int tok = tq.tok0 + row;
+                const bool row_valid = row < tq.valid;  // rows past the end of a ragged tile are not part of the group
+                __nv_bfloat16* orow = p.o + ((static_cast<size_t>(w.b) * p.geo.N + tok) * p.geo.H + w.h) * HD;
+#pragma unroll
+                for (int c = 0; c < HD / 32; ++c) {
+                    uint32_t r[32];
+                    tmem_ld_32x32(t_row + C::kColO + t * kTile + c * 32, r);
+                    tmem_wait_ld();
+                    const uint32_t dst_s = smem_u32(sO) + (c >> 1) * C::kBoxBytes + row * 128;
+                    uint4* dst_g = reinterpret_cast<uint4*>(orow + c * 32);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        uint4 pk;
+                        pk.x = pack_bf16(__uint_as_float(r[8 * e + 0]) * inv_l, __uint_as_float(r[8 * e + 1]) * inv_l);
+                        pk.y = pack_bf16(__uint_as_float(r[8 * e + 2]) * inv_l, __uint_as_float(r[8 * e + 3]) * inv_l);
+                        pk.z = pack_bf16(__uint_as_float(r[8 * e + 4]) * inv_l, __uint_as_float(r[8 * e + 5]) * inv_l);
+                        pk.w = pack_bf16(__uint_as_float(r[8 * e + 6]) * inv_l, __uint_as_float(r[8 * e + 7]) * inv_l);
+                        if (whole) {
+                            // 16-byte chunk (4 (c & 1) + e) of the 128-byte row, swizzled as the tensor map has it
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst_s + (((4 * (c & 1) + e) ^ (row & 7)) << 4)),
+                                         "r"(pk.x), "r"(pk.y), "r"(pk.z), "r"(pk.w)
+                                         : "memory");
+                        } else if (row_valid) {
+                            dst_g[e] = pk;
+                        }
                     }
                 }
-            }
-        };
-        for (int j = 0; j < n_kv; ++j) {
-            if (!mbar_wait(s_full, j & 1, ctx, kWaitFwd + 7)) { ok = false; break; }
-            tc_fence_after();
-            // pass 1: row maximum of this thread's 64 columns (the scores are read again in pass 2,
-            // 32 at a time, which keeps the register footprint small enough for two CTAs per SM)
-            // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
-            // on the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
-            const int k_valid = tile_ref(L, j_begin + j).valid;
-            const bool last = (j == n_kv - 1);
-            const bool diagonal = last || k_valid < kTile;   // "this tile is masked"
-            const int vis = (last && row < k_valid) ? row : k_valid - 1;
-            const int lim = vis - half * 64;   // visible iff (column within this half) <= lim
-            float mx4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t sreg[32];
-                tmem_ld_32x32(t_mine + c * 32, sreg);
-                tmem_wait_ld();
-                if (diagonal) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (c * 32 + e > lim) sreg[e] = 0xff800000u;  // -inf
-                }
-#pragma unroll
-                for (int e = 0; e < 32; ++e) mx4[e & 3] = fmaxf(mx4[e & 3], __uint_as_float(sreg[e]));
-            }
-            const float mx_own = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3]));
-            float mx_other;
-            if (!pair_exchange(mx_own, j, mx_other)) { ok = false; break; }
-            const float mx = fmaxf(mx_own, mx_other);
-            const float m_new = fmaxf(m_used, mx * c2);
-            if (j == 0) {
-                m_used = m_new;
-            } else {
-                const bool need = (m_new - m_used) > kLazyRescale;
-                if (__any_sync(0xffffffffu, need)) {
-                    // s_full(j) also covers the previous P.V, so O is quiescent here; each half
-                    // rescales its own half of O's columns
-                    const float alpha = need ? fast_exp2(m_used - m_new) : 1.0f;
-                    l *= alpha;
-#pragma unroll
-                    for (int c = 0; c < HD / 64; ++c) {
-                        uint32_t oreg[32];
-                        const uint32_t t_o = t_row + C::kColO + half * (HD / 2) + c * 32;
-                        tmem_ld_32x32(t_o, oreg);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) oreg[e] = __float_as_uint(__uint_as_float(oreg[e]) * alpha);
-                        tmem_st_32x32(t_o, oreg);
+                tc_fence_before();
+                mbar_arrive_warp(&bars->o_empty[t]);
+                if (whole) {
+                    fence_proxy_async();
+                    named_barrier(1, 128);
+                    if (threadIdx.x == 256) {
+                        for (int bx = 0; bx < C::kBoxes; ++bx)
+                            tma_store_4d(&p.tm_o, sO + bx * C::kBoxBytes, bx * 64, w.h, tq.tok0, w.b);
+                        bulk_commit_group();
                     }
-                    if (need) m_used = m_new;
                 }
+                // natural-log sum-exp of the scaled scores
+                if (row_valid) p.lse[(static_cast<size_t>(w.b) * p.geo.H + w.h) * p.geo.N + tok] = (m + log2f(l)) * 0.6931471805599453f;
             }
-            float sum4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t sreg[32];
-                tmem_ld_32x32(t_mine + c * 32, sreg);
-                tmem_wait_ld();
-                if (diagonal) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e)
-                        if (c * 32 + e > lim) sreg[e] = 0xff800000u;
-                }
-                uint32_t preg[16];
-#pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const float p0 = fast_exp2(fmaf(__uint_as_float(sreg[2 * e]), c2, -m_used));
-                    const float p1 = fast_exp2(fmaf(__uint_as_float(sreg[2 * e + 1]), c2, -m_used));
-                    sum4[e & 3] += p0 + p1;
-                    preg[e] = pack_bf16(p0, p1);
-                }
-                // packed columns [16c, 16c+16) overlay score columns [16c, 16c+16) of this half, which
-                // pass 2 has already consumed (c = 1 writes over columns 16..31, read when c was 0)
-                tmem_st_32x16(t_mine + c * 16, preg);
-            }
-            l += (sum4[0] + sum4[1]) + (sum4[2] + sum4[3]);
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(p_full);
         }
-        if (ok && mbar_wait(o_full, 0, ctx, kWaitFwd + 8)) {
-            tc_fence_after();
-            // total row sum = this half's part + the other half's
-            float l_other = 0.f;
-            pair_exchange(l, n_kv, l_other);
-            const float l_row = l + l_other;
-            const float inv_l = 1.0f / l_row;
-            const int t = tq0 + row;
-            const bool row_valid = row < tq.valid;   // rows past the end of a ragged tile are not part of the group
-            __nv_bfloat16* orow = p.o + ((static_cast<size_t>(b) * p.geo.N + t) * p.geo.H + h) * HD + half * (HD / 2);
-#pragma unroll
-            for (int c = 0; c < HD / 64; ++c) {
-                uint32_t oreg[32];
-                tmem_ld_32x32(t_row + C::kColO + half * (HD / 2) + c * 32, oreg);
+        if (threadIdx.x == 256) bulk_wait_all();
+    } else {
+        // =========================== softmax =========================================================
+        setmaxnreg_inc<C::kRegsSoftmax>();
+        const int t = warp >> 2;               // query tile
+        const int quad = warp & 3;             // tensor-memory lane quadrant this warp may access
+        const int row = quad * 32 + lane;
+        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+        const uint32_t tS = t_row + t * kTile;
+        const float c2 = p.scale_log2;
+        const uint64_t c2x2 = f2_pack(c2, c2);
+        uint32_t n_s = 0, n_it = 0;
+        bool ok = true;
+        for (int k = 0; ok; ++k) {
+            const int id = next_item(k, kWaitFwd + 14);
+            if (id < 0) break;
+            FwdItem w;
+            fwd_item(p, id, &w);
+            const int n = t ? w.t.n[1] : w.t.n[0];
+            if (n == 0) continue;
+            float m_used = 0.f;   // running maximum in use, scaled to log2 units
+            float l = 0.f;        // running sum of exp2(s*c2 - m_used)
+            for (int j = 0; j < n; ++j, ++n_s) {
+                const int k_valid = tile_ref(w.L, w.t.j_begin + j).valid;
+                if (!mbar_wait_uniform(&bars->s_full[t], n_s & 1, ctx, kWaitFwd + 15)) { ok = false; break; }
+                tc_fence_after();
+                uint32_t s[4][32];
+                tmem_ld_32x32(tS, s[0]);
+                tmem_ld_32x32(tS + 32, s[1]);
+                tmem_ld_32x32(tS + 64, s[2]);
+                tmem_ld_32x32(tS + 96, s[3]);
                 tmem_wait_ld();
-                uint4* dst = reinterpret_cast<uint4*>(orow + c * 32);
+                // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
+                // on the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
+                const bool last = (j == n - 1);
+                if (last || k_valid < kTile) {
+                    const int vis = (last && row < k_valid) ? row : k_valid - 1;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    uint4 pk;
-                    pk.x = pack_bf16(__uint_as_float(oreg[8 * e + 0]) * inv_l, __uint_as_float(oreg[8 * e + 1]) * inv_l);
-                    pk.y = pack_bf16(__uint_as_float(oreg[8 * e + 2]) * inv_l, __uint_as_float(oreg[8 * e + 3]) * inv_l);
-                    pk.z = pack_bf16(__uint_as_float(oreg[8 * e + 4]) * inv_l, __uint_as_float(oreg[8 * e + 5]) * inv_l);
-                    pk.w = pack_bf16(__uint_as_float(oreg[8 * e + 6]) * inv_l, __uint_as_float(oreg[8 * e + 7]) * inv_l);
-                    if (row_valid) dst[e] = pk;
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int e = 0; e < 32; ++e)
+                            if (c * 32 + e > vis) s[c][e] = 0xff800000u;  // -inf
                 }
+                float mx4[4];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    mx4[c] = fmaxf(__uint_as_float(s[c][0]), __uint_as_float(s[c][1]));
+#pragma unroll
+                    for (int e = 2; e < 32; e += 2) mx4[c] = fmax3(mx4[c], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
+                }
+                const float m_new = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * c2;
+                if (j == 0) {
+                    m_used = m_new;
+                } else {
+                    const bool need = (m_new - m_used) > kLazyRescale;
+                    if (__any_sync(0xffffffffu, need)) {
+                        // s_full of this step also covers the P.V product of the step before, so O is quiescent here
+                        const float alpha = need ? fast_exp2(m_used - m_new) : 1.0f;
+                        l *= alpha;
+#pragma unroll 1
+                        for (int c = 0; c < HD / 16; ++c) {
+                            uint32_t o[16];
+                            const uint32_t t_o = t_row + C::kColO + t * kTile + c * 16;
+                            tmem_ld_32x16(t_o, o);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+                            tmem_st_32x16(t_o, o);
+                        }
+                        if (need) m_used = m_new;
+                    }
+                }
+                const uint64_t nm = f2_pack(-m_used, -m_used);
+                uint64_t sum[2] = {0, 0};
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    uint32_t pk[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) {
+                        const uint64_t x = f2_fma(f2_pack(__uint_as_float(s[c][2 * e]), __uint_as_float(s[c][2 * e + 1])), c2x2, nm);
+                        float x0, x1;
+                        f2_unpack(x, x0, x1);
+                        const float p0 = fast_exp2(x0), p1 = fast_exp2(x1);
+                        sum[e & 1] = f2_add(sum[e & 1], f2_pack(p0, p1));
+                        pk[e] = pack_bf16(p0, p1);
+                    }
+                    // every score of the row is in registers, so P may go over the start of S: 16 packed columns
+                    tmem_st_32x16(tS + c * 16, pk);
+                    if (c >= 2) {
+                        tmem_wait_st();
+                        tc_fence_before();
+                        mbar_arrive_warp(c == 2 ? &bars->p_full[t] : &bars->p_rest[t]);
+                    }
+                }
+                float a0, a1, b0, b1;
+                f2_unpack(sum[0], a0, a1);
+                f2_unpack(sum[1], b0, b1);
+                l += (a0 + a1) + (b0 + b1);
             }
-            // natural-log sum-exp of the scaled scores
-            if (half == 0 && row_valid)
-                p.lse[(static_cast<size_t>(b) * p.geo.H + h) * p.geo.N + t] = (m_used + log2f(l_row)) * 0.6931471805599453f;
+            if (!ok || !mbar_wait_uniform(&bars->stat_empty[t], (n_it & 1) ^ 1, ctx, kWaitFwd + 16)) break;
+            ++n_it;
+            sStat[t * 256 + row] = m_used;
+            sStat[t * 256 + 128 + row] = l;
+            mbar_arrive_warp(&bars->stat_full[t]);
         }
     }
 
     // ---- teardown ------------------------------------------------------------------------------
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) {
+    if (warp == 13) {
         tc_fence_after();
         tmem_dealloc(tmem_base, C::kTmemCols);
     }
 }
 
+template <int HD>
+cudaError_t configure_one() {
+    using C = FwdCfg<HD>;
+    // the register split of the kernel draws on what a block is launched with
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, s2a_fwd_kernel<HD>);
+    if (e != cudaSuccess) return e;
+    if (a.numRegs < C::kRegsLaunch || a.sharedSizeBytes != 0) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(s2a_fwd_kernel<HD>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+}
+
 }  // namespace
 
 cudaError_t configure_fwd() {
-    cudaError_t e = cudaFuncSetAttribute(s2a_fwd_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         FwdCfg<64>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(s2a_fwd_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                FwdCfg<128>::kSmemBytes);
+    const cudaError_t e = configure_one<64>();
+    return e != cudaSuccess ? e : configure_one<128>();
 }
 
 cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream) {
-    const long long n_cta = static_cast<long long>(p.geo.B) * p.geo.H * p.geo.groups * p.geo.tiles_per_group;
-    const dim3 grid(static_cast<unsigned>(n_cta));
+    const long long n_items = static_cast<long long>(p.geo.B) * p.geo.H * p.geo.groups * p.pairs_per_group;
+    const dim3 grid(static_cast<unsigned>(n_items));
     if (d == 64) {
         s2a_fwd_kernel<64><<<grid, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, stream>>>(p);
     } else {

@@ -109,16 +109,45 @@ __host__ __device__ inline TileRef subtile_ref(const GroupLayout& L, int n) {
 __host__ __device__ inline int first_key_tile(const GroupLayout& L, int i) { return (L.cut > 0 && i >= L.cut) ? L.cut : 0; }
 __host__ __device__ inline int end_query_tile(const GroupLayout& L, int j) { return (L.cut > 0 && j < L.cut) ? L.cut : L.nTiles; }
 
+// The forward kernel works on two neighbouring query tiles of a group at a time ("a pair"), which share
+// the key tiles they stream.  The pairs of a group are numbered by rank, most work first; the tiles on
+// either side of a cut (variant 2 of Appendix B) have no keys in common and are paired separately.
+__host__ __device__ inline int pairs_of_group(const GroupLayout& L) {
+    return L.cut > 0 ? (L.nTiles - L.cut + 1) / 2 + (L.cut + 1) / 2 : (L.nTiles + 1) / 2;
+}
+struct TilePair {
+    int i[2];     // query tiles (i[0] = i[1] - 1)
+    int j_begin;  // first key tile; tile t attends key tiles [j_begin, i[t]]
+    int n[2];     // key tiles each attends: n[1] = n[0] + 1, n[0] = 0 when there is no second tile
+};
+__host__ __device__ inline TilePair tile_pair(const GroupLayout& L, int rank) {
+    int lo = 0, hi = L.nTiles;  // tiles [lo, hi) hold this pair
+    if (L.cut > 0) {
+        const int upper = (L.nTiles - L.cut + 1) / 2;
+        if (rank < upper) lo = L.cut;
+        else hi = L.cut, rank -= upper;
+    }
+    TilePair t;
+    t.j_begin = lo;
+    t.i[1] = hi - 1 - 2 * rank;
+    t.i[0] = t.i[1] - 1;
+    t.n[1] = t.i[1] + 1 - lo;
+    t.n[0] = t.i[0] + 1 - lo;  // 0 when i[1] is the first tile of its range
+    return t;
+}
+
 struct alignas(64) FwdParams {
     CUtensorMap tm_q;  // bf16 (d, H,   N, B), box (64, 1, 128, 1), 128-byte swizzle
     CUtensorMap tm_k;  // bf16 (d, Hkv, N, B), same box
     CUtensorMap tm_v;
+    CUtensorMap tm_o;  // like tm_q, for the stores of whole tiles
     __nv_bfloat16* o;
     float* lse;
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
-    float scale_log2;  // softmax scale * log2(e)
+    int pairs_per_group;  // largest number of query tile pairs any group has
+    float scale_log2;     // softmax scale * log2(e)
 };
 
 struct PreParams {

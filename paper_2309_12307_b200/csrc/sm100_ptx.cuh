@@ -88,10 +88,22 @@ __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, 
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
     return mbar_wait_limit(bar, parity, ctx, where, kWaitLimitCycles);
 }
-// All 32 lanes wait; the outcome is made warp-uniform so the warp can keep executing warp-wide
-// instructions (or leave its loop) together.
+// All 32 lanes wait; the outcome is warp-uniform, so the warp can keep executing warp-wide
+// instructions (or leave its loop) together.  The vote comes first and decides the branch: a wait that
+// each lane branches on by itself costs the warp about 200 clocks even when the phase is complete.
 __device__ __forceinline__ bool mbar_wait_uniform(uint64_t* bar, uint32_t parity, const WaitCtx& ctx, int where) {
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, ctx, where) ? 1 : 0) != 0;
+    if (__builtin_expect(__all_sync(0xffffffffu, mbar_try_wait(bar, parity) ? 1 : 0), 1)) return true;
+    const long long t0 = clock64();
+    for (uint32_t spins = 1;; ++spins) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity) ? 1 : 0)) return true;
+        if ((spins & 63u) == 0) {
+            if (__any_sync(0xffffffffu, *ctx.abort_flag != 0)) return false;
+            if (__any_sync(0xffffffffu, clock64() - t0 > kWaitLimitCycles)) {
+                report_expiry(ctx, where);
+                return false;
+            }
+        }
+    }
 }
 // One lane of a fully active warp (the same lane every time for a given warp).
 __device__ __forceinline__ bool elect_one() {
@@ -104,6 +116,12 @@ __device__ __forceinline__ bool elect_one() {
         "}\n"
         : "=r"(pred));
     return pred != 0;
+}
+
+// One arrival on behalf of a whole warp, after everything its lanes did before.
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* bar) {
+    __syncwarp();
+    if (elect_one()) mbar_arrive(bar);
 }
 
 // Teardown helper for an aborting CTA: wait (time-limited, ignoring the abort flag) for an
@@ -136,6 +154,84 @@ __device__ __forceinline__ void bulk_load_1d(void* smem_dst, const void* gmem_sr
                      smem_u32(smem_dst)),
                  "l"(gmem_src), "r"(bytes), "r"(smem_u32(bar))
                  : "memory");
+}
+
+// 4-D tiled store shared -> global; ordered after this thread's writes by fence_proxy_async().
+__device__ __forceinline__ void tma_store_4d(const CUtensorMap* tmap, const void* smem_src, int c0, int c1, int c2, int c3) {
+    asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%2, %3, %4, %5}], [%1];" ::"l"(tmap),
+                 "r"(smem_u32(smem_src)), "r"(c0), "r"(c1), "r"(c2), "r"(c3)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit_group() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+// all but the newest kLeft bulk stores this thread committed have read their shared memory
+template <int kLeft>
+__device__ __forceinline__ void bulk_wait_read() {
+    asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kLeft) : "memory");
+}
+// every bulk store this thread committed has completed
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+// make this thread's shared-memory writes visible to the asynchronous proxy
+__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// barrier over `threads` threads (whole warps), other than __syncthreads()
+__device__ __forceinline__ void named_barrier(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+// the same, and whether `ok` holds for every thread of it
+__device__ __forceinline__ bool named_barrier_and(int id, int threads, bool ok) {
+    uint32_t all;
+    asm volatile(
+        "{\n"
+        ".reg .pred p, q;\n"
+        "setp.ne.u32 p, %3, 0;\n"
+        "bar.red.and.pred q, %1, %2, p;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n"
+        : "=r"(all)
+        : "r"(id), "r"(threads), "r"(ok ? 1u : 0u)
+        : "memory");
+    return all != 0;
+}
+
+// ---------------------------------------------------------------------------------------------
+// Work stealing between the blocks of a grid (cluster launch control)
+// ---------------------------------------------------------------------------------------------
+// Ask for a block of this grid that has not been launched yet: the 16-byte answer lands in `resp` and
+// is counted on `bar` (expect 16 bytes).  A block that was granted will not be launched: the asking
+// block does its work.
+__device__ __forceinline__ void clc_try_cancel(void* resp, uint64_t* bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                     smem_u32(resp)),
+                 "r"(smem_u32(bar))
+                 : "memory");
+}
+// Block index (x) of the granted block, or -1: nothing is left, and no further request may be made.
+__device__ __forceinline__ int clc_granted_block(const void* resp) {
+    uint32_t ok, x = 0;
+    asm volatile(
+        "{\n"
+        ".reg .b128 h;\n"
+        ".reg .pred p;\n"
+        "ld.shared.b128 h, [%2];\n"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "mov.u32 %1, 0;\n"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n"
+        "}\n"
+        : "=r"(ok), "=r"(x)
+        : "r"(smem_u32(resp))
+        : "memory");
+    return ok ? static_cast<int>(x) : -1;
+}
+
+// Registers per thread of the executing warpgroup.  The shares of a block's warpgroups must not add up
+// to more than the block was launched with.
+template <int kRegs>
+__device__ __forceinline__ void setmaxnreg_inc() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs));
+}
+template <int kRegs>
+__device__ __forceinline__ void setmaxnreg_dec() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -320,6 +416,11 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar) {
 __device__ __forceinline__ float fast_exp2(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float fmax3(float a, float b, float c) {
+    float y;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(y) : "f"(a), "f"(b), "f"(c));
     return y;
 }
 // Packed fp32 pairs (one 64-bit register pair, one instruction for two lanes of arithmetic):
