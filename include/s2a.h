@@ -90,9 +90,9 @@ int s2a_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
  *   in : q, k, v, o, lse (o and lse exactly as s2a_fwd produced them), dO
  *   out: dq, dk, dv (overwritten, not accumulated into)
  *   workspace: caller-owned device scratch of at least s2a_bwd_workspace_bytes(...) bytes,
- *              256-byte aligned; holds D[b,h,t] = dO[b,t,h,:] . o[b,t,h,:] in fp32, the work counters of
- *              the persistent kernels and, if it is large enough, the spilled dS (below).  Its contents
- *              before the call do not matter; calls that can overlap on the GPU need a workspace each.
+ *              256-byte aligned; holds D[b,h,t] = dO[b,t,h,:] . o[b,t,h,:] in fp32, 256 reserved bytes and,
+ *              if it is large enough, the spilled dS (below).  Its contents before the call do not
+ *              matter; calls that can overlap on the GPU need a workspace each.
  * dk and dv sum over the H/Hkv query heads that share a KV head inside one thread block, and every dq
  * row is summed by one thread block in a fixed order, so the results are deterministic (no atomics).
  *
@@ -104,7 +104,7 @@ int s2a_fwd(const void* q, const void* k, const void* v, void* o, float* lse,
  *     the very values it multiplies with q) in the workspace and dq = scale * dS k is a plain product
  *     that reads them back: nothing is computed twice, at the price of 2 bytes of scratch per attended
  *     pair, written once and read once.  If the workspace holds the dS of only some of the KV heads,
- *     the KV heads are worked off in several passes (two launches and one 4-byte memset per pass).
+ *     the KV heads are worked off in several passes (two launches per pass).
  *   dk and dv are bit-identical either way; dq agrees to rounding (the fp32 sums inside the score
  *   products run in a different order).
  */
@@ -179,9 +179,8 @@ int s2a_bwd_packed(const void* qkv, const void* o, const float* lse, const void*
  * initialisation.  s2a_bwd wants a workspace from such a caller; this variant does not.
  *
  * It computes exactly what s2a_bwd computes with a minimum workspace (same kernels, same results), but keeps
- * D = rowsum(dO * o) and the work counter of its persistent kernel in an array that is part of the
- * library image: 2^20 fp32 values and 256 bytes (4 MiB in all) on every GPU that loads the library,
- * held until the process exits.  It calls no allocation routine of any kind.
+ * D = rowsum(dO * o) in an array that is part of the library image: 2^20 fp32 values and 256 reserved
+ * bytes (4 MiB in all) on every GPU that loads the library, held until the process exits.  It calls no allocation routine of any kind.
  *
  *   Limit     : B * H * N <= s2a_bwd_noalloc_max_rows() (= 1,048,576; e.g. B=1, H=32, N=32768).
  *               Larger problems return S2A_ERR_TOO_LARGE and enqueue nothing; use s2a_bwd.
@@ -192,8 +191,7 @@ int s2a_bwd_packed(const void* qkv, const void* o, const float* lse, const void*
  *               or different host threads on different streams) overwrite each other's D and
  *               give wrong gradients: serialise them, or use s2a_bwd with separate workspaces.
  *   Contents  : the array keeps whatever the previous call left; every value of D a call reads is
- *               first rewritten by that same call, and the work counter is set to zero by a 4-byte
- *               memset on `stream` ahead of the kernel that counts with it, so the caller clears nothing.
+ *               first rewritten by that same call, so the caller clears nothing.
  * Other arguments, shapes, errors and the meaning of `stream` are those of s2a_bwd.
  */
 int s2a_bwd_noalloc(const void* q, const void* k, const void* v, const void* o, const float* lse, const void* dO,

@@ -37,7 +37,6 @@ struct DeviceState {
     int* status_ptr = nullptr;        // device address of g_status_word
     volatile int* host_word = nullptr;  // this device's mirror, host address
     int* host_word_dev = nullptr;     // the same word as the device sees it
-    int n_sm = 0;                     // multiprocessors (grid of the persistent kernel)
     // s2a_fwd_bwd_host only: copy streams and the events that order them against the caller's stream
     bool host_path_ready = false;
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
@@ -71,8 +70,6 @@ int prepare_device(DeviceState** out) {
         e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
         if (e != cudaSuccess) return cuda_fail(e);
         if (major != 10) return S2A_ERR_UNSUPPORTED;
-        e = cudaDeviceGetAttribute(&ds.n_sm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return cuda_fail(e);
         if (!g_encode) {
             void* fn = nullptr;
             cudaDriverEntryPointQueryResult qres;
@@ -293,9 +290,9 @@ int s2a_fwd(const void* q, const void* k, const void* v, void* o, float* lse, in
 }
 
 namespace {
-// Workspace layout: D [B, H, N] fp32 padded to 256 bytes, 256 bytes of work counters for the persistent
-// kernels (together the minimum), then the spill area.
-constexpr size_t kCounterBytes = 256;
+// Workspace layout: D [B, H, N] fp32 padded to 256 bytes, 256 reserved bytes (together the minimum; the
+// sizes callers were told stay what they were), then the spill area.
+constexpr size_t kReservedBytes = 256;
 size_t d_bytes(int B, int N, int H) {
     return (static_cast<size_t>(B) * H * N * sizeof(float) + 255) & ~static_cast<size_t>(255);
 }
@@ -304,7 +301,7 @@ size_t d_bytes(int B, int N, int H) {
 size_t s2a_bwd_workspace_bytes(int B, int N, int H, int Hkv, int d, int G) {
     if (B <= 0 || N <= 0 || H <= 0 || Hkv <= 0 || d <= 0 || G <= 0) return 0;
     if (N % G != 0 || H % Hkv != 0) return 0;
-    return d_bytes(B, N, H) + kCounterBytes;
+    return d_bytes(B, N, H) + kReservedBytes;
 }
 
 namespace {
@@ -368,6 +365,8 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     if ((rc = make_tmap(&pk.tm_v, v, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
     if ((rc = make_tmap(&pk.tm_q, q, d, H, N, B, kSubTile, ts.q)) != S2A_OK) return rc;
     if ((rc = make_tmap(&pk.tm_do, dO, d, H, N, B, kSubTile)) != S2A_OK) return rc;
+    if ((rc = make_tmap(&pk.tm_dk, dk, d, Hkv, N, B, 32, ts.dkv)) != S2A_OK) return rc;
+    if ((rc = make_tmap(&pk.tm_dv, dv, d, Hkv, N, B, 32, ts.dkv)) != S2A_OK) return rc;
     pk.dkv_tok_stride = ts.dkv ? ts.dkv : static_cast<long long>(Hkv) * d;
     pk.lse = lse, pk.Dsum = Dsum;
     pk.dk = static_cast<__nv_bfloat16*>(dk), pk.dv = static_cast<__nv_bfloat16*>(dv);
@@ -392,8 +391,6 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     if (stages != kStageAll && nk_fit < static_cast<size_t>(Hkv)) nk_fit = 0;
 
     char* base = static_cast<char*>(workspace);
-    int* counters = reinterpret_cast<int*>(base + d_bytes(B, N, H));  // [0] dK,dV kernel, [1] dQ-from-spill kernel
-    pk.counter = counters;
     cudaError_t e;
     if (stages & kStagePre) {
         e = launch_bwd_preprocess(pp, d, st);
@@ -401,9 +398,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     }
     if (nk_fit == 0) {
         if (stages & kStageDkDv) {
-            e = cudaMemsetAsync(counters, 0, sizeof(int), st);
-            if (e != cudaSuccess) return cuda_fail(e);
-            e = launch_bwd_dkdv(pk, d, ds->n_sm, st);
+            e = launch_bwd_dkdv(pk, d, st);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         if (stages & kStageDq) {
@@ -417,23 +412,21 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     BwdDqSpillParams ps;
     memset(&ps, 0, sizeof ps);
     ps.tm_k = pq.tm_k;
+    if ((rc = make_tmap(&ps.tm_dq, dq, d, H, N, B, 32, ts.dq)) != S2A_OK) return rc;
+    ps.pairs_per_group = most_pairs(geo);
     ps.spill = pk.spill;
-    ps.dq = pq.dq, ps.dq_tok_stride = pq.dq_tok_stride, ps.counter = counters + 1;
+    ps.dq = pq.dq, ps.dq_tok_stride = pq.dq_tok_stride;
     ps.status = ds->status_ptr, ps.host_status = ds->host_word_dev, ps.geo = geo, ps.scale = scale;
     for (int hk0 = 0; hk0 < Hkv; hk0 += static_cast<int>(nk_fit)) {
         const int nk = Hkv - hk0 < static_cast<int>(nk_fit) ? Hkv - hk0 : static_cast<int>(nk_fit);
         pk.pass.hk0 = hk0, pk.pass.nk = nk;
         ps.pass = pk.pass;
         if (stages & kStageDkDv) {
-            e = cudaMemsetAsync(counters, 0, sizeof(int), st);
-            if (e != cudaSuccess) return cuda_fail(e);
-            e = launch_bwd_dkdv(pk, d, ds->n_sm, st);
+            e = launch_bwd_dkdv(pk, d, st);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         if (stages & kStageDq) {
-            e = cudaMemsetAsync(counters + 1, 0, sizeof(int), st);
-            if (e != cudaSuccess) return cuda_fail(e);
-            e = launch_bwd_dq_spill(ps, d, ds->n_sm, st);
+            e = launch_bwd_dq_spill(ps, d, st);
             if (e != cudaSuccess) return cuda_fail(e);
         }
     }
@@ -610,11 +603,11 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
 // ---------------------------------------------------------------------------------------------
 namespace {
 
-// Built-in home for D = rowsum(dO * o) and the work counters when the caller cannot provide a
-// workspace: 2^20 fp32 rows and 256 bytes (4 MiB in all), which every GPU that loads this library keeps
+// Built-in home for D = rowsum(dO * o) when the caller cannot provide a workspace: 2^20 fp32 rows and
+// the reserved bytes of a workspace (4 MiB in all), which every GPU that loads this library keeps
 // resident until the process exits.
 constexpr size_t kBuiltinScratchRows = size_t(1) << 20;
-static __device__ __align__(256) float g_builtin_scratch[kBuiltinScratchRows + kCounterBytes / sizeof(float)];
+static __device__ __align__(256) float g_builtin_scratch[kBuiltinScratchRows + kReservedBytes / sizeof(float)];
 
 // In host code `g_builtin_scratch` is only a handle for the runtime, not an address a kernel may
 // use; the device address is looked up once per device, with that device current.
@@ -649,10 +642,9 @@ int s2a_bwd_noalloc(const void* q, const void* k, const void* v, const void* o, 
     const int rc = builtin_scratch(&scratch);
     if (rc != S2A_OK) return rc;
     // Every row of D that the two gradient kernels read is rewritten by the first kernel of this
-    // call and the work counter is cleared by a memset ahead of its kernel, so nothing left in the
-    // array by an earlier call matters.
+    // call, so nothing left in the array by an earlier call matters.
     return bwd_impl(q, k, v, o, lse, dO, dq, dk, dv, B, N, H, Hkv, d, G, 1.0f / sqrtf(static_cast<float>(d)), H / 2,
-                    G / 2, scratch, kBuiltinScratchRows * sizeof(float) + kCounterBytes, stream, kStageAll, 0u, TokStrides(), false);
+                    G / 2, scratch, kBuiltinScratchRows * sizeof(float) + kReservedBytes, stream, kStageAll, 0u, TokStrides(), false);
 }
 
 size_t s2a_bwd_noalloc_max_rows(void) { return kBuiltinScratchRows; }

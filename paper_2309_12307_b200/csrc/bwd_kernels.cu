@@ -18,11 +18,12 @@
 // The roll of the shifted heads and the group boundaries are folded into TMA coordinates exactly
 // as in the forward kernel; all results are stored at original token rows.
 //
-// Kernels 2 and 3 use the same warp roles (384 threads, one CTA per SM, all 512 tensor-memory columns):
+// Kernels 2 and 3 share their warp roles (one CTA per SM, all 512 tensor-memory columns):
 // warp 0 loads with TMA; warp 1 issues the score MMAs and warp 2 the gradient MMAs (a single issuing
 // warp spends so long on its own barrier waits that the tensor pipe runs dry in between; with two, one
-// can issue while the other waits); warp 3 owns the tensor-memory allocation; warps 4-11 do the
-// elementwise work with one tensor-memory lane and half of the columns per thread.  dP (dP^T) has a
+// can issue while the other waits); warp 3 owns the tensor-memory allocation (and loads K and V in kernel
+// 3); warps 4-11 do the elementwise work with one tensor-memory lane and half of the columns per thread;
+// kernel 3 has four more warps that write finished accumulators out.  dP (dP^T) has a
 // single buffer: the elementwise warps copy their part of it into registers and release it at once,
 // which leaves the columns for two score buffers (and, in kernel 3, for K as a tensor-memory operand),
 // so that the score products of the next step run while the elementwise warps work on the current one.
@@ -36,8 +37,9 @@ namespace {
 constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ int mod_pos(int x, int n) {
-    int r = x % n;
-    return r < 0 ? r + n : r;
+    // x in (-n, 2 n)
+    if (x < 0) x += n;
+    return x >= n ? x - n : x;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -76,11 +78,11 @@ __global__ void __launch_bounds__(256) s2a_bwd_preprocess_kernel(const PreParams
 }
 
 // ------------------------------------------------------------------------------------------------
-// shared configuration of the two tensor-core kernels
+// configuration of the dK,dV kernel, accumulator read-out
 // ------------------------------------------------------------------------------------------------
 template <int HD>
 struct BwdCfg {
-    static constexpr int kThreads = 384;  // TMA warp, two MMA warps, one spare, 8 elementwise warps
+    static constexpr int kThreads = 512;  // 4 load and issue warps, 8 elementwise warps, 4 epilogue warps
     static constexpr int kBoxes = HD / 64;
     static constexpr int kBigBoxBytes = kTile * 128;            // 128-row box
     static constexpr int kSubBoxBytes = kSubTile * 128;         // 64-row box
@@ -89,11 +91,15 @@ struct BwdCfg {
     static constexpr int kStages = 4;
     static constexpr int kStatBytes = kSubTile * 4;             // lse or D of one streamed tile
     static constexpr int kStageBytes = 2 * kSubTileBytes;       // two streamed operands per stage
-    static constexpr int kBarBytes = 512;
-    static constexpr int kNeeded = 1024 + 2 * kBigTileBytes + kStages * kStageBytes + kStages * 2 * kStatBytes + kBarBytes;
+    static constexpr int kOutBytes = 4 * 2 * 4096;              // two staging buffers for each epilogue warp
+    static constexpr int kBarBytes = 1024;
+    static constexpr int kNeeded = 2 * kBigTileBytes + kStages * kStageBytes + kOutBytes + kStages * 2 * kStatBytes + kBarBytes;
     // at least 120 KB so that only one CTA fits on an SM: each CTA allocates all of tensor memory
     static constexpr int kSmemBytes = kNeeded > 120 * 1024 ? kNeeded : 120 * 1024;
     static constexpr int kTmemCols = 512;
+    // registers per thread after the split; the launch gives kRegsLaunch to each of the 512
+    static constexpr int kRegsLaunch = 128, kRegsElem = 152, kRegsOther = 104;
+    static_assert(2 * kRegsElem + 2 * kRegsOther <= 4 * kRegsLaunch, "register split");
 };
 
 // Store COLS consecutive fp32 accumulator columns of this thread's tensor-memory lane (times `mul`)
@@ -114,6 +120,57 @@ __device__ __forceinline__ void store_acc_cols(uint32_t t_addr, float mul, __nv_
             pk.z = pack_bf16(__uint_as_float(r[8 * e + 4]) * mul, __uint_as_float(r[8 * e + 5]) * mul);
             pk.w = pack_bf16(__uint_as_float(r[8 * e + 6]) * mul, __uint_as_float(r[8 * e + 7]) * mul);
             if (row_valid) dst[e] = pk;
+        }
+    }
+}
+
+// Write 32 accumulator rows of HD columns (times `mul`) as bf16: this warp's tensor-memory lanes at
+// `t_addr` go to tokens tok0 .. tok0+31 of `head`, 64 columns at a time through the warp's staging buffers
+// (2 x 4 KB of shared memory at `stage`, `used` counts their uses) and a TMA store.  Storing 16 bytes a lane
+// straight to rows that lie heads * d apart touches 32 lines with every instruction, 4096 clocks for
+// a 128 x 256 tile.  Only the first `valid` rows exist; rows of a ragged tile are stored directly
+// (`row_ptr`: this lane's row).  `tm`: box (64, 1, 32, 1).  `done()` runs when the accumulator has been read.
+template <int HD, typename Done>
+__device__ __forceinline__ void store_acc_rows(const CUtensorMap* tm, uint8_t* stage, uint32_t& used, uint32_t t_addr, float mul,
+                                               __nv_bfloat16* row_ptr, int head, int tok0, int b, int valid, Done done) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int c = 0; c < HD / 64; ++c) {
+        uint32_t r[64];
+        tmem_ld_32x32(t_addr + c * 64, *reinterpret_cast<uint32_t(*)[32]>(&r[0]));
+        tmem_ld_32x32(t_addr + c * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&r[32]));
+        tmem_wait_ld();
+        if (c == HD / 64 - 1) done();
+        uint8_t* buf = stage + (used & 1) * 4096;
+        if (valid >= 32) {
+            if (lane == 0) bulk_wait_read<1>();  // the store before the last one has left this buffer
+            __syncwarp();
+        }
+        const uint32_t dst_s = smem_u32(buf) + lane * 128;
+        uint4* dst_g = reinterpret_cast<uint4*>(row_ptr + c * 64);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            uint4 pk;
+            pk.x = pack_bf16(__uint_as_float(r[8 * e + 0]) * mul, __uint_as_float(r[8 * e + 1]) * mul);
+            pk.y = pack_bf16(__uint_as_float(r[8 * e + 2]) * mul, __uint_as_float(r[8 * e + 3]) * mul);
+            pk.z = pack_bf16(__uint_as_float(r[8 * e + 4]) * mul, __uint_as_float(r[8 * e + 5]) * mul);
+            pk.w = pack_bf16(__uint_as_float(r[8 * e + 6]) * mul, __uint_as_float(r[8 * e + 7]) * mul);
+            if (valid >= 32) {
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst_s + ((e ^ (lane & 7)) << 4)), "r"(pk.x), "r"(pk.y),
+                             "r"(pk.z), "r"(pk.w)
+                             : "memory");
+            } else if (lane < valid) {
+                dst_g[e] = pk;
+            }
+        }
+        if (valid >= 32) {
+            fence_proxy_async();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_4d(tm, buf, c * 64, head, tok0, b);
+                bulk_commit_group();
+            }
+            ++used;
         }
     }
 }
@@ -142,7 +199,7 @@ struct DqCfg {
     static constexpr int kRingK = 3;
     static constexpr int kRingV = 2;
     static constexpr int kBarBytes = 512;
-    static constexpr int kNeeded = 1024 + (2 + kRingK + kRingV) * kTileBytes + kBarBytes;
+    static constexpr int kNeeded = (2 + kRingK + kRingV) * kTileBytes + kBarBytes;
     // at least 120 KB so that only one CTA fits on an SM: each CTA allocates all of tensor memory
     static constexpr int kSmemBytes = kNeeded > 120 * 1024 ? kNeeded : 120 * 1024;
     static constexpr int kTmemCols = 512;
@@ -166,8 +223,8 @@ struct DqBars {
 template <int HD>
 __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(const __grid_constant__ BwdDqParams p) {
     using C = DqCfg<HD>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = smem_raw;                          // 1024-byte aligned: nothing precedes the dynamic array
     uint8_t* sQ = smem;                                // resident: Q_i
     uint8_t* sDO = sQ + C::kTileBytes;                 // resident: dO_i
     uint8_t* sK = sDO + C::kTileBytes;                 // ring of K tiles
@@ -179,10 +236,10 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
 
     // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
     // then return at once instead of each running into its own time limit.
-    __shared__ int s_poisoned;
-    if (threadIdx.x == 0) s_poisoned = *reinterpret_cast<volatile int*>(p.status);
+    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
     __syncthreads();
-    if (s_poisoned != 0) return;
+    if (bars->abort_flag != 0) return;
+    __syncthreads();
     const Geometry& geo = p.geo;
 
     const int Tg = geo.tiles_per_group;
@@ -207,10 +264,10 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->drain2, 1);
         mbar_init(&bars->dp_ready, 1);
-        mbar_init(&bars->dp_free, 256);
+        mbar_init(&bars->dp_free, 8);  // one arrival per elementwise warp
         for (int x = 0; x < 2; ++x) {
             mbar_init(&bars->s_ready[x], 1);
-            mbar_init(&bars->p_full[x], 256);
+            mbar_init(&bars->p_full[x], 8);
             mbar_init(&bars->buf_free[x], 1);
             mbar_init(&bars->v_full[x], 1);
             mbar_init(&bars->v_empty[x], 1);
@@ -374,19 +431,19 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
         // n+1 at the END of step n (dP_{n+1} has been complete for a long time by then), so that dP_{n+2}
         // and S_{n+2} can be issued while step n+1 is still being worked on.
         auto fetch_dp = [&](int m) -> bool {
-            if (!mbar_wait(&bars->dp_ready, m & 1, ctx, kWaitBwdDq + 5)) return false;
+            if (!mbar_wait_uniform(&bars->dp_ready, m & 1, ctx, kWaitBwdDq + 5)) return false;
             tc_fence_after();
             tmem_ld_32x32(t_row + kColP + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&dp[0]));
             tmem_ld_32x32(t_row + kColP + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&dp[32]));
             tmem_wait_ld();
             tc_fence_before();
-            mbar_arrive(&bars->dp_free);
+            mbar_arrive_warp(&bars->dp_free);
             return true;
         };
         ok = fetch_dp(0);
         for (int n = 0; ok && n < n_steps; ++n) {
             const int st = n & 1;
-            if (!mbar_wait(&bars->s_ready[st], (n >> 1) & 1, ctx, kWaitBwdDq + 11)) { ok = false; break; }
+            if (!mbar_wait_uniform(&bars->s_ready[st], (n >> 1) & 1, ctx, kWaitBwdDq + 11)) { ok = false; break; }
             tc_fence_after();
             // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
             // in the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
@@ -433,7 +490,7 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
             }
             tmem_wait_st();
             tc_fence_before();
-            mbar_arrive(&bars->p_full[st]);
+            mbar_arrive_warp(&bars->p_full[st]);
             if (n + 1 < n_steps && !fetch_dp(n + 1)) { ok = false; break; }
         }
         if (ok && mbar_wait(&bars->acc_full, 0, ctx, kWaitBwdDq + 6)) {
@@ -476,7 +533,7 @@ __device__ __forceinline__ HeadWalk head_walk(const Geometry& geo, int hq, int t
     const int pos = mod_pos(tk0 - s, geo.N);
     w.g = pos / geo.G;
     w.L = group_layout(geo, s, w.g);
-    const int in_group = pos % geo.G;
+    const int in_group = pos - w.g * geo.G;
     const int nB = w.L.nTiles - w.L.nA;
     w.j = in_group < w.L.lenA ? (w.L.swapped ? nB : 0) + in_group / kTile
                               : (w.L.swapped ? 0 : w.L.nA) + (in_group - w.L.lenA) / kTile;
@@ -515,37 +572,44 @@ __device__ __forceinline__ DkDvItem dkdv_item(const Geometry& geo, const SpillPa
     return t;
 }
 
-// Barriers of the persistent dK,dV kernel.  Steps are counted through all items of the CTA (`it`), so
-// the rings of stages and score buffers simply carry on from one item to the next.
+// Barriers of the dK,dV kernel.  Steps are counted through all items of the CTA (`it`), so the rings of
+// stages and score buffers simply carry on from one item to the next.
 template <int kStages>
 struct DkDvBars {
-    uint64_t res_full;            // K and V of an item landed (one phase per item)
+    uint64_t k_full, v_full;      // K / V of an item landed (one phase per item)
     uint64_t kt_full;             // K of an item has been copied into tensor memory
-    uint64_t kv_empty;            // the score products of an item are done: K and V may be overwritten
+    uint64_t v_empty;             // the dP^T products of an item are done: V may be overwritten
+    uint64_t s_done;              // all score products of an item are done: the copy of K may be overwritten
     uint64_t acc_full;            // all gradient MMAs of an item are done
     uint64_t acc_empty;           // the accumulators of an item have been read out
     uint64_t drain;               // abort path only (gradient MMA warp)
     uint64_t drain2;              // abort path only (score MMA warp)
-    uint64_t s_full[3];           // S^T of a step is in tensor memory (buffer it % 3)
-    uint64_t p_full[3];           // bf16 P^T and dS^T of a step are in tensor memory
-    uint64_t buf_free[3];         // gradient MMAs that read a score buffer's bf16 operands are done
+    uint64_t s_full[2];           // S^T (and dP^T) of a step is in tensor memory (buffer it % 2)
+    uint64_t p_full[2];           // bf16 P^T and dS^T of a step are in tensor memory
+    uint64_t buf_free[2];         // gradient MMAs that read a score buffer's bf16 operands are done
     uint64_t dp_free;             // the elementwise threads of a step hold their dP^T in registers
     uint64_t st_full[kStages];    // streamed operands of a stage landed
     uint64_t st_empty[kStages];   // MMAs reading a stage are done
-    uint64_t sched_full[8];       // a work item id has been published
-    long long item[8];
+    uint64_t sched_full[8];       // a work item has been published
+    uint64_t clc;
+    alignas(16) uint8_t clc_resp[16];
+    DkDvItem item[8];             // total_steps = 0: no more items
     uint32_t tmem_slot;
     int abort_flag;
 };
 
 // kSpill: every step's dS^T also goes to global memory (see SpillPass) for s2a_bwd_dq_spill_kernel.
 //
-// Persistent: one CTA per SM draws key tiles, heaviest first, from a counter in global memory.  The TMA
-// warp runs ahead across items (the K and V of the next item are fetched as soon as the last score
-// product of the current one has been issued and completed, its first query sub-tiles right behind),
-// so that barrier set-up, tensor-memory allocation, the first loads and the pipeline fill are paid
-// once per SM instead of once per key tile, and the score products of the next item run while the
-// accumulators of the finished one are written out.
+// Persistent: one CTA per SM takes over key tiles, heaviest first, by cluster launch control.  Everything
+// that belongs to the change from one item to the next runs beside the steps: the ids and the streamed
+// tiles are requested ahead (warp 0); K of the next item is loaded as soon as the current one has been
+// copied to tensor memory, V as soon as the last dP^T product is done (warp 3); the copy of K and the
+// read-out of the accumulators have four warps of their own, so that the elementwise warps go straight on
+// with the next item's first steps.  With the elementwise warps doing it and every warp decoding the item
+// for itself (64-bit divisions, one after the other), the change of item cost 10,000 to 17,000 clocks, as
+// much as ten steps.  Before and after, spilling form, us a launch in a loop: Llama2-7B 8k 354 and 325, 4 x 2048
+// tokens with groups of 512 178 and 146, 4 x 2000 with groups of 200 (head size 64) 53 and 43, 32k 4380 and 4290
+// (there the part is at its power limit).
 template <int HD, bool kSpill>
 __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(const __grid_constant__ BwdDkDvParams p) {
     using C = BwdCfg<HD>;
@@ -554,12 +618,13 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     constexpr int kCols = 32;  // query columns per elementwise thread and step: two threads share a key row
     constexpr int kChunks = kCols / 16;
     constexpr int kSched = 8;  // item ids in flight: the TMA warp is at most five items ahead of the read-out
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = smem_raw;                          // 1024-byte aligned: nothing precedes the dynamic array
     uint8_t* sK = smem;                                // resident: K_j
     uint8_t* sV = sK + C::kBigTileBytes;               // resident: V_j
     uint8_t* sStage = sV + C::kBigTileBytes;           // per stage: Q_n then dO_n
-    float* sStat = reinterpret_cast<float*>(sStage + C::kStages * C::kStageBytes);  // per stage: lse[64], D[64]
+    uint8_t* sOut = sStage + C::kStages * C::kStageBytes;  // staging buffers of the epilogue warps
+    float* sStat = reinterpret_cast<float*>(sOut + C::kOutBytes);  // per stage: lse[64], D[64]
     Bars* bars = reinterpret_cast<Bars*>(reinterpret_cast<uint8_t*>(sStat) + C::kStages * 2 * C::kStatBytes);
     static_assert(sizeof(Bars) <= C::kBarBytes, "barrier block");
 
@@ -568,21 +633,23 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
 
     // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
     // then return at once instead of each running into its own time limit.
-    __shared__ int s_poisoned;
-    if (threadIdx.x == 0) s_poisoned = *reinterpret_cast<volatile int*>(p.status);
+    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
     __syncthreads();
-    if (s_poisoned != 0) return;
+    if (bars->abort_flag != 0) return;
+    __syncthreads();
     const Geometry& geo = p.geo;
     const int rep = geo.H / geo.Hkv;
     const int Tg = geo.tiles_per_group;
-    const long long n_items = static_cast<long long>(geo.B) * p.pass.nk * geo.groups * Tg;
 
     if (threadIdx.x == 0) {
-        mbar_init(&bars->res_full, 1);
-        mbar_init(&bars->kt_full, 256);
-        mbar_init(&bars->kv_empty, 1);
+        // hand-offs by whole warps count one arrival per warp
+        mbar_init(&bars->k_full, 1);
+        mbar_init(&bars->v_full, 1);
+        mbar_init(&bars->kt_full, 4);
+        mbar_init(&bars->v_empty, 1);
+        mbar_init(&bars->s_done, 1);
         mbar_init(&bars->acc_full, 1);
-        mbar_init(&bars->acc_empty, 256);
+        mbar_init(&bars->acc_empty, 4);
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->drain2, 1);
         for (int x = 0; x < kBufs; ++x) {
@@ -596,12 +663,15 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             mbar_init(&bars->st_empty[st], 1);
         }
         for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
+        mbar_init(&bars->clc, 1);
         bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
         tma_prefetch_desc(&p.tm_do);
         tma_prefetch_desc(&p.tm_k);
         tma_prefetch_desc(&p.tm_v);
+        tma_prefetch_desc(&p.tm_dk);
+        tma_prefetch_desc(&p.tm_dv);
     }
     if (warp == 3) {
         tmem_alloc(&bars->tmem_slot, C::kTmemCols);
@@ -614,175 +684,201 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
     constexpr uint32_t kColDV = 0, kColDK = 128, kColS = 256, kColP = 384, kColKt = 448;
 
-    // Every consumer role walks the same sequence of items: wait for the k-th id, stop at the end marker.
-    auto next_item = [&](int k, int where, long long* id) -> bool {
-        if (!mbar_wait(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return false;
-        *id = bars->item[k % kSched];
-        return *id < n_items;
+    // Every consumer warp walks the same sequence of items, as the scheduling thread has decoded them (the
+    // divisions cost a warp more than a step): the k-th one, false = the end (or aborting).
+    auto next_item = [&](int k, int where, DkDvItem* t) -> bool {
+        if (!mbar_wait_uniform(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return false;
+        *t = bars->item[k % kSched];
+        return t->total_steps > 0;
     };
 
-    if (warp == 0) {
-        if (lane == 0) {
-            int it = 0;
-            int last_res = -1;  // newest item whose K and V were requested
-            bool ok = true;
-            for (int k = 0; ok; ++k) {
-                // draw the next item that has work; the other warps only see real items and the end marker
-                long long id;
-                DkDvItem t;
-                do {
-                    id = static_cast<long long>(atomicAdd(p.counter, 1));
-                    if (id >= n_items) break;
-                    t = dkdv_item(geo, p.pass, id);
-                } while (t.total_steps == 0);
-                bars->item[k % kSched] = id;
-                mbar_arrive(&bars->sched_full[k % kSched]);  // release: the id is visible to whoever sees the phase
-                if (id >= n_items) break;
-                // K and V of the item: their buffers are free once the score products of the previous item are done
-                if (k > 0 && !mbar_wait(&bars->kv_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 10)) break;
-                mbar_expect_tx(&bars->res_full, 2 * C::kBigTileBytes);
-                for (int bx = 0; bx < C::kBoxes; ++bx) {
-                    tma_load_4d(sK + bx * C::kBigBoxBytes, &p.tm_k, &bars->res_full, bx * 64, t.hk, t.tk0, t.b);
-                    tma_load_4d(sV + bx * C::kBigBoxBytes, &p.tm_v, &bars->res_full, bx * 64, t.hk, t.tk0, t.b);
-                }
-                last_res = k;
-                const int hq0 = t.hk * rep;
-                for (int hq = hq0; ok && hq < hq0 + rep; ++hq) {
-                    const HeadWalk w = head_walk(geo, hq, t.tk0);
-                    for (int n = w.n_begin; n < w.n_end; ++n, ++it) {
-                        const int st = it % C::kStages;
-                        const uint32_t ph = (it / C::kStages) & 1;
-                        const TileRef tq = subtile_ref(w.L, n);
-                        const int tq0 = tq.tok0;
-                        // statistics of the valid rows only (a multiple of 4 rows, so of 16 bytes): a ragged
-                        // sub-tile must not read past the end of the arrays
-                        const uint32_t stat_bytes = static_cast<uint32_t>(tq.valid) * 4u;
-                        if (!mbar_wait(&bars->st_empty[st], ph ^ 1, ctx, kWaitBwdDkDv + 1)) { ok = false; break; }
-                        mbar_expect_tx(&bars->st_full[st], C::kStageBytes + 2 * stat_bytes);
-                        uint8_t* sQ = sStage + st * C::kStageBytes;
-                        uint8_t* sDO = sQ + C::kSubTileBytes;
-                        for (int bx = 0; bx < C::kBoxes; ++bx) {
-                            tma_load_4d(sQ + bx * C::kSubBoxBytes, &p.tm_q, &bars->st_full[st], bx * 64, hq, tq0, t.b);
-                            tma_load_4d(sDO + bx * C::kSubBoxBytes, &p.tm_do, &bars->st_full[st], bx * 64, hq, tq0, t.b);
-                        }
-                        const size_t stat_idx = (static_cast<size_t>(t.b) * geo.H + hq) * geo.N + tq0;
-                        if (stat_bytes != 0) {
-                            bulk_load_1d(sStat + st * 2 * kSubTile, p.lse + stat_idx, stat_bytes, &bars->st_full[st]);
-                            bulk_load_1d(sStat + st * 2 * kSubTile + kSubTile, p.Dsum + stat_idx, stat_bytes, &bars->st_full[st]);
+    if (warp < 4) {
+        setmaxnreg_dec<C::kRegsOther>();
+        if (warp == 0) {
+            // ---- work items and streamed query sub-tiles
+            if (lane == 0) {
+                int it = 0;
+                bool ok = true;
+                ItemSource items{&bars->clc, bars->clc_resp};
+                int id = static_cast<int>(blockIdx.x);
+                for (int k = 0; ok; ++k) {
+                    // the next item that has work; the other warps only see real items and the end marker
+                    DkDvItem t;
+                    while (id >= 0 && (t = dkdv_item(geo, p.pass, id)).total_steps == 0) {
+                        id = items.next(ctx, kWaitBwdDkDv + 10, &ok);
+                    }
+                    if (id < 0) t.total_steps = 0;
+                    bars->item[k % kSched] = t;
+                    mbar_arrive(&bars->sched_full[k % kSched]);  // release: the item is visible to whoever sees the phase
+                    if (id < 0) break;
+                    const int hq0 = t.hk * rep;
+                    for (int hq = hq0; ok && hq < hq0 + rep; ++hq) {
+                        const HeadWalk w = head_walk(geo, hq, t.tk0);
+                        for (int n = w.n_begin; n < w.n_end; ++n, ++it) {
+                            const int st = it % C::kStages;
+                            const uint32_t ph = (it / C::kStages) & 1;
+                            const TileRef tq = subtile_ref(w.L, n);
+                            const int tq0 = tq.tok0;
+                            // statistics of the valid rows only (a multiple of 4 rows, so of 16 bytes): a ragged
+                            // sub-tile must not read past the end of the arrays
+                            const uint32_t stat_bytes = static_cast<uint32_t>(tq.valid) * 4u;
+                            if (!mbar_wait(&bars->st_empty[st], ph ^ 1, ctx, kWaitBwdDkDv + 1)) { ok = false; break; }
+                            mbar_expect_tx(&bars->st_full[st], C::kStageBytes + 2 * stat_bytes);
+                            uint8_t* sQ = sStage + st * C::kStageBytes;
+                            uint8_t* sDO = sQ + C::kSubTileBytes;
+                            for (int bx = 0; bx < C::kBoxes; ++bx) {
+                                tma_load_4d(sQ + bx * C::kSubBoxBytes, &p.tm_q, &bars->st_full[st], bx * 64, hq, tq0, t.b);
+                                tma_load_4d(sDO + bx * C::kSubBoxBytes, &p.tm_do, &bars->st_full[st], bx * 64, hq, tq0, t.b);
+                            }
+                            const size_t stat_idx = (static_cast<size_t>(t.b) * geo.H + hq) * geo.N + tq0;
+                            if (stat_bytes != 0) {
+                                bulk_load_1d(sStat + st * 2 * kSubTile, p.lse + stat_idx, stat_bytes, &bars->st_full[st]);
+                                bulk_load_1d(sStat + st * 2 * kSubTile + kSubTile, p.Dsum + stat_idx, stat_bytes, &bars->st_full[st]);
+                            }
                         }
                     }
+                    if (ok) id = items.next(ctx, kWaitBwdDkDv + 10, &ok);
+                }
+                if (bars->abort_flag != 0) {
+                    // let loads that are still in flight land before the CTA gives its memory back
+                    for (int nn = (it > C::kStages ? it - C::kStages : 0); nn < it; ++nn)
+                        mbar_wait_drain(&bars->st_full[nn % C::kStages], (nn / C::kStages) & 1);
                 }
             }
-            if (bars->abort_flag != 0) {
-                // let loads that are still in flight land before the CTA gives its memory back: K and V of
-                // the newest item and the stages issued last
-                if (last_res >= 0) mbar_wait_drain(&bars->res_full, last_res & 1);
-                for (int nn = (it > C::kStages ? it - C::kStages : 0); nn < it; ++nn)
-                    mbar_wait_drain(&bars->st_full[nn % C::kStages], (nn / C::kStages) & 1);
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ---- score MMAs of step `it`: dP^T = V dO^T into the single dP^T buffer (free as soon as the
-        // elementwise warps hold the previous one in registers), then S^T = K Q^T into buffer it % 3
-        // (warp-uniform loop, one elected lane issues; see the dQ kernel)
-        constexpr uint32_t idesc_sc = idesc_bf16(128, kSubTile, 0, 0);
-        const uint32_t dV = desc_lo_k_major(smem_u32(sV));
-        const uint32_t tP = tmem_base + kColP, tKt = tmem_base + kColKt;
-        int it = 0;
-        bool ok = true;
-        for (int k = 0; ok; ++k) {
-            long long id = n_items;
-            if (!__all_sync(0xffffffffu, next_item(k, kWaitBwdDkDv + 11, &id) ? 1 : 0)) break;  // warp-uniform outcome
-            const DkDvItem t = dkdv_item(geo, p.pass, id);
-            if (!mbar_wait_uniform(&bars->res_full, k & 1, ctx, kWaitBwdDkDv + 3)) break;
-            if (!mbar_wait_uniform(&bars->kt_full, k & 1, ctx, kWaitBwdDkDv + 16)) break;
-            for (int x = 0; x < t.total_steps; ++x, ++it) {
-                const int st = it % C::kStages;
-                const int bf = it % kBufs;
-                if (!mbar_wait_uniform(&bars->st_full[st], (it / C::kStages) & 1, ctx, kWaitBwdDkDv + 2)) { ok = false; break; }
-                if (it >= 1 && !mbar_wait_uniform(&bars->dp_free, (it - 1) & 1, ctx, kWaitBwdDkDv + 9)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
-                const uint32_t dQ = desc_lo_k_major(aQ), dDO = desc_lo_k_major(aQ + C::kSubTileBytes);
-                if (elect_one()) {
+            __syncwarp();
+        } else if (warp == 1) {
+            // ---- score MMAs of step `it`: dP^T = V dO^T into the single dP^T buffer (free as soon as the
+            // elementwise warps hold the previous one in registers) and S^T = K Q^T into buffer it % 2
+            // (warp-uniform loop, one elected lane issues; see the dQ kernel).  In an item's first step S^T
+            // goes first: it needs only K, while V may still be on its way.
+            constexpr uint32_t idesc_sc = idesc_bf16(128, kSubTile, 0, 0);
+            const uint32_t dV = desc_lo_k_major(smem_u32(sV));
+            const uint32_t tP = tmem_base + kColP, tKt = tmem_base + kColKt;
+            int it = 0;
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
+                DkDvItem t;
+                if (!next_item(k, kWaitBwdDkDv + 11, &t)) break;
+                const int steps = t.total_steps;
+                if (!mbar_wait_uniform(&bars->kt_full, k & 1, ctx, kWaitBwdDkDv + 16)) break;
+                for (int x = 0; ok && x < steps; ++x, ++it) {
+                    const int st = it % C::kStages;
+                    const int bf = it % kBufs;
+                    const bool last = x == steps - 1;
+                    if (!mbar_wait_uniform(&bars->st_full[st], (it / C::kStages) & 1, ctx, kWaitBwdDkDv + 2)) { ok = false; break; }
+                    const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
+                    const uint32_t dQ = desc_lo_k_major(aQ), dDO = desc_lo_k_major(aQ + C::kSubTileBytes);
+                    const uint32_t tS = tmem_base + kColS + bf * kSubTile;
+                    if (x == 0 && !mbar_wait_uniform(&bars->v_full, k & 1, ctx, kWaitBwdDkDv + 3)) { ok = false; break; }
+                    if (it >= 1 && !mbar_wait_uniform(&bars->dp_free, (it - 1) & 1, ctx, kWaitBwdDkDv + 9)) { ok = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < HD / 16; ++kk)
-                        mma_ss(tP, dV + desc_step_k_major(kk, C::kBigBoxBytes), dDO + desc_step_k_major(kk, C::kSubBoxBytes),
-                               idesc_sc, kk > 0);
-                }
-                __syncwarp();
-                if (it >= kBufs && !mbar_wait_uniform(&bars->buf_free[bf], ((it / kBufs) & 1) ^ 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t tS = tmem_base + kColS + bf * kSubTile;
-                if (elect_one()) {
+                        for (int kk = 0; kk < HD / 16; ++kk)
+                            mma_ss(tP, dV + desc_step_k_major(kk, C::kBigBoxBytes), dDO + desc_step_k_major(kk, C::kSubBoxBytes),
+                                   idesc_sc, kk > 0);
+                        if (last) mma_commit(&bars->v_empty);
+                    }
+                    __syncwarp();
+                    if (it >= kBufs && !mbar_wait_uniform(&bars->buf_free[bf], ((it / kBufs) & 1) ^ 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
+                    tc_fence_after();
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < HD / 16; ++kk)
-                        mma_ts(tS, tKt + 8 * kk, dQ + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
-                    mma_commit(&bars->s_full[bf]);
-                    if (x == t.total_steps - 1) mma_commit(&bars->kv_empty);  // nothing reads this item's K and V any more
+                        for (int kk = 0; kk < HD / 16; ++kk)
+                            mma_ts(tS, tKt + 8 * kk, dQ + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
+                    }
+                    __syncwarp();
+                    if (!ok) break;
+                    if (elect_one()) {
+                        mma_commit(&bars->s_full[bf]);
+                        if (last) mma_commit(&bars->s_done);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
-        }
-        if (__any_sync(0xffffffffu, bars->abort_flag != 0)) {
-            if (elect_one()) {
-                mma_commit(&bars->drain2);
-                mbar_wait_drain(&bars->drain2, 0);
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
+                if (elect_one()) {
+                    mma_commit(&bars->drain2);
+                    mbar_wait_drain(&bars->drain2, 0);
+                }
             }
-        }
-        __syncwarp();
-    } else if (warp == 2) {
-        // ---- gradient MMAs: dV += P^T dO and dK += dS^T Q of step `it`; both bf16 operands sit in
-        // the step's S^T buffer
-        constexpr uint32_t idesc_acc = idesc_bf16(128, HD, 0, 1);
-        int it = 0;
-        bool ok = true;
-        for (int k = 0; ok; ++k) {
-            long long id = n_items;
-            if (!__all_sync(0xffffffffu, next_item(k, kWaitBwdDkDv + 12, &id) ? 1 : 0)) break;  // warp-uniform outcome
-            const DkDvItem t = dkdv_item(geo, p.pass, id);
-            for (int x = 0; x < t.total_steps; ++x, ++it) {
-                const int st = it % C::kStages;
-                const int bf = it % kBufs;
-                if (!mbar_wait_uniform(&bars->p_full[bf], (it / kBufs) & 1, ctx, kWaitBwdDkDv + 4)) { ok = false; break; }
+            __syncwarp();
+        } else if (warp == 2) {
+            // ---- gradient MMAs: dV += P^T dO and dK += dS^T Q of step `it`; both bf16 operands sit in
+            // the step's S^T buffer
+            constexpr uint32_t idesc_acc = idesc_bf16(128, HD, 0, 1);
+            int it = 0;
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
+                DkDvItem t;
+                if (!next_item(k, kWaitBwdDkDv + 12, &t)) break;
+                const int steps = t.total_steps;
                 // the first products of an item overwrite the accumulators: the previous item's must have been read out
-                if (x == 0 && k > 0 && !mbar_wait_uniform(&bars->acc_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 13)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
-                const uint32_t dQmn = desc_lo_mn_major(aQ, C::kSubBoxBytes);
-                const uint32_t dDOmn = desc_lo_mn_major(aQ + C::kSubTileBytes, C::kSubBoxBytes);
-                // the 16 queries of K slice kk: P^T in packed columns [16 kk, +8) of the buffer, dS^T in [16 kk + 8, +8)
-                const uint32_t tPt = tmem_base + kColS + bf * kSubTile;
-                if (elect_one()) {
+                if (k > 0 && !mbar_wait_uniform(&bars->acc_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 13)) break;
+                for (int x = 0; x < steps; ++x, ++it) {
+                    const int st = it % C::kStages;
+                    const int bf = it % kBufs;
+                    if (!mbar_wait_uniform(&bars->p_full[bf], (it / kBufs) & 1, ctx, kWaitBwdDkDv + 4)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
+                    const uint32_t dQmn = desc_lo_mn_major(aQ, C::kSubBoxBytes);
+                    const uint32_t dDOmn = desc_lo_mn_major(aQ + C::kSubTileBytes, C::kSubBoxBytes);
+                    // the 16 queries of K slice kk: P^T in packed columns [16 kk, +8) of the buffer, dS^T in [16 kk + 8, +8)
+                    const uint32_t tPt = tmem_base + kColS + bf * kSubTile;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kSubTile / 16; ++kk)
-                        mma_ts(tmem_base + kColDV, tPt + 16 * kk, dDOmn + kk * kDescStepMn, idesc_acc, (x > 0) || (kk > 0));
+                        for (int kk = 0; kk < kSubTile / 16; ++kk)
+                            mma_ts(tmem_base + kColDV, tPt + 16 * kk, dDOmn + kk * kDescStepMn, idesc_acc, (x > 0) || (kk > 0));
 #pragma unroll
-                    for (int kk = 0; kk < kSubTile / 16; ++kk)
-                        mma_ts(tmem_base + kColDK, tPt + 16 * kk + 8, dQmn + kk * kDescStepMn, idesc_acc, (x > 0) || (kk > 0));
-                    mma_commit(&bars->st_empty[st]);
-                    mma_commit(&bars->buf_free[bf]);
-                    if (x == t.total_steps - 1) mma_commit(&bars->acc_full);
+                        for (int kk = 0; kk < kSubTile / 16; ++kk)
+                            mma_ts(tmem_base + kColDK, tPt + 16 * kk + 8, dQmn + kk * kDescStepMn, idesc_acc, (x > 0) || (kk > 0));
+                        mma_commit(&bars->st_empty[st]);
+                        mma_commit(&bars->buf_free[bf]);
+                        if (x == steps - 1) mma_commit(&bars->acc_full);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
-        }
-        if (__any_sync(0xffffffffu, bars->abort_flag != 0)) {
-            if (elect_one()) {
-                mma_commit(&bars->drain);
-                mbar_wait_drain(&bars->drain, 0);
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
+                if (elect_one()) {
+                    mma_commit(&bars->drain);
+                    mbar_wait_drain(&bars->drain, 0);
+                }
             }
+            __syncwarp();
+        } else {
+            // ---- K and V of every item (and the tensor-memory allocation)
+            if (lane == 0) {
+                int n_k = 0, n_v = 0;  // K and V tiles requested so far
+                for (int k = 0;; ++k) {
+                    if (!mbar_wait(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, kWaitBwdDkDv + 15)) break;
+                    const DkDvItem t = bars->item[k % kSched];
+                    if (t.total_steps == 0) break;
+                    if (k > 0 && !mbar_wait(&bars->kt_full, (k - 1) & 1, ctx, kWaitBwdDkDv + 19)) break;
+                    mbar_expect_tx(&bars->k_full, C::kBigTileBytes);
+                    for (int bx = 0; bx < C::kBoxes; ++bx)
+                        tma_load_4d(sK + bx * C::kBigBoxBytes, &p.tm_k, &bars->k_full, bx * 64, t.hk, t.tk0, t.b);
+                    ++n_k;
+                    if (k > 0 && !mbar_wait(&bars->v_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 20)) break;
+                    mbar_expect_tx(&bars->v_full, C::kBigTileBytes);
+                    for (int bx = 0; bx < C::kBoxes; ++bx)
+                        tma_load_4d(sV + bx * C::kBigBoxBytes, &p.tm_v, &bars->v_full, bx * 64, t.hk, t.tk0, t.b);
+                    ++n_v;
+                }
+                if (bars->abort_flag != 0) {
+                    if (n_k > 0) mbar_wait_drain(&bars->k_full, (n_k - 1) & 1);
+                    if (n_v > 0) mbar_wait_drain(&bars->v_full, (n_v - 1) & 1);
+                }
+            }
+            __syncwarp();
         }
-        __syncwarp();
-    } else if (warp == 3) {
-        // spare warp: owns the tensor-memory allocation only
-    } else {
+    } else if (warp < 12) {
         // ---- elementwise.  Thread (quad, lane, group) owns key row 32 quad + lane and the query columns
         // [32 group, +32) of every step.  (Letting the two groups of four warps take alternate steps with a
         // whole row per thread was measured too: with two S^T buffers the chain S^T -> elementwise ->
         // gradient MMAs of a buffer is what a step waits for, and half the columns per thread halve its
         // elementwise part: 3.33 against 3.53 ms on the Llama2-7B 32k shape.)
+        setmaxnreg_inc<C::kRegsElem>();
         const int quad = warp & 3;
         const int group = (warp - 4) >> 2;
         const int row = quad * 32 + lane;  // key row of the tile owned by this thread
@@ -796,33 +892,9 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "r"(a));
             return r;
         };
-        // K of item k goes from its shared-memory tile into tensor memory, where it is the A operand of
-        // S^T = K Q^T: an A operand in shared memory would be read again by every step (4 KB per MMA
-        // against 2 KB of B), and shared-memory bandwidth is what bounds this kernel.  Row `row`, columns
-        // [64 group, +64) of d: eight 16-byte chunks of the 128-byte-swizzled row, 32 packed columns.
-        auto copy_k = [&](int k) -> bool {
-            if (!mbar_wait(&bars->res_full, k & 1, ctx, kWaitBwdDkDv + 17)) return false;
-            if (group * 64 < HD) {
-                const uint32_t src = smem_u32(sK) + group * C::kBigBoxBytes + row * 128;
-                uint32_t kr[32];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(kr[4 * c]), "=r"(kr[4 * c + 1]), "=r"(kr[4 * c + 2]), "=r"(kr[4 * c + 3])
-                                 : "r"(src + ((c ^ (row & 7)) << 4)));
-                }
-                tmem_st_32x32(t_row + kColKt + group * 32, kr);
-                tmem_wait_st();
-            }
-            tc_fence_before();
-            mbar_arrive(&bars->kt_full);
-            return true;
-        };
         for (int k = 0; ok; ++k) {
-            long long id;
-            if (!next_item(k, kWaitBwdDkDv + 14, &id)) break;
-            if (k == 0 && !copy_k(0)) break;   // later items: copied at the end of the item before
-            const DkDvItem t = dkdv_item(geo, p.pass, id);
+            DkDvItem t;
+            if (!next_item(k, kWaitBwdDkDv + 14, &t)) break;
             const bool key_valid = row < t.k_valid;  // rows past the end of a ragged tile belong to other tiles
             const int hq0 = t.hk * rep;
             for (int hq = hq0; ok && hq < hq0 + rep; ++hq) {
@@ -840,8 +912,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     const int st = it % C::kStages;
                     const int bf = it % kBufs;
                     // The statistics of this step travel with its stage.  s_full covers dP^T of this step as
-                    // well: its MMAs were issued before those of S^T by the same thread, and a commit completes
-                    // after everything issued before it.
+                    // well: its MMAs were issued by the same thread before the commit.
                     if (!mbar_wait(&bars->st_full[st], (it / C::kStages) & 1, ctx, kWaitBwdDkDv + 5) ||
                         !mbar_wait(&bars->s_full[bf], (it / kBufs) & 1, ctx, kWaitBwdDkDv + 6)) {
                         ok = false;
@@ -939,26 +1010,58 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     mbar_arrive(&bars->p_full[bf]);
                 }
             }
-            if (!ok) break;
-            // K of the next item, if there is one, while the last gradient MMAs of this one run: the TMA
-            // warp fetched it as soon as the last score product of this item was done (which also means that
-            // nothing reads the old copy any more)
-            {
-                long long next_id;
-                if (next_item(k + 1, kWaitBwdDkDv + 18, &next_id)) {
-                    if (!copy_k(k + 1)) break;
-                } else if (bars->abort_flag != 0) {
-                    break;
+        }
+    } else {
+        // ---- epilogue: the copy of K into tensor memory and the read-out of the accumulators
+        setmaxnreg_dec<C::kRegsOther>();
+        const int quad = warp & 3;
+        const int row = quad * 32 + lane;
+        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+        uint8_t* stage = sOut + quad * 8192;
+        uint32_t used = 0;
+        // K of item k goes from its shared-memory tile into tensor memory, where it is the A operand of
+        // S^T = K Q^T: an A operand in shared memory would be read again by every step (4 KB per MMA
+        // against 2 KB of B), and shared-memory bandwidth is what bounds this kernel.  One key row per thread:
+        // the 16-byte chunks of the 128-byte-swizzled rows, 32 packed columns for each 64 values.
+        auto copy_k = [&](int k) -> bool {
+            if (!mbar_wait_uniform(&bars->k_full, k & 1, ctx, kWaitBwdDkDv + 17)) return false;
+            if (k > 0 && !mbar_wait_uniform(&bars->s_done, (k - 1) & 1, ctx, kWaitBwdDkDv + 21)) return false;
+            tc_fence_after();
+#pragma unroll
+            for (int bx = 0; bx < C::kBoxes; ++bx) {
+                const uint32_t src = smem_u32(sK) + bx * C::kBigBoxBytes + row * 128;
+                uint32_t kr[32];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                 : "=r"(kr[4 * c]), "=r"(kr[4 * c + 1]), "=r"(kr[4 * c + 2]), "=r"(kr[4 * c + 3])
+                                 : "r"(src + ((c ^ (row & 7)) << 4)));
                 }
+                tmem_st_32x32(t_row + kColKt + bx * 32, kr);
             }
-            if (!mbar_wait(&bars->acc_full, k & 1, ctx, kWaitBwdDkDv + 7)) break;
+            tmem_wait_st();
+            tc_fence_before();
+            mbar_arrive_warp(&bars->kt_full);
+            return true;
+        };
+        DkDvItem next;
+        bool more = next_item(0, kWaitBwdDkDv + 18, &next) && copy_k(0);
+        for (int k = 0; more; ++k) {
+            const DkDvItem t = next;
+            // K of the next item, if there is one, as soon as this item's score products are done
+            more = next_item(k + 1, kWaitBwdDkDv + 18, &next);
+            if (more && !copy_k(k + 1)) break;
+            if (!mbar_wait_uniform(&bars->acc_full, k & 1, ctx, kWaitBwdDkDv + 7)) break;
             tc_fence_after();
             const size_t out_row = (static_cast<size_t>(t.b) * geo.N + t.tk0 + row) * p.dkv_tok_stride + static_cast<size_t>(t.hk) * HD;
-            if (group == 0) store_acc_cols<HD>(t_row + kColDV, 1.0f, p.dv + out_row, key_valid);
-            else store_acc_cols<HD>(t_row + kColDK, p.scale, p.dk + out_row, key_valid);
-            tc_fence_before();
-            mbar_arrive(&bars->acc_empty);
+            const int tok0 = t.tk0 + quad * 32, valid = t.k_valid - quad * 32;
+            store_acc_rows<HD>(&p.tm_dv, stage, used, t_row + kColDV, 1.0f, p.dv + out_row, t.hk, tok0, t.b, valid, [] {});
+            store_acc_rows<HD>(&p.tm_dk, stage, used, t_row + kColDK, p.scale, p.dk + out_row, t.hk, tok0, t.b, valid, [&] {
+                tc_fence_before();
+                mbar_arrive_warp(&bars->acc_empty);
+            });
         }
+        if (lane == 0) bulk_wait_all();
     }
 
     tc_fence_before();
@@ -976,10 +1079,13 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
 // the blocks the spilling dK,dV kernel wrote: nothing is recomputed, the kernel is a chain of
 // 128x128x128 products whose A operand streams from global memory once (memory bound).
 //
-// Persistent: one CTA per SM takes (unit, query tile) work items, heaviest first, from a counter in
-// global memory.  Warp 0 draws the items and loads with TMA (it runs ahead across item boundaries, so
-// the ring never drains between items), warp 1 issues the MMAs into one of two accumulators in tensor
-// memory, warps 2-5 write the finished accumulator out while the next item is being multiplied.
+// Persistent: one CTA per SM takes pairs of neighbouring query tiles of a unit, heaviest first, by cluster
+// launch control.  The two tiles of a pair share the K tiles they stream: 48 instead of 64 KB through L2
+// and shared memory for every product.  Warp 0 draws the items and loads with TMA (it runs ahead across item boundaries,
+// so the ring never drains between items), warp 1 issues the MMAs into one of two pairs of accumulators in
+// tensor memory, warps 2-5 write the finished accumulators out while the next item is being multiplied.
+// Bound by reading dS (8.7 GB on Llama2-7B 32k: 1.33 ms at the measured copy rate, 1.50 taken; a tile at a time
+// took 1.60).
 // A block (j, n) is copied to shared memory as it lies in global memory (one bulk copy for the blocks
 // (j, 2i) and (j, 2i+1), which are neighbours): chunk-major, i.e. the 16-byte chunk c (8 queries) of
 // key row r at byte (c * 128 + r) * 16.  Eight key rows of one chunk are 128 contiguous bytes: the
@@ -993,91 +1099,90 @@ struct DqSpillCfg {
     static constexpr int kBoxes = HD / 64;
     static constexpr int kKBoxBytes = kTile * 128;
     static constexpr int kKBytes = kBoxes * kKBoxBytes;
-    static constexpr int kDsBlockBytes = kSpillBlockElems * 2;
-    static constexpr int kStageBytes = 2 * kDsBlockBytes + kKBytes;
-    static constexpr int kStages = 3;
+    static constexpr int kDsBytes = 2 * kSpillBlockElems * 2;  // dS of one query tile against one key tile
+    static constexpr int kSlotBytes = 32768;                   // a K tile or a dS tile
+    static_assert(kKBytes <= kSlotBytes && kDsBytes <= kSlotBytes, "slot size");
+    static constexpr int kRing = 6;   // K_j, dS_1j, dS_0j, K_{j+1}, ...
     static constexpr int kSched = 8;  // work items the producer can be ahead of the epilogue: at most 5
-    static constexpr int kBarBytes = 512;
-    static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kBarBytes;
-    static constexpr int kTmemCols = 256;  // two accumulators of 128 columns
-};
-
-struct DqSpillBars {
-    uint64_t full[3], empty[3];
-    uint64_t acc_full[2], acc_empty[2];
-    uint64_t sched_full[8];
-    uint64_t drain;
-    long long item[8];
-    uint32_t tmem_slot;
-    int abort_flag;
+    static constexpr int kOutBytes = 4 * 2 * 4096;
+    static constexpr int kBarBytes = 1024;
+    static constexpr int kSmemBytes = kRing * kSlotBytes + kOutBytes + kBarBytes;
+    static constexpr int kTmemCols = 512;  // two pairs of accumulators of 128 columns
 };
 
 struct DqSpillItem {
-    int b, h, hk, i, j_begin, n_steps, tq0, q_valid;
+    int b, h, hk;
     long long unit;
     GroupLayout L;
+    TilePair t;
 };
-// Work item `id` (heaviest query tiles of a chunk of units first, as in the other kernels).  n_steps = 0
-// marks a slot of a group that has fewer tiles than the largest one.
-__device__ __forceinline__ DqSpillItem dq_spill_item(const Geometry& geo, const SpillPass& pass, long long id) {
-    DqSpillItem t;
+struct DqSpillBars {
+    uint64_t full[6], empty[6];
+    uint64_t acc_full[2], acc_empty[2];
+    uint64_t sched_full[8];
+    uint64_t drain, clc;
+    alignas(16) uint8_t clc_resp[16];
+    DqSpillItem item[8];  // b = -1: no more items
+    uint32_t tmem_slot;
+    int abort_flag;
+};
+static_assert(sizeof(DqSpillBars) <= 1024, "barrier block");
+
+// Work item `id`: a pair of query tiles, the heaviest of a chunk of units first, as in the other kernels.
+// Units are taken from the last one down: the dS^T that was written last may still be in L2.  false marks
+// a slot of a group that has fewer pairs than the largest one.
+__device__ __forceinline__ bool dq_spill_item(const BwdDqSpillParams& p, int id, DqSpillItem* w) {
+    const Geometry& geo = p.geo;
     const int rep = geo.H / geo.Hkv;
-    const int heads = pass.nk * rep;
+    const int heads = p.pass.nk * rep;
+    const int units = geo.B * heads * geo.groups;
     int unit, rank;
-    decode_block(id, geo.B * heads * geo.groups, geo.tiles_per_group, &unit, &rank);
+    decode_block(id, units, p.pairs_per_group, &unit, &rank);
+    unit = units - 1 - unit;
     const int g = unit % geo.groups;
-    t.h = pass.hk0 * rep + (unit / geo.groups) % heads;
-    t.b = unit / (geo.groups * heads);
-    t.hk = t.h / rep;
-    t.unit = unit;
-    const int s = (t.h < geo.n_unshifted) ? 0 : geo.shift;
-    t.L = group_layout(geo, s, g);
-    t.i = t.L.nTiles - 1 - rank;
-    if (t.i < 0) {
-        t.n_steps = 0;
-        t.j_begin = 0, t.tq0 = 0, t.q_valid = 0;
-        return t;
-    }
-    t.j_begin = first_key_tile(t.L, t.i);
-    t.n_steps = t.i + 1 - t.j_begin;
-    const TileRef tq = tile_ref(t.L, t.i);
-    t.tq0 = tq.tok0;
-    t.q_valid = tq.valid;
-    return t;
+    w->h = p.pass.hk0 * rep + (unit / geo.groups) % heads;
+    w->b = unit / (geo.groups * heads);
+    w->hk = w->h / rep;
+    w->unit = unit;
+    w->L = group_layout(geo, (w->h < geo.n_unshifted) ? 0 : geo.shift, g);
+    if (rank >= pairs_of_group(w->L)) return false;
+    w->t = tile_pair(w->L, rank);
+    return true;
 }
 
 template <int HD>
 __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_kernel(const __grid_constant__ BwdDqSpillParams p) {
     using C = DqSpillCfg<HD>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    DqSpillBars* bars = reinterpret_cast<DqSpillBars*>(smem + C::kStages * C::kStageBytes);
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    uint8_t* smem = smem_raw;  // 1024-byte aligned: nothing precedes the dynamic array
+    uint8_t* sOut = smem + C::kRing * C::kSlotBytes;
+    DqSpillBars* bars = reinterpret_cast<DqSpillBars*>(sOut + C::kOutBytes);
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    __shared__ int s_poisoned;
-    if (threadIdx.x == 0) s_poisoned = *reinterpret_cast<volatile int*>(p.status);
+    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
     __syncthreads();
-    if (s_poisoned != 0) return;
-    const Geometry& geo = p.geo;
-    const int Tg = geo.tiles_per_group;
-    const long long n_items = static_cast<long long>(geo.B) * p.pass.nk * (geo.H / geo.Hkv) * geo.groups * Tg;
+    if (bars->abort_flag != 0) return;
+    __syncthreads();
+    const int Tg = p.geo.tiles_per_group;
 
     if (threadIdx.x == 0) {
-        for (int x = 0; x < C::kStages; ++x) {
+        for (int x = 0; x < C::kRing; ++x) {
             mbar_init(&bars->full[x], 1);
             mbar_init(&bars->empty[x], 1);
         }
         for (int x = 0; x < 2; ++x) {
             mbar_init(&bars->acc_full[x], 1);
-            mbar_init(&bars->acc_empty[x], 128);
+            mbar_init(&bars->acc_empty[x], 4);  // one arrival per epilogue warp
         }
         for (int x = 0; x < C::kSched; ++x) mbar_init(&bars->sched_full[x], 1);
         mbar_init(&bars->drain, 1);
+        mbar_init(&bars->clc, 1);
         bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_k);
+        tma_prefetch_desc(&p.tm_dq);
     }
     if (warp == 1) {
         tmem_alloc(&bars->tmem_slot, C::kTmemCols);
@@ -1088,81 +1193,103 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
+    auto next_item = [&](int k, int where, DqSpillItem* w) -> bool {
+        if (!mbar_wait_uniform(&bars->sched_full[k % C::kSched], (k / C::kSched) & 1, ctx, where)) return false;
+        *w = bars->item[k % C::kSched];
+        return w->b >= 0;
+    };
 
     if (warp == 0) {
-        // ---- scheduler + TMA producer -------------------------------------------------------------
+        // ---- work items + TMA producer ------------------------------------------------------------
         if (lane == 0) {
-            long long it = 0;  // stage uses so far
+            uint32_t x = 0;  // ring slots filled so far
             bool ok = true;
-            for (int k = 0; ok; ++k) {
-                // draw the next item that has work (slots of groups with fewer tiles than the largest are
-                // skipped here, so the other warps only ever see real items and the end marker)
-                long long id;
-                DqSpillItem t;
-                do {
-                    id = static_cast<long long>(atomicAdd(p.counter, 1));
-                    if (id >= n_items) break;
-                    t = dq_spill_item(geo, p.pass, id);
-                } while (t.n_steps == 0);
-                bars->item[k % C::kSched] = id;
-                mbar_arrive(&bars->sched_full[k % C::kSched]);  // release: the id is visible to whoever sees the phase
-                if (id >= n_items) break;
-                for (int n = 0; n < t.n_steps; ++n, ++it) {
-                    const int st = static_cast<int>(it % C::kStages);
-                    const uint32_t ph = static_cast<uint32_t>(it / C::kStages) & 1u;
-                    if (!mbar_wait(&bars->empty[st], ph ^ 1, ctx, kWaitBwdDqSpill + 1)) { ok = false; break; }
-                    const int j = t.j_begin + n;
-                    uint8_t* sDs = smem + st * C::kStageBytes;
-                    uint8_t* sK = sDs + 2 * C::kDsBlockBytes;
-                    mbar_expect_tx(&bars->full[st], C::kStageBytes);
-                    const long long blk = spill_block(t.unit, Tg, j, 2 * t.i);
-                    bulk_load_1d(sDs, p.spill + blk * kSpillBlockElems, 2 * C::kDsBlockBytes, &bars->full[st]);
-                    const int tk0 = tile_ref(t.L, j).tok0;
-                    for (int bx = 0; bx < C::kBoxes; ++bx)
-                        tma_load_4d(sK + bx * C::kKBoxBytes, &p.tm_k, &bars->full[st], bx * 64, t.hk, tk0, t.b);
+            ItemSource items{&bars->clc, bars->clc_resp};
+            int id = static_cast<int>(blockIdx.x);
+            auto slot = [&](uint32_t bytes) -> uint8_t* {
+                const uint32_t st = x % C::kRing;
+                if (!mbar_wait(&bars->empty[st], ((x / C::kRing) & 1) ^ 1, ctx, kWaitBwdDqSpill + 1)) {
+                    ok = false;
+                    return nullptr;
                 }
+                mbar_expect_tx(&bars->full[st], bytes);
+                return smem + st * C::kSlotBytes;
+            };
+            for (int k = 0; ok; ++k) {
+                DqSpillItem w;
+                while (id >= 0 && !dq_spill_item(p, id, &w)) {  // skip the empty slots of smaller groups
+                    id = items.next(ctx, kWaitBwdDqSpill + 7, &ok);
+                }
+                if (id < 0) w.b = -1;
+                bars->item[k % C::kSched] = w;
+                mbar_arrive(&bars->sched_full[k % C::kSched]);  // release: the item is visible to whoever sees the phase
+                if (id < 0) break;
+                for (int n = 0; ok && n < w.t.n[1]; ++n) {
+                    const int j = w.t.j_begin + n;
+                    const int tk0 = tile_ref(w.L, j).tok0;
+                    uint8_t* dst = slot(C::kKBytes);
+                    if (!ok) break;
+                    for (int bx = 0; bx < C::kBoxes; ++bx)
+                        tma_load_4d(dst + bx * C::kKBoxBytes, &p.tm_k, &bars->full[x % C::kRing], bx * 64, w.hk, tk0, w.b);
+                    ++x;
+                    for (int t = 1; t >= 0 && n < w.t.n[t]; --t) {
+                        dst = slot(C::kDsBytes);
+                        if (!ok) break;
+                        bulk_load_1d(dst, p.spill + spill_block(w.unit, Tg, j, 2 * w.t.i[t]) * kSpillBlockElems, C::kDsBytes,
+                                     &bars->full[x % C::kRing]);
+                        ++x;
+                    }
+                }
+                if (ok) id = items.next(ctx, kWaitBwdDqSpill + 7, &ok);
             }
             if (bars->abort_flag != 0) {
-                for (long long nn = (it > C::kStages ? it - C::kStages : 0); nn < it; ++nn)
-                    mbar_wait_drain(&bars->full[nn % C::kStages], static_cast<uint32_t>(nn / C::kStages) & 1u);
+                for (uint32_t y = (x > C::kRing ? x - C::kRing : 0); y < x; ++y)
+                    mbar_wait_drain(&bars->full[y % C::kRing], (y / C::kRing) & 1);
             }
         }
         __syncwarp();
     } else if (warp == 1) {
         // ---- MMA issuer (warp-uniform loop, one elected lane issues) ------------------------------
         constexpr uint32_t idesc = idesc_bf16(128, HD, 1, 1);
-        long long it = 0;
+        uint32_t x = 0;
         bool ok = true;
-        int used = 0;  // accumulator uses so far
+        auto wait_slot = [&](uint32_t y) -> bool {
+            return mbar_wait_uniform(&bars->full[y % C::kRing], (y / C::kRing) & 1, ctx, kWaitBwdDqSpill + 4);
+        };
         for (int k = 0; ok; ++k) {
-            if (!mbar_wait_uniform(&bars->sched_full[k % C::kSched], (k / C::kSched) & 1, ctx, kWaitBwdDqSpill + 2)) break;
-            const long long id = bars->item[k % C::kSched];
-            if (id >= n_items) break;
-            const DqSpillItem t = dq_spill_item(geo, p.pass, id);
-            const int buf = used & 1;
-            if (!mbar_wait_uniform(&bars->acc_empty[buf], ((used >> 1) & 1) ^ 1, ctx, kWaitBwdDqSpill + 3)) break;
-            tc_fence_after();
-            const uint32_t tAcc = tmem_base + buf * 128;
-            for (int n = 0; n < t.n_steps; ++n, ++it) {
-                const int st = static_cast<int>(it % C::kStages);
-                if (!mbar_wait_uniform(&bars->full[st], static_cast<uint32_t>(it / C::kStages) & 1u, ctx, kWaitBwdDqSpill + 4)) { ok = false; break; }
-                tc_fence_after();
-                const uint32_t aDs = smem_u32(smem + st * C::kStageBytes);
-                const uint32_t dA = desc_lo_mn_major_plain(aDs, 128);
-                const uint32_t dB = desc_lo_mn_major(aDs + 2 * C::kDsBlockBytes, C::kKBoxBytes);
-                if (elect_one()) {
+            DqSpillItem w;
+            if (!next_item(k, kWaitBwdDqSpill + 2, &w)) break;
+            const int buf = k & 1;
+            if (!mbar_wait_uniform(&bars->acc_empty[buf], ((k >> 1) & 1) ^ 1, ctx, kWaitBwdDqSpill + 3)) break;
+            for (int n = 0; ok && n < w.t.n[1]; ++n) {
+                const uint32_t xk = x++;
+                ok = wait_slot(xk);
+                const uint32_t dB = desc_lo_mn_major(smem_u32(smem + (xk % C::kRing) * C::kSlotBytes), C::kKBoxBytes);
+#pragma unroll 1
+                for (int t = 1; ok && t >= 0; --t) {
+                    const int n_t = t ? w.t.n[1] : w.t.n[0];
+                    if (n >= n_t) break;
+                    const uint32_t xd = x++;
+                    ok = wait_slot(xd);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t dA = desc_lo_mn_major_plain(smem_u32(smem + (xd % C::kRing) * C::kSlotBytes), 128);
+                    const uint32_t tAcc = tmem_base + buf * 256 + t * 128;
+                    const bool last_t = t == 0 || n >= w.t.n[0];  // last product with this K tile
+                    if (elect_one()) {
 #pragma unroll
-                    for (int kk = 0; kk < kTile / 16; ++kk)
-                        mma_ss_hi(tAcc, dA + kk * (256u >> 4), desc_hi_plain(2048), dB + kk * kDescStepMn, kDescHi, idesc,
-                                  (n > 0) || (kk > 0));
-                    mma_commit(&bars->empty[st]);
-                    if (n == t.n_steps - 1) mma_commit(&bars->acc_full[buf]);
+                        for (int kk = 0; kk < kTile / 16; ++kk)
+                            mma_ss_hi(tAcc, dA + kk * (256u >> 4), desc_hi_plain(2048), dB + kk * kDescStepMn, kDescHi, idesc,
+                                      (n > 0) || (kk > 0));
+                        mma_commit(&bars->empty[xd % C::kRing]);
+                        if (last_t) mma_commit(&bars->empty[xk % C::kRing]);
+                        if (last_t && n == w.t.n[1] - 1) mma_commit(&bars->acc_full[buf]);
+                    }
+                    __syncwarp();
                 }
-                __syncwarp();
             }
-            ++used;
         }
-        if (__any_sync(0xffffffffu, bars->abort_flag != 0)) {
+        if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
             if (elect_one()) {
                 mma_commit(&bars->drain);
                 mbar_wait_drain(&bars->drain, 0);
@@ -1174,21 +1301,28 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-        int used = 0;
+        uint8_t* stage = sOut + quad * 8192;
+        uint32_t used = 0;
         for (int k = 0;; ++k) {
-            if (!mbar_wait(&bars->sched_full[k % C::kSched], (k / C::kSched) & 1, ctx, kWaitBwdDqSpill + 5)) break;
-            const long long id = bars->item[k % C::kSched];
-            if (id >= n_items) break;
-            const DqSpillItem t = dq_spill_item(geo, p.pass, id);
-            const int buf = used & 1;
-            if (!mbar_wait(&bars->acc_full[buf], (used >> 1) & 1, ctx, kWaitBwdDqSpill + 6)) break;
+            DqSpillItem w;
+            if (!next_item(k, kWaitBwdDqSpill + 5, &w)) break;
+            const int buf = k & 1;
+            if (!mbar_wait_uniform(&bars->acc_full[buf], (k >> 1) & 1, ctx, kWaitBwdDqSpill + 6)) break;
             tc_fence_after();
-            __nv_bfloat16* dst = p.dq + (static_cast<size_t>(t.b) * geo.N + t.tq0 + row) * p.dq_tok_stride + static_cast<size_t>(t.h) * HD;
-            store_acc_cols<HD>(t_row + buf * 128, p.scale, dst, row < t.q_valid);
-            tc_fence_before();
-            mbar_arrive(&bars->acc_empty[buf]);
-            ++used;
+#pragma unroll 1
+            for (int t = w.t.n[0] > 0 ? 0 : 1; t < 2; ++t) {
+                const TileRef tq = tile_ref(w.L, t ? w.t.i[1] : w.t.i[0]);
+                __nv_bfloat16* dst = p.dq + (static_cast<size_t>(w.b) * p.geo.N + tq.tok0 + row) * p.dq_tok_stride + static_cast<size_t>(w.h) * HD;
+                store_acc_rows<HD>(&p.tm_dq, stage, used, t_row + buf * 256 + t * 128, p.scale, dst, w.h, tq.tok0 + quad * 32, w.b,
+                                   tq.valid - quad * 32, [&] {
+                                       if (t == 1) {
+                                           tc_fence_before();
+                                           mbar_arrive_warp(&bars->acc_empty[buf]);
+                                       }
+                                   });
+            }
         }
+        if (lane == 0) bulk_wait_all();
     }
 
     tc_fence_before();
@@ -1201,24 +1335,30 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
 
 }  // namespace
 
+namespace {
+// The kernels place their tiles from the start of the dynamic array, and the register split of the dK,dV
+// kernel draws on what a block is launched with (min_regs).
+template <typename Kernel>
+cudaError_t configure_one(Kernel kernel, int smem_bytes, int min_regs) {
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+    if (e != cudaSuccess) return e;
+    if (a.numRegs < min_regs || a.sharedSizeBytes != 0) return cudaErrorInvalidConfiguration;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+}
+template <int HD>
+cudaError_t configure_all() {
+    cudaError_t e = configure_one(s2a_bwd_dq_kernel<HD>, DqCfg<HD>::kSmemBytes, 0);
+    if (e == cudaSuccess) e = configure_one(s2a_bwd_dkdv_kernel<HD, false>, BwdCfg<HD>::kSmemBytes, BwdCfg<HD>::kRegsLaunch);
+    if (e == cudaSuccess) e = configure_one(s2a_bwd_dkdv_kernel<HD, true>, BwdCfg<HD>::kSmemBytes, BwdCfg<HD>::kRegsLaunch);
+    if (e == cudaSuccess) e = configure_one(s2a_bwd_dq_spill_kernel<HD>, DqSpillCfg<HD>::kSmemBytes, 0);
+    return e;
+}
+}  // namespace
+
 cudaError_t configure_bwd() {
-    cudaError_t e;
-    e = cudaFuncSetAttribute(s2a_bwd_dq_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<64>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dq_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqCfg<128>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dkdv_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<64>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dkdv_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<128>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dkdv_kernel<64, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<64>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dkdv_kernel<128, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, BwdCfg<128>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(s2a_bwd_dq_spill_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, DqSpillCfg<64>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(s2a_bwd_dq_spill_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                DqSpillCfg<128>::kSmemBytes);
+    const cudaError_t e = configure_all<64>();
+    return e != cudaSuccess ? e : configure_all<128>();
 }
 
 cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream) {
@@ -1237,10 +1377,9 @@ cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, int n_sm, cudaStream_t stream) {
+cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, cudaStream_t stream) {
     const Geometry& g = p.geo;
-    const long long items = static_cast<long long>(g.B) * p.pass.nk * g.groups * g.tiles_per_group;
-    const unsigned grid = static_cast<unsigned>(items < n_sm ? items : n_sm);
+    const unsigned grid = static_cast<unsigned>(static_cast<long long>(g.B) * p.pass.nk * g.groups * g.tiles_per_group);
     if (p.spill != nullptr) {
         if (d == 64) s2a_bwd_dkdv_kernel<64, true><<<grid, BwdCfg<64>::kThreads, BwdCfg<64>::kSmemBytes, stream>>>(p);
         else s2a_bwd_dkdv_kernel<128, true><<<grid, BwdCfg<128>::kThreads, BwdCfg<128>::kSmemBytes, stream>>>(p);
@@ -1251,10 +1390,9 @@ cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, int n_sm, cudaStream_
     return cudaGetLastError();
 }
 
-cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, int n_sm, cudaStream_t stream) {
+cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream) {
     const Geometry& g = p.geo;
-    const long long items = static_cast<long long>(g.B) * p.pass.nk * (g.H / g.Hkv) * g.groups * g.tiles_per_group;
-    const unsigned grid = static_cast<unsigned>(items < n_sm ? items : n_sm);
+    const unsigned grid = static_cast<unsigned>(static_cast<long long>(g.B) * p.pass.nk * (g.H / g.Hkv) * g.groups * p.pairs_per_group);
     if (d == 64) s2a_bwd_dq_spill_kernel<64><<<grid, DqSpillCfg<64>::kThreads, DqSpillCfg<64>::kSmemBytes, stream>>>(p);
     else s2a_bwd_dq_spill_kernel<128><<<grid, DqSpillCfg<128>::kThreads, DqSpillCfg<128>::kSmemBytes, stream>>>(p);
     return cudaGetLastError();

@@ -22,11 +22,16 @@
 // are fetched once for the 256 query rows, which halves their L2 and shared-memory traffic.
 // Tensor memory: S0 [0,128)  S1 [128,256)  O0 [256,256+HD)  O1 [384,384+HD); P (bf16) over S.
 //
+// The last work items of a launch decide how long it takes, so blocks ask for the next one late (when they
+// have issued their loads), and one thread decodes it for all warps.  Asking an item ahead and decoding it in
+// every warp with 64-bit divisions cost 86 against 73 us on 4 x 2048 tokens with groups of 512, 101 against 80
+// on a grouped-query shape (2 x 4096, groups of 1024, head size 64), 2 % on Llama2-7B 32k.
+//
 // What bounds it: the chain scores -> softmax -> P V -> next scores of a tile (clock stamps: about 2400
 // clocks in the softmax and 1100 in the two products of a step, with the other tile's step alongside); the
 // special-function unit and the tensor pipe are each busy about half of the time.  Measured against the
 // form it replaces (one query tile per block, two blocks per SM, two threads per row, scores read twice):
-// Llama2-7B 32k 2.04 against 2.38 ms a call, 8k 0.177 against 0.211, head size 64 at 32k 1.55 against 1.80.
+// Llama2-7B 32k 1.94 against 2.38 ms a call, 8k 0.161 against 0.211, groups of 512 0.073 against 0.099.
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -41,7 +46,8 @@ struct FwdCfg {
     static constexpr int kBoxBytes = kTile * 128;           // 128 rows x 128 bytes
     static constexpr int kTileBytes = kBoxes * kBoxBytes;   // one Q, K, V or O tile
     static constexpr int kRing = (HD == 128) ? 4 : 8;       // K and V tiles in flight: K_0 V_0 K_1 V_1 ...
-    static constexpr int kBarBytes = 512 + 2 * 2 * kTile * 4;  // barriers + row statistics handed to the epilogue
+    static constexpr int kStatBytes = 2 * 2 * kTile * 4;     // row statistics handed to the epilogue
+    static constexpr int kBarBytes = 1024 + kStatBytes;
     static constexpr int kSmemBytes = (2 + kRing + 1) * kTileBytes + kBarBytes;
     static constexpr int kTmemCols = 512;
     static constexpr int kColO = 256;
@@ -50,8 +56,13 @@ struct FwdCfg {
     static_assert(2 * kRegsSoftmax + kRegsEpilogue + kRegsIssue <= 4 * kRegsLaunch, "register split");
 };
 
-constexpr int kSched = 8;  // item ids in flight: the producer is at most five items ahead of the epilogue
+constexpr int kSched = 8;  // items in flight: the producer is at most five items ahead of the epilogue
 
+struct FwdItem {
+    int b, h, hk;
+    GroupLayout L;
+    TilePair t;
+};
 struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t s_full[2];              // S of a tile's step is in tensor memory
@@ -63,21 +74,16 @@ struct FwdBars {
     uint64_t sched_full[kSched];
     uint64_t clc, drain[2];
     alignas(16) uint8_t clc_resp[16];
-    int item[kSched];
+    FwdItem item[kSched];  // b = -1: no more items
     uint32_t tmem_slot;
     int abort_flag;
 };
-static_assert(sizeof(FwdBars) <= 512, "barrier block");
+static_assert(sizeof(FwdBars) <= 1024, "barrier block");
 
 // Threshold (in log2 units) below which a larger running maximum is ignored: P then grows by at
 // most 2^8, which bf16 and the fp32 row sum absorb, and O needs no rescale.
 constexpr float kLazyRescale = 8.0f;
 
-struct FwdItem {
-    int b, h, hk;
-    GroupLayout L;
-    TilePair t;
-};
 // Work item `id`; false marks a slot of a group that has fewer pairs than the largest one.
 __device__ __forceinline__ bool fwd_item(const FwdParams& p, int id, FwdItem* w) {
     int unit, rank;
@@ -100,7 +106,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
     uint8_t* sKV = sQ + 2 * C::kTileBytes;             // ring of K and V tiles
     uint8_t* sO = sKV + C::kRing * C::kTileBytes;      // one output tile on its way out
     FwdBars* bars = reinterpret_cast<FwdBars*>(sO + C::kTileBytes);
-    float* sStat = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 512);  // [tile][m, l][128 rows]
+    float* sStat = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);  // [tile][m, l][128 rows]
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -114,10 +120,10 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             atomicCAS(p.status, 0, bad);
             *reinterpret_cast<volatile int*>(p.host_status) = bad;
         }
-        bars->item[0] = bad;
+        bars->abort_flag = bad;
     }
     __syncthreads();
-    if (bars->item[0] != 0) return;
+    if (bars->abort_flag != 0) return;
     __syncthreads();
 
     if (threadIdx.x == 0) {
@@ -158,10 +164,12 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
     const uint32_t tmem_base = bars->tmem_slot;
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
 
-    // Every consumer warp walks the same sequence of items: the k-th id, -1 = the end (or aborting).
-    auto next_item = [&](int k, int where) -> int {
-        if (!mbar_wait_uniform(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return -1;
-        return *reinterpret_cast<volatile int*>(&bars->item[k % kSched]);
+    // Every consumer warp walks the same sequence of items, as the scheduling thread has decoded them (the
+    // divisions of fwd_item cost a warp about a thousand clocks): the k-th one, false = the end (or aborting).
+    auto next_item = [&](int k, int where, FwdItem* w) -> bool {
+        if (!mbar_wait_uniform(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return false;
+        *w = bars->item[k % kSched];
+        return w->b >= 0;
     };
 
     if (warp >= 12) {
@@ -171,25 +179,9 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             if (lane == 0) {
                 uint32_t kv = 0;              // K and V tiles requested so far
                 uint32_t n_q[2] = {0, 0};     // query tiles requested so far
-                uint32_t n_clc = 0;
-                bool ok = true, asked = false;
+                bool ok = true;
+                ItemSource items{&bars->clc, bars->clc_resp};
                 int id = static_cast<int>(blockIdx.x);
-                auto ask = [&]() {
-                    mbar_expect_tx(&bars->clc, 16);
-                    clc_try_cancel(bars->clc_resp, &bars->clc);
-                    asked = true;
-                };
-                auto answer = [&]() -> int {
-                    asked = false;
-                    if (!mbar_wait(&bars->clc, n_clc & 1, ctx, kWaitFwd + 1)) {
-                        ok = false;
-                        return -1;
-                    }
-                    ++n_clc;
-                    const int x = clc_granted_block(bars->clc_resp);
-                    fence_proxy_async();  // the answer has been read before the next one is written
-                    return x;
-                };
                 auto load_q = [&](const FwdItem& w, int t) {
                     if (!mbar_wait(&bars->q_empty[t], (n_q[t] & 1) ^ 1, ctx, kWaitFwd + 2)) { ok = false; return; }
                     mbar_expect_tx(&bars->q_full[t], C::kTileBytes);
@@ -207,14 +199,13 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     ++kv;
                 };
                 for (int k = 0; ok; ++k) {
-                    if (id >= 0) ask();
                     FwdItem w;
                     while (id >= 0 && !fwd_item(p, id, &w)) {  // skip the empty slots of smaller groups
-                        id = answer();
-                        if (id >= 0) ask();
+                        id = items.next(ctx, kWaitFwd + 1, &ok);
                     }
-                    bars->item[k % kSched] = id;
-                    mbar_arrive(&bars->sched_full[k % kSched]);  // release: the id is visible to whoever sees the phase
+                    if (id < 0) w.b = -1;
+                    bars->item[k % kSched] = w;
+                    mbar_arrive(&bars->sched_full[k % kSched]);  // release: the item is visible to whoever sees the phase
                     if (id < 0) break;
                     for (int j = 0; ok && j < w.t.n[1]; ++j) {
                         const int tok0 = tile_ref(w.L, w.t.j_begin + j).tok0;
@@ -223,10 +214,9 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                         if (j == 0 && ok) load_q(w, 1);
                         if (ok) load_kv(w, &p.tm_v, tok0);
                     }
-                    if (ok) id = answer();
+                    if (ok) id = items.next(ctx, kWaitFwd + 1, &ok);
                 }
-                // Nothing may land after the block has gone: the pending answer, and the loads when aborting.
-                if (asked) mbar_wait_drain(&bars->clc, n_clc & 1);
+                // nothing may land after the block has gone
                 if (bars->abort_flag != 0) {
                     for (int t = 0; t < 2; ++t)
                         if (n_q[t] > 0) mbar_wait_drain(&bars->q_full[t], (n_q[t] - 1) & 1);
@@ -256,11 +246,9 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             int k = 0;
             int n = 0, n1 = 0, m = 0, m1 = 0;  // steps of this tile and of tile 1: this item, the next one
             auto fetch = [&]() -> bool {
-                const int id = next_item(k++, kWaitFwd + 10);
-                m = 0;
-                if (id < 0) return false;
                 FwdItem w;
-                fwd_item(p, id, &w);
+                m = 0;
+                if (!next_item(k++, kWaitFwd + 10, &w)) return false;
                 m1 = w.t.n[1];
                 m = t ? m1 : w.t.n[0];
                 return true;
@@ -345,11 +333,9 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         uint32_t n_o[2] = {0, 0};
         bool ok = true;
         for (int k = 0; ok; ++k) {
-            const int id = next_item(k, kWaitFwd + 11);
-            // the four warps leave together, or the ones that stay would wait for the others below
-            if (!named_barrier_and(1, 128, id >= 0)) break;
             FwdItem w;
-            fwd_item(p, id, &w);
+            // the four warps leave together, or the ones that stay would wait for the others below
+            if (!named_barrier_and(1, 128, next_item(k, kWaitFwd + 11, &w))) break;
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
                 if (w.t.n[t] == 0) continue;
@@ -422,10 +408,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         uint32_t n_s = 0, n_it = 0;
         bool ok = true;
         for (int k = 0; ok; ++k) {
-            const int id = next_item(k, kWaitFwd + 14);
-            if (id < 0) break;
             FwdItem w;
-            fwd_item(p, id, &w);
+            if (!next_item(k, kWaitFwd + 14, &w)) break;
             const int n = t ? w.t.n[1] : w.t.n[0];
             if (n == 0) continue;
             float m_used = 0.f;   // running maximum in use, scaled to log2 units

@@ -26,13 +26,15 @@ enum WaitCode : int {
 // start first, and the tail of the grid consists of the lightest tiles only.
 constexpr int kUnitChunk = 8;
 __host__ __device__ inline void decode_block(long long idx, int units, int tiles, int* unit, int* rank) {
-    const long long per_chunk = static_cast<long long>(kUnitChunk) * tiles;
-    const int chunk = static_cast<int>(idx / per_chunk);
-    const int within = static_cast<int>(idx % per_chunk);
-    const int first = chunk * kUnitChunk;
+    // 32-bit arithmetic (the entry points admit fewer than 2^31 tiles): this runs on one thread between two
+    // work items, where a 64-bit division is a subroutine of several hundred clocks
+    const uint32_t i = static_cast<uint32_t>(idx), per_chunk = static_cast<uint32_t>(kUnitChunk) * tiles;
+    const uint32_t chunk = i / per_chunk;
+    const uint32_t within = i - chunk * per_chunk;
+    const int first = static_cast<int>(chunk) * kUnitChunk;
     const int in_chunk = (units - first) < kUnitChunk ? (units - first) : kUnitChunk;
-    *rank = within / in_chunk;
-    *unit = first + within % in_chunk;
+    *rank = static_cast<int>(within / static_cast<uint32_t>(in_chunk));
+    *unit = first + static_cast<int>(within) - *rank * in_chunk;
 }
 
 // Geometry of the shifted grouping (Algorithm 1): common to every kernel.
@@ -61,9 +63,10 @@ struct GroupLayout {
 };
 __host__ __device__ inline GroupLayout group_layout(const Geometry& geo, int s, int g) {
     GroupLayout L;
-    long long a = (static_cast<long long>(g) * geo.G + s) % geo.N;
+    int a = g * geo.G + s;  // in (-N, 2 N), and 2 N < 2^31
     if (a < 0) a += geo.N;
-    L.a0 = static_cast<int>(a);
+    if (a >= geo.N) a -= geo.N;
+    L.a0 = a;
     L.lenA = (geo.N - L.a0 < geo.G) ? geo.N - L.a0 : geo.G;
     L.lenB = geo.G - L.lenA;
     L.nA = (L.lenA + kTile - 1) / kTile;
@@ -109,8 +112,8 @@ __host__ __device__ inline TileRef subtile_ref(const GroupLayout& L, int n) {
 __host__ __device__ inline int first_key_tile(const GroupLayout& L, int i) { return (L.cut > 0 && i >= L.cut) ? L.cut : 0; }
 __host__ __device__ inline int end_query_tile(const GroupLayout& L, int j) { return (L.cut > 0 && j < L.cut) ? L.cut : L.nTiles; }
 
-// The forward kernel works on two neighbouring query tiles of a group at a time ("a pair"), which share
-// the key tiles they stream.  The pairs of a group are numbered by rank, most work first; the tiles on
+// The forward kernel and the dQ product kernel work on two neighbouring query tiles of a group at a time
+// ("a pair"), which share the key tiles they stream.  The pairs of a group are numbered by rank, most work first; the tiles on
 // either side of a cut (variant 2 of Appendix B) have no keys in common and are paired separately.
 __host__ __device__ inline int pairs_of_group(const GroupLayout& L) {
     return L.cut > 0 ? (L.nTiles - L.cut + 1) / 2 + (L.cut + 1) / 2 : (L.nTiles + 1) / 2;
@@ -191,6 +194,7 @@ constexpr int kSpillBlockElems = kTile * kSubTile;  // bf16 values per block
 struct alignas(64) BwdDkDvParams {
     CUtensorMap tm_k, tm_v;   // box (64, 1, 128, 1): the resident key tile
     CUtensorMap tm_q, tm_do;  // box (64, 1,  64, 1): streamed query sub-tiles
+    CUtensorMap tm_dk, tm_dv; // box (64, 1,  32, 1): stores, 32 key rows at a time
     const float* lse;
     const float* Dsum;
     __nv_bfloat16* dk;
@@ -198,24 +202,24 @@ struct alignas(64) BwdDkDvParams {
     long long dkv_tok_stride;  // elements between consecutive tokens of dk and dv (Hkv * d when dense)
     __nv_bfloat16* spill;      // dS^T blocks of this pass (spilling variant only)
     SpillPass pass;            // KV heads this launch covers (all of them when nothing is spilled)
-    int* counter;              // next work item; zero when the kernel starts
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
     float scale, scale_log2;
 };
 
-// dQ from spilled dS^T: dQ_i = scale * sum_j dS_ij K_j, one CTA per 128-query tile.
+// dQ from spilled dS^T: dQ_i = scale * sum_j dS_ij K_j, two neighbouring query tiles at a time.
 struct alignas(64) BwdDqSpillParams {
     CUtensorMap tm_k;   // box (64, 1, 128, 1): streamed key tiles
+    CUtensorMap tm_dq;  // box (64, 1,  32, 1): stores, 32 query rows at a time
     const __nv_bfloat16* spill;  // the blocks the dK,dV kernel of this pass wrote
     __nv_bfloat16* dq;
     long long dq_tok_stride;
-    int* counter;  // next work item; zero when the kernel starts
     SpillPass pass;
     int* status;
     int* host_status;
     Geometry geo;
+    int pairs_per_group;  // largest number of query tile pairs any group has
     float scale;
 };
 
@@ -223,8 +227,8 @@ struct alignas(64) BwdDqSpillParams {
 cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream);
 cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream);
 cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream);
-cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, int n_sm, cudaStream_t stream);  // persistent; p.spill != nullptr: spilling variant
-cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, int n_sm, cudaStream_t stream);  // persistent: one CTA per SM
+cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, cudaStream_t stream);  // p.spill != nullptr: spilling variant
+cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream);
 
 // Per-device kernel attribute set-up (dynamic shared memory sizes).
 cudaError_t configure_fwd();

@@ -223,6 +223,29 @@ __device__ __forceinline__ int clc_granted_block(const void* resp) {
     return ok ? static_cast<int>(x) : -1;
 }
 
+// The work items of a persistent block, for its one scheduling thread: the next block index, or -1 =
+// none left (not to be called again), or the wait expired (*ok becomes false).  To be called as late as the
+// answer's latency allows: a block that reserves its next item while it is still busy with a heavy one
+// takes it from a block that could start on it at once.
+struct ItemSource {
+    uint64_t* bar;  // one arrival
+    void* resp;     // 16 bytes of shared memory, 16-byte aligned
+    uint32_t n = 0;
+    __device__ __forceinline__ int next(const WaitCtx& ctx, int where, bool* ok) {
+        mbar_expect_tx(bar, 16);
+        clc_try_cancel(resp, bar);
+        if (!mbar_wait(bar, n & 1, ctx, where)) {
+            mbar_wait_drain(bar, n & 1);  // the answer must not land after the block has gone
+            *ok = false;
+            return -1;
+        }
+        ++n;
+        const int x = clc_granted_block(resp);
+        fence_proxy_async();  // the answer has been read before the next one is written
+        return x;
+    }
+};
+
 // Registers per thread of the executing warpgroup.  The shares of a block's warpgroups must not add up
 // to more than the block was launched with.
 template <int kRegs>

@@ -1,0 +1,53 @@
+"""The kernels' work items at the edges of their tiles, against the CPU oracle: groups of one tile, of an odd
+number of tiles (a query tile without a partner), last tiles that end inside, at and just past the 32 rows
+that one TMA store covers, more items than blocks and fewer.
+
+Tolerances as everywhere: bf16 results of fp32 sums against fp64 (one bf16 rounding of an o of up to 4 is
+8e-3 plus the rounding of the probabilities: 2e-2; 1e-2 relative L2 on the gradients).
+"""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import s2a_oracle as orc
+from paper_2309_12307_b200.inputs import make_inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def rel_l2(got, want):
+    return float(np.linalg.norm(got - want) / max(np.linalg.norm(want), 1e-30))
+
+
+@pytest.mark.parametrize("B,N,G,H,Hkv,d,kw", [
+    (1, 128, 128, 2, 2, 128, {}),                       # the smallest: one group, its shifted heads of two half tiles
+    (1, 256, 128, 2, 1, 64, {"n_unshifted": 2}),        # one tile per group, nothing shifted
+    (1, 768, 384, 4, 2, 128, {}),                       # three tiles
+    (1, 320, 160, 2, 2, 64, {}),                        # 32 rows in the last tile
+    (2, 336, 168, 2, 2, 128, {}),                       # 40 rows, 84-row runs where the group wraps
+    (1, 384, 192, 2, 2, 128, {"leak_free": True}),      # a cut inside a pair of tiles
+    (1, 1920, 640, 4, 4, 64, {"leak_free": True}),      # five tiles, cut after the third
+    (1, 640, 320, 2, 2, 128, {"swap_wrapped": True}),
+    (3, 1536, 128, 10, 2, 64, {"n_unshifted": 5}),      # more units than blocks
+    (1, 4992, 1664, 12, 12, 64, {}),                    # 13 tiles: more pairs than blocks, the last one single
+])
+def test_tile_edges_match_oracle(B, N, G, H, Hkv, d, kw):
+    from paper_2309_12307_b200 import binding as s2a
+
+    q, k, v, dO = make_inputs(B, N, H, Hkv, d, seed=31)
+    o_ref, lse_ref = orc.fwd(q, k, v, G, **kw)
+    grads_ref = orc.bwd(q, k, v, dO, G, **kw)
+    qd, kd, vd, dOd = (x.cuda() for x in (q, k, v, dO))
+    o, lse = (torch.full(s, float("nan"), dtype=t, device="cuda") for s, t in ((qd.shape, torch.bfloat16), ((B, H, N), torch.float32)))
+    s2a.s2a_fwd_ex(qd, kd, vd, G, o=o, lse=lse, **kw)
+    assert np.abs(o.double().cpu().numpy() - o_ref).max() <= 2e-2
+    assert np.abs(lse.double().cpu().numpy() - lse_ref).max() <= 2e-3
+    for fast in (False, True):
+        grads = tuple(torch.full_like(x, float("nan")) for x in (qd, kd, vd))
+        s2a.s2a_bwd_ex(qd, kd, vd, o, lse, dOd, G, fast=fast, dq=grads[0], dk=grads[1], dv=grads[2], **kw)
+        for got, want, name in zip(grads, grads_ref, ("dq", "dk", "dv")):
+            err = rel_l2(got.double().cpu().numpy(), want)
+            assert math.isfinite(err) and err <= 1e-2, (name, fast, err)
+    assert s2a.device_status() == (0, 0)
