@@ -2,29 +2,14 @@
 
 `s2_attn(q, k, v, G)` behaves like a differentiable function of q [B,N,H,d] and k, v [B,N,Hkv,d]
 (bf16, CUDA, contiguous): the forward runs `s2a_fwd_ex`, the backward `s2a_bwd_ex`.  Everything is
-computed by the CUDA library; torch only records the graph and owns the tensors.
+computed by the CUDA library; torch only records the graph (a C++ autograd function in
+csrc/torch_binding.cpp, so that the backward does not come back to Python) and owns the tensors.
 """
 from __future__ import annotations
 
 import torch
 
 from . import binding
-
-
-class _S2Attn(torch.autograd.Function):
-    @staticmethod
-    def forward(ctx, q, k, v, G, opts, fast_backward):
-        q, k, v = q.contiguous(), k.contiguous(), v.contiguous()
-        o, lse = binding.s2a_fwd_ex(q, k, v, G, **opts)
-        ctx.save_for_backward(q, k, v, o, lse)
-        ctx.G, ctx.opts, ctx.fast_backward = G, opts, fast_backward
-        return o
-
-    @staticmethod
-    def backward(ctx, dO):
-        q, k, v, o, lse = ctx.saved_tensors
-        dq, dk, dv = binding.s2a_bwd_ex(q, k, v, o, lse, dO.contiguous(), ctx.G, fast=ctx.fast_backward, **ctx.opts)
-        return dq, dk, dv, None, None, None
 
 
 def s2_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, G: int, *, scale: float | None = None,
@@ -39,5 +24,10 @@ def s2_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, G: int, *, scale:
     attended pair of a tile, within half of the free device memory) so that dq is a plain product, False
     the minimum (4 bytes per query row; dq then recomputes the scores).
     """
-    opts = dict(scale=scale, n_unshifted=n_unshifted, shift=shift, leak_free=leak_free, swap_wrapped=swap_wrapped)
-    return _S2Attn.apply(q, k, v, G, opts, fast_backward)
+    hot = binding._hot or binding._hot_for(_check, q, k, v)
+    o = hot.s2_attn(q, k, v, G, scale, n_unshifted, shift, binding._flags(leak_free, swap_wrapped), fast_backward)
+    return binding._result(o, "s2_attn", _check, q, k, v) if o is None else o
+
+
+def _check(q, k, v) -> None:
+    binding._dims(*(t.contiguous() for t in (q, k, v)))

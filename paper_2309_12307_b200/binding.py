@@ -1,13 +1,15 @@
-"""Python binding of the C-ABI in include/s2a.h (ctypes; argument marshalling only).
+"""Python binding of the C-ABI in include/s2a.h (argument marshalling only).
 
-torch is used for device memory and streams.  Every step of the operator runs in the CUDA
+The forward and backward entry points go through _s2a_torch.so (csrc/torch_binding.cpp), which checks the
+arguments, makes the outputs and calls the library without a trip through Python for each of them; the rest
+is ctypes.  torch is used for device memory and streams.  Every step of the operator runs in the CUDA
 library; there is no fallback: if libs2a.so is missing or a call fails, an exception is raised.
 Operation: S2-Attn, Algorithm 1 / Section 3.2 of the LongLoRA paper (see include/s2a.h).
 """
 from __future__ import annotations
 
 import ctypes
-import math
+import importlib.util
 import os
 
 import torch
@@ -28,7 +30,10 @@ EXPORTS = [
     "s2a_selftest_wait_expiry", "s2a_device_status", "s2a_status_string", "s2a_last_cuda_error", "s2a_version",
 ]
 
+TORCH_LIB_PATH = os.path.join(_PKG, "_s2a_torch.so")
+
 _lib = None
+_hot = None  # the module _s2a_torch
 
 
 class S2AError(RuntimeError):
@@ -82,6 +87,21 @@ def load() -> ctypes.CDLL:
     return lib
 
 
+def load_hot():
+    """Load _s2a_torch.so (built by paper_2309_12307_b200/build.py).  Raises if it is not there."""
+    global _hot
+    if _hot is None:
+        load()
+        if not os.path.exists(TORCH_LIB_PATH):
+            raise FileNotFoundError(
+                f"{TORCH_LIB_PATH} not found: build it with `python -m paper_2309_12307_b200.build` (needs g++)")
+        spec = importlib.util.spec_from_file_location("_s2a_torch", TORCH_LIB_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _hot = module
+    return _hot
+
+
 def status_string(status: int) -> str:
     return load().s2a_status_string(int(status)).decode()
 
@@ -98,6 +118,31 @@ def _stream_ptr(stream) -> int:
     if stream is None:
         stream = torch.cuda.current_stream()
     return int(stream.cuda_stream)
+
+
+def _given_stream(stream):
+    """What _s2a_torch takes for a stream: None (the current one) or its handle."""
+    return None if stream is None else int(stream.cuda_stream)
+
+
+def _hot_for(check, *args, **kw):
+    """The module _s2a_torch; if it has not been built, bad arguments are still named first."""
+    try:
+        return load_hot()
+    except FileNotFoundError:
+        check(*args, **kw)
+        raise
+
+
+def _result(r, what: str, check, *args, **kw):
+    """What a function of _s2a_torch returned: its tensors, the library's status if that is an error, or
+    None for an argument that the kernels would misread, which `check` names."""
+    if r is None:
+        check(*args, **kw)
+        raise RuntimeError(f"{what}: arguments refused")
+    if r.__class__ is int:
+        raise S2AError(r, what)
+    return r
 
 
 def _check(rc: int, what: str) -> None:
@@ -138,16 +183,29 @@ def _dims(q, k, v, cuda: bool = True):
 
 def _check_fwd_out(q, o, lse):
     B, N, H, d = q.shape
+    if o is not None:
+        _require(o, torch.bfloat16, "o", shape=q.shape, device=q.device)
+    if lse is not None:
+        _require(lse, torch.float32, "lse", shape=(B, H, N), device=q.device)
+
+
+def _check_fwd(q, k, v, o=None, lse=None):
+    _dims(q, k, v)
+    _check_fwd_out(q, o, lse)
+
+
+def _check_bwd(q, k, v, o, lse, dO, dq, dk, dv, workspace=None, optional=True):
+    """Every tensor of a backward; with `optional` the gradients may be None (they are made then)."""
+    _dims(q, k, v)
+    B, N, H, d = q.shape
     _require(o, torch.bfloat16, "o", shape=q.shape, device=q.device)
     _require(lse, torch.float32, "lse", shape=(B, H, N), device=q.device)
-
-
-def _check_bwd(q, k, o, lse, dO, dq, dk, dv):
-    _check_fwd_out(q, o, lse)
     _require(dO, torch.bfloat16, "dO", shape=q.shape, device=q.device)
-    _require(dq, torch.bfloat16, "dq", shape=q.shape, device=q.device)
-    _require(dk, torch.bfloat16, "dk", shape=k.shape, device=q.device)
-    _require(dv, torch.bfloat16, "dv", shape=k.shape, device=q.device)
+    for t, name, like in ((dq, "dq", q), (dk, "dk", k), (dv, "dv", k)):
+        if t is not None or not optional:
+            _require(t, torch.bfloat16, name, shape=like.shape, device=q.device)
+    if workspace is not None:
+        _check_workspace(workspace, q.device)
 
 
 def _check_workspace(ws, device):
@@ -165,66 +223,20 @@ def bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, budget: int) -> int:
     return int(load().s2a_bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, int(budget)))
 
 
-# Part of the device memory below which a fast workspace is taken without asking how much is free.
-_UNASKED_PART = 32
-_total_memory: dict[int, int] = {}
-
-
-def _default_workspace(B, N, H, Hkv, d, G, device, fast=True):
-    """Workspace for a call that was given none: the fast size within half of the free device memory,
-    or the minimum with fast=False.
-
-    Asking the driver for the free memory takes 70 to 220 us and more while the GPU is busy, longer than the
-    whole backward of a small problem (4 x 2000 tokens, 16 heads: 90 us).  So a workspace that is a small part
-    of the device's memory (5.7 GB of 180: Llama2-7B up to 16k tokens) is simply allocated, and the question
-    asked only when it is larger or that allocation fails."""
-    least = max(bwd_workspace_bytes(B, N, H, Hkv, d, G), 256)
-    if not fast:
-        return torch.empty(least, dtype=torch.uint8, device=device)
-    total = _total_memory.get(device.index)
-    if total is None:
-        total = _total_memory[device.index] = torch.cuda.get_device_properties(device).total_memory
-    need = bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, 1 << 62)
-    if need <= total // _UNASKED_PART:
-        try:
-            return torch.empty(max(need, least), dtype=torch.uint8, device=device)
-        except torch.OutOfMemoryError:
-            pass
-    free, _ = torch.cuda.mem_get_info(device)
-    need = max(least, bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, free // 2))
-    return torch.empty(need, dtype=torch.uint8, device=device)
-
-
 def s2a_fwd(q, k, v, G, o=None, lse=None, stream=None):
     """o [B,N,H,d] bf16 and lse [B,H,N] fp32 of S2-Attn (second half of the heads shifted by G/2)."""
-    B, N, H, Hkv, d = _dims(q, k, v)
-    if o is None:
-        o = torch.empty_like(q)
-    if lse is None:
-        lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device)
-    _check_fwd_out(q, o, lse)
-    rc = load().s2a_fwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), B, N, H, Hkv, d, G,
-                        _stream_ptr(stream))
-    _check(rc, "s2a_fwd")
-    return o, lse
+    hot = _hot or _hot_for(_check_fwd, q, k, v, o, lse)
+    r = hot.fwd(q, k, v, G, o, lse, _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_fwd", _check_fwd, q, k, v, o, lse)
 
 
 def s2a_bwd(q, k, v, o, lse, dO, G, dq=None, dk=None, dv=None, workspace=None, stream=None, fast=True):
     """dq, dk, dv (bf16) of sum(o * dO).  Without a workspace one is allocated: large enough for the
-    spilling backward (fast=True) or the minimum (fast=False: dq recomputes the scores)."""
-    B, N, H, Hkv, d = _dims(q, k, v)
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    _check_bwd(q, k, o, lse, dO, dq, dk, dv)
-    if workspace is None:
-        workspace = _default_workspace(B, N, H, Hkv, d, G, q.device, fast)
-    _check_workspace(workspace, q.device)
-    rc = load().s2a_bwd(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), dO.data_ptr(),
-                        dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), B, N, H, Hkv, d, G, workspace.data_ptr(),
-                        workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-    _check(rc, "s2a_bwd")
-    return dq, dk, dv
+    spilling backward within half of the free device memory (fast=True) or the minimum (fast=False: dq
+    recomputes the scores)."""
+    hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    r = hot.bwd(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, fast, _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_bwd", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
 
 
 def bwd_noalloc_max_rows() -> int:
@@ -238,57 +250,44 @@ def s2a_bwd_noalloc(q, k, v, o, lse, dO, G, dq, dk, dv, stream=None):
     tensor.  B*H*N must not exceed bwd_noalloc_max_rows().  Calls that may overlap on the GPU
     share the array and must be serialised (see include/s2a.h).
     """
-    B, N, H, Hkv, d = _dims(q, k, v)
-    _check_bwd(q, k, o, lse, dO, dq, dk, dv)
-    rc = load().s2a_bwd_noalloc(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(),
-                                dO.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), B, N, H, Hkv, d, G,
-                                _stream_ptr(stream))
-    _check(rc, "s2a_bwd_noalloc")
-    return dq, dk, dv
+    hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, optional=False)
+    r = hot.bwd_noalloc(q, k, v, o, lse, dO, G, dq, dk, dv, _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_bwd_noalloc", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, optional=False)
 
 
-def _packed_dims(qkv):
+def _check_packed(qkv, o=None, lse=None, dO=None, dqkv=None, workspace=None, backward=False):
     _require(qkv, torch.bfloat16, "qkv")
     if qkv.dim() != 5 or qkv.shape[2] != 3:
         raise ValueError(f"qkv must be [B, N, 3, H, d], not {tuple(qkv.shape)}")
     B, N, _, H, d = qkv.shape
-    return B, N, H, d
+    for t, name, dtype, shape in ((o, "o", torch.bfloat16, (B, N, H, d)), (lse, "lse", torch.float32, (B, H, N)),
+                                  (dO, "dO", torch.bfloat16, (B, N, H, d))):
+        if t is not None or backward:
+            _require(t, dtype, name, shape=shape, device=qkv.device)
+    if dqkv is not None:
+        _require(dqkv, torch.bfloat16, "dqkv", shape=qkv.shape, device=qkv.device)
+    if workspace is not None:
+        _check_workspace(workspace, qkv.device)
 
 
 def s2a_fwd_packed(qkv, G, o=None, lse=None, stream=None):
     """Forward on a packed qkv tensor [B, N, 3, H, d] (the calling convention of Algorithm 1)."""
-    B, N, H, d = _packed_dims(qkv)
-    o = torch.empty((B, N, H, d), dtype=torch.bfloat16, device=qkv.device) if o is None else o
-    lse = torch.empty((B, H, N), dtype=torch.float32, device=qkv.device) if lse is None else lse
-    _require(o, torch.bfloat16, "o", shape=(B, N, H, d), device=qkv.device)
-    _require(lse, torch.float32, "lse", shape=(B, H, N), device=qkv.device)
-    rc = load().s2a_fwd_packed(qkv.data_ptr(), o.data_ptr(), lse.data_ptr(), B, N, H, d, G, _stream_ptr(stream))
-    _check(rc, "s2a_fwd_packed")
-    return o, lse
+    hot = _hot or _hot_for(_check_packed, qkv, o, lse)
+    r = hot.fwd_packed(qkv, G, o, lse, _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_fwd_packed", _check_packed, qkv, o, lse)
 
 
 def s2a_bwd_packed(qkv, o, lse, dO, G, dqkv=None, workspace=None, stream=None, fast=True):
     """Backward on a packed qkv tensor; returns dqkv [B, N, 3, H, d]."""
-    B, N, H, d = _packed_dims(qkv)
-    dqkv = torch.empty_like(qkv) if dqkv is None else dqkv
-    _require(dqkv, torch.bfloat16, "dqkv", shape=qkv.shape, device=qkv.device)
-    _require(o, torch.bfloat16, "o", shape=(B, N, H, d), device=qkv.device)
-    _require(dO, torch.bfloat16, "dO", shape=(B, N, H, d), device=qkv.device)
-    _require(lse, torch.float32, "lse", shape=(B, H, N), device=qkv.device)
-    if workspace is None:
-        workspace = _default_workspace(B, N, H, H, d, G, qkv.device, fast)
-    _check_workspace(workspace, qkv.device)
-    rc = load().s2a_bwd_packed(qkv.data_ptr(), o.data_ptr(), lse.data_ptr(), dO.data_ptr(), dqkv.data_ptr(), B, N, H, d, G,
-                               workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-    _check(rc, "s2a_bwd_packed")
-    return dqkv
+    hot = _hot or _hot_for(_check_packed, qkv, o, lse, dO, dqkv, workspace, backward=True)
+    r = hot.bwd_packed(qkv, o, lse, dO, G, dqkv, workspace, fast, _given_stream(stream))
+    return _result(r, "s2a_bwd_packed", _check_packed, qkv, o, lse, dO, dqkv, workspace, backward=True)
 
 
 def s2a_bwd_stage(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, stage, stream=None):
     """Enqueue one kernel of the backward: 0 = D preprocess, 1 = dk/dv, 2 = dq (profiling aid)."""
     B, N, H, Hkv, d = _dims(q, k, v)
-    _check_bwd(q, k, o, lse, dO, dq, dk, dv)
-    _check_workspace(workspace, q.device)
+    _check_bwd(q, k, v, o, lse, dO, dq, dk, dv, workspace, optional=False)
     rc = load().s2a_bwd_stage(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), dO.data_ptr(),
                               dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), B, N, H, Hkv, d, G, workspace.data_ptr(),
                               workspace.numel() * workspace.element_size(), int(stage), _stream_ptr(stream))
@@ -308,37 +307,17 @@ def s2a_fwd_ex(q, k, v, G, scale=None, n_unshifted=None, shift=None, leak_free=F
     """Generalised forward: heads [0, n_unshifted) unshifted, the rest rolled by -shift tokens;
     leak_free=True cuts the wrapped group of the shifted heads at the wrap (Appendix B, variant 2);
     swap_wrapped=True makes its two parts change places (variant 3)."""
-    B, N, H, Hkv, d = _dims(q, k, v)
-    scale = 1.0 / math.sqrt(d) if scale is None else scale
-    n_unshifted = H // 2 if n_unshifted is None else n_unshifted
-    shift = G // 2 if shift is None else shift
-    o = torch.empty_like(q) if o is None else o
-    lse = torch.empty((B, H, N), dtype=torch.float32, device=q.device) if lse is None else lse
-    _check_fwd_out(q, o, lse)
-    rc = load().s2a_fwd_ex(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), B, N, H, Hkv, d, G,
-                           scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), _stream_ptr(stream))
-    _check(rc, "s2a_fwd_ex")
-    return o, lse
+    hot = _hot or _hot_for(_check_fwd, q, k, v, o, lse)
+    r = hot.fwd_ex(q, k, v, G, scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), o, lse, _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_fwd_ex", _check_fwd, q, k, v, o, lse)
 
 
 def s2a_bwd_ex(q, k, v, o, lse, dO, G, scale=None, n_unshifted=None, shift=None, leak_free=False, workspace=None,
                stream=None, dq=None, dk=None, dv=None, swap_wrapped=False, fast=True):
-    B, N, H, Hkv, d = _dims(q, k, v)
-    scale = 1.0 / math.sqrt(d) if scale is None else scale
-    n_unshifted = H // 2 if n_unshifted is None else n_unshifted
-    shift = G // 2 if shift is None else shift
-    dq = torch.empty_like(q) if dq is None else dq
-    dk = torch.empty_like(k) if dk is None else dk
-    dv = torch.empty_like(v) if dv is None else dv
-    _check_bwd(q, k, o, lse, dO, dq, dk, dv)
-    if workspace is None:
-        workspace = _default_workspace(B, N, H, Hkv, d, G, q.device, fast)
-    _check_workspace(workspace, q.device)
-    rc = load().s2a_bwd_ex(q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(), lse.data_ptr(), dO.data_ptr(),
-                           dq.data_ptr(), dk.data_ptr(), dv.data_ptr(), B, N, H, Hkv, d, G, scale, n_unshifted, shift,
-                           _flags(leak_free, swap_wrapped), workspace.data_ptr(), workspace.numel() * workspace.element_size(), _stream_ptr(stream))
-    _check(rc, "s2a_bwd_ex")
-    return dq, dk, dv
+    hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    r = hot.bwd_ex(q, k, v, o, lse, dO, G, scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), dq, dk, dv, workspace, fast,
+                   _given_stream(stream))
+    return r if r.__class__ is tuple else _result(r, "s2a_bwd_ex", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
 
 
 def s2a_fwd_bwd_host(host_in, host_out, dev, G, workspace, stream=None):

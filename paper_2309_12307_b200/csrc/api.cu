@@ -152,6 +152,25 @@ int check_default_shape(int N, int H, int d, int G) {
     return S2A_OK;
 }
 
+// Largest value of `count` over the groups of both partitions.  All groups of a partition are alike but the
+// one that wraps around the end of the sequence, so two of them are looked at however many there are.
+template <typename Count>
+int most_over_groups(const Geometry& g, Count count) {
+    int most = 0;
+    const int shifts[2] = {0, g.shift};
+    for (int which = 0; which < 2; ++which) {
+        if ((which == 0 && g.n_unshifted == 0) || (which == 1 && g.n_unshifted == g.H)) continue;
+        const int s = shifts[which], r = ((s % g.G) + g.G) % g.G;
+        // the group that starts at token N - G + r: it wraps unless r = 0
+        const int wraps = ((g.N - g.G + r - s) / g.G % g.groups + g.groups) % g.groups;
+        for (int grp : {wraps, (wraps + 1) % g.groups}) {
+            const int n = count(group_layout(g, s, grp));
+            if (n > most) most = n;
+        }
+    }
+    return most;
+}
+
 Geometry make_geometry(int B, int N, int H, int Hkv, int G, int n_unshifted, int shift, unsigned flags = 0u) {
     Geometry g;
     g.B = B, g.N = N, g.H = H, g.Hkv = Hkv, g.G = G;
@@ -161,30 +180,12 @@ Geometry make_geometry(int B, int N, int H, int Hkv, int G, int n_unshifted, int
     g.leak_free = (flags & S2A_FLAG_LEAK_FREE) ? 1 : 0;
     g.swap_wrapped = (flags & S2A_FLAG_SWAP_WRAPPED) ? 1 : 0;
     // the grid has one slot per (unit, tile rank); groups with fewer tiles leave their last slots idle
-    g.tiles_per_group = 0;
-    const int shifts[2] = {0, shift};
-    for (int which = 0; which < 2; ++which) {
-        if ((which == 0 && n_unshifted == 0) || (which == 1 && n_unshifted == H)) continue;
-        for (int grp = 0; grp < g.groups; ++grp) {
-            const int n = group_layout(g, shifts[which], grp).nTiles;
-            if (n > g.tiles_per_group) g.tiles_per_group = n;
-        }
-    }
+    g.tiles_per_group = most_over_groups(g, [](const GroupLayout& L) { return L.nTiles; });
     return g;
 }
-
 // Largest number of query tile pairs any group has (see tile_pair).
 int most_pairs(const Geometry& g) {
-    int most = 0;
-    const int shifts[2] = {0, g.shift};
-    for (int which = 0; which < 2; ++which) {
-        if ((which == 0 && g.n_unshifted == 0) || (which == 1 && g.n_unshifted == g.H)) continue;
-        for (int grp = 0; grp < g.groups; ++grp) {
-            const int n = pairs_of_group(group_layout(g, shifts[which], grp));
-            if (n > most) most = n;
-        }
-    }
-    return most;
+    return most_over_groups(g, [](const GroupLayout& L) { return pairs_of_group(L); });
 }
 
 constexpr float kLog2eHost = 1.4426950408889634f;
@@ -349,16 +350,6 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     const Geometry geo = make_geometry(B, N, H, Hkv, G, n_unshifted, shift, flags);
     float* Dsum = static_cast<float*>(workspace);
 
-    BwdDqParams pq;
-    memset(&pq, 0, sizeof pq);
-    if ((rc = make_tmap(&pq.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
-    if ((rc = make_tmap(&pq.tm_do, dO, d, H, N, B, kTile)) != S2A_OK) return rc;
-    if ((rc = make_tmap(&pq.tm_k, k, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
-    if ((rc = make_tmap(&pq.tm_v, v, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
-    pq.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
-    pq.lse = lse, pq.Dsum = Dsum, pq.dq = static_cast<__nv_bfloat16*>(dq);
-    pq.status = ds->status_ptr, pq.host_status = ds->host_word_dev, pq.geo = geo, pq.scale = scale, pq.scale_log2 = scale * kLog2eHost;
-
     BwdDkDvParams pk;
     memset(&pk, 0, sizeof pk);
     if ((rc = make_tmap(&pk.tm_k, k, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
@@ -402,6 +393,14 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
             if (e != cudaSuccess) return cuda_fail(e);
         }
         if (stages & kStageDq) {
+            BwdDqParams pq;
+            memset(&pq, 0, sizeof pq);
+            if ((rc = make_tmap(&pq.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
+            if ((rc = make_tmap(&pq.tm_do, dO, d, H, N, B, kTile)) != S2A_OK) return rc;
+            pq.tm_k = pk.tm_k, pq.tm_v = pk.tm_v;
+            pq.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
+            pq.lse = lse, pq.Dsum = Dsum, pq.dq = static_cast<__nv_bfloat16*>(dq);
+            pq.status = ds->status_ptr, pq.host_status = ds->host_word_dev, pq.geo = geo, pq.scale = scale, pq.scale_log2 = scale * kLog2eHost;
             e = launch_bwd_dq(pq, d, st);
             if (e != cudaSuccess) return cuda_fail(e);
         }
@@ -411,11 +410,11 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     pk.spill = reinterpret_cast<__nv_bfloat16*>(base + min_bytes);
     BwdDqSpillParams ps;
     memset(&ps, 0, sizeof ps);
-    ps.tm_k = pq.tm_k;
+    ps.tm_k = pk.tm_k;
     if ((rc = make_tmap(&ps.tm_dq, dq, d, H, N, B, 32, ts.dq)) != S2A_OK) return rc;
     ps.pairs_per_group = most_pairs(geo);
     ps.spill = pk.spill;
-    ps.dq = pq.dq, ps.dq_tok_stride = pq.dq_tok_stride;
+    ps.dq = static_cast<__nv_bfloat16*>(dq), ps.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
     ps.status = ds->status_ptr, ps.host_status = ds->host_word_dev, ps.geo = geo, ps.scale = scale;
     for (int hk0 = 0; hk0 < Hkv; hk0 += static_cast<int>(nk_fit)) {
         const int nk = Hkv - hk0 < static_cast<int>(nk_fit) ? Hkv - hk0 : static_cast<int>(nk_fit);
