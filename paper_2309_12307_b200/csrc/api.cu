@@ -37,6 +37,7 @@ struct DeviceState {
     int* status_ptr = nullptr;        // device address of g_status_word
     volatile int* host_word = nullptr;  // this device's mirror, host address
     int* host_word_dev = nullptr;     // the same word as the device sees it
+    int n_sm = 0;                     // multiprocessors
     // s2a_fwd_bwd_host only: copy streams and the events that order them against the caller's stream
     bool host_path_ready = false;
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
@@ -70,6 +71,8 @@ int prepare_device(DeviceState** out) {
         e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
         if (e != cudaSuccess) return cuda_fail(e);
         if (major != 10) return S2A_ERR_UNSUPPORTED;
+        e = cudaDeviceGetAttribute(&ds.n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return cuda_fail(e);
         if (!g_encode) {
             void* fn = nullptr;
             cudaDriverEntryPointQueryResult qres;
@@ -184,8 +187,20 @@ Geometry make_geometry(int B, int N, int H, int Hkv, int G, int n_unshifted, int
     return g;
 }
 // Largest number of query tile pairs any group has (see tile_pair).
-int most_pairs(const Geometry& g) {
-    return most_over_groups(g, [](const GroupLayout& L) { return pairs_of_group(L); });
+int most_pairs(const Geometry& g, bool single) {
+    return most_over_groups(g, [single](const GroupLayout& L) { return pairs_of_group(L, single); });
+}
+// Whether the kernels that work on pairs of query tiles take single tiles instead: when the pairs of `heads`
+// heads are fewer than the multiprocessors.
+bool take_single_tiles(const Geometry& g, int heads, int n_sm) {
+    return static_cast<long long>(g.B) * heads * g.groups * most_pairs(g, false) <= n_sm;
+}
+
+// Whether launches are so short (some 50 us at most) that starting them early pays, see launch_kernel(): up to
+// 32 pairs of a query and a key tile, counted for head size 128, for each multiprocessor.
+bool is_short(const Geometry& g, int d, int n_sm) {
+    const double T = g.tiles_per_group;
+    return static_cast<double>(g.B) * g.H * g.groups * T * (T + 1) / 2 * d / 128 <= 32.0 * n_sm;
 }
 
 constexpr float kLog2eHost = 1.4426950408889634f;
@@ -261,9 +276,11 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     p.status = ds->status_ptr;
     p.host_status = ds->host_word_dev;
     p.geo = make_geometry(B, N, H, Hkv, G, n_unshifted, shift, flags);
-    p.pairs_per_group = most_pairs(p.geo);
+    p.single = take_single_tiles(p.geo, H, ds->n_sm);
+    p.pairs_per_group = most_pairs(p.geo, p.single);
+    p.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * 4);  // q, k, v, o
     p.scale_log2 = scale * kLog2eHost;
-    cudaError_t e = launch_fwd(p, d, static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_fwd(p, d, static_cast<cudaStream_t>(stream), is_short(p.geo, d, ds->n_sm));
     return e == cudaSuccess ? S2A_OK : cuda_fail(e);
 }
 }  // namespace
@@ -364,6 +381,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     pk.status = ds->status_ptr, pk.host_status = ds->host_word_dev, pk.geo = geo, pk.scale = scale, pk.scale_log2 = scale * kLog2eHost;
     pk.spill = nullptr;
     pk.pass.hk0 = 0, pk.pass.nk = Hkv;
+    pk.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * (2 * (H / Hkv) + 2));  // q and dO of every query head, k, v
 
     PreParams pp;
     pp.o = static_cast<const __nv_bfloat16*>(o), pp.dO = static_cast<const __nv_bfloat16*>(dO), pp.Dsum = Dsum;
@@ -381,10 +399,11 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     if (nk_fit > static_cast<size_t>(Hkv)) nk_fit = Hkv;
     if (stages != kStageAll && nk_fit < static_cast<size_t>(Hkv)) nk_fit = 0;
 
+    const bool overlap = is_short(geo, d, ds->n_sm);
     char* base = static_cast<char*>(workspace);
     cudaError_t e;
     if (stages & kStagePre) {
-        e = launch_bwd_preprocess(pp, d, st);
+        e = launch_bwd_preprocess(pp, d, st, overlap);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     if (nk_fit == 0) {
@@ -401,7 +420,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
             pq.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
             pq.lse = lse, pq.Dsum = Dsum, pq.dq = static_cast<__nv_bfloat16*>(dq);
             pq.status = ds->status_ptr, pq.host_status = ds->host_word_dev, pq.geo = geo, pq.scale = scale, pq.scale_log2 = scale * kLog2eHost;
-            e = launch_bwd_dq(pq, d, st);
+            e = launch_bwd_dq(pq, d, st, overlap);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         return S2A_OK;
@@ -412,20 +431,22 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     memset(&ps, 0, sizeof ps);
     ps.tm_k = pk.tm_k;
     if ((rc = make_tmap(&ps.tm_dq, dq, d, H, N, B, 32, ts.dq)) != S2A_OK) return rc;
-    ps.pairs_per_group = most_pairs(geo);
     ps.spill = pk.spill;
     ps.dq = static_cast<__nv_bfloat16*>(dq), ps.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
     ps.status = ds->status_ptr, ps.host_status = ds->host_word_dev, ps.geo = geo, ps.scale = scale;
+    ps.chunk = kUnitChunk;  // what streams through this kernel, dS, is read once: 4 to 16 units make no difference
     for (int hk0 = 0; hk0 < Hkv; hk0 += static_cast<int>(nk_fit)) {
         const int nk = Hkv - hk0 < static_cast<int>(nk_fit) ? Hkv - hk0 : static_cast<int>(nk_fit);
         pk.pass.hk0 = hk0, pk.pass.nk = nk;
         ps.pass = pk.pass;
+        ps.single = take_single_tiles(geo, nk * (H / Hkv), ds->n_sm);
+        ps.pairs_per_group = most_pairs(geo, ps.single);
         if (stages & kStageDkDv) {
             e = launch_bwd_dkdv(pk, d, st);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         if (stages & kStageDq) {
-            e = launch_bwd_dq_spill(ps, d, st);
+            e = launch_bwd_dq_spill(ps, d, st, overlap);
             if (e != cudaSuccess) return cuda_fail(e);
         }
     }

@@ -49,6 +49,8 @@ __device__ __forceinline__ int mod_pos(int x, int n) {
 template <int HD>
 __global__ void __launch_bounds__(256) s2a_bwd_preprocess_kernel(const PreParams p) {
     constexpr int kThreadsPerRow = HD / 8;
+    release_successor();
+    wait_for_predecessor();
     const long long n_rows = static_cast<long long>(p.B) * p.N * p.H;
     const long long gtid = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     const long long row = gtid / kThreadsPerRow;  // (b * N + t) * H + h
@@ -234,12 +236,6 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
-    // then return at once instead of each running into its own time limit.
-    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
-    __syncthreads();
-    if (bars->abort_flag != 0) return;
-    __syncthreads();
     const Geometry& geo = p.geo;
 
     const int Tg = geo.tiles_per_group;
@@ -276,7 +272,6 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
             mbar_init(&bars->k_full[x], 1);
             mbar_init(&bars->k_empty[x], 1);
         }
-        bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
         tma_prefetch_desc(&p.tm_do);
@@ -287,10 +282,19 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
         tmem_alloc(&bars->tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
+    wait_for_predecessor();
+    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
+    // then return at once instead of each running into its own time limit.
+    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    release_successor();
     const uint32_t tmem_base = bars->tmem_slot;
+    if (bars->abort_flag != 0) {
+        if (warp == 3) tmem_dealloc(tmem_base, C::kTmemCols);
+        return;
+    }
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
     constexpr uint32_t kColAcc = 0, kColS = 128, kColP = 384;
 
@@ -548,10 +552,12 @@ __device__ __forceinline__ HeadWalk head_walk(const Geometry& geo, int hq, int t
 struct DkDvItem {
     int b, hk, tk0, k_valid, total_steps;
 };
-__device__ __forceinline__ DkDvItem dkdv_item(const Geometry& geo, const SpillPass& pass, long long id) {
+__device__ __forceinline__ DkDvItem dkdv_item(const BwdDkDvParams& p, long long id) {
+    const Geometry& geo = p.geo;
+    const SpillPass& pass = p.pass;
     DkDvItem t;
     int unit, j0;
-    decode_block(id, geo.B * pass.nk * geo.groups, geo.tiles_per_group, &unit, &j0);
+    decode_block(id, geo.B * pass.nk * geo.groups, geo.tiles_per_group, &unit, &j0, p.chunk);
     const int g0 = unit % geo.groups;
     const int rep = geo.H / geo.Hkv;
     t.hk = pass.hk0 + (unit / geo.groups) % pass.nk;
@@ -704,7 +710,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                 for (int k = 0; ok; ++k) {
                     // the next item that has work; the other warps only see real items and the end marker
                     DkDvItem t;
-                    while (id >= 0 && (t = dkdv_item(geo, p.pass, id)).total_steps == 0) {
+                    while (id >= 0 && (t = dkdv_item(p, id)).total_steps == 0) {
                         id = items.next(ctx, kWaitBwdDkDv + 10, &ok);
                     }
                     if (id < 0) t.total_steps = 0;
@@ -1137,7 +1143,7 @@ __device__ __forceinline__ bool dq_spill_item(const BwdDqSpillParams& p, int id,
     const int heads = p.pass.nk * rep;
     const int units = geo.B * heads * geo.groups;
     int unit, rank;
-    decode_block(id, units, p.pairs_per_group, &unit, &rank);
+    decode_block(id, units, p.pairs_per_group, &unit, &rank, p.chunk);
     unit = units - 1 - unit;
     const int g = unit % geo.groups;
     w->h = p.pass.hk0 * rep + (unit / geo.groups) % heads;
@@ -1145,8 +1151,8 @@ __device__ __forceinline__ bool dq_spill_item(const BwdDqSpillParams& p, int id,
     w->hk = w->h / rep;
     w->unit = unit;
     w->L = group_layout(geo, (w->h < geo.n_unshifted) ? 0 : geo.shift, g);
-    if (rank >= pairs_of_group(w->L)) return false;
-    w->t = tile_pair(w->L, rank);
+    if (rank >= pairs_of_group(w->L, p.single)) return false;
+    w->t = tile_pair(w->L, rank, p.single);
     return true;
 }
 
@@ -1161,10 +1167,6 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
 
-    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
-    __syncthreads();
-    if (bars->abort_flag != 0) return;
-    __syncthreads();
     const int Tg = p.geo.tiles_per_group;
 
     if (threadIdx.x == 0) {
@@ -1179,7 +1181,6 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
         for (int x = 0; x < C::kSched; ++x) mbar_init(&bars->sched_full[x], 1);
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->clc, 1);
-        bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_k);
         tma_prefetch_desc(&p.tm_dq);
@@ -1188,10 +1189,19 @@ __global__ void __launch_bounds__(DqSpillCfg<HD>::kThreads, 1) s2a_bwd_dq_spill_
         tmem_alloc(&bars->tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
+    wait_for_predecessor();
+    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later CTAs
+    // then return at once instead of each running into its own time limit.
+    if (threadIdx.x == 0) bars->abort_flag = *reinterpret_cast<volatile int*>(p.status);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    release_successor();
     const uint32_t tmem_base = bars->tmem_slot;
+    if (bars->abort_flag != 0) {
+        if (warp == 1) tmem_dealloc(tmem_base, C::kTmemCols);
+        return;
+    }
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
     auto next_item = [&](int k, int where, DqSpillItem* w) -> bool {
         if (!mbar_wait_uniform(&bars->sched_full[k % C::kSched], (k / C::kSched) & 1, ctx, where)) return false;
@@ -1361,41 +1371,39 @@ cudaError_t configure_bwd() {
     return e != cudaSuccess ? e : configure_all<128>();
 }
 
-cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream) {
+cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream, bool overlap) {
     const long long threads = static_cast<long long>(p.B) * p.N * p.H * (d / 8);
     const unsigned grid = static_cast<unsigned>((threads + 255) / 256);
-    if (d == 64) s2a_bwd_preprocess_kernel<64><<<grid, 256, 0, stream>>>(p);
-    else s2a_bwd_preprocess_kernel<128><<<grid, 256, 0, stream>>>(p);
-    return cudaGetLastError();
+    return d == 64 ? launch_kernel(s2a_bwd_preprocess_kernel<64>, grid, 256, 0, stream, p, overlap)
+                   : launch_kernel(s2a_bwd_preprocess_kernel<128>, grid, 256, 0, stream, p, overlap);
 }
 
-cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream) {
+cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream, bool overlap) {
     const Geometry& g = p.geo;
     const unsigned grid = static_cast<unsigned>(static_cast<long long>(g.B) * g.H * g.groups * g.tiles_per_group);
-    if (d == 64) s2a_bwd_dq_kernel<64><<<grid, DqCfg<64>::kThreads, DqCfg<64>::kSmemBytes, stream>>>(p);
-    else s2a_bwd_dq_kernel<128><<<grid, DqCfg<128>::kThreads, DqCfg<128>::kSmemBytes, stream>>>(p);
-    return cudaGetLastError();
+    return d == 64 ? launch_kernel(s2a_bwd_dq_kernel<64>, grid, DqCfg<64>::kThreads, DqCfg<64>::kSmemBytes, stream, p, overlap)
+                   : launch_kernel(s2a_bwd_dq_kernel<128>, grid, DqCfg<128>::kThreads, DqCfg<128>::kSmemBytes, stream, p, overlap);
 }
+
+namespace {
+template <int HD>
+cudaError_t launch_dkdv(const BwdDkDvParams& p, unsigned grid, cudaStream_t stream) {
+    return p.spill != nullptr ? launch_kernel(s2a_bwd_dkdv_kernel<HD, true>, grid, BwdCfg<HD>::kThreads, BwdCfg<HD>::kSmemBytes, stream, p, false)
+                              : launch_kernel(s2a_bwd_dkdv_kernel<HD, false>, grid, BwdCfg<HD>::kThreads, BwdCfg<HD>::kSmemBytes, stream, p, false);
+}
+}  // namespace
 
 cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, cudaStream_t stream) {
     const Geometry& g = p.geo;
     const unsigned grid = static_cast<unsigned>(static_cast<long long>(g.B) * p.pass.nk * g.groups * g.tiles_per_group);
-    if (p.spill != nullptr) {
-        if (d == 64) s2a_bwd_dkdv_kernel<64, true><<<grid, BwdCfg<64>::kThreads, BwdCfg<64>::kSmemBytes, stream>>>(p);
-        else s2a_bwd_dkdv_kernel<128, true><<<grid, BwdCfg<128>::kThreads, BwdCfg<128>::kSmemBytes, stream>>>(p);
-    } else {
-        if (d == 64) s2a_bwd_dkdv_kernel<64, false><<<grid, BwdCfg<64>::kThreads, BwdCfg<64>::kSmemBytes, stream>>>(p);
-        else s2a_bwd_dkdv_kernel<128, false><<<grid, BwdCfg<128>::kThreads, BwdCfg<128>::kSmemBytes, stream>>>(p);
-    }
-    return cudaGetLastError();
+    return d == 64 ? launch_dkdv<64>(p, grid, stream) : launch_dkdv<128>(p, grid, stream);
 }
 
-cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream) {
+cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream, bool overlap) {
     const Geometry& g = p.geo;
     const unsigned grid = static_cast<unsigned>(static_cast<long long>(g.B) * p.pass.nk * (g.H / g.Hkv) * g.groups * p.pairs_per_group);
-    if (d == 64) s2a_bwd_dq_spill_kernel<64><<<grid, DqSpillCfg<64>::kThreads, DqSpillCfg<64>::kSmemBytes, stream>>>(p);
-    else s2a_bwd_dq_spill_kernel<128><<<grid, DqSpillCfg<128>::kThreads, DqSpillCfg<128>::kSmemBytes, stream>>>(p);
-    return cudaGetLastError();
+    return d == 64 ? launch_kernel(s2a_bwd_dq_spill_kernel<64>, grid, DqSpillCfg<64>::kThreads, DqSpillCfg<64>::kSmemBytes, stream, p, overlap)
+                   : launch_kernel(s2a_bwd_dq_spill_kernel<128>, grid, DqSpillCfg<128>::kThreads, DqSpillCfg<128>::kSmemBytes, stream, p, overlap);
 }
 
 }  // namespace s2a

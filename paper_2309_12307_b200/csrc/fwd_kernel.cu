@@ -87,14 +87,14 @@ constexpr float kLazyRescale = 8.0f;
 // Work item `id`; false marks a slot of a group that has fewer pairs than the largest one.
 __device__ __forceinline__ bool fwd_item(const FwdParams& p, int id, FwdItem* w) {
     int unit, rank;
-    decode_block(id, p.geo.B * p.geo.H * p.geo.groups, p.pairs_per_group, &unit, &rank);
+    decode_block(id, p.geo.B * p.geo.H * p.geo.groups, p.pairs_per_group, &unit, &rank, p.chunk);
     const int g = unit % p.geo.groups;
     w->h = (unit / p.geo.groups) % p.geo.H;
     w->b = unit / (p.geo.groups * p.geo.H);
     w->hk = w->h / (p.geo.H / p.geo.Hkv);
     w->L = group_layout(p.geo, (w->h < p.geo.n_unshifted) ? 0 : p.geo.shift, g);
-    if (rank >= pairs_of_group(w->L)) return false;
-    w->t = tile_pair(w->L, rank);
+    if (rank >= pairs_of_group(w->L, p.single)) return false;
+    w->t = tile_pair(w->L, rank, p.single);
     return true;
 }
 
@@ -110,21 +110,6 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-
-    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later blocks
-    // then return at once instead of each running into its own time limit.
-    if (threadIdx.x == 0) {
-        int bad = *reinterpret_cast<volatile int*>(p.status);
-        if ((smem_u32(smem) & 1023u) != 0) {  // cannot happen: nothing precedes the dynamic array
-            bad = kWaitFwd + 99;
-            atomicCAS(p.status, 0, bad);
-            *reinterpret_cast<volatile int*>(p.host_status) = bad;
-        }
-        bars->abort_flag = bad;
-    }
-    __syncthreads();
-    if (bars->abort_flag != 0) return;
-    __syncthreads();
 
     if (threadIdx.x == 0) {
         for (int t = 0; t < 2; ++t) {
@@ -147,7 +132,6 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         }
         for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
         mbar_init(&bars->clc, 1);
-        bars->abort_flag = 0;
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
         tma_prefetch_desc(&p.tm_k);
@@ -158,10 +142,27 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         tmem_alloc(&bars->tmem_slot, C::kTmemCols);
         tmem_relinquish();
     }
+    wait_for_predecessor();
+    // A bounded wait that expired earlier (in any kernel) leaves the status word set: later blocks
+    // then return at once instead of each running into its own time limit.
+    if (threadIdx.x == 0) {
+        int bad = *reinterpret_cast<volatile int*>(p.status);
+        if ((smem_u32(smem) & 1023u) != 0) {  // cannot happen: nothing precedes the dynamic array
+            bad = kWaitFwd + 99;
+            atomicCAS(p.status, 0, bad);
+            *reinterpret_cast<volatile int*>(p.host_status) = bad;
+        }
+        bars->abort_flag = bad;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    release_successor();
     const uint32_t tmem_base = bars->tmem_slot;
+    if (bars->abort_flag != 0) {
+        if (warp == 13) tmem_dealloc(tmem_base, C::kTmemCols);
+        return;
+    }
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
 
     // Every consumer warp walks the same sequence of items, as the scheduling thread has decoded them (the
@@ -253,6 +254,15 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 m = t ? m1 : w.t.n[0];
                 return true;
             };
+            // K and V tiles that only the other query tile attends: each of them is handed back by both
+            // issuers, and only once it has landed (the hand-back belongs to the current use of its slot)
+            auto hand_back = [&](uint32_t from, uint32_t to) -> bool {
+                for (uint32_t x = from; x < to; ++x) {
+                    if (!wait_kv(x, kWaitFwd + 17)) return false;
+                    if (lane == 0) mbar_arrive(&bars->kv_empty[x % C::kRing]);
+                }
+                return true;
+            };
             // Item by item, one turn a step: P.V of the step, then the scores of the next one, which may be
             // the next item's first.  (The first pass, n = n1 = 0, only issues the first item's first scores.)
             uint32_t kv = 0;  // ring position of the item's K_0
@@ -260,6 +270,9 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             while (ok && more) {
                 const uint32_t kv_next = kv + 2 * n1;
                 const int turns = n > 0 ? n : 1;
+                // an item without this tile: its K and V first, or the scheduling thread, which publishes the next
+                // item when it has loaded all of them, and the wait for that item would wait for each other
+                if (n == 0) ok = hand_back(kv, kv_next);
 #pragma unroll 1
                 for (int j = 0; ok && j < turns; ++j) {
                     if (j == turns - 1) more = fetch();
@@ -307,12 +320,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                         __syncwarp();
                     }
                 }
-                // K and V tiles that only the other query tile attends: each of them is handed back by both
-                // issuers, and only once it has landed (the hand-back belongs to the current use of its slot)
-                for (uint32_t x = kv + 2 * n; ok && x < kv_next; ++x) {
-                    ok = wait_kv(x, kWaitFwd + 17);
-                    if (ok && lane == 0) mbar_arrive(&bars->kv_empty[x % C::kRing]);
-                }
+                if (ok && n > 0) ok = hand_back(kv + 2 * n, kv_next);
                 kv = kv_next, n = m, n1 = m1;
             }
             // MMAs already issued must finish before tensor memory is released
@@ -526,15 +534,11 @@ cudaError_t configure_fwd() {
     return e != cudaSuccess ? e : configure_one<128>();
 }
 
-cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream) {
+cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream, bool overlap) {
     const long long n_items = static_cast<long long>(p.geo.B) * p.geo.H * p.geo.groups * p.pairs_per_group;
-    const dim3 grid(static_cast<unsigned>(n_items));
-    if (d == 64) {
-        s2a_fwd_kernel<64><<<grid, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, stream>>>(p);
-    } else {
-        s2a_fwd_kernel<128><<<grid, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, stream>>>(p);
-    }
-    return cudaGetLastError();
+    const unsigned grid = static_cast<unsigned>(n_items);
+    return d == 64 ? launch_kernel(s2a_fwd_kernel<64>, grid, FwdCfg<64>::kThreads, FwdCfg<64>::kSmemBytes, stream, p, overlap)
+                   : launch_kernel(s2a_fwd_kernel<128>, grid, FwdCfg<128>::kThreads, FwdCfg<128>::kSmemBytes, stream, p, overlap);
 }
 
 }  // namespace s2a

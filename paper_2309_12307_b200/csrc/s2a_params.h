@@ -20,19 +20,32 @@ enum WaitCode : int {
 };
 
 // Block order shared by the tensor-core kernels.  A "unit" is one (batch, head, group); it has
-// `tiles` tiles whose cost falls with their rank (rank 0 = most work).  Units are taken in chunks of
-// kUnitChunk: inside a chunk all rank-0 tiles come first, then all rank-1 tiles, and so on.  So the
+// `tiles` tiles whose cost falls with their rank (rank 0 = most work).  Units are taken in chunks:
+// inside a chunk all rank-0 tiles come first, then all rank-1 tiles, and so on.  So the
 // blocks that run together belong to a few units (their streamed operands stay in L2), heavy tiles
 // start first, and the tail of the grid consists of the lightest tiles only.
 constexpr int kUnitChunk = 8;
-__host__ __device__ inline void decode_block(long long idx, int units, int tiles, int* unit, int* rank) {
+// Units in a chunk where their operands are what the L2 is for (`unit_bytes` each): as many as keep them
+// within a quarter of it, rounded down to a power of two (most counts of units divide by it), at least two.
+// A chunk's first tiles are its heavy ones, and those of the last chunk start when the launch is nearly over:
+// the more units it has, the more light tiles are left to even out the ends.  Measured with chunks of 8 and of
+// this rule: dK,dV 153 and 138 us on 4 x 2048 tokens with groups of 512 (64 units), 138 and 127 on a grouped-query
+// shape (16 units).  Chunks that overflow the L2 cost more than the ends: 32k, units of 8 MB, forward 1.98 ms
+// with 3, 1.99 with 8, 2.10 with 24; 100k, units of 26 MB, 17.4 ms with 2, 18.1 with 8, 20.6 with 64.
+constexpr long long kChunkBytes = 32ll << 20;
+__host__ __device__ inline int unit_chunk(long long unit_bytes) {
+    int n = 2;
+    while (n < 4096 && 2 * n * unit_bytes <= kChunkBytes) n *= 2;
+    return n;
+}
+__host__ __device__ inline void decode_block(long long idx, int units, int tiles, int* unit, int* rank, int unit_chunk = kUnitChunk) {
     // 32-bit arithmetic (the entry points admit fewer than 2^31 tiles): this runs on one thread between two
     // work items, where a 64-bit division is a subroutine of several hundred clocks
-    const uint32_t i = static_cast<uint32_t>(idx), per_chunk = static_cast<uint32_t>(kUnitChunk) * tiles;
+    const uint32_t i = static_cast<uint32_t>(idx), per_chunk = static_cast<uint32_t>(unit_chunk < units ? unit_chunk : units) * tiles;
     const uint32_t chunk = i / per_chunk;
     const uint32_t within = i - chunk * per_chunk;
-    const int first = static_cast<int>(chunk) * kUnitChunk;
-    const int in_chunk = (units - first) < kUnitChunk ? (units - first) : kUnitChunk;
+    const int first = static_cast<int>(chunk) * unit_chunk;
+    const int in_chunk = (units - first) < unit_chunk ? (units - first) : unit_chunk;
     *rank = static_cast<int>(within / static_cast<uint32_t>(in_chunk));
     *unit = first + static_cast<int>(within) - *rank * in_chunk;
 }
@@ -114,8 +127,11 @@ __host__ __device__ inline int end_query_tile(const GroupLayout& L, int j) { ret
 
 // The forward kernel and the dQ product kernel work on two neighbouring query tiles of a group at a time
 // ("a pair"), which share the key tiles they stream.  The pairs of a group are numbered by rank, most work first; the tiles on
-// either side of a cut (variant 2 of Appendix B) have no keys in common and are paired separately.
-__host__ __device__ inline int pairs_of_group(const GroupLayout& L) {
+// either side of a cut (variant 2 of Appendix B) have no keys in common and are paired separately.  Where
+// a problem has fewer pairs than the GPU has multiprocessors the kernels take single tiles instead
+// (`single`; a pair of which only the second tile exists).
+__host__ __device__ inline int pairs_of_group(const GroupLayout& L, bool single = false) {
+    if (single) return L.nTiles;
     return L.cut > 0 ? (L.nTiles - L.cut + 1) / 2 + (L.cut + 1) / 2 : (L.nTiles + 1) / 2;
 }
 struct TilePair {
@@ -123,7 +139,16 @@ struct TilePair {
     int j_begin;  // first key tile; tile t attends key tiles [j_begin, i[t]]
     int n[2];     // key tiles each attends: n[1] = n[0] + 1, n[0] = 0 when there is no second tile
 };
-__host__ __device__ inline TilePair tile_pair(const GroupLayout& L, int rank) {
+__host__ __device__ inline TilePair tile_pair(const GroupLayout& L, int rank, bool single = false) {
+    if (single) {
+        TilePair t;
+        t.i[1] = L.nTiles - 1 - rank;
+        t.i[0] = t.i[1] - 1;
+        t.j_begin = first_key_tile(L, t.i[1]);
+        t.n[1] = t.i[1] + 1 - t.j_begin;
+        t.n[0] = 0;
+        return t;
+    }
     int lo = 0, hi = L.nTiles;  // tiles [lo, hi) hold this pair
     if (L.cut > 0) {
         const int upper = (L.nTiles - L.cut + 1) / 2;
@@ -150,6 +175,8 @@ struct alignas(64) FwdParams {
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
     int pairs_per_group;  // largest number of query tile pairs any group has
+    bool single;          // work items are single tiles (see tile_pair)
+    int chunk;            // units in a chunk of the block order
     float scale_log2;     // softmax scale * log2(e)
 };
 
@@ -202,6 +229,7 @@ struct alignas(64) BwdDkDvParams {
     long long dkv_tok_stride;  // elements between consecutive tokens of dk and dv (Hkv * d when dense)
     __nv_bfloat16* spill;      // dS^T blocks of this pass (spilling variant only)
     SpillPass pass;            // KV heads this launch covers (all of them when nothing is spilled)
+    int chunk;                 // units in a chunk of the block order
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
@@ -220,15 +248,38 @@ struct alignas(64) BwdDqSpillParams {
     int* host_status;
     Geometry geo;
     int pairs_per_group;  // largest number of query tile pairs any group has
+    bool single;          // work items are single tiles (see tile_pair)
+    int chunk;            // units in a chunk of the block order
     float scale;
 };
 
+// With `overlap`, programmatic stream serialisation: the kernel's blocks may be set up (barriers, tensor memory,
+// descriptors) while the kernel before it in the stream runs its last blocks; see wait_for_predecessor().  The
+// entry points ask for it where a launch is short: a forward and a backward of 1024 tokens, 4 heads take 25.6 instead
+// of 31.7 us, of 4 x 2000 tokens in groups of 200 96 instead of 102, of 2 x 4096 tokens (grouped query) 275 instead
+// of 278.  On larger problems nothing is gained (Llama2-7B 8k: 647 against 629).  The dK,dV kernel is always
+// launched plainly: with the two instructions in it it was 2 to 3 % slower from 4 x 2048 tokens upwards.
+template <typename Params>
+cudaError_t launch_kernel(void (*kernel)(Params), unsigned grid, int threads, int smem_bytes, cudaStream_t stream, const Params& p, bool overlap) {
+    cudaLaunchConfig_t config = {};
+    config.gridDim = dim3(grid);
+    config.blockDim = dim3(static_cast<unsigned>(threads));
+    config.dynamicSmemBytes = static_cast<size_t>(smem_bytes);
+    config.stream = stream;
+    cudaLaunchAttribute attribute = {};
+    attribute.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attribute.val.programmaticStreamSerializationAllowed = 1;
+    config.attrs = &attribute;
+    config.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&config, kernel, p);
+}
+
 // Enqueue one kernel each on `stream`; return the launch error, if any.
-cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream);
-cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream);
-cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream);
+cudaError_t launch_fwd(const FwdParams& p, int d, cudaStream_t stream, bool overlap);
+cudaError_t launch_bwd_preprocess(const PreParams& p, int d, cudaStream_t stream, bool overlap);
+cudaError_t launch_bwd_dq(const BwdDqParams& p, int d, cudaStream_t stream, bool overlap);
 cudaError_t launch_bwd_dkdv(const BwdDkDvParams& p, int d, cudaStream_t stream);  // p.spill != nullptr: spilling variant
-cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream);
+cudaError_t launch_bwd_dq_spill(const BwdDqSpillParams& p, int d, cudaStream_t stream, bool overlap);
 
 // Per-device kernel attribute set-up (dynamic shared memory sizes).
 cudaError_t configure_fwd();

@@ -246,6 +246,12 @@ struct ItemSource {
     }
 };
 
+// Programmatic dependent launch: a kernel that launch_kernel() overlaps may start while its predecessor
+// in the stream is still running.  It waits here, before it touches global memory, until the predecessor is
+// done and its writes are visible, and lets its own successor start as early as it can.
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void release_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Registers per thread of the executing warpgroup.  The shares of a block's warpgroups must not add up
 // to more than the block was launched with.
 template <int kRegs>

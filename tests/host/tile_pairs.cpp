@@ -1,5 +1,6 @@
 // Host-side check of the forward kernel's work items (tile_pair in s2a_params.h): every query tile of a
-// group is in exactly one pair, with exactly the key tiles it attends, heaviest pair of a range first.
+// group is in exactly one pair (or is a single item of its own), with exactly the key tiles it attends,
+// heaviest of a range first.
 // Prints "ok" and returns 0, or says what failed.
 #include <cstdio>
 #include <vector>
@@ -18,12 +19,13 @@ int main() {
                     geo.B = 1, geo.N = G * groups, geo.H = 2, geo.Hkv = 2, geo.G = G, geo.groups = groups, geo.shift = shift;
                     geo.leak_free = variant == 1, geo.swap_wrapped = variant == 2;
                     for (int g = 0; g < groups; ++g) {
+                      for (bool single : {false, true}) {
                         const GroupLayout L = group_layout(geo, shift, g);
                         std::vector<int> seen(L.nTiles, 0);
                         int prev = 1 << 30;
-                        for (int r = 0; r < pairs_of_group(L); ++r) {
-                            const TilePair t = tile_pair(L, r);
-                            if (t.n[1] < 1 || t.n[0] != t.n[1] - 1 || t.i[0] != t.i[1] - 1) return std::printf("FAIL shape %d %d %d\n", G, g, r), 1;
+                        for (int r = 0; r < pairs_of_group(L, single); ++r) {
+                            const TilePair t = tile_pair(L, r, single);
+                            if (t.n[1] < 1 || t.n[0] != (single ? 0 : t.n[1] - 1) || t.i[0] != t.i[1] - 1) return std::printf("FAIL shape %d %d %d\n", G, g, r), 1;
                             const bool new_range = L.cut > 0 && t.i[1] == L.cut - 1;
                             if (t.n[1] > prev && !new_range) return std::printf("FAIL order %d %d %d\n", G, g, r), 1;
                             prev = t.n[1];
@@ -36,6 +38,7 @@ int main() {
                         }
                         for (int s : seen)
                             if (s != 1) return std::printf("FAIL tile left out %d %d\n", G, g), 1;
+                      }
                     }
                 }
     std::printf("ok\n");
