@@ -17,21 +17,26 @@
 //   warps 8-11       epilogue: O / l -> bf16 -> shared memory -> TMA store (or row stores, ragged tiles)
 //   warp 12          work items (cluster launch control: a block takes over blocks that were not launched
 //                    yet, heaviest first) and TMA loads, running ahead across items
-//   warps 13, 14     tcgen05 MMAs of query tile 0 / 1:  O += P V_j, S = Q K_{j+1}^T, O += P V_{j+1}, ...
+//   warps 13, 14     tcgen05 MMAs: the score products S = Q K_j^T of both tiles in turn / the products O += P V_j
 // While one tile's scores are in the softmax, the tensor cores work for the other tile; K and V tiles
 // are fetched once for the 256 query rows, which halves their L2 and shared-memory traffic.
-// Tensor memory: S0 [0,128)  S1 [128,256)  O0 [256,256+HD)  O1 [384,384+HD); P (bf16) over S.
+// The scores of a step are in registers 150 clocks after they are complete, and P has tensor memory columns of
+// its own, so a tile's next scores are computed while its softmax works on the present ones.  (With P over S the
+// chain scores -> softmax -> P V -> next scores of a tile, about 3700 clocks for a step of either tile, was what
+// bounded the kernel, with the special-function unit and the tensor pipe each busy half of the time.)
+// Tensor memory: O of either tile, P of either tile, then one score buffer (HD = 128) or two.
 //
 // The last work items of a launch decide how long it takes, so blocks ask for the next one late (when they
 // have issued their loads), and one thread decodes it for all warps.  Asking an item ahead and decoding it in
 // every warp with 64-bit divisions cost 86 against 73 us on 4 x 2048 tokens with groups of 512, 101 against 80
 // on a grouped-query shape (2 x 4096, groups of 1024, head size 64), 2 % on Llama2-7B 32k.
 //
-// What bounds it: the chain scores -> softmax -> P V -> next scores of a tile (clock stamps: about 2400
-// clocks in the softmax and 1100 in the two products of a step, with the other tile's step alongside); the
-// special-function unit and the tensor pipe are each busy about half of the time.  Measured against the
-// form it replaces (one query tile per block, two blocks per SM, two threads per row, scores read twice):
-// Llama2-7B 32k 1.94 against 2.38 ms a call, 8k 0.161 against 0.211, groups of 512 0.073 against 0.099.
+// What bounds it: the softmax (a step of both tiles keeps the special-function unit busy for 2048 clocks and the
+// tensor pipe for 2048) and, sustained, the power limit: 1244 TFLOP/s on Llama2-7B 32k, 0.92 of what the cuBLAS
+// loop sustains.  Microseconds a call in a loop: first form (one query tile per block, two blocks per SM, two threads
+// per row, scores read twice), two tiles with P over S, this form:
+//   Llama2-7B 32k 2383, 1982, 1768; 8k 211, 162, 145; causal 8k 610, 497, 449;
+//   groups of 512 99, 73, 70; groups of 200 (head size 64) 40, 32, 29; head size 64 at 32k 1800, 1514, 1374
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -49,8 +54,13 @@ struct FwdCfg {
     static constexpr int kStatBytes = 2 * 2 * kTile * 4;     // row statistics handed to the epilogue
     static constexpr int kBarBytes = 1024 + kStatBytes;
     static constexpr int kSmemBytes = (2 + kRing + 1) * kTileBytes + kBarBytes;
+    // Tensor memory columns: O of either tile, P of either tile (bf16, 64 columns), scores.  The scores of a step are
+    // in registers soon after they are complete, so for HD = 128, where O takes half of the columns, one
+    // score buffer serves both tiles in turn.
     static constexpr int kTmemCols = 512;
-    static constexpr int kColO = 256;
+    static constexpr int kColO = 0, kColP = 2 * HD, kColS = 2 * HD + 2 * 64;
+    static constexpr int kScoreBufs = (HD == 128) ? 1 : 2;
+    static_assert(kColS + kScoreBufs * kTile <= kTmemCols, "tensor memory");
     // registers per thread after the split; the launch gives kRegsLaunch to each of the 512
     static constexpr int kRegsLaunch = 128, kRegsSoftmax = 176, kRegsEpilogue = 80, kRegsIssue = 80;
     static_assert(2 * kRegsSoftmax + kRegsEpilogue + kRegsIssue <= 4 * kRegsLaunch, "register split");
@@ -66,8 +76,10 @@ struct FwdItem {
 struct FwdBars {
     uint64_t q_full[2], q_empty[2];
     uint64_t s_full[2];              // S of a tile's step is in tensor memory
+    uint64_t s_empty[2];             // a score buffer has been read into registers
     uint64_t p_full[2];              // P of keys [0, 96) of the step is in tensor memory (and O is rescaled)
     uint64_t p_rest[2];              // the other 32 keys
+    uint64_t p_empty[2];             // the P.V product of the step is done: P and O may be written
     uint64_t o_full[2], o_empty[2];  // an item's O is complete / has been read out
     uint64_t stat_full[2], stat_empty[2];
     uint64_t kv_full[8], kv_empty[8];
@@ -118,6 +130,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             mbar_init(&bars->q_full[t], 1);
             mbar_init(&bars->q_empty[t], 1);
             mbar_init(&bars->s_full[t], 1);
+            mbar_init(&bars->s_empty[t], 4);
+            mbar_init(&bars->p_empty[t], 1);
             mbar_init(&bars->p_full[t], 4);
             mbar_init(&bars->p_rest[t], 4);
             mbar_init(&bars->o_full[t], 1);
@@ -128,7 +142,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         }
         for (int x = 0; x < C::kRing; ++x) {
             mbar_init(&bars->kv_full[x], 1);
-            mbar_init(&bars->kv_empty[x], 2);  // one hand-back by each tile's issuer
+            mbar_init(&bars->kv_empty[x], 1);
         }
         for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
         mbar_init(&bars->clc, 1);
@@ -227,107 +241,82 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             }
             __syncwarp();
         } else if (warp <= 14) {
-            // ======================= MMA issuers: warp 13 for tile 0, warp 14 for tile 1 ==================
+            // ======================= MMA issuers: warp 13 for S = Q K^T, warp 14 for O += P V ============
             // The whole warp walks the loop so that addresses and descriptors stay warp-uniform values;
-            // only the MMA and commit instructions themselves are issued by one elected lane.  One warp
-            // for each tile: while one waits for a barrier the other keeps the tensor pipe fed (one warp for
-            // both tiles: 2.07 to 2.18 ms at 32k against 2.04).  A wait costs 100 to 200 clocks even when its
-            // phase is complete (barriers share shared memory with the operand reads), so K and V are waited
-            // for ahead of P: between P and the products that follow it, which are on the tile's critical
-            // path, there is only the wait for the rest of P.
+            // only the MMA and commit instructions themselves are issued by one elected lane.  Both take the
+            // tiles in turn: tile 0, tile 1 of key tile j, then of j + 1 (tile 0 has no products with the
+            // last key tile).  K tiles are in the even slots of the ring, V tiles in the odd ones.
             constexpr uint32_t idesc_s = idesc_bf16(128, kTile, 0, 0);  // S = Q K^T   (both K-major)
             constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);     // O += P V    (V is MN-major)
-            const int t = warp - 13;
-            const uint32_t dQ = desc_lo_k_major(smem_u32(sQ + t * C::kTileBytes)), aKV = smem_u32(sKV);
-            const uint32_t tS = tmem_base + t * kTile, tO = tmem_base + C::kColO + t * kTile;
-            uint32_t n_step = 0, n_q = 0, n_o = 0;  // P.V products, query tiles, outputs of this tile so far
-            auto wait_kv = [&](uint32_t x, int where) -> bool {
-                return mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, where);
-            };
-            int k = 0;
-            int n = 0, n1 = 0, m = 0, m1 = 0;  // steps of this tile and of tile 1: this item, the next one
-            auto fetch = [&]() -> bool {
+            const bool is_s = warp == 13;
+            const uint32_t aKV = smem_u32(sKV), dQ0 = desc_lo_k_major(smem_u32(sQ));
+            uint32_t kv = 0;                    // ring position of the item's K_0
+            uint32_t n_it[2] = {0, 0};          // items of either tile so far
+            uint32_t n_st[2] = {0, 0}, n_s = 0; // steps of either tile, score products
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
                 FwdItem w;
-                m = 0;
-                if (!next_item(k++, kWaitFwd + 10, &w)) return false;
-                m1 = w.t.n[1];
-                m = t ? m1 : w.t.n[0];
-                return true;
-            };
-            // K and V tiles that only the other query tile attends: each of them is handed back by both
-            // issuers, and only once it has landed (the hand-back belongs to the current use of its slot)
-            auto hand_back = [&](uint32_t from, uint32_t to) -> bool {
-                for (uint32_t x = from; x < to; ++x) {
-                    if (!wait_kv(x, kWaitFwd + 17)) return false;
-                    if (lane == 0) mbar_arrive(&bars->kv_empty[x % C::kRing]);
-                }
-                return true;
-            };
-            // Item by item, one turn a step: P.V of the step, then the scores of the next one, which may be
-            // the next item's first.  (The first pass, n = n1 = 0, only issues the first item's first scores.)
-            uint32_t kv = 0;  // ring position of the item's K_0
-            bool more = true, ok = true;
-            while (ok && more) {
-                const uint32_t kv_next = kv + 2 * n1;
-                const int turns = n > 0 ? n : 1;
-                // an item without this tile: its K and V first, or the scheduling thread, which publishes the next
-                // item when it has loaded all of them, and the wait for that item would wait for each other
-                if (n == 0) ok = hand_back(kv, kv_next);
+                if (!next_item(k, kWaitFwd + 10, &w)) break;
+                const int n1 = w.t.n[1], n0 = w.t.n[0];
 #pragma unroll 1
-                for (int j = 0; ok && j < turns; ++j) {
-                    if (j == turns - 1) more = fetch();
-                    const bool same = j + 1 < n, next = j == turns - 1 && m > 0, do_s = same || next, do_pv = j < n;
-                    const uint32_t xv = kv + 2 * j + 1, xk = same ? kv + 2 * (j + 1) : kv_next;
-                    if (do_pv) {
-                        if (j == 0 && !mbar_wait_uniform(&bars->o_empty[t], (n_o++ & 1) ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
-                        if (!wait_kv(xv, kWaitFwd + 6)) { ok = false; break; }
-                    }
-                    if (do_s) {
-                        if (next && !mbar_wait_uniform(&bars->q_full[t], n_q++ & 1, ctx, kWaitFwd + 4)) { ok = false; break; }
-                        if (!wait_kv(xk, kWaitFwd + 5)) { ok = false; break; }
-                    }
-                    if (do_pv) {
-                        const uint32_t dV = desc_lo_mn_major(aKV + (xv % C::kRing) * C::kTileBytes, C::kBoxBytes);
-                        if (!mbar_wait_uniform(&bars->p_full[t], n_step & 1, ctx, kWaitFwd + 8)) { ok = false; break; }
+                for (int h = 0; ok && h < 2 * n1; ++h) {
+                    const int t = h & 1, j = h >> 1, n = t ? n1 : n0;
+                    if (j >= n) continue;
+                    const uint32_t x = kv + 2 * j + (is_s ? 0 : 1);
+                    // what tile 0 has used, tile 1 need not wait for again
+                    if ((t == 0 || j >= n0) && !mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, kWaitFwd + 5)) { ok = false; break; }
+                    const uint32_t it = t ? n_it[1] : n_it[0], st = t ? n_st[1] : n_st[0];
+                    if (is_s) {
+                        if (j == 0 && !mbar_wait_uniform(&bars->q_full[t], it & 1, ctx, kWaitFwd + 4)) { ok = false; break; }
+                        const int buf = C::kScoreBufs == 1 ? 0 : t;
+                        const uint32_t use = C::kScoreBufs == 1 ? n_s : st;
+                        if (!mbar_wait_uniform(&bars->s_empty[buf], (use & 1) ^ 1, ctx, kWaitFwd + 6)) { ok = false; break; }
                         tc_fence_after();
-                        if (elect_one()) {
-#pragma unroll
-                            for (int kk = 0; kk < 6; ++kk) mma_ts(tO, tS + kk * 8, dV + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
-                        }
-                        __syncwarp();
-                        if (!mbar_wait_uniform(&bars->p_rest[t], n_step & 1, ctx, kWaitFwd + 9)) { ok = false; break; }
-                        ++n_step;
-                        tc_fence_after();
-                        if (elect_one()) {
-#pragma unroll
-                            for (int kk = 6; kk < 8; ++kk) mma_ts(tO, tS + kk * 8, dV + kk * kDescStepMn, idesc_o, 1);
-                            mma_commit(&bars->kv_empty[xv % C::kRing]);
-                            if (j == n - 1) mma_commit(&bars->o_full[t]);
-                        }
-                        __syncwarp();
-                    }
-                    if (do_s) {
-                        const uint32_t dK = desc_lo_k_major(aKV + (xk % C::kRing) * C::kTileBytes);
-                        tc_fence_after();
+                        const uint32_t dQ = dQ0 + t * (C::kTileBytes >> 4);
+                        const uint32_t dK = desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes);
+                        const uint32_t tS = tmem_base + C::kColS + buf * kTile;
                         if (elect_one()) {
 #pragma unroll
                             for (int kk = 0; kk < HD / 16; ++kk)
                                 mma_ss(tS, dQ + desc_step_k_major(kk, C::kBoxBytes), dK + desc_step_k_major(kk, C::kBoxBytes), idesc_s, kk > 0);
                             mma_commit(&bars->s_full[t]);
-                            mma_commit(&bars->kv_empty[xk % C::kRing]);
-                            if (same ? j + 2 == n : m == 1) mma_commit(&bars->q_empty[t]);
+                            if (t == 1) mma_commit(&bars->kv_empty[x % C::kRing]);  // tile 1 uses every K and V tile, and uses it last
+                            if (j == n - 1) mma_commit(&bars->q_empty[t]);
+                        }
+                        __syncwarp();
+                        ++n_s;
+                    } else {
+                        if (j == 0 && !mbar_wait_uniform(&bars->o_empty[t], (it & 1) ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
+                        const uint32_t dV = desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
+                        const uint32_t tP = tmem_base + C::kColP + t * 64, tO = tmem_base + C::kColO + t * HD;
+                        if (!mbar_wait_uniform(&bars->p_full[t], st & 1, ctx, kWaitFwd + 8)) { ok = false; break; }
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 0; kk < 6; ++kk) mma_ts(tO, tP + kk * 8, dV + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
+                        }
+                        __syncwarp();
+                        if (!mbar_wait_uniform(&bars->p_rest[t], st & 1, ctx, kWaitFwd + 9)) { ok = false; break; }
+                        tc_fence_after();
+                        if (elect_one()) {
+#pragma unroll
+                            for (int kk = 6; kk < 8; ++kk) mma_ts(tO, tP + kk * 8, dV + kk * kDescStepMn, idesc_o, 1);
+                            mma_commit(&bars->p_empty[t]);
+                            if (t == 1) mma_commit(&bars->kv_empty[x % C::kRing]);
+                            if (j == n - 1) mma_commit(&bars->o_full[t]);
                         }
                         __syncwarp();
                     }
+                    if (t) ++n_st[1], n_it[1] += j == n - 1;
+                    else ++n_st[0], n_it[0] += j == n - 1;
                 }
-                if (ok && n > 0) ok = hand_back(kv + 2 * n, kv_next);
-                kv = kv_next, n = m, n1 = m1;
+                kv += 2 * n1;
             }
             // MMAs already issued must finish before tensor memory is released
             if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
                 if (elect_one()) {
-                    mma_commit(&bars->drain[t]);
-                    mbar_wait_drain(&bars->drain[t], 0);
+                    mma_commit(&bars->drain[is_s]);
+                    mbar_wait_drain(&bars->drain[is_s], 0);
                 }
             }
             __syncwarp();
@@ -366,7 +355,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
 #pragma unroll
                 for (int c = 0; c < HD / 32; ++c) {
                     uint32_t r[32];
-                    tmem_ld_32x32(t_row + C::kColO + t * kTile + c * 32, r);
+                    tmem_ld_32x32(t_row + C::kColO + t * HD + c * 32, r);
                     tmem_wait_ld();
                     const uint32_t dst_s = smem_u32(sO) + (c >> 1) * C::kBoxBytes + row * 128;
                     uint4* dst_g = reinterpret_cast<uint4*>(orow + c * 32);
@@ -410,7 +399,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         const int quad = warp & 3;             // tensor-memory lane quadrant this warp may access
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-        const uint32_t tS = t_row + t * kTile;
+        const uint32_t tS = t_row + C::kColS + (C::kScoreBufs == 1 ? 0 : t * kTile), tP = t_row + C::kColP + t * 64;
         const float c2 = p.scale_log2;
         const uint64_t c2x2 = f2_pack(c2, c2);
         uint32_t n_s = 0, n_it = 0;
@@ -432,6 +421,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 tmem_ld_32x32(tS + 64, s[2]);
                 tmem_ld_32x32(tS + 96, s[3]);
                 tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive_warp(&bars->s_empty[C::kScoreBufs == 1 ? 0 : t]);
                 // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
                 // on the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
                 const bool last = (j == n - 1);
@@ -451,18 +442,20 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     for (int e = 2; e < 32; e += 2) mx4[c] = fmax3(mx4[c], __uint_as_float(s[c][e]), __uint_as_float(s[c][e + 1]));
                 }
                 const float m_new = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * c2;
+                // the P.V product of this tile's step before is done: P and O may be written
+                if (n_s > 0 && !mbar_wait_uniform(&bars->p_empty[t], (n_s - 1) & 1, ctx, kWaitFwd + 17)) { ok = false; break; }
+                tc_fence_after();
                 if (j == 0) {
                     m_used = m_new;
                 } else {
                     const bool need = (m_new - m_used) > kLazyRescale;
                     if (__any_sync(0xffffffffu, need)) {
-                        // s_full of this step also covers the P.V product of the step before, so O is quiescent here
                         const float alpha = need ? fast_exp2(m_used - m_new) : 1.0f;
                         l *= alpha;
 #pragma unroll 1
                         for (int c = 0; c < HD / 16; ++c) {
                             uint32_t o[16];
-                            const uint32_t t_o = t_row + C::kColO + t * kTile + c * 16;
+                            const uint32_t t_o = t_row + C::kColO + t * HD + c * 16;
                             tmem_ld_32x16(t_o, o);
                             tmem_wait_ld();
 #pragma unroll
@@ -486,8 +479,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                         sum[e & 1] = f2_add(sum[e & 1], f2_pack(p0, p1));
                         pk[e] = pack_bf16(p0, p1);
                     }
-                    // every score of the row is in registers, so P may go over the start of S: 16 packed columns
-                    tmem_st_32x16(tS + c * 16, pk);
+                    tmem_st_32x16(tP + c * 16, pk);
                     if (c >= 2) {
                         tmem_wait_st();
                         tc_fence_before();
