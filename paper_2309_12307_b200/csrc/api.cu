@@ -417,6 +417,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
             if ((rc = make_tmap(&pq.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
             if ((rc = make_tmap(&pq.tm_do, dO, d, H, N, B, kTile)) != S2A_OK) return rc;
             pq.tm_k = pk.tm_k, pq.tm_v = pk.tm_v;
+            pq.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * 4);  // q, dO, k, v
             pq.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
             pq.lse = lse, pq.Dsum = Dsum, pq.dq = static_cast<__nv_bfloat16*>(dq);
             pq.status = ds->status_ptr, pq.host_status = ds->host_word_dev, pq.geo = geo, pq.scale = scale, pq.scale_log2 = scale * kLog2eHost;

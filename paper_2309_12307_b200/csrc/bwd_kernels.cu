@@ -180,19 +180,25 @@ __device__ __forceinline__ void store_acc_rows(const CUtensorMap* tm, uint8_t* s
 // ------------------------------------------------------------------------------------------------
 // 2. dQ
 // ------------------------------------------------------------------------------------------------
-// One CTA per 128-row query tile; it walks the 128-key tiles j_begin..i of its group (keys <= query).
-// Per key tile n:  S_n = Q K_n^T,  dP_n = dO V_n^T,  dS_n = P_n o (dP_n - D) as bf16 written over the
-// start of S_n's columns,  dQ += dS_n K_n  (K_n is MN-major in the tile that served Q K_n^T).
+// A work item is a 128-row query tile; it walks the 128-key tiles j_begin..i of its group (keys <= query).
+// Per key tile n:  S_n = Q K_n^T,  dP_n = dO V_n^T,  dS_n = P_n o (dP_n - D) as bf16,
+// dQ += dS_n K_n  (K_n is MN-major in the tile that served Q K_n^T).
 // Full 128x128 score products: a 64-column product re-reads the 128-row A operand from shared memory
 // for half the work and runs at 48 instead of 32 clocks per K step.
 //
-// Tensor memory columns: dQ [0,HD)   S buffers [128,256) [256,384)   dP [384,512)
-// Only one dP buffer fits, so the elementwise warps copy their part of dP_{n+1} into registers as soon
-// as they are done with step n and release the buffer at once: dP_{n+2} (and S_{n+2}, into the S
-// buffer that the dQ MMAs of step n give back) run while they work on step n+1.  Shared memory: Q_i and dO_i resident, a ring of three K tiles and a ring of two V tiles.
+// Tensor memory columns: dQ [0,HD)   S [128,256)   dP [256,384)   dS (bf16, two buffers) [384,448) [448,512)
+// The elementwise warps copy S and dP into registers at the start of a step and release them at once, so the
+// score products of the next step run while they work.  Shared memory: Q and dO of the item resident, a ring
+// of three K tiles and a ring of two V tiles.
+//
+// Persistent, like the dK,dV kernel: items by cluster launch control, the loads of the next item behind those
+// of the last one, the accumulator read out by four warps of their own beside the next item's first steps.
+// Before (a block for each tile, dS over S, dP copied ahead) and after, us a launch in a loop: Llama2-7B 8k 246 and
+// 202, 16k 808 and 677, 32k 2720 and 2580 (at the power limit), 4 x 2000 tokens with groups of 200 48 and 27,
+// grouped query 2 x 4096 125 and 84.
 template <int HD>
 struct DqCfg {
-    static constexpr int kThreads = 384;  // TMA warp, two MMA warps, one spare, 8 elementwise warps
+    static constexpr int kThreads = 512;  // 4 load and issue warps, 8 elementwise warps, 4 epilogue warps
     static constexpr int kBoxes = HD / 64;
     static constexpr int kBoxBytes = kTile * 128;          // 128 rows x 128 bytes
     static constexpr int kTileBytes = kBoxes * kBoxBytes;  // one Q, dO, K or V tile
@@ -200,31 +206,63 @@ struct DqCfg {
     // around the issue of S_{n+1}, V_n only until dP_n is done.
     static constexpr int kRingK = 3;
     static constexpr int kRingV = 2;
-    static constexpr int kBarBytes = 512;
+    static constexpr int kBarBytes = 1024;
     static constexpr int kNeeded = (2 + kRingK + kRingV) * kTileBytes + kBarBytes;
     // at least 120 KB so that only one CTA fits on an SM: each CTA allocates all of tensor memory
     static constexpr int kSmemBytes = kNeeded > 120 * 1024 ? kNeeded : 120 * 1024;
     static constexpr int kTmemCols = 512;
+    // registers per thread after the split; the launch gives kRegsLaunch to each of the 512
+    static constexpr int kRegsLaunch = 128, kRegsElem = 168, kRegsOther = 88;
+    static_assert(2 * kRegsElem + 2 * kRegsOther <= 4 * kRegsLaunch, "register split");
 };
 
+struct DqItem {
+    int b, h, hk;     // b = -1: no more items
+    int tq0, q_valid; // the query tile
+    int j_begin, n_steps;
+    GroupLayout L;
+};
+// Work item `id` (heaviest query tiles of a chunk of units first); false marks a slot of a group that has
+// fewer tiles than the largest one.
+__device__ __forceinline__ bool dq_item(const BwdDqParams& p, int id, DqItem* t) {
+    const Geometry& geo = p.geo;
+    int unit, rank;
+    decode_block(id, geo.B * geo.H * geo.groups, geo.tiles_per_group, &unit, &rank, p.chunk);
+    const int g = unit % geo.groups;
+    t->h = (unit / geo.groups) % geo.H;
+    t->b = unit / (geo.groups * geo.H);
+    t->hk = t->h / (geo.H / geo.Hkv);
+    t->L = group_layout(geo, (t->h < geo.n_unshifted) ? 0 : geo.shift, g);
+    const int i = t->L.nTiles - 1 - rank;
+    if (i < 0) return false;
+    t->j_begin = first_key_tile(t->L, i);
+    t->n_steps = i + 1 - t->j_begin;
+    const TileRef tq = tile_ref(t->L, i);
+    t->tq0 = tq.tok0, t->q_valid = tq.valid;
+    return true;
+}
+
 struct DqBars {
-    uint64_t res_full;     // Q_i and dO_i landed
-    uint64_t acc_full;     // all dQ MMAs done
-    uint64_t drain;        // abort path only (gradient MMA warp)
-    uint64_t drain2;       // abort path only (score MMA warp)
-    uint64_t dp_ready;     // dP_n is in tensor memory
-    uint64_t s_ready[2];   // S_n is in tensor memory (buffer n & 1)
-    uint64_t dp_free;      // every elementwise thread holds its part of dP_n in registers
-    uint64_t p_full[2];    // bf16 dS_n is in tensor memory
-    uint64_t buf_free[2];  // the dQ MMAs that read an S buffer's bf16 dS are done
+    uint64_t res_full, res_empty;    // Q and dO of an item landed / the score products of the item are done
+    uint64_t acc_full, acc_empty;    // dQ of an item is complete / has been read out
+    uint64_t drain, drain2;          // abort path only (gradient / score MMA warp)
+    uint64_t s_full;                 // S_n and dP_n are in tensor memory
+    uint64_t s_free;                 // the elementwise threads hold them in registers
+    uint64_t p_full[2], p_free[2];   // bf16 dS_n is in tensor memory / the dQ MMAs that read it are done
     uint64_t k_full[3], k_empty[3], v_full[2], v_empty[2];
+    uint64_t sched_full[8];
+    uint64_t clc;
+    alignas(16) uint8_t clc_resp[16];
+    DqItem item[8];
     uint32_t tmem_slot;
     int abort_flag;
 };
+static_assert(sizeof(DqBars) <= 1024, "barrier block");
 
 template <int HD>
 __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(const __grid_constant__ BwdDqParams p) {
     using C = DqCfg<HD>;
+    constexpr int kSched = 8;  // items in flight
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = smem_raw;                          // 1024-byte aligned: nothing precedes the dynamic array
     uint8_t* sQ = smem;                                // resident: Q_i
@@ -235,36 +273,21 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
-
     const Geometry& geo = p.geo;
 
-    const int Tg = geo.tiles_per_group;
-    int unit, rank;
-    decode_block(blockIdx.x, geo.B * geo.H * geo.groups, Tg, &unit, &rank);
-    const int g = unit % geo.groups;
-    const int h = (unit / geo.groups) % geo.H;
-    const int b = unit / (geo.groups * geo.H);
-    const int hk = h / (geo.H / geo.Hkv);
-    const int s = (h < geo.n_unshifted) ? 0 : geo.shift;
-    const GroupLayout L = group_layout(geo, s, g);
-    const int i = L.nTiles - 1 - rank;  // heaviest query tiles first
-    if (i < 0) return;                  // this group has fewer tiles than the largest one
-    const int j_begin = first_key_tile(L, i);
-    const int n_steps = i + 1 - j_begin;  // key tiles j_begin .. i of the group (j_begin = 0 by default)
-    const TileRef tq = tile_ref(L, i);
-    const int tq0 = tq.tok0;
-
     if (threadIdx.x == 0) {
+        // hand-offs by whole warps count one arrival per warp
         mbar_init(&bars->res_full, 1);
+        mbar_init(&bars->res_empty, 1);
         mbar_init(&bars->acc_full, 1);
+        mbar_init(&bars->acc_empty, 4);
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->drain2, 1);
-        mbar_init(&bars->dp_ready, 1);
-        mbar_init(&bars->dp_free, 8);  // one arrival per elementwise warp
+        mbar_init(&bars->s_full, 1);
+        mbar_init(&bars->s_free, 8);
         for (int x = 0; x < 2; ++x) {
-            mbar_init(&bars->s_ready[x], 1);
             mbar_init(&bars->p_full[x], 8);
-            mbar_init(&bars->buf_free[x], 1);
+            mbar_init(&bars->p_free[x], 1);
             mbar_init(&bars->v_full[x], 1);
             mbar_init(&bars->v_empty[x], 1);
         }
@@ -272,6 +295,8 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
             mbar_init(&bars->k_full[x], 1);
             mbar_init(&bars->k_empty[x], 1);
         }
+        for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
+        mbar_init(&bars->clc, 1);
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
         tma_prefetch_desc(&p.tm_do);
@@ -296,211 +321,245 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
         return;
     }
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
-    constexpr uint32_t kColAcc = 0, kColS = 128, kColP = 384;
+    constexpr uint32_t kColAcc = 0, kColS = 128, kColP = 256, kColDs = 384;
 
-    if (warp == 0) {
-        if (lane == 0) {
-            mbar_expect_tx(&bars->res_full, 2 * C::kTileBytes);
-            for (int bx = 0; bx < C::kBoxes; ++bx) {
-                tma_load_4d(sQ + bx * C::kBoxBytes, &p.tm_q, &bars->res_full, bx * 64, h, tq0, b);
-                tma_load_4d(sDO + bx * C::kBoxBytes, &p.tm_do, &bars->res_full, bx * 64, h, tq0, b);
-            }
-            int n = 0;
-            for (; n < n_steps; ++n) {
-                const int st = n & 1;
-                const uint32_t ph = (n >> 1) & 1;
-                const int tk0 = tile_ref(L, j_begin + n).tok0;
-                if (!mbar_wait(&bars->v_empty[st], ph ^ 1, ctx, kWaitBwdDq + 1)) break;
-                mbar_expect_tx(&bars->v_full[st], C::kTileBytes);
-                for (int bx = 0; bx < C::kBoxes; ++bx)
-                    tma_load_4d(sV + st * C::kTileBytes + bx * C::kBoxBytes, &p.tm_v, &bars->v_full[st], bx * 64, hk, tk0, b);
-                const int sk = n % C::kRingK;
-                const uint32_t phk = (n / C::kRingK) & 1;
-                if (!mbar_wait(&bars->k_empty[sk], phk ^ 1, ctx, kWaitBwdDq + 8)) {
-                    mbar_wait_drain(&bars->v_full[st], ph);
-                    break;
+    // Every consumer warp walks the same sequence of items: the k-th one, false = the end (or aborting).
+    auto next_item = [&](int k, int where, DqItem* t) -> bool {
+        if (!mbar_wait_uniform(&bars->sched_full[k % kSched], (k / kSched) & 1, ctx, where)) return false;
+        *t = bars->item[k % kSched];
+        return t->b >= 0;
+    };
+
+    if (warp < 4) {
+        setmaxnreg_dec<C::kRegsOther>();
+        if (warp == 0) {
+            // ---- work items and TMA loads
+            if (lane == 0) {
+                int it = 0;     // key tiles requested so far
+                int n_res = 0;  // items whose Q and dO were requested
+                bool ok = true;
+                ItemSource items{&bars->clc, bars->clc_resp};
+                int id = static_cast<int>(blockIdx.x);
+                for (int k = 0; ok; ++k) {
+                    DqItem t;
+                    while (id >= 0 && !dq_item(p, id, &t)) id = items.next(ctx, kWaitBwdDq + 12, &ok);
+                    if (id < 0) t.b = -1;
+                    bars->item[k % kSched] = t;
+                    mbar_arrive(&bars->sched_full[k % kSched]);  // release: the item is visible to whoever sees the phase
+                    if (id < 0) break;
+                    for (int n = 0; ok && n < t.n_steps; ++n, ++it) {
+                        const int st = it % C::kRingV, sk = it % C::kRingK;
+                        const int tk0 = tile_ref(t.L, t.j_begin + n).tok0;
+                        if (!mbar_wait(&bars->v_empty[st], ((it / C::kRingV) & 1) ^ 1, ctx, kWaitBwdDq + 1)) { ok = false; break; }
+                        mbar_expect_tx(&bars->v_full[st], C::kTileBytes);
+                        for (int bx = 0; bx < C::kBoxes; ++bx)
+                            tma_load_4d(sV + st * C::kTileBytes + bx * C::kBoxBytes, &p.tm_v, &bars->v_full[st], bx * 64, t.hk, tk0, t.b);
+                        if (n == 0) {
+                            if (!mbar_wait(&bars->res_empty, (k & 1) ^ 1, ctx, kWaitBwdDq + 13)) {
+                                mbar_wait_drain(&bars->v_full[st], (it / C::kRingV) & 1);
+                                ok = false;
+                                break;
+                            }
+                            mbar_expect_tx(&bars->res_full, 2 * C::kTileBytes);
+                            for (int bx = 0; bx < C::kBoxes; ++bx) {
+                                tma_load_4d(sQ + bx * C::kBoxBytes, &p.tm_q, &bars->res_full, bx * 64, t.h, t.tq0, t.b);
+                                tma_load_4d(sDO + bx * C::kBoxBytes, &p.tm_do, &bars->res_full, bx * 64, t.h, t.tq0, t.b);
+                            }
+                            ++n_res;
+                        }
+                        if (!mbar_wait(&bars->k_empty[sk], ((it / C::kRingK) & 1) ^ 1, ctx, kWaitBwdDq + 8)) {
+                            mbar_wait_drain(&bars->v_full[st], (it / C::kRingV) & 1);
+                            ok = false;
+                            break;
+                        }
+                        mbar_expect_tx(&bars->k_full[sk], C::kTileBytes);
+                        for (int bx = 0; bx < C::kBoxes; ++bx)
+                            tma_load_4d(sK + sk * C::kTileBytes + bx * C::kBoxBytes, &p.tm_k, &bars->k_full[sk], bx * 64, t.hk, tk0, t.b);
+                    }
+                    if (ok) id = items.next(ctx, kWaitBwdDq + 12, &ok);
                 }
-                mbar_expect_tx(&bars->k_full[sk], C::kTileBytes);
-                for (int bx = 0; bx < C::kBoxes; ++bx)
-                    tma_load_4d(sK + sk * C::kTileBytes + bx * C::kBoxBytes, &p.tm_k, &bars->k_full[sk], bx * 64, hk, tk0, b);
-            }
-            if (bars->abort_flag != 0) {
-                // let loads that are still in flight land before the CTA gives its memory back
-                mbar_wait_drain(&bars->res_full, 0);
-                for (int nn = (n > C::kRingK ? n - C::kRingK : 0); nn < n; ++nn)
-                    mbar_wait_drain(&bars->k_full[nn % C::kRingK], (nn / C::kRingK) & 1);
-                for (int nn = (n > C::kRingV ? n - C::kRingV : 0); nn < n; ++nn)
-                    mbar_wait_drain(&bars->v_full[nn & 1], (nn >> 1) & 1);
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ---- score MMAs: dP_n = dO V_n^T first (its buffer is free as soon as the elementwise warps
-        // hold dP_{n-1} in registers), then S_n = Q K_n^T into S buffer n & 1 (free once the dQ MMAs
-        // of step n-2 are done).  The whole warp walks the loop so that addresses and descriptors
-        // stay warp-uniform values; only the MMA and commit instructions are issued by one elected lane.
-        constexpr uint32_t idesc_sc = idesc_bf16(128, kTile, 0, 0);
-        const uint32_t dQ = desc_lo_k_major(smem_u32(sQ)), dDO = desc_lo_k_major(smem_u32(sDO));
-        const uint32_t tP = tmem_base + kColP;
-        bool ok = mbar_wait_uniform(&bars->res_full, 0, ctx, kWaitBwdDq + 3);
-        for (int n = 0; ok && n < n_steps; ++n) {
-            const int st = n & 1;
-            const uint32_t ph = (n >> 1) & 1;
-            const int sk = n % C::kRingK;
-            // the two TMA barriers first: they have usually completed long ago, and every wait that sits
-            // between the two groups of MMAs below is time the tensor pipe idles
-            if (!mbar_wait_uniform(&bars->v_full[st], ph, ctx, kWaitBwdDq + 2)) break;
-            if (!mbar_wait_uniform(&bars->k_full[sk], (n / C::kRingK) & 1, ctx, kWaitBwdDq + 10)) break;
-            if (n >= 1 && !mbar_wait_uniform(&bars->dp_free, (n - 1) & 1, ctx, kWaitBwdDq + 9)) break;
-            tc_fence_after();
-            const uint32_t dV = desc_lo_k_major(smem_u32(sV + st * C::kTileBytes));
-            if (elect_one()) {
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk)
-                    mma_ss(tP, dDO + desc_step_k_major(kk, C::kBoxBytes), dV + desc_step_k_major(kk, C::kBoxBytes), idesc_sc, kk > 0);
-                mma_commit(&bars->v_empty[st]);
-                mma_commit(&bars->dp_ready);
+                if (bars->abort_flag != 0) {
+                    // let loads that are still in flight land before the CTA gives its memory back
+                    if (n_res > 0) mbar_wait_drain(&bars->res_full, (n_res - 1) & 1);
+                    for (int nn = (it > C::kRingK ? it - C::kRingK : 0); nn < it; ++nn)
+                        mbar_wait_drain(&bars->k_full[nn % C::kRingK], (nn / C::kRingK) & 1);
+                    for (int nn = (it > C::kRingV ? it - C::kRingV : 0); nn < it; ++nn)
+                        mbar_wait_drain(&bars->v_full[nn % C::kRingV], (nn / C::kRingV) & 1);
+                }
             }
             __syncwarp();
-            if (n >= 2 && !mbar_wait_uniform(&bars->buf_free[st], ph ^ 1, ctx, kWaitBwdDq + 7)) break;
-            tc_fence_after();
-            const uint32_t dK = desc_lo_k_major(smem_u32(sK + sk * C::kTileBytes));
-            const uint32_t tS = tmem_base + kColS + st * kTile;
-            if (elect_one()) {
+        } else if (warp == 1) {
+            // ---- score MMAs: dP_n = dO V_n^T and S_n = Q K_n^T, as soon as the elementwise warps hold those of the
+            // step before in registers.  The whole warp walks the loop so that addresses and descriptors
+            // stay warp-uniform values; only the MMA and commit instructions are issued by one elected lane.
+            constexpr uint32_t idesc_sc = idesc_bf16(128, kTile, 0, 0);
+            const uint32_t dQ = desc_lo_k_major(smem_u32(sQ)), dDO = desc_lo_k_major(smem_u32(sDO));
+            const uint32_t tP = tmem_base + kColP, tS = tmem_base + kColS;
+            int it = 0;
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
+                DqItem t;
+                if (!next_item(k, kWaitBwdDq + 14, &t)) break;
+                if (!mbar_wait_uniform(&bars->res_full, k & 1, ctx, kWaitBwdDq + 3)) break;
+                for (int n = 0; n < t.n_steps; ++n, ++it) {
+                    const int st = it % C::kRingV, sk = it % C::kRingK;
+                    // the two TMA barriers first: they have usually completed long ago
+                    if (!mbar_wait_uniform(&bars->v_full[st], (it / C::kRingV) & 1, ctx, kWaitBwdDq + 2) ||
+                        !mbar_wait_uniform(&bars->k_full[sk], (it / C::kRingK) & 1, ctx, kWaitBwdDq + 10)) { ok = false; break; }
+                    if (it >= 1 && !mbar_wait_uniform(&bars->s_free, (it - 1) & 1, ctx, kWaitBwdDq + 9)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t dV = desc_lo_k_major(smem_u32(sV + st * C::kTileBytes));
+                    const uint32_t dK = desc_lo_k_major(smem_u32(sK + sk * C::kTileBytes));
+                    if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk)
-                    mma_ss(tS, dQ + desc_step_k_major(kk, C::kBoxBytes), dK + desc_step_k_major(kk, C::kBoxBytes), idesc_sc, kk > 0);
-                mma_commit(&bars->s_ready[st]);
+                        for (int kk = 0; kk < HD / 16; ++kk)
+                            mma_ss(tP, dDO + desc_step_k_major(kk, C::kBoxBytes), dV + desc_step_k_major(kk, C::kBoxBytes), idesc_sc, kk > 0);
+                        mma_commit(&bars->v_empty[st]);
+#pragma unroll
+                        for (int kk = 0; kk < HD / 16; ++kk)
+                            mma_ss(tS, dQ + desc_step_k_major(kk, C::kBoxBytes), dK + desc_step_k_major(kk, C::kBoxBytes), idesc_sc, kk > 0);
+                        mma_commit(&bars->s_full);
+                        if (n == t.n_steps - 1) mma_commit(&bars->res_empty);
+                    }
+                    __syncwarp();
+                }
+            }
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
+                if (elect_one()) {
+                    mma_commit(&bars->drain2);
+                    mbar_wait_drain(&bars->drain2, 0);
+                }
+            }
+            __syncwarp();
+        } else if (warp == 2) {
+            // ---- gradient MMAs: dQ += dS_n K_n
+            constexpr uint32_t idesc_acc = idesc_bf16(128, HD, 0, 1);
+            int it = 0;
+            bool ok = true;
+            for (int k = 0; ok; ++k) {
+                DqItem t;
+                if (!next_item(k, kWaitBwdDq + 15, &t)) break;
+                // the first product of an item overwrites the accumulator: the previous item's must have been read out
+                if (k > 0 && !mbar_wait_uniform(&bars->acc_empty, (k - 1) & 1, ctx, kWaitBwdDq + 7)) break;
+                for (int n = 0; n < t.n_steps; ++n, ++it) {
+                    const int bf = it & 1, sk = it % C::kRingK;
+                    if (!mbar_wait_uniform(&bars->p_full[bf], (it >> 1) & 1, ctx, kWaitBwdDq + 4)) { ok = false; break; }
+                    tc_fence_after();
+                    const uint32_t dKmn = desc_lo_mn_major(smem_u32(sK + sk * C::kTileBytes), C::kBoxBytes);
+                    const uint32_t tdS = tmem_base + kColDs + bf * 64;
+                    if (elect_one()) {
+#pragma unroll
+                        for (int kk = 0; kk < kTile / 16; ++kk)
+                            mma_ts(tmem_base + kColAcc, tdS + kk * 8, dKmn + kk * kDescStepMn, idesc_acc, (n > 0) || (kk > 0));
+                        mma_commit(&bars->k_empty[sk]);
+                        mma_commit(&bars->p_free[bf]);
+                        if (n == t.n_steps - 1) mma_commit(&bars->acc_full);
+                    }
+                    __syncwarp();
+                }
+            }
+            if (__any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&bars->abort_flag) != 0)) {
+                // MMAs already issued must finish before tensor memory is released
+                if (elect_one()) {
+                    mma_commit(&bars->drain);
+                    mbar_wait_drain(&bars->drain, 0);
+                }
             }
             __syncwarp();
         }
-        if (__any_sync(0xffffffffu, bars->abort_flag != 0)) {
-            if (elect_one()) {
-                mma_commit(&bars->drain2);
-                mbar_wait_drain(&bars->drain2, 0);
-            }
-        }
-        __syncwarp();
-    } else if (warp == 2) {
-        // ---- gradient MMAs: dQ += dS_n K_n
-        constexpr uint32_t idesc_acc = idesc_bf16(128, HD, 0, 1);
-        for (int n = 0; n < n_steps; ++n) {
-            const int st = n & 1;
-            if (!mbar_wait_uniform(&bars->p_full[st], (n >> 1) & 1, ctx, kWaitBwdDq + 4)) break;
-            tc_fence_after();
-            const int sk = n % C::kRingK;
-            const uint32_t dKmn = desc_lo_mn_major(smem_u32(sK + sk * C::kTileBytes), C::kBoxBytes);
-            const uint32_t tdS = tmem_base + kColS + st * kTile;  // bf16 dS over the S buffer
-            if (elect_one()) {
-#pragma unroll
-                for (int kk = 0; kk < kTile / 16; ++kk)
-                    mma_ts(tmem_base + kColAcc, tdS + (kk >> 2) * 64 + (kk & 3) * 8, dKmn + kk * kDescStepMn, idesc_acc,
-                           (n > 0) || (kk > 0));
-                mma_commit(&bars->k_empty[sk]);
-                mma_commit(&bars->buf_free[st]);
-                if (n == n_steps - 1) mma_commit(&bars->acc_full);
-            }
-            __syncwarp();
-        }
-        if (__any_sync(0xffffffffu, bars->abort_flag != 0)) {
-            // MMAs already issued (by either MMA warp) must finish before tensor memory is released
-            if (elect_one()) {
-                mma_commit(&bars->drain);
-                mbar_wait_drain(&bars->drain, 0);
-            }
-        }
-        __syncwarp();
-    } else if (warp == 3) {
-        // spare warp: owns the tensor-memory allocation only
-    } else {
-        // ---- elementwise: thread (quad, lane, half) owns columns [64 half, +64) of score row
-        // 32 quad + lane.  Its 64 bf16 dS values (32 packed columns) go over the first 32 of its own
-        // columns, so the two halves never write into columns the other half still has to read: the
-        // 128 K values of the dS operand sit at packed columns [0,32) and [64,96) of the S buffer.
+        // warp 3: owns the tensor-memory allocation only
+    } else if (warp < 12) {
+        // ---- elementwise: thread (quad, lane, half) owns columns [64 half, +64) of score row 32 quad + lane
+        setmaxnreg_inc<C::kRegsElem>();
         const int quad = warp & 3;
         const int half = (warp - 4) >> 2;
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-        // rows past the end of a ragged tile are not part of the group: they are computed on whatever
-        // the box holds there and never stored
-        const bool row_valid = row < tq.valid;
-        const size_t stat_idx = (static_cast<size_t>(b) * geo.H + h) * geo.N + tq0 + row;
-        const float neg_lse2 = row_valid ? -p.lse[stat_idx] * kLog2e : 0.f;
-        const float Drow = row_valid ? p.Dsum[stat_idx] : 0.f;
         const float c2 = p.scale_log2;
-        const uint64_t c2x2 = f2_pack(c2, c2), nlx2 = f2_pack(neg_lse2, neg_lse2), Dx2 = f2_pack(Drow, Drow);
+        const uint64_t c2x2 = f2_pack(c2, c2);
+        int it = 0;
         bool ok = true;
-        uint32_t dp[64];  // this thread's part of dP_n
-        // Copy dP_m out of tensor memory and release its buffer.  Done for step 0 up front and for step
-        // n+1 at the END of step n (dP_{n+1} has been complete for a long time by then), so that dP_{n+2}
-        // and S_{n+2} can be issued while step n+1 is still being worked on.
-        auto fetch_dp = [&](int m) -> bool {
-            if (!mbar_wait_uniform(&bars->dp_ready, m & 1, ctx, kWaitBwdDq + 5)) return false;
-            tc_fence_after();
-            tmem_ld_32x32(t_row + kColP + half * 64, *reinterpret_cast<uint32_t(*)[32]>(&dp[0]));
-            tmem_ld_32x32(t_row + kColP + half * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&dp[32]));
-            tmem_wait_ld();
-            tc_fence_before();
-            mbar_arrive_warp(&bars->dp_free);
-            return true;
-        };
-        ok = fetch_dp(0);
-        for (int n = 0; ok && n < n_steps; ++n) {
-            const int st = n & 1;
-            if (!mbar_wait_uniform(&bars->s_ready[st], (n >> 1) & 1, ctx, kWaitBwdDq + 11)) { ok = false; break; }
-            tc_fence_after();
-            // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
-            // in the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
-            const int k_valid = tile_ref(L, j_begin + n).valid;
-            const bool last = (n == n_steps - 1);
-            const bool masked = last || k_valid < kTile;
-            const int vis = (last && row < k_valid) ? row : k_valid - 1;
-            const int lim = vis - half * 64;  // visible iff (column within this half) <= lim
-            const uint32_t tS = t_row + kColS + st * kTile + half * 64;
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t sr[32];
-                tmem_ld_32x32(tS + c * 32, sr);
+        for (int k = 0; ok; ++k) {
+            DqItem t;
+            if (!next_item(k, kWaitBwdDq + 16, &t)) break;
+            // rows past the end of a ragged tile are not part of the group: they are computed on whatever
+            // the box holds there and never stored
+            const bool row_valid = row < t.q_valid;
+            const size_t stat_idx = (static_cast<size_t>(t.b) * geo.H + t.h) * geo.N + t.tq0 + row;
+            const float neg_lse2 = row_valid ? -p.lse[stat_idx] * kLog2e : 0.f;
+            const float Drow = row_valid ? p.Dsum[stat_idx] : 0.f;
+            const uint64_t nlx2 = f2_pack(neg_lse2, neg_lse2), Dx2 = f2_pack(Drow, Drow);
+            for (int n = 0; n < t.n_steps; ++n, ++it) {
+                const int bf = it & 1;
+                // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
+                // in the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
+                const int k_valid = tile_ref(t.L, t.j_begin + n).valid;
+                if (!mbar_wait_uniform(&bars->s_full, it & 1, ctx, kWaitBwdDq + 11)) { ok = false; break; }
+                tc_fence_after();
+                uint32_t sr[2][32], dp[2][32];
+                tmem_ld_32x32(t_row + kColS + half * 64, sr[0]);
+                tmem_ld_32x32(t_row + kColS + half * 64 + 32, sr[1]);
+                tmem_ld_32x32(t_row + kColP + half * 64, dp[0]);
+                tmem_ld_32x32(t_row + kColP + half * 64 + 32, dp[1]);
                 tmem_wait_ld();
-                uint32_t pk[16];
-                if (masked) {
+                tc_fence_before();
+                mbar_arrive_warp(&bars->s_free);
+                if (it >= 2 && !mbar_wait_uniform(&bars->p_free[bf], ((it >> 1) & 1) ^ 1, ctx, kWaitBwdDq + 5)) { ok = false; break; }
+                tc_fence_after();
+                const bool last = (n == t.n_steps - 1);
+                const bool masked = last || k_valid < kTile;
+                const int vis = (last && row < k_valid) ? row : k_valid - 1;
+                const int lim = vis - half * 64;  // visible iff (column within this half) <= lim
+                const uint32_t tdS = t_row + kColDs + bf * 64 + half * 32;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        float pe0 = fast_exp2(fmaf(__uint_as_float(sr[2 * e]), c2, neg_lse2));
-                        float pe1 = fast_exp2(fmaf(__uint_as_float(sr[2 * e + 1]), c2, neg_lse2));
-                        if (c * 32 + 2 * e > lim) pe0 = 0.f;
-                        if (c * 32 + 2 * e + 1 > lim) pe1 = 0.f;
-                        pk[e] = pack_bf16(pe0 * (__uint_as_float(dp[c * 32 + 2 * e]) - Drow),
-                                          pe1 * (__uint_as_float(dp[c * 32 + 2 * e + 1]) - Drow));
-                    }
-                } else {
-                    // two columns per instruction for the multiply-adds
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t pk[16];
+                    if (masked) {
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const uint64_t x = f2_fma(f2_pack(__uint_as_float(sr[2 * e]), __uint_as_float(sr[2 * e + 1])), c2x2, nlx2);
-                        float x0, x1;
-                        f2_unpack(x, x0, x1);
-                        // part of the exponentials goes to the FMA pipe (see poly_exp2_x2)
-                        const uint64_t pe = ((kPolyExpMask >> e) & 1u) ? poly_exp2_x2(x) : f2_pack(fast_exp2(x0), fast_exp2(x1));
-                        const uint64_t t = f2_sub(f2_pack(__uint_as_float(dp[c * 32 + 2 * e]), __uint_as_float(dp[c * 32 + 2 * e + 1])), Dx2);
-                        float d0, d1;
-                        f2_unpack(f2_mul(pe, t), d0, d1);
-                        pk[e] = pack_bf16(d0, d1);
+                        for (int e = 0; e < 16; ++e) {
+                            float pe0 = fast_exp2(fmaf(__uint_as_float(sr[c][2 * e]), c2, neg_lse2));
+                            float pe1 = fast_exp2(fmaf(__uint_as_float(sr[c][2 * e + 1]), c2, neg_lse2));
+                            if (c * 32 + 2 * e > lim) pe0 = 0.f;
+                            if (c * 32 + 2 * e + 1 > lim) pe1 = 0.f;
+                            pk[e] = pack_bf16(pe0 * (__uint_as_float(dp[c][2 * e]) - Drow), pe1 * (__uint_as_float(dp[c][2 * e + 1]) - Drow));
+                        }
+                    } else {
+                        // two columns per instruction for the multiply-adds
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) {
+                            const uint64_t x = f2_fma(f2_pack(__uint_as_float(sr[c][2 * e]), __uint_as_float(sr[c][2 * e + 1])), c2x2, nlx2);
+                            float x0, x1;
+                            f2_unpack(x, x0, x1);
+                            // part of the exponentials goes to the FMA pipe (see poly_exp2_x2)
+                            const uint64_t pe = ((kPolyExpMask >> e) & 1u) ? poly_exp2_x2(x) : f2_pack(fast_exp2(x0), fast_exp2(x1));
+                            const uint64_t u = f2_sub(f2_pack(__uint_as_float(dp[c][2 * e]), __uint_as_float(dp[c][2 * e + 1])), Dx2);
+                            float d0, d1;
+                            f2_unpack(f2_mul(pe, u), d0, d1);
+                            pk[e] = pack_bf16(d0, d1);
+                        }
                     }
+                    tmem_st_32x16(tdS + c * 16, pk);
                 }
-                // packed columns [16c, 16c+16) overlay score columns [16c, 16c+16) of this half, which
-                // have been read already (c = 1 writes over columns 16..31, read when c was 0)
-                tmem_st_32x16(tS + c * 16, pk);
+                tmem_wait_st();
+                tc_fence_before();
+                mbar_arrive_warp(&bars->p_full[bf]);
             }
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive_warp(&bars->p_full[st]);
-            if (n + 1 < n_steps && !fetch_dp(n + 1)) { ok = false; break; }
         }
-        if (ok && mbar_wait(&bars->acc_full, 0, ctx, kWaitBwdDq + 6)) {
+    } else {
+        // ---- epilogue: thread owns accumulator row 32 quad + lane
+        setmaxnreg_dec<C::kRegsOther>();
+        const int quad = warp & 3;
+        const int row = quad * 32 + lane;
+        const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
+        for (int k = 0;; ++k) {
+            DqItem t;
+            if (!next_item(k, kWaitBwdDq + 17, &t)) break;
+            if (!mbar_wait_uniform(&bars->acc_full, k & 1, ctx, kWaitBwdDq + 6)) break;
             tc_fence_after();
-            __nv_bfloat16* dst = p.dq + (static_cast<size_t>(b) * geo.N + tq0 + row) * p.dq_tok_stride + static_cast<size_t>(h) * HD;
-            store_acc_cols<HD / 2>(t_row + kColAcc + half * (HD / 2), p.scale, dst + half * (HD / 2), row_valid);
+            __nv_bfloat16* dst = p.dq + (static_cast<size_t>(t.b) * geo.N + t.tq0 + row) * p.dq_tok_stride + static_cast<size_t>(t.h) * HD;
+            store_acc_cols<HD>(t_row + kColAcc, p.scale, dst, row < t.q_valid);
+            tc_fence_before();
+            mbar_arrive_warp(&bars->acc_empty);
         }
     }
 
@@ -1358,7 +1417,7 @@ cudaError_t configure_one(Kernel kernel, int smem_bytes, int min_regs) {
 }
 template <int HD>
 cudaError_t configure_all() {
-    cudaError_t e = configure_one(s2a_bwd_dq_kernel<HD>, DqCfg<HD>::kSmemBytes, 0);
+    cudaError_t e = configure_one(s2a_bwd_dq_kernel<HD>, DqCfg<HD>::kSmemBytes, DqCfg<HD>::kRegsLaunch);
     if (e == cudaSuccess) e = configure_one(s2a_bwd_dkdv_kernel<HD, false>, BwdCfg<HD>::kSmemBytes, BwdCfg<HD>::kRegsLaunch);
     if (e == cudaSuccess) e = configure_one(s2a_bwd_dkdv_kernel<HD, true>, BwdCfg<HD>::kSmemBytes, BwdCfg<HD>::kRegsLaunch);
     if (e == cudaSuccess) e = configure_one(s2a_bwd_dq_spill_kernel<HD>, DqSpillCfg<HD>::kSmemBytes, 0);

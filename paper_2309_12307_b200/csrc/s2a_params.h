@@ -194,6 +194,7 @@ struct alignas(64) BwdDqParams {
     const float* Dsum;        // [B, H, N]
     __nv_bfloat16* dq;
     long long dq_tok_stride;  // elements between consecutive tokens of dq (H * d when dense)
+    int chunk;                // units in a chunk of the block order
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
