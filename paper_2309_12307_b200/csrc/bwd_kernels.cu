@@ -23,10 +23,9 @@
 // warp spends so long on its own barrier waits that the tensor pipe runs dry in between; with two, one
 // can issue while the other waits); warp 3 owns the tensor-memory allocation (and loads K and V in kernel
 // 3); warps 4-11 do the elementwise work with one tensor-memory lane and half of the columns per thread;
-// kernel 3 has four more warps that write finished accumulators out.  dP (dP^T) has a
-// single buffer: the elementwise warps copy their part of it into registers and release it at once,
-// which leaves the columns for two score buffers (and, in kernel 3, for K as a tensor-memory operand),
-// so that the score products of the next step run while the elementwise warps work on the current one.
+// warps 12-15 write finished accumulators out.  S and dP (S^T and dP^T) need one buffer only: the elementwise
+// warps copy their part into registers and release it at once, so that the score products of the next
+// step run while they work on the current one, and write their bf16 results to columns of their own.
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -574,12 +573,14 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
 // ------------------------------------------------------------------------------------------------
 // 3. dK, dV
 // ------------------------------------------------------------------------------------------------
-// Tensor memory columns: dV [0,HD)  dK [128,128+HD)  S^T buffers [256,320) [320,384)  dP^T [384,448)
-//                        K (bf16, the A operand of the score products) [448,448+HD/2)
-// One dP^T buffer is enough because the elementwise warps copy their part of it into registers at the
-// start of a step and release the buffer at once; that leaves room for a third S^T
-// buffer, and with three steps in flight the chain scores -> elementwise -> gradient MMAs of one
-// buffer no longer leaves the tensor pipe idle.
+// Tensor memory columns: dV, dK (HD each), S^T, dP^T (64 each), P^T and dS^T (bf16, 64 together; two buffers where
+//                        HD = 64 leaves room), K (bf16, HD/2: the A operand of S^T = K Q^T)
+// One buffer of S^T and dP^T is enough: the elementwise warps copy them into registers at the start of a step
+// and release them at once, so the score products of the next step run while they work.  P^T and dS^T are
+// written when the gradient MMAs are done with what the buffer held.  With P^T and dS^T over S^T, in two
+// buffers, the score products waited some 400 clocks a step for the gradient MMAs.  Microseconds a launch in a
+// loop, before and after (plain / spilling): Llama2-7B 32k 3670 and 3475 / 4270 and 4150, 16k 992 and 943 / 1149 and
+// 1094, 8k 281 and 275 / 328 and 313; head size 64 at 32k 2557 and 2503 / 3151 and 3053.
 //
 // The CTA owns key tile (b, hk, original tokens tk0 .. tk0+127).  For every query head hq that
 // reads KV head hk (shift s): the tile sits at rolled position (tk0 - s) mod N, i.e. in group g at
@@ -649,10 +650,10 @@ struct DkDvBars {
     uint64_t acc_empty;           // the accumulators of an item have been read out
     uint64_t drain;               // abort path only (gradient MMA warp)
     uint64_t drain2;              // abort path only (score MMA warp)
-    uint64_t s_full[2];           // S^T (and dP^T) of a step is in tensor memory (buffer it % 2)
-    uint64_t p_full[2];           // bf16 P^T and dS^T of a step are in tensor memory
-    uint64_t buf_free[2];         // gradient MMAs that read a score buffer's bf16 operands are done
-    uint64_t dp_free;             // the elementwise threads of a step hold their dP^T in registers
+    uint64_t s_full;              // S^T and dP^T of a step are in tensor memory
+    uint64_t s_free;              // the elementwise threads of a step hold their S^T and dP^T in registers
+    uint64_t p_full[2];           // bf16 P^T and dS^T of a step are in tensor memory (buffer it % kPBufs)
+    uint64_t p_free[2];           // the gradient MMAs that read them are done
     uint64_t st_full[kStages];    // streamed operands of a stage landed
     uint64_t st_empty[kStages];   // MMAs reading a stage are done
     uint64_t sched_full[8];       // a work item has been published
@@ -679,7 +680,7 @@ template <int HD, bool kSpill>
 __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(const __grid_constant__ BwdDkDvParams p) {
     using C = BwdCfg<HD>;
     using Bars = DkDvBars<C::kStages>;
-    constexpr int kBufs = 2;   // S^T buffers in flight
+    constexpr int kPBufs = HD == 64 ? 2 : 1;  // buffers of P^T and dS^T
     constexpr int kCols = 32;  // query columns per elementwise thread and step: two threads share a key row
     constexpr int kChunks = kCols / 16;
     constexpr int kSched = 8;  // item ids in flight: the TMA warp is at most five items ahead of the read-out
@@ -717,12 +718,12 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
         mbar_init(&bars->acc_empty, 4);
         mbar_init(&bars->drain, 1);
         mbar_init(&bars->drain2, 1);
-        for (int x = 0; x < kBufs; ++x) {
-            mbar_init(&bars->s_full[x], 1);
-            mbar_init(&bars->p_full[x], 256);
-            mbar_init(&bars->buf_free[x], 1);
+        mbar_init(&bars->s_full, 2);  // the score MMAs are done; their issuer has seen the stage land
+        mbar_init(&bars->s_free, 8);
+        for (int x = 0; x < kPBufs; ++x) {
+            mbar_init(&bars->p_full[x], 8);
+            mbar_init(&bars->p_free[x], 1);
         }
-        mbar_init(&bars->dp_free, 256);
         for (int st = 0; st < C::kStages; ++st) {
             mbar_init(&bars->st_full[st], 1);
             mbar_init(&bars->st_empty[st], 1);
@@ -747,7 +748,8 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
-    constexpr uint32_t kColDV = 0, kColDK = 128, kColS = 256, kColP = 384, kColKt = 448;
+    constexpr uint32_t kColDV = 0, kColDK = HD, kColS = 2 * HD, kColP = kColS + 64, kColPdS = kColP + 64, kColKt = kColPdS + 64 * kPBufs;
+    static_assert(kColKt + HD / 2 <= C::kTmemCols, "tensor memory");
 
     // Every consumer warp walks the same sequence of items, as the scheduling thread has decoded them (the
     // divisions cost a warp more than a step): the k-th one, false = the end (or aborting).
@@ -812,10 +814,8 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             }
             __syncwarp();
         } else if (warp == 1) {
-            // ---- score MMAs of step `it`: dP^T = V dO^T into the single dP^T buffer (free as soon as the
-            // elementwise warps hold the previous one in registers) and S^T = K Q^T into buffer it % 2
-            // (warp-uniform loop, one elected lane issues; see the dQ kernel).  In an item's first step S^T
-            // goes first: it needs only K, while V may still be on its way.
+            // ---- score MMAs of step `it`: dP^T = V dO^T and S^T = K Q^T, as soon as the elementwise warps hold those
+            // of the step before in registers (warp-uniform loop, one elected lane issues; see the dQ kernel)
             constexpr uint32_t idesc_sc = idesc_bf16(128, kSubTile, 0, 0);
             const uint32_t dV = desc_lo_k_major(smem_u32(sV));
             const uint32_t tP = tmem_base + kColP, tKt = tmem_base + kColKt;
@@ -828,34 +828,26 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                 if (!mbar_wait_uniform(&bars->kt_full, k & 1, ctx, kWaitBwdDkDv + 16)) break;
                 for (int x = 0; ok && x < steps; ++x, ++it) {
                     const int st = it % C::kStages;
-                    const int bf = it % kBufs;
                     const bool last = x == steps - 1;
                     if (!mbar_wait_uniform(&bars->st_full[st], (it / C::kStages) & 1, ctx, kWaitBwdDkDv + 2)) { ok = false; break; }
                     const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
                     const uint32_t dQ = desc_lo_k_major(aQ), dDO = desc_lo_k_major(aQ + C::kSubTileBytes);
-                    const uint32_t tS = tmem_base + kColS + bf * kSubTile;
+                    const uint32_t tS = tmem_base + kColS;
                     if (x == 0 && !mbar_wait_uniform(&bars->v_full, k & 1, ctx, kWaitBwdDkDv + 3)) { ok = false; break; }
-                    if (it >= 1 && !mbar_wait_uniform(&bars->dp_free, (it - 1) & 1, ctx, kWaitBwdDkDv + 9)) { ok = false; break; }
+                    if (it >= 1 && !mbar_wait_uniform(&bars->s_free, (it - 1) & 1, ctx, kWaitBwdDkDv + 9)) { ok = false; break; }
+                    if (kPBufs > 1 && it >= kPBufs && !mbar_wait_uniform(&bars->p_free[it % kPBufs], ((it / kPBufs) & 1) ^ 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
                     tc_fence_after();
                     if (elect_one()) {
+                        mbar_arrive(&bars->s_full);  // (the phase of the step before was over when s_free was)
 #pragma unroll
                         for (int kk = 0; kk < HD / 16; ++kk)
                             mma_ss(tP, dV + desc_step_k_major(kk, C::kBigBoxBytes), dDO + desc_step_k_major(kk, C::kSubBoxBytes),
                                    idesc_sc, kk > 0);
                         if (last) mma_commit(&bars->v_empty);
-                    }
-                    __syncwarp();
-                    if (it >= kBufs && !mbar_wait_uniform(&bars->buf_free[bf], ((it / kBufs) & 1) ^ 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
-                    tc_fence_after();
-                    if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < HD / 16; ++kk)
                             mma_ts(tS, tKt + 8 * kk, dQ + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
-                    }
-                    __syncwarp();
-                    if (!ok) break;
-                    if (elect_one()) {
-                        mma_commit(&bars->s_full[bf]);
+                        mma_commit(&bars->s_full);
                         if (last) mma_commit(&bars->s_done);
                     }
                     __syncwarp();
@@ -869,8 +861,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             }
             __syncwarp();
         } else if (warp == 2) {
-            // ---- gradient MMAs: dV += P^T dO and dK += dS^T Q of step `it`; both bf16 operands sit in
-            // the step's S^T buffer
+            // ---- gradient MMAs: dV += P^T dO and dK += dS^T Q of step `it`
             constexpr uint32_t idesc_acc = idesc_bf16(128, HD, 0, 1);
             int it = 0;
             bool ok = true;
@@ -882,14 +873,14 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                 if (k > 0 && !mbar_wait_uniform(&bars->acc_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 13)) break;
                 for (int x = 0; x < steps; ++x, ++it) {
                     const int st = it % C::kStages;
-                    const int bf = it % kBufs;
-                    if (!mbar_wait_uniform(&bars->p_full[bf], (it / kBufs) & 1, ctx, kWaitBwdDkDv + 4)) { ok = false; break; }
+                    const int bf = it % kPBufs;
+                    if (!mbar_wait_uniform(&bars->p_full[bf], (it / kPBufs) & 1, ctx, kWaitBwdDkDv + 4)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
                     const uint32_t dQmn = desc_lo_mn_major(aQ, C::kSubBoxBytes);
                     const uint32_t dDOmn = desc_lo_mn_major(aQ + C::kSubTileBytes, C::kSubBoxBytes);
                     // the 16 queries of K slice kk: P^T in packed columns [16 kk, +8) of the buffer, dS^T in [16 kk + 8, +8)
-                    const uint32_t tPt = tmem_base + kColS + bf * kSubTile;
+                    const uint32_t tPt = tmem_base + kColPdS + bf * 64;
                     if (elect_one()) {
 #pragma unroll
                         for (int kk = 0; kk < kSubTile / 16; ++kk)
@@ -898,7 +889,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                         for (int kk = 0; kk < kSubTile / 16; ++kk)
                             mma_ts(tmem_base + kColDK, tPt + 16 * kk + 8, dQmn + kk * kDescStepMn, idesc_acc, (x > 0) || (kk > 0));
                         mma_commit(&bars->st_empty[st]);
-                        mma_commit(&bars->buf_free[bf]);
+                        mma_commit(&bars->p_free[bf]);
                         if (x == steps - 1) mma_commit(&bars->acc_full);
                     }
                     __syncwarp();
@@ -975,29 +966,20 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                 for (int n = w.n_begin; n < w.n_end; ++n, ++it) {
                     const int cg0 = 2 * group;   // first 16-column chunk of this thread
                     const int st = it % C::kStages;
-                    const int bf = it % kBufs;
-                    // The statistics of this step travel with its stage.  s_full covers dP^T of this step as
-                    // well: its MMAs were issued by the same thread before the commit.
-                    if (!mbar_wait(&bars->st_full[st], (it / C::kStages) & 1, ctx, kWaitBwdDkDv + 5) ||
-                        !mbar_wait(&bars->s_full[bf], (it / kBufs) & 1, ctx, kWaitBwdDkDv + 6)) {
-                        ok = false;
-                        break;
-                    }
+                    // The statistics of this step travel with its stage; the score MMA warp's arrival on s_full says that
+                    // it has seen the stage land.  (Every wait here is 5 % of a step with head size 64.)
+                    if (!mbar_wait(&bars->s_full, it & 1, ctx, kWaitBwdDkDv + 6)) { ok = false; break; }
                     tc_fence_after();
-                    // copy this thread's part of dP^T into registers and release the single dP^T buffer as soon
-                    // as the copy has landed, so that the dP^T product of the next step runs while this step is
-                    // worked on
+                    // copy this thread's part of dP^T and S^T into registers and release their buffers as soon as the
+                    // copies have landed, so that the score products of the next step run while this one is worked on
                     uint32_t pr[kCols];
                     tmem_ld_32x32(t_row + kColP + 16 * cg0, pr);
-                    // S^T in two chunks of 16 columns; the bf16 results of a chunk go back over its 16 columns:
-                    // P^T into the first 8 (packed), dS^T into the other 8
-                    const uint32_t tS = t_row + kColS + bf * kSubTile;
                     uint32_t sbuf[2][16];
-                    tmem_ld_32x16(tS + 16 * cg0, sbuf[0]);
-                    tmem_ld_32x16(tS + 16 * (cg0 + 1), sbuf[1]);
+                    tmem_ld_32x16(t_row + kColS + 16 * cg0, sbuf[0]);
+                    tmem_ld_32x16(t_row + kColS + 16 * (cg0 + 1), sbuf[1]);
                     tmem_wait_ld();
                     tc_fence_before();
-                    mbar_arrive(&bars->dp_free);
+                    mbar_arrive_warp(&bars->s_free);
                     const uint32_t stat_sa = smem_u32(sStat + st * 2 * kSubTile);  // lse[64] then D[64] of this stage
                     // query x of this sub-tile sees key row r iff x is a valid row of the sub-tile and, in the
                     // diagonal tile, 128 j + r <= 64 n + x
@@ -1006,11 +988,21 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     const int lim = (n < w.n_begin + 2) ? row - (n & 1) * kSubTile : -64;  // visible iff lim <= x < q_valid
                     uint4* spill_dst = nullptr;
                     if constexpr (kSpill) spill_dst = spill_head + static_cast<size_t>(n - w.n_begin) * (kSpillBlockElems / 8);
+                    uint32_t pk[kChunks][2][8];  // bf16 P^T and dS^T
+                    // P^T of chunk cg goes to the packed columns [16 cg, +8), dS^T to [16 cg + 8, +8): at once where
+                    // there are two buffers (the score MMAs of this step were held back until this one was free),
+                    // else at the end of the step, when the gradient MMAs of the step before are done with it
+                    const int bf = it % kPBufs;
+                    const uint32_t tPdS = t_row + kColPdS + bf * 64 + 16 * cg0;
+                    auto store_chunk = [&](int c) {
+                        tmem_st_32x8(tPdS + 16 * c, pk[c][0]);
+                        tmem_st_32x8(tPdS + 16 * c + 8, pk[c][1]);
+                    };
 #pragma unroll
                     for (int c = 0; c < kChunks; ++c) {
                         const int cg = cg0 + c;   // chunk within the sub-tile: queries [16 cg, +16)
                         const uint32_t (&sr)[16] = sbuf[c];
-                        uint32_t pkP[8], pkS[8];
+                        uint32_t (&pkP)[8] = pk[c][0], (&pkS)[8] = pk[c][1];
                         if (masked) {
                             // masked sub-tiles: scalar path.  Statistics of rows that are not valid were never
                             // loaded, so a masked entry is set to zero, never multiplied by zero.
@@ -1058,8 +1050,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                                 }
                             }
                         }
-                        tmem_st_32x8(tS + 16 * cg, pkP);
-                        tmem_st_32x8(tS + 16 * cg + 8, pkS);
+                        if constexpr (kPBufs > 1) store_chunk(c);
                         if constexpr (kSpill) {
                             // streaming stores: written once, read once by the dQ kernel much later
 #pragma unroll
@@ -1070,9 +1061,15 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                             }
                         }
                     }
+                    if constexpr (kPBufs == 1) {
+                        if (it >= 1 && !mbar_wait(&bars->p_free[0], (it - 1) & 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
+                        tc_fence_after();
+#pragma unroll
+                        for (int c = 0; c < kChunks; ++c) store_chunk(c);
+                    }
                     tmem_wait_st();
                     tc_fence_before();
-                    mbar_arrive(&bars->p_full[bf]);
+                    mbar_arrive_warp(&bars->p_full[bf]);
                 }
             }
         }
