@@ -182,6 +182,8 @@ Geometry make_geometry(int B, int N, int H, int Hkv, int G, int n_unshifted, int
     g.groups = N / G;
     g.leak_free = (flags & S2A_FLAG_LEAK_FREE) ? 1 : 0;
     g.swap_wrapped = (flags & S2A_FLAG_SWAP_WRAPPED) ? 1 : 0;
+    g.rep = H / Hkv;
+    g.by_group = FastDiv(G), g.by_groups = FastDiv(g.groups), g.by_rep = FastDiv(g.rep);
     // the grid has one slot per (unit, tile rank); groups with fewer tiles leave their last slots idle
     g.tiles_per_group = most_over_groups(g, [](const GroupLayout& L) { return L.nTiles; });
     return g;
@@ -278,7 +280,8 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     p.geo = make_geometry(B, N, H, Hkv, G, n_unshifted, shift, flags);
     p.single = take_single_tiles(p.geo, H, ds->n_sm);
     p.pairs_per_group = most_pairs(p.geo, p.single);
-    p.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * 4);  // q, k, v, o
+    p.order = BlockOrder(B * H * p.geo.groups, p.pairs_per_group, unit_chunk(static_cast<long long>(G) * d * 2 * 4));  // q, k, v, o
+    p.by_heads = FastDiv(H);
     p.scale_log2 = scale * kLog2eHost;
     cudaError_t e = launch_fwd(p, d, static_cast<cudaStream_t>(stream), is_short(p.geo, d, ds->n_sm));
     return e == cudaSuccess ? S2A_OK : cuda_fail(e);
@@ -381,7 +384,8 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     pk.status = ds->status_ptr, pk.host_status = ds->host_word_dev, pk.geo = geo, pk.scale = scale, pk.scale_log2 = scale * kLog2eHost;
     pk.spill = nullptr;
     pk.pass.hk0 = 0, pk.pass.nk = Hkv;
-    pk.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * (2 * (H / Hkv) + 2));  // q and dO of every query head, k, v
+    const int chunk_kv = unit_chunk(static_cast<long long>(G) * d * 2 * (2 * (H / Hkv) + 2));  // q and dO of every query head, k, v
+    pk.order = BlockOrder(B * Hkv * geo.groups, geo.tiles_per_group, chunk_kv), pk.by_heads = FastDiv(Hkv);
 
     PreParams pp;
     pp.o = static_cast<const __nv_bfloat16*>(o), pp.dO = static_cast<const __nv_bfloat16*>(dO), pp.Dsum = Dsum;
@@ -417,7 +421,8 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
             if ((rc = make_tmap(&pq.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
             if ((rc = make_tmap(&pq.tm_do, dO, d, H, N, B, kTile)) != S2A_OK) return rc;
             pq.tm_k = pk.tm_k, pq.tm_v = pk.tm_v;
-            pq.chunk = unit_chunk(static_cast<long long>(G) * d * 2 * 4);  // q, dO, k, v
+            pq.order = BlockOrder(B * H * geo.groups, geo.tiles_per_group, unit_chunk(static_cast<long long>(G) * d * 2 * 4));  // q, dO, k, v
+            pq.by_heads = FastDiv(H);
             pq.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
             pq.lse = lse, pq.Dsum = Dsum, pq.dq = static_cast<__nv_bfloat16*>(dq);
             pq.status = ds->status_ptr, pq.host_status = ds->host_word_dev, pq.geo = geo, pq.scale = scale, pq.scale_log2 = scale * kLog2eHost;
@@ -435,13 +440,16 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     ps.spill = pk.spill;
     ps.dq = static_cast<__nv_bfloat16*>(dq), ps.dq_tok_stride = ts.dq ? ts.dq : static_cast<long long>(H) * d;
     ps.status = ds->status_ptr, ps.host_status = ds->host_word_dev, ps.geo = geo, ps.scale = scale;
-    ps.chunk = kUnitChunk;  // what streams through this kernel, dS, is read once: 4 to 16 units make no difference
     for (int hk0 = 0; hk0 < Hkv; hk0 += static_cast<int>(nk_fit)) {
         const int nk = Hkv - hk0 < static_cast<int>(nk_fit) ? Hkv - hk0 : static_cast<int>(nk_fit);
         pk.pass.hk0 = hk0, pk.pass.nk = nk;
         ps.pass = pk.pass;
         ps.single = take_single_tiles(geo, nk * (H / Hkv), ds->n_sm);
         ps.pairs_per_group = most_pairs(geo, ps.single);
+        pk.order = BlockOrder(B * nk * geo.groups, geo.tiles_per_group, chunk_kv), pk.by_heads = FastDiv(nk);
+        // what streams through the product kernel, dS, is read once: chunks of 4 to 16 units make no difference
+        ps.by_heads = FastDiv(nk * (H / Hkv));
+        ps.order = BlockOrder(B * nk * (H / Hkv) * geo.groups, ps.pairs_per_group, kUnitChunk);
         if (stages & kStageDkDv) {
             e = launch_bwd_dkdv(pk, d, st);
             if (e != cudaSuccess) return cuda_fail(e);

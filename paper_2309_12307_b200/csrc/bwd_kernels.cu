@@ -225,12 +225,10 @@ struct DqItem {
 // fewer tiles than the largest one.
 __device__ __forceinline__ bool dq_item(const BwdDqParams& p, int id, DqItem* t) {
     const Geometry& geo = p.geo;
-    int unit, rank;
-    decode_block(id, geo.B * geo.H * geo.groups, geo.tiles_per_group, &unit, &rank, p.chunk);
-    const int g = unit % geo.groups;
-    t->h = (unit / geo.groups) % geo.H;
-    t->b = unit / (geo.groups * geo.H);
-    t->hk = t->h / (geo.H / geo.Hkv);
+    int unit, rank, g;
+    p.order.decode(id, &unit, &rank);
+    t->b = p.by_heads(geo.by_groups(unit, &g), &t->h);
+    t->hk = geo.by_rep(t->h);
     t->L = group_layout(geo, (t->h < geo.n_unshifted) ? 0 : geo.shift, g);
     const int i = t->L.nTiles - 1 - rank;
     if (i < 0) return false;
@@ -595,9 +593,9 @@ __device__ __forceinline__ HeadWalk head_walk(const Geometry& geo, int hq, int t
     HeadWalk w;
     const int s = (hq < geo.n_unshifted) ? 0 : geo.shift;
     const int pos = mod_pos(tk0 - s, geo.N);
-    w.g = pos / geo.G;
+    int in_group;
+    w.g = geo.by_group(pos, &in_group);
     w.L = group_layout(geo, s, w.g);
-    const int in_group = pos - w.g * geo.G;
     const int nB = w.L.nTiles - w.L.nA;
     w.j = in_group < w.L.lenA ? (w.L.swapped ? nB : 0) + in_group / kTile
                               : (w.L.swapped ? 0 : w.L.nA) + (in_group - w.L.lenA) / kTile;
@@ -616,12 +614,11 @@ __device__ __forceinline__ DkDvItem dkdv_item(const BwdDkDvParams& p, long long 
     const Geometry& geo = p.geo;
     const SpillPass& pass = p.pass;
     DkDvItem t;
-    int unit, j0;
-    decode_block(id, geo.B * pass.nk * geo.groups, geo.tiles_per_group, &unit, &j0, p.chunk);
-    const int g0 = unit % geo.groups;
-    const int rep = geo.H / geo.Hkv;
-    t.hk = pass.hk0 + (unit / geo.groups) % pass.nk;
-    t.b = unit / (geo.groups * pass.nk);
+    int unit, j0, g0;
+    p.order.decode(static_cast<int>(id), &unit, &j0);
+    const int rep = geo.rep;
+    t.b = p.by_heads(geo.by_groups(unit, &g0), &t.hk);
+    t.hk += pass.hk0;
     const int hq0 = t.hk * rep;
     const int s0 = (hq0 < geo.n_unshifted) ? 0 : geo.shift;
     const GroupLayout L0 = group_layout(geo, s0, g0);
@@ -704,7 +701,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     if (bars->abort_flag != 0) return;
     __syncthreads();
     const Geometry& geo = p.geo;
-    const int rep = geo.H / geo.Hkv;
+    const int rep = geo.rep;
     const int Tg = geo.tiles_per_group;
 
     if (threadIdx.x == 0) {
@@ -1195,16 +1192,12 @@ static_assert(sizeof(DqSpillBars) <= 1024, "barrier block");
 // a slot of a group that has fewer pairs than the largest one.
 __device__ __forceinline__ bool dq_spill_item(const BwdDqSpillParams& p, int id, DqSpillItem* w) {
     const Geometry& geo = p.geo;
-    const int rep = geo.H / geo.Hkv;
-    const int heads = p.pass.nk * rep;
-    const int units = geo.B * heads * geo.groups;
-    int unit, rank;
-    decode_block(id, units, p.pairs_per_group, &unit, &rank, p.chunk);
-    unit = units - 1 - unit;
-    const int g = unit % geo.groups;
-    w->h = p.pass.hk0 * rep + (unit / geo.groups) % heads;
-    w->b = unit / (geo.groups * heads);
-    w->hk = w->h / rep;
+    int unit, rank, g;
+    p.order.decode(id, &unit, &rank);
+    unit = p.order.units - 1 - unit;
+    w->b = p.by_heads(geo.by_groups(unit, &g), &w->h);
+    w->h += p.pass.hk0 * geo.rep;
+    w->hk = geo.by_rep(w->h);
     w->unit = unit;
     w->L = group_layout(geo, (w->h < geo.n_unshifted) ? 0 : geo.shift, g);
     if (rank >= pairs_of_group(w->L, p.single)) return false;

@@ -98,12 +98,10 @@ constexpr float kLazyRescale = 8.0f;
 
 // Work item `id`; false marks a slot of a group that has fewer pairs than the largest one.
 __device__ __forceinline__ bool fwd_item(const FwdParams& p, int id, FwdItem* w) {
-    int unit, rank;
-    decode_block(id, p.geo.B * p.geo.H * p.geo.groups, p.pairs_per_group, &unit, &rank, p.chunk);
-    const int g = unit % p.geo.groups;
-    w->h = (unit / p.geo.groups) % p.geo.H;
-    w->b = unit / (p.geo.groups * p.geo.H);
-    w->hk = w->h / (p.geo.H / p.geo.Hkv);
+    int unit, rank, g;
+    p.order.decode(id, &unit, &rank);
+    w->b = p.by_heads(p.geo.by_groups(unit, &g), &w->h);
+    w->hk = p.geo.by_rep(w->h);
     w->L = group_layout(p.geo, (w->h < p.geo.n_unshifted) ? 0 : p.geo.shift, g);
     if (rank >= pairs_of_group(w->L, p.single)) return false;
     w->t = tile_pair(w->L, rank, p.single);

@@ -38,16 +38,55 @@ __host__ __device__ inline int unit_chunk(long long unit_bytes) {
     while (n < 4096 && 2 * n * unit_bytes <= kChunkBytes) n *= 2;
     return n;
 }
-__host__ __device__ inline void decode_block(long long idx, int units, int tiles, int* unit, int* rank, int unit_chunk = kUnitChunk) {
-    // 32-bit arithmetic (the entry points admit fewer than 2^31 tiles): this runs on one thread between two
-    // work items, where a 64-bit division is a subroutine of several hundred clocks
-    const uint32_t i = static_cast<uint32_t>(idx), per_chunk = static_cast<uint32_t>(unit_chunk < units ? unit_chunk : units) * tiles;
-    const uint32_t chunk = i / per_chunk;
-    const uint32_t within = i - chunk * per_chunk;
-    const int first = static_cast<int>(chunk) * unit_chunk;
-    const int in_chunk = (units - first) < unit_chunk ? (units - first) : unit_chunk;
-    *rank = static_cast<int>(within / static_cast<uint32_t>(in_chunk));
-    *unit = first + static_cast<int>(within) - *rank * in_chunk;
+// n / d for 0 <= n < 2^31 as a multiplication (d, and with it the multiplier, is known when the kernel is
+// launched): decoding a work item takes about seven divisions one after the other, on one thread, while the
+// other warps wait for the item.  dK,dV kernel, division and multiplication, us a launch in a loop: Llama2-7B 16k 951
+// and 909, 8k 275 and 264, 4 x 2048 tokens with groups of 512 120 and 113.
+struct FastDiv {
+    uint32_t d = 1, m = 0;
+    int s = 0;
+    FastDiv() = default;
+    explicit FastDiv(int divisor) : d(static_cast<uint32_t>(divisor)) {
+        if (divisor <= 1) return;
+        int l = 1;  // 2^(l-1) < d <= 2^l
+        while ((1ull << l) < d) ++l;
+        m = static_cast<uint32_t>(((1ull << (31 + l)) + d - 1) / d);  // n m / 2^(31+l) is exact for n < 2^31
+        s = l - 1;
+    }
+    __host__ __device__ int operator()(int n) const {
+        if (d <= 1) return n;
+#ifdef __CUDA_ARCH__
+        return static_cast<int>(__umulhi(static_cast<uint32_t>(n), m) >> s);
+#else
+        return static_cast<int>((static_cast<uint64_t>(static_cast<uint32_t>(n)) * m) >> 32 >> s);
+#endif
+    }
+    // n / d; *rest = n % d
+    __host__ __device__ int operator()(int n, int* rest) const {
+        const int q = (*this)(n);
+        *rest = n - q * static_cast<int>(d);
+        return q;
+    }
+};
+
+// The block order of a launch: `units` units of `tiles` tiles in chunks of `chunk` units.
+struct BlockOrder {
+    int units = 0, chunk = 1, tail = 0;  // tail: first unit of the last chunk, which can be smaller
+    FastDiv per_chunk, in_chunk, in_tail;
+    BlockOrder() = default;
+    BlockOrder(int units_, int tiles, int chunk_) : units(units_), chunk(chunk_ < units_ ? chunk_ : units_) {
+        tail = (units - 1) / chunk * chunk;
+        per_chunk = FastDiv(chunk * tiles), in_chunk = FastDiv(chunk), in_tail = FastDiv(units - tail);
+    }
+    __host__ __device__ void decode(int idx, int* unit, int* rank) const {
+        int within, at;
+        const int first = per_chunk(idx, &within) * chunk;
+        *rank = first == tail ? in_tail(within, &at) : in_chunk(within, &at);
+        *unit = first + at;
+    }
+};
+inline void decode_block(long long idx, int units, int tiles, int* unit, int* rank, int unit_chunk = kUnitChunk) {
+    BlockOrder(units, tiles, unit_chunk).decode(static_cast<int>(idx), unit, rank);
 }
 
 // Geometry of the shifted grouping (Algorithm 1): common to every kernel.
@@ -59,6 +98,8 @@ struct Geometry {
     int groups;           // N / G
     int leak_free;        // variant 2 of Appendix B: cut the wrapped group of a shifted head at the wrap
     int swap_wrapped;     // variant 3 of Appendix B: the two runs of the wrapped group change places
+    int rep;              // query heads of a KV head, H / Hkv
+    FastDiv by_group, by_groups, by_rep;  // divisions by G, by groups and by rep
 };
 
 // Where the tokens of one group live.  Group g of a head with shift s holds rolled positions
@@ -176,7 +217,8 @@ struct alignas(64) FwdParams {
     Geometry geo;
     int pairs_per_group;  // largest number of query tile pairs any group has
     bool single;          // work items are single tiles (see tile_pair)
-    int chunk;            // units in a chunk of the block order
+    BlockOrder order;     // of the pairs of (batch, head, group)
+    FastDiv by_heads;     // division by H
     float scale_log2;     // softmax scale * log2(e)
 };
 
@@ -194,7 +236,8 @@ struct alignas(64) BwdDqParams {
     const float* Dsum;        // [B, H, N]
     __nv_bfloat16* dq;
     long long dq_tok_stride;  // elements between consecutive tokens of dq (H * d when dense)
-    int chunk;                // units in a chunk of the block order
+    BlockOrder order;         // of the query tiles of (batch, head, group)
+    FastDiv by_heads;         // division by H
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
@@ -230,7 +273,8 @@ struct alignas(64) BwdDkDvParams {
     long long dkv_tok_stride;  // elements between consecutive tokens of dk and dv (Hkv * d when dense)
     __nv_bfloat16* spill;      // dS^T blocks of this pass (spilling variant only)
     SpillPass pass;            // KV heads this launch covers (all of them when nothing is spilled)
-    int chunk;                 // units in a chunk of the block order
+    BlockOrder order;          // of the key tiles of (batch, KV head of the pass, group)
+    FastDiv by_heads;          // division by the KV heads of the pass
     int* status;       // device status word (see WaitCtx)
     int* host_status;  // its mirror in mapped host memory
     Geometry geo;
@@ -250,7 +294,8 @@ struct alignas(64) BwdDqSpillParams {
     Geometry geo;
     int pairs_per_group;  // largest number of query tile pairs any group has
     bool single;          // work items are single tiles (see tile_pair)
-    int chunk;            // units in a chunk of the block order
+    BlockOrder order;     // of the pairs of (batch, query head of the pass, group)
+    FastDiv by_heads;     // division by the query heads of the pass
     float scale;
 };
 
