@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "../../include/s2a.h"
+#include "host_plan.h"
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -31,7 +32,6 @@ bool g_host_status_registered = false;
 thread_local int tl_last_cuda_error = 0;
 
 constexpr int kMaxDevices = 64;
-constexpr int kMaxHostChunks = 16;
 struct DeviceState {
     bool ready = false;
     int* status_ptr = nullptr;        // device address of g_status_word
@@ -42,7 +42,7 @@ struct DeviceState {
     bool host_path_ready = false;
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
     cudaEvent_t ev_start = nullptr, ev_done = nullptr, ev_in_done = nullptr;
-    cudaEvent_t ev_in[kMaxHostChunks] = {}, ev_compute[kMaxHostChunks] = {};
+    cudaEvent_t ev_qkv = nullptr, ev_do = nullptr, ev_fwd = nullptr, ev_bwd = nullptr;  // recorded again for every chunk
 };
 DeviceState g_dev[kMaxDevices];
 static_assert(kMaxDevices == kMaxDevicesMirror, "one mirror word per device");
@@ -517,54 +517,17 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
     if (!ds->host_path_ready) {
         if ((e = cudaStreamCreateWithFlags(&ds->copy_in, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(e);
         if ((e = cudaStreamCreateWithFlags(&ds->copy_out, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaEventCreateWithFlags(&ds->ev_start, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaEventCreateWithFlags(&ds->ev_done, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
-        if ((e = cudaEventCreateWithFlags(&ds->ev_in_done, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
-        for (int c = 0; c < kMaxHostChunks; ++c) {
-            if ((e = cudaEventCreateWithFlags(&ds->ev_in[c], cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaEventCreateWithFlags(&ds->ev_compute[c], cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
-        }
+        for (cudaEvent_t* ev : {&ds->ev_start, &ds->ev_done, &ds->ev_in_done, &ds->ev_qkv, &ds->ev_do, &ds->ev_fwd, &ds->ev_bwd})
+            if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
         ds->host_path_ready = true;
     }
     lock.unlock();
-    // Heads are independent, so the job is cut into chunks of whole KV heads (with their query heads):
-    // while chunk c is computed, chunk c+1 travels to the device and the results of chunk c-1 travel
-    // back.  Only the first chunk's upload and the last chunk's download cannot be hidden, so the
-    // chunks at both ends are small and grow towards the middle, where wide rows keep the strided
-    // copies efficient: 2,2,4,8,8,4,2,2 KV heads for Hkv = 32 (a chunk of a single 256-byte head row per
-    // token copies at well under the link's rate, which costs more than its shorter exposure saves).
-    // Chunk c holds the KV
-    // heads [kv0[c], kv0[c] + kvn[c]) and sits densely ([B, N, heads of the chunk, d]) at the matching
-    // offset of the caller's device buffers.
+    // Heads and groups are independent, so the job is cut into chunks (host_plan.h): while chunk c is
+    // computed, chunk c + 1 travels to the device and the results of chunk c - 1 travel back.  The forward
+    // pass of a chunk runs while its dO is on its way, and o goes back while its backward pass runs.
     const int rep = H / Hkv;
-    int kv0[kMaxHostChunks], kvn[kMaxHostChunks];
-    int chunks = 0;
-    {
-        int left[kMaxHostChunks / 2], right[kMaxHostChunks / 2], nl = 0, nr = 0;
-        const int first = Hkv >= 32 ? Hkv / 16 : 1;
-        int remaining = Hkv, size = first, uses = 0;
-        const int cap = Hkv >= 8 ? Hkv / 4 : 1;
-        while (remaining > 0) {
-            const int a = size < remaining ? size : remaining;
-            if (nl <= nr) left[nl++] = a; else right[nr++] = a;
-            remaining -= a;
-            if (++uses == (size == first ? 4 : 2)) {   // the smallest size twice at each end, then every size once per end
-                uses = 0;
-                if (size * 2 <= cap) size *= 2;
-            }
-            if (nl + nr == kMaxHostChunks - 1 && remaining > 0) {   // out of slots: the rest in one chunk
-                if (nl <= nr) left[nl++] = remaining; else right[nr++] = remaining;
-                remaining = 0;
-            }
-        }
-        int at_kv = 0;
-        for (int x = 0; x < nl; ++x) kv0[chunks] = at_kv, kvn[chunks] = left[x], at_kv += left[x], ++chunks;
-        for (int x = nr - 1; x >= 0; --x) kv0[chunks] = at_kv, kvn[chunks] = right[x], at_kv += right[x], ++chunks;
-    }
-    const size_t rows = static_cast<size_t>(B) * N;
-    const size_t hb = static_cast<size_t>(d) * 2;                                              // bytes of one head of one token
-    const size_t pq = static_cast<size_t>(H) * d * 2, pk = static_cast<size_t>(Hkv) * d * 2;   // host pitches
-    const size_t pl = static_cast<size_t>(H) * N * sizeof(float);
+    const size_t hb = static_cast<size_t>(d) * 2;  // bytes of one head of one token
+    const float scale = 1.0f / sqrtf(static_cast<float>(d));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     auto at = [](const void* base, size_t bytes) { return const_cast<char*>(static_cast<const char*>(base)) + bytes; };
 
@@ -581,40 +544,67 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
     auto enqueue_all = [&]() -> int {
         if ((e = cudaStreamWaitEvent(ds->copy_in, ds->ev_start, 0)) != cudaSuccess) return cuda_fail(e);
         if ((e = cudaStreamWaitEvent(ds->copy_out, ds->ev_start, 0)) != cudaSuccess) return cuda_fail(e);
-        for (int c = 0; c < chunks; ++c) {
-            const int kvc = kvn[c], hc = kvc * rep, h0 = kv0[c] * rep;   // KV heads, query heads, first query head of the chunk
-            const size_t wq = hc * hb, wk = kvc * hb;                    // bytes per token of the chunk
-            const size_t wl = static_cast<size_t>(hc) * N * sizeof(float);
-            const size_t oq = rows * h0 * hb, ok_ = rows * kv0[c] * hb, ol = static_cast<size_t>(B) * h0 * N * sizeof(float);
-            void *cq = at(d_q, oq), *ck = at(d_k, ok_), *cv = at(d_v, ok_), *cdo = at(d_dO, oq), *co = at(d_o, oq);
-            void *cdq = at(d_dq, oq), *cdk = at(d_dk, ok_), *cdv = at(d_dv, ok_);
-            float* cl = reinterpret_cast<float*>(at(d_lse, ol));
-            // host -> device: the chunk's heads of every token
-            if ((e = cudaMemcpy2DAsync(cq, wq, at(h_q, h0 * hb), pq, wq, rows, cudaMemcpyHostToDevice, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(ck, wk, at(h_k, kv0[c] * hb), pk, wk, rows, cudaMemcpyHostToDevice, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(cv, wk, at(h_v, kv0[c] * hb), pk, wk, rows, cudaMemcpyHostToDevice, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(cdo, wq, at(h_dO, h0 * hb), pq, wq, rows, cudaMemcpyHostToDevice, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaEventRecord(ds->ev_in[c], ds->copy_in)) != cudaSuccess) return cuda_fail(e);
-            // compute on the caller's stream; the second half of ALL heads is shifted
-            if ((e = cudaStreamWaitEvent(st, ds->ev_in[c], 0)) != cudaSuccess) return cuda_fail(e);
-            int n_unshifted = H / 2 - h0;
-            n_unshifted = n_unshifted < 0 ? 0 : (n_unshifted > hc ? hc : n_unshifted);
-            const float scale = 1.0f / sqrtf(static_cast<float>(d));
-            int rc2 = fwd_impl(cq, ck, cv, co, cl, B, N, hc, kvc, d, G, scale, n_unshifted, G / 2, 0u, stream, TokStrides());
+        size_t at_q = 0, at_kv = 0;  // (token, head) rows of the chunks before this one
+        return cut_host_job(B, N, H, Hkv, d, G, [&](const HostChunk& c) -> int {
+            const int n = c.tokens(), hc = c.kvn * rep, h0 = c.kv0 * rep;
+            void *cq = at(d_q, at_q * hb), *ck = at(d_k, at_kv * hb), *cv = at(d_v, at_kv * hb), *cdo = at(d_dO, at_q * hb);
+            void *co = at(d_o, at_q * hb), *cdq = at(d_dq, at_q * hb), *cdk = at(d_dk, at_kv * hb), *cdv = at(d_dv, at_kv * hb);
+            float* cl = d_lse + at_q;
+            at_q += static_cast<size_t>(c.bn) * n * hc, at_kv += static_cast<size_t>(c.bn) * n * c.kvn;
+            // `heads` heads from `first` on, of a tensor with `all` heads, for the chunk's tokens; several batch items come with all N
+            auto copy = [&](cudaMemcpyKind kind, const void* host, void* dev, int all, int first, int heads) -> cudaError_t {
+                const size_t w = heads * hb, pitch = all * hb;
+                size_t row = 0;
+                for (int r = 0; r < 2; ++r) {
+                    if (c.n[r] == 0) continue;
+                    void* h = at(host, (static_cast<size_t>(c.b0) * N + c.from[r]) * pitch + first * hb);
+                    void* g = at(dev, row * w);
+                    const size_t rows = static_cast<size_t>(c.bn) * c.n[r];
+                    const cudaError_t ec = kind == cudaMemcpyHostToDevice
+                                               ? cudaMemcpy2DAsync(g, w, h, pitch, w, rows, kind, ds->copy_in)
+                                               : cudaMemcpy2DAsync(h, pitch, g, w, w, rows, kind, ds->copy_out);
+                    if (ec != cudaSuccess) return ec;
+                    row += rows;
+                }
+                return cudaSuccess;
+            };
+            auto copy_lse = [&]() -> cudaError_t {
+                float* h = h_lse + (static_cast<size_t>(c.b0) * H + h0) * N;
+                const size_t f = sizeof(float);
+                if (n == N) return cudaMemcpy2DAsync(h, H * f * N, cl, hc * f * N, hc * f * N, c.bn, cudaMemcpyDeviceToHost, ds->copy_out);
+                for (int r = 0, row = 0; r < 2; row += c.n[r], ++r) {
+                    if (c.n[r] == 0) continue;
+                    const cudaError_t ec = cudaMemcpy2DAsync(h + c.from[r], f * N, cl + row, f * n, f * c.n[r], hc, cudaMemcpyDeviceToHost, ds->copy_out);
+                    if (ec != cudaSuccess) return ec;
+                }
+                return cudaSuccess;
+            };
+            auto after = [](cudaStream_t waiting, cudaEvent_t ev, cudaStream_t done) -> cudaError_t {
+                const cudaError_t ec = cudaEventRecord(ev, done);
+                return ec != cudaSuccess ? ec : cudaStreamWaitEvent(waiting, ev, 0);
+            };
+            // host -> device, and the forward pass behind q, k, v
+            if ((e = copy(cudaMemcpyHostToDevice, h_q, cq, H, h0, hc)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyHostToDevice, h_k, ck, Hkv, c.kv0, c.kvn)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyHostToDevice, h_v, cv, Hkv, c.kv0, c.kvn)) != cudaSuccess) return cuda_fail(e);
+            if ((e = after(st, ds->ev_qkv, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyHostToDevice, h_dO, cdo, H, h0, hc)) != cudaSuccess) return cuda_fail(e);
+            int rc2 = fwd_impl(cq, ck, cv, co, cl, c.bn, n, hc, c.kvn, d, G, scale, c.n_unshifted, c.shift, 0u, stream, TokStrides());
             if (rc2 != S2A_OK) return rc2;
-            rc2 = bwd_impl(cq, ck, cv, co, cl, cdo, cdq, cdk, cdv, B, N, hc, kvc, d, G, scale, n_unshifted, G / 2, workspace,
+            // o and lse go back while the backward pass runs behind dO
+            if ((e = after(ds->copy_out, ds->ev_fwd, st)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyDeviceToHost, h_o, co, H, h0, hc)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy_lse()) != cudaSuccess) return cuda_fail(e);
+            if ((e = after(st, ds->ev_do, ds->copy_in)) != cudaSuccess) return cuda_fail(e);
+            rc2 = bwd_impl(cq, ck, cv, co, cl, cdo, cdq, cdk, cdv, c.bn, n, hc, c.kvn, d, G, scale, c.n_unshifted, c.shift, workspace,
                            workspace_bytes, stream, kStageAll);
             if (rc2 != S2A_OK) return rc2;
-            if ((e = cudaEventRecord(ds->ev_compute[c], st)) != cudaSuccess) return cuda_fail(e);
-            // device -> host
-            if ((e = cudaStreamWaitEvent(ds->copy_out, ds->ev_compute[c], 0)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(at(h_o, h0 * hb), pq, co, wq, wq, rows, cudaMemcpyDeviceToHost, ds->copy_out)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(at(h_lse, static_cast<size_t>(h0) * N * sizeof(float)), pl, cl, wl, wl, B, cudaMemcpyDeviceToHost, ds->copy_out)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(at(h_dq, h0 * hb), pq, cdq, wq, wq, rows, cudaMemcpyDeviceToHost, ds->copy_out)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(at(h_dk, kv0[c] * hb), pk, cdk, wk, wk, rows, cudaMemcpyDeviceToHost, ds->copy_out)) != cudaSuccess) return cuda_fail(e);
-            if ((e = cudaMemcpy2DAsync(at(h_dv, kv0[c] * hb), pk, cdv, wk, wk, rows, cudaMemcpyDeviceToHost, ds->copy_out)) != cudaSuccess) return cuda_fail(e);
-        }
-        return S2A_OK;
+            if ((e = after(ds->copy_out, ds->ev_bwd, st)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyDeviceToHost, h_dq, cdq, H, h0, hc)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyDeviceToHost, h_dk, cdk, Hkv, c.kv0, c.kvn)) != cudaSuccess) return cuda_fail(e);
+            if ((e = copy(cudaMemcpyDeviceToHost, h_dv, cdv, Hkv, c.kv0, c.kvn)) != cudaSuccess) return cuda_fail(e);
+            return S2A_OK;
+        });
     };
     rc = enqueue_all();
     // the caller's stream is done when the last copy back is (also after a failure part-way)

@@ -51,3 +51,29 @@ def test_tile_edges_match_oracle(B, N, G, H, Hkv, d, kw):
             err = rel_l2(got.double().cpu().numpy(), want)
             assert math.isfinite(err) and err <= 1e-2, (name, fast, err)
     assert s2a.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("B,N,G,H,Hkv,d", [(1, 8192, 2048, 32, 32, 64),   # groups and heads cut
+                                           (1, 6000, 600, 16, 8, 128),    # ragged tiles; two groups in the chunk that wraps
+                                           (2, 4096, 4096, 16, 4, 128),   # one group: heads cut only
+                                           (1, 8192, 1024, 6, 3, 128),    # a KV head with shifted and unshifted query heads
+                                           (20, 1024, 512, 4, 4, 128)])   # several batch items to a chunk, not the same number
+@pytest.mark.parametrize("fast", [False, True])
+def test_host_chunks_equal_device_path(B, N, G, H, Hkv, d, fast):
+    """A chunk of the host entry point cuts its groups into the tiles of the whole job, so nothing differs by a bit."""
+    from paper_2309_12307_b200 import binding as s2a
+    dev = torch.device("cuda:0")
+    gen = torch.Generator(device=dev).manual_seed(5)
+    q, dO = (torch.randn(B, N, H, d, generator=gen, device=dev).bfloat16() for _ in range(2))
+    k, v = (torch.randn(B, N, Hkv, d, generator=gen, device=dev).bfloat16() for _ in range(2))
+    o, lse = s2a.s2a_fwd(q, k, v, G)
+    need = s2a.bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, 1 << 40) if fast else s2a.bwd_workspace_bytes(B, N, H, Hkv, d, G)
+    ws = torch.empty(need, dtype=torch.uint8, device=dev)
+    want = (o, lse, *s2a.s2a_bwd(q, k, v, o, lse, dO, G, workspace=ws))
+    host_in = [x.cpu().pin_memory() for x in (q, k, v, dO)]
+    host_out = [torch.full(x.shape, float("nan"), dtype=x.dtype).pin_memory() for x in want]
+    s2a.s2a_fwd_bwd_host(host_in, host_out, [torch.empty_like(x) for x in (q, k, v, dO, *want)], G, ws)
+    torch.cuda.synchronize()
+    assert s2a.device_status()[0] == 0
+    for got, ref in zip(host_out, want):
+        assert torch.equal(got, ref.cpu())

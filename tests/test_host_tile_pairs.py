@@ -12,7 +12,7 @@ CUDA_INC = os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include
 
 
 @pytest.mark.skipif(shutil.which("g++") is None or not os.path.isdir(CUDA_INC), reason="needs g++ and the CUDA headers")
-@pytest.mark.parametrize("program", ["tile_pairs", "fast_div"])
+@pytest.mark.parametrize("program", ["tile_pairs", "fast_div", "host_plan"])
 def test_work_items_decode_to_every_tile_once(tmp_path, program):
     exe = str(tmp_path / program)
     src = os.path.join(ROOT, "tests", "host", program + ".cpp")
