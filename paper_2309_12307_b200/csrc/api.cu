@@ -389,7 +389,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
 
     PreParams pp;
     pp.o = static_cast<const __nv_bfloat16*>(o), pp.dO = static_cast<const __nv_bfloat16*>(dO), pp.Dsum = Dsum;
-    pp.B = B, pp.N = N, pp.H = H;
+    pp.rows = B * N * H, pp.N = N, pp.H = H, pp.by_heads = FastDiv(H), pp.by_tokens = FastDiv(N);
 
     // How many KV heads' worth of dS^T the workspace can hold beyond D: with room for at least one, the
     // dK,dV kernel spills dS^T and dQ is a plain product (several passes over the KV heads if they do

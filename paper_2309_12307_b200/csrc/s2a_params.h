@@ -226,7 +226,9 @@ struct PreParams {
     const __nv_bfloat16* o;
     const __nv_bfloat16* dO;
     float* Dsum;  // [B, H, N]
-    int B, N, H;
+    int rows;     // B N H: o and dO of 2^31 rows would be 550 GB
+    int N, H;
+    FastDiv by_heads, by_tokens;
 };
 
 struct alignas(64) BwdDqParams {

@@ -28,6 +28,8 @@ def rel_l2(got, want):
     (1, 320, 160, 2, 2, 64, {}),                        # 32 rows in the last tile
     (2, 336, 168, 2, 2, 128, {}),                       # 40 rows, 84-row runs where the group wraps
     (1, 384, 192, 2, 2, 128, {"leak_free": True}),      # a cut inside a pair of tiles
+    (1, 168, 168, 2, 2, 128, {}),                       # D's last block has half of its rows
+    (3, 136, 136, 2, 2, 64, {}),                        # and three quarters
     (1, 1920, 640, 4, 4, 64, {"leak_free": True}),      # five tiles, cut after the third
     (1, 640, 320, 2, 2, 128, {"swap_wrapped": True}),
     (3, 1536, 128, 10, 2, 64, {"n_unshifted": 5}),      # more units than blocks
