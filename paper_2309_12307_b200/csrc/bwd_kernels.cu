@@ -5,8 +5,8 @@
 //     dQ = scale * dS K    dK = scale * dS^T Q
 // Four kernels:
 //   1. preprocess: D[b,h,t] = sum_c dO[b,t,h,c] * o[b,t,h,c]                     (memory bound)
-//   2. dQ, recomputing: one CTA per 128-row query tile, walks the 128-key tiles of its group (keys <=
-//            query) and computes S, dP, dS again
+//   2. dQ, recomputing: persistent; a work item is one 128-row query tile, which walks the 128-key tiles of
+//            its group (keys <= query) and computes S, dP, dS again
 //   3. dK,dV: persistent; a work item is one 128-row key tile, against which the 64-query sub-tiles of
 //            every query head that shares the KV head (queries >= key) are streamed, so the sum over
 //            those heads stays in tensor memory and needs no atomics.  It works on the transposed
@@ -939,8 +939,8 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     } else if (warp < 12) {
         // ---- elementwise.  Thread (quad, lane, group) owns key row 32 quad + lane and the query columns
         // [32 group, +32) of every step.  (Letting the two groups of four warps take alternate steps with a
-        // whole row per thread was measured too: with two S^T buffers the chain S^T -> elementwise ->
-        // gradient MMAs of a buffer is what a step waits for, and half the columns per thread halve its
+        // whole row per thread was measured in an earlier form with two S^T buffers: the chain S^T ->
+        // elementwise -> gradient MMAs is what a step waits for, and half the columns per thread halve its
         // elementwise part: 3.33 against 3.53 ms on the Llama2-7B 32k shape.)
         setmaxnreg_inc<C::kRegsElem>();
         const int quad = warp & 3;
