@@ -101,6 +101,18 @@ int prepare_device(DeviceState** out) {
     return S2A_OK;
 }
 
+int encode_tmap(CUtensorMap* tm, const void* base, int rank, const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    const CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void*>(base), dims, strides, box, estr,
+                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) {
+        tl_last_cuda_error = static_cast<int>(cudaErrorInvalidValue);
+        return S2A_ERR_CUDA;
+    }
+    return S2A_OK;
+}
+
 // bf16 tensor [B, N, heads, d] viewed as (d, heads, N, B); box = 64 columns x `box_rows` tokens of
 // one head, written to shared memory with the 128-byte swizzle the MMA descriptors expect.
 // `tok_stride` = elements between consecutive tokens (heads * d when the tensor is dense; 3 * H * d for
@@ -110,15 +122,18 @@ int make_tmap(CUtensorMap* tm, const void* base, int d, int heads, int N, int B,
     const cuuint64_t dims[4] = {(cuuint64_t)d, (cuuint64_t)heads, (cuuint64_t)N, (cuuint64_t)B};
     const cuuint64_t strides[3] = {(cuuint64_t)d * 2, (cuuint64_t)tok_stride * 2, (cuuint64_t)N * tok_stride * 2};
     const cuuint32_t box[4] = {64, 1, (cuuint32_t)box_rows, 1};
-    const cuuint32_t estr[4] = {1, 1, 1, 1};
-    CUresult r = g_encode(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
-                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) {
-        tl_last_cuda_error = static_cast<int>(cudaErrorInvalidValue);
-        return S2A_ERR_CUDA;
-    }
-    return S2A_OK;
+    return encode_tmap(tm, base, 4, dims, strides, box);
+}
+
+// The same tensor and swizzle with boxes of 64 columns x 128 tokens in the order 0 2 1 3, 4 6 5 7, ... (N % 4 = 0): a
+// group of four tokens is two dimensions of two.
+int make_tmap_exchanged(CUtensorMap* tm, const void* base, int d, int heads, int N, int B, long long tok_stride = 0) {
+    if (tok_stride == 0) tok_stride = static_cast<long long>(heads) * d;
+    const cuuint64_t tok = (cuuint64_t)tok_stride * 2;
+    const cuuint64_t dims[5] = {(cuuint64_t)heads * d, 2, 2, (cuuint64_t)N / 4, (cuuint64_t)B};
+    const cuuint64_t strides[4] = {2 * tok, tok, 4 * tok, N * tok};
+    const cuuint32_t box[5] = {64, 2, 2, kTile / 4, 1};
+    return encode_tmap(tm, base, 5, dims, strides, box);
 }
 
 // variants 2 and 3 of Appendix B exclude each other; no other bits are defined
@@ -270,7 +285,7 @@ int fwd_impl(const void* q, const void* k, const void* v, void* o, float* lse, i
     FwdParams p;
     memset(&p, 0, sizeof p);
     if ((rc = make_tmap(&p.tm_q, q, d, H, N, B, kTile, ts.q)) != S2A_OK) return rc;
-    if ((rc = make_tmap(&p.tm_k, k, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
+    if ((rc = make_tmap_exchanged(&p.tm_k, k, d, Hkv, N, B, ts.kv)) != S2A_OK) return rc;
     if ((rc = make_tmap(&p.tm_v, v, d, Hkv, N, B, kTile, ts.kv)) != S2A_OK) return rc;
     if ((rc = make_tmap(&p.tm_o, o, d, H, N, B, kTile)) != S2A_OK) return rc;
     p.o = static_cast<__nv_bfloat16*>(o);

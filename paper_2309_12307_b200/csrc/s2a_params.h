@@ -207,8 +207,8 @@ __host__ __device__ inline TilePair tile_pair(const GroupLayout& L, int rank, bo
 
 struct alignas(64) FwdParams {
     CUtensorMap tm_q;  // bf16 (d, H,   N, B), box (64, 1, 128, 1), 128-byte swizzle
-    CUtensorMap tm_k;  // bf16 (d, Hkv, N, B), same box
-    CUtensorMap tm_v;
+    CUtensorMap tm_k;  // bf16 (Hkv * d, 2 tokens apart by two, 2 by one, N / 4, B), box (64, 2, 2, 32, 1): see key_of_column()
+    CUtensorMap tm_v;  // bf16 (d, Hkv, N, B), box as tm_q
     CUtensorMap tm_o;  // like tm_q, for the stores of whole tiles
     __nv_bfloat16* o;
     float* lse;

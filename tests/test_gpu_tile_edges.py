@@ -79,3 +79,33 @@ def test_host_chunks_equal_device_path(B, N, G, H, Hkv, d, fast):
     assert s2a.device_status()[0] == 0
     for got, ref in zip(host_out, want):
         assert torch.equal(got, ref.cpu())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_row_sums_add_neighbouring_columns_first(d):
+    """One key with weight 1 ahead of keys with weight 2^-24, half an ulp of it: added one by one to the 1 they are lost, added
+    in pairs first they count.  The sum of each half tile is four chains of pairs; l = 1 + x is known, and lse = log(l) to
+    1 ulp of log2 and the 2^-22 of an exponential, of x (a chain for each column parity misses x by 1/128 to 1/2)."""
+    from paper_2309_12307_b200 import binding as s2a
+
+    N, f = 256, np.float32
+    scale = next(x for x in (f(np.log(2)) + f(i) * f(2) ** -25 for i in range(-8, 9)) if f(x) * f(1.4426950408889634) == f(1))
+    q, k = torch.zeros(1, N, 2, d), torch.zeros(1, N, 2, d)
+    q[..., 0], k[:, 1:, :, 0] = 1, -24
+    q, k = q.bfloat16().cuda(), k.bfloat16().cuda()
+    _, lse = s2a.s2a_fwd_ex(q, k, k, N, scale=float(scale), n_unshifted=2, shift=0)
+    want = np.zeros(N)
+    for row in range(N):
+        l = [f(0), f(0)]
+        for tile in range(row // 128 + 1):
+            p = [f(0) if 128 * tile + x > row else f(1) if tile + x == 0 else f(2) ** -24 for x in range(128)]
+            for half in range(2):
+                chains = [f(0)] * 4
+                for pair in range(32):
+                    at = 64 * half + 2 * pair
+                    chains[pair % 4] = f(chains[pair % 4] + f(p[at] + p[at + 1]))
+                l[half] = f(l[half] + f(f(chains[0] + chains[1]) + f(chains[2] + chains[3])))
+        want[row] = np.log(np.float64(f(l[0] + l[1])))
+    got = lse[0].double().cpu().numpy()
+    assert want[-1] > 200 * 2.0 ** -24
+    assert np.abs(got - want).max() <= 2e-6 * want.max(), (got[0, :8], want[:8])
