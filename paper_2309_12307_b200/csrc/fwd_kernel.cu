@@ -66,7 +66,10 @@ struct FwdCfg {
     static_assert(2 * kRegsSoftmax + kRegsEpilogue + kRegsIssue <= 4 * kRegsLaunch, "register split");
 };
 
-constexpr int kSched = 8;  // items in flight: the producer is at most five items ahead of the epilogue
+// Items in flight.  A warp that has a part in an item holds the next loads back, so the producer is at most six items
+// ahead of it.  The softmax warps of tile 0 have no part in an item without that tile (the last pair of an odd number of
+// tiles, single tiles), so they walk a list of their own, of the items that have it.
+constexpr int kSched = 8;
 
 struct FwdItem {
     int b, h, hk;
@@ -84,9 +87,11 @@ struct FwdBars {
     uint64_t stat_full[2], stat_empty[2];
     uint64_t kv_full[8], kv_empty[8];
     uint64_t sched_full[kSched];
+    uint64_t pair_full[kSched];      // the same for the softmax warps of tile 0: items with two tiles only
     uint64_t clc, drain[2];
     alignas(16) uint8_t clc_resp[16];
     FwdItem item[kSched];  // b = -1: no more items
+    int pair_slot[kSched];  // where the items counted on pair_full are
     uint32_t tmem_slot;
     int abort_flag;
 };
@@ -151,7 +156,10 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             mbar_init(&bars->kv_full[x], 1);
             mbar_init(&bars->kv_empty[x], 1);
         }
-        for (int x = 0; x < kSched; ++x) mbar_init(&bars->sched_full[x], 1);
+        for (int x = 0; x < kSched; ++x) {
+            mbar_init(&bars->sched_full[x], 1);
+            mbar_init(&bars->pair_full[x], 1);
+        }
         mbar_init(&bars->clc, 1);
         fence_barrier_init();
         tma_prefetch_desc(&p.tm_q);
@@ -204,6 +212,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 bool ok = true;
                 ItemSource items{&bars->clc, bars->clc_resp};
                 int id = static_cast<int>(blockIdx.x);
+                uint32_t n_pairs = 0;  // items with two tiles so far
                 auto load_q = [&](const FwdItem& w, int t) {
                     if (!mbar_wait(&bars->q_empty[t], (n_q[t] & 1) ^ 1, ctx, kWaitFwd + 2)) { ok = false; return; }
                     mbar_expect_tx(&bars->q_full[t], C::kTileBytes);
@@ -231,6 +240,10 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     if (id < 0) w.b = -1;
                     bars->item[k % kSched] = w;
                     mbar_arrive(&bars->sched_full[k % kSched]);  // release: the item is visible to whoever sees the phase
+                    if (id < 0 || w.t.n[0] > 0) {
+                        bars->pair_slot[n_pairs % kSched] = k % kSched;
+                        mbar_arrive(&bars->pair_full[n_pairs++ % kSched]);
+                    }
                     if (id < 0) break;
                     for (int j = 0; ok && j < w.t.n[1]; ++j) {
                         const int tok0 = tile_ref(w.L, w.t.j_begin + j).tok0;
@@ -414,11 +427,12 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         const uint64_t c2x2 = f2_pack(c2, c2);
         uint32_t n_s = 0, n_it = 0;
         bool ok = true;
+        uint64_t* full = t ? bars->sched_full : bars->pair_full;
         for (int k = 0; ok; ++k) {
-            FwdItem w;
-            if (!next_item(k, kWaitFwd + 14, &w)) break;
+            if (!mbar_wait_uniform(&full[k % kSched], (k / kSched) & 1, ctx, kWaitFwd + 14)) break;
+            const FwdItem w = bars->item[t ? k % kSched : bars->pair_slot[k % kSched]];
+            if (w.b < 0) break;
             const int n = t ? w.t.n[1] : w.t.n[0];
-            if (n == 0) continue;
             float m_used = 0.f;   // running maximum in use, scaled to log2 units
             // running sum of exp2(s*c2 - m_used) over the keys [0, 64) and [64, 128) of the tiles
             float l[2] = {0.f, 0.f};

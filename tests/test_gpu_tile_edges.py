@@ -33,6 +33,7 @@ def rel_l2(got, want):
     (1, 1920, 640, 4, 4, 64, {"leak_free": True}),      # five tiles, cut after the third
     (1, 640, 320, 2, 2, 128, {"swap_wrapped": True}),
     (3, 1536, 128, 10, 2, 64, {"n_unshifted": 5}),      # more units than blocks
+    (2, 16384, 128, 8, 8, 64, {"n_unshifted": 8}),      # 14 items to a block, none with a second query tile
     (1, 4992, 1664, 12, 12, 64, {}),                    # 13 tiles: more pairs than blocks, the last one single
 ])
 def test_tile_edges_match_oracle(B, N, G, H, Hkv, d, kw):
