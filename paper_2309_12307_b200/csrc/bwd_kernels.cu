@@ -976,7 +976,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     const int st = it % C::kStages;
                     // The statistics of this step travel with its stage; the score MMA warp's arrival on s_full says that
                     // it has seen the stage land.  (Every wait here is 5 % of a step with head size 64.)
-                    if (!mbar_wait(&bars->s_full, it & 1, ctx, kWaitBwdDkDv + 6)) { ok = false; break; }
+                    if (!mbar_wait_uniform(&bars->s_full, it & 1, ctx, kWaitBwdDkDv + 6)) { ok = false; break; }
                     tc_fence_after();
                     // copy this thread's part of dP^T and S^T into registers and release their buffers as soon as the
                     // copies have landed, so that the score products of the next step run while this one is worked on
@@ -1070,7 +1070,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                         }
                     }
                     if constexpr (kPBufs == 1) {
-                        if (it >= 1 && !mbar_wait(&bars->p_free[0], (it - 1) & 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
+                        if (it >= 1 && !mbar_wait_uniform(&bars->p_free[0], (it - 1) & 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
                         tc_fence_after();
 #pragma unroll
                         for (int c = 0; c < kChunks; ++c) store_chunk(c);
