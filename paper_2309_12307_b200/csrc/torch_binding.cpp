@@ -10,6 +10,7 @@
 #include <torch/extension.h>
 
 #include <ATen/cuda/CUDAContext.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <cuda_runtime_api.h>
 
@@ -57,6 +58,37 @@ Tensor new_stats(const Sizes& s, const Tensor& like) { return at::empty({s.B, s.
 Tensor new_like(const Tensor& t) { return at::empty(t.sizes(), t.options()); }
 
 void* current_stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+// The stream of a call of binding.py: the one it was given, or torch's current one.  What is made for a call on another
+// stream than the current one (the workspace, outputs that were not given) belongs to that stream in the caching
+// allocator.  From the current stream's memory it could take a block that work still queued there uses, and the
+// workspace, which goes back when the call returns, could be handed out and overwritten before the kernels ran.
+class CallStream {
+public:
+    CallStream(std::optional<int64_t> given, const Tensor& like)
+        : stream_(given ? reinterpret_cast<cudaStream_t>(*given) : c10::cuda::getCurrentCUDAStream().stream()) {
+        const auto current = c10::cuda::getCurrentCUDAStream(like.device().index());
+        if (given && stream_ != current.stream()) {
+            caller_ = current;
+            guard_.reset_stream(c10::cuda::getStreamFromExternal(stream_, like.device().index()));
+        }
+    }
+    // an output: the caller will go on with it on the current stream
+    Tensor output(Tensor t) const {
+        if (caller_) t.record_stream(*caller_);
+        return t;
+    }
+    // to be called when everything has been made
+    void* begin() {
+        guard_.reset();
+        return stream_;
+    }
+
+private:
+    cudaStream_t stream_;
+    std::optional<c10::cuda::CUDAStream> caller_;
+    c10::cuda::OptionalCUDAStreamGuard guard_;
+};
 
 // Workspace for a call that was given none: the fast size within half of the free device memory, or the
 // minimum.  How much is free is asked only for a workspace that is a large part of the device's memory, or
@@ -130,22 +162,22 @@ struct Arg {
     }
 };
 
-void* stream_of(const std::optional<int64_t>& stream) { return stream ? reinterpret_cast<void*>(*stream) : current_stream(); }
-
 py::object fwd_any(py::handle q_, py::handle k_, py::handle v_, int G, py::handle o_, py::handle lse_, const Options* ex,
                    std::optional<int64_t> stream) {
     Arg q(q_), k(k_), v(v_), o(o_), lse(lse_);
     if (q.bad || k.bad || v.bad || o.bad || lse.bad) return py::none();
     const auto s = sizes_of(q.t, k.t, v.t);
     if (!s) return py::none();
-    if (!o.given) o.t = new_like(q.t);
+    CallStream on(stream, q.t);
+    if (!o.given) o.t = on.output(new_like(q.t));
     else if (!same_shape(o.t, q.t.sizes(), q.t, at::kBFloat16)) return py::none();
-    if (!lse.given) lse.t = new_stats(*s, q.t);
+    if (!lse.given) lse.t = on.output(new_stats(*s, q.t));
     else if (!is_stats(lse.t, *s, q.t)) return py::none();
+    void* st = on.begin();
     int rc;
     {
         py::gil_scoped_release nogil;
-        rc = call_fwd(q.t, k.t, v.t, o.t, lse.t, *s, G, ex, stream_of(stream));
+        rc = call_fwd(q.t, k.t, v.t, o.t, lse.t, *s, G, ex, st);
     }
     if (rc != S2A_OK) return py::int_(rc);
     return py::make_tuple(o.t, lse.t);
@@ -169,6 +201,7 @@ py::object bwd_any(py::handle q_, py::handle k_, py::handle v_, py::handle o_, p
     if (!s || !same_shape(o.t, q.t.sizes(), q.t, at::kBFloat16) || !is_stats(lse.t, *s, q.t) ||
         !same_shape(dO.t, q.t.sizes(), q.t, at::kBFloat16))
         return py::none();
+    CallStream on(stream, q.t);
     const struct {
         Arg* out;
         const Tensor* like;
@@ -176,7 +209,7 @@ py::object bwd_any(py::handle q_, py::handle k_, py::handle v_, py::handle o_, p
     for (const auto& x : outs) {
         if (!x.out->given) {
             if (noalloc) return py::none();
-            x.out->t = new_like(*x.like);
+            x.out->t = on.output(new_like(*x.like));
         } else if (!same_shape(x.out->t, x.like->sizes(), q.t, at::kBFloat16)) {
             return py::none();
         }
@@ -185,10 +218,10 @@ py::object bwd_any(py::handle q_, py::handle k_, py::handle v_, py::handle o_, p
         if (!ws.given) ws.t = new_workspace(*s, G, q.t, fast);
         else if (!is_dense(ws.t, at::kByte) || ws.t.device() != q.t.device()) return py::none();
     }
+    void* st = on.begin();
     int rc;
     {
         py::gil_scoped_release nogil;
-        void* st = stream_of(stream);
         if (noalloc)
             rc = s2a_bwd_noalloc(q.t.data_ptr(), k.t.data_ptr(), v.t.data_ptr(), o.t.data_ptr(), static_cast<const float*>(lse.t.data_ptr()),
                                  dO.t.data_ptr(), dq.t.data_ptr(), dk.t.data_ptr(), dv.t.data_ptr(), s->B, s->N, s->H, s->Hkv, s->d, G, st);
@@ -228,14 +261,16 @@ py::object fwd_packed(py::handle qkv_, int G, py::handle o_, py::handle lse_, st
     if (qkv.bad || o.bad || lse.bad) return py::none();
     const auto s = packed_sizes(qkv.t);
     if (!s) return py::none();
-    if (!o.given) o.t = at::empty({s->B, s->N, s->H, s->d}, qkv.t.options());
+    CallStream on(stream, qkv.t);
+    if (!o.given) o.t = on.output(at::empty({s->B, s->N, s->H, s->d}, qkv.t.options()));
     else if (!same_shape(o.t, {s->B, s->N, s->H, s->d}, qkv.t, at::kBFloat16)) return py::none();
-    if (!lse.given) lse.t = new_stats(*s, qkv.t);
+    if (!lse.given) lse.t = on.output(new_stats(*s, qkv.t));
     else if (!is_stats(lse.t, *s, qkv.t)) return py::none();
+    void* st = on.begin();
     int rc;
     {
         py::gil_scoped_release nogil;
-        rc = s2a_fwd_packed(qkv.t.data_ptr(), o.t.data_ptr(), static_cast<float*>(lse.t.data_ptr()), s->B, s->N, s->H, s->d, G, stream_of(stream));
+        rc = s2a_fwd_packed(qkv.t.data_ptr(), o.t.data_ptr(), static_cast<float*>(lse.t.data_ptr()), s->B, s->N, s->H, s->d, G, st);
     }
     if (rc != S2A_OK) return py::int_(rc);
     return py::make_tuple(o.t, lse.t);
@@ -250,15 +285,17 @@ py::object bwd_packed(py::handle qkv_, py::handle o_, py::handle lse_, py::handl
     if (!s || !same_shape(o.t, {s->B, s->N, s->H, s->d}, qkv.t, at::kBFloat16) || !is_stats(lse.t, *s, qkv.t) ||
         !same_shape(dO.t, {s->B, s->N, s->H, s->d}, qkv.t, at::kBFloat16))
         return py::none();
-    if (!dqkv.given) dqkv.t = new_like(qkv.t);
+    CallStream on(stream, qkv.t);
+    if (!dqkv.given) dqkv.t = on.output(new_like(qkv.t));
     else if (!same_shape(dqkv.t, qkv.t.sizes(), qkv.t, at::kBFloat16)) return py::none();
     if (!ws.given) ws.t = new_workspace(*s, G, qkv.t, fast);
     else if (!is_dense(ws.t, at::kByte) || ws.t.device() != qkv.t.device()) return py::none();
+    void* st = on.begin();
     int rc;
     {
         py::gil_scoped_release nogil;
         rc = s2a_bwd_packed(qkv.t.data_ptr(), o.t.data_ptr(), static_cast<const float*>(lse.t.data_ptr()), dO.t.data_ptr(), dqkv.t.data_ptr(), s->B,
-                            s->N, s->H, s->d, G, ws.t.data_ptr(), static_cast<size_t>(ws.t.numel()), stream_of(stream));
+                            s->N, s->H, s->d, G, ws.t.data_ptr(), static_cast<size_t>(ws.t.numel()), st);
     }
     if (rc != S2A_OK) return py::int_(rc);
     return py::cast(dqkv.t);
