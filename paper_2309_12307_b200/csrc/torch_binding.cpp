@@ -341,7 +341,10 @@ struct S2Attn : public torch::autograd::Function<S2Attn> {
         const int G = static_cast<int>(ctx->saved_data["G"].toInt());
         const Tensor dO = grads[0].contiguous();
         const auto s = sizes_of(q, k, v);
-        TORCH_CHECK_VALUE(s && same_shape(dO, q.sizes(), q, at::kBFloat16), "dO must be a bf16 CUDA tensor of the shape of q");
+        // saved-tensor hooks decide what comes back
+        TORCH_CHECK_VALUE(s && same_shape(o, q.sizes(), q, at::kBFloat16) && is_stats(lse, *s, q),
+                          "the saved q, k, v, o and lse have come back with another type, shape, layout or device");
+        TORCH_CHECK_VALUE(same_shape(dO, q.sizes(), q, at::kBFloat16), "dO must be a bf16 CUDA tensor of the shape of q");
         at::NoGradGuard no_grad;
         Tensor dq = new_like(q), dk = new_like(k), dv = new_like(v);
         const Tensor ws = new_workspace(*s, G, q, ctx->saved_data["fast"].toBool());

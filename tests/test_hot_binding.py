@@ -45,3 +45,21 @@ def test_s2_attn_takes_strided_inputs_and_gradients():
     got = (o.detach(), *torch.autograd.grad(o, strided, dO.transpose(1, 2).contiguous().transpose(1, 2)))
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("change", [lambda t: t.half(), lambda t: t[..., ::2], lambda t: t[..., :32].contiguous(), lambda t: t.cpu(),
+                                    lambda t: t.transpose(1, 2).contiguous().transpose(1, 2)])
+@pytest.mark.parametrize("which", range(5))
+def test_backward_refuses_saved_tensors_that_come_back_changed(change, which):
+    """q, k, v, o, lse pass through saved-tensor hooks; the kernels read them by their raw pointers."""
+    q, k, v, dO = (x.cuda() for x in make_inputs(1, 512, 4, 2, 64, seed=7))
+    for t in (q, k, v):
+        t.requires_grad_()
+    saved = []
+    with torch.autograd.graph.saved_tensors_hooks(lambda t: saved.append(t) or len(saved) - 1,
+                                                  lambda i: change(saved[i].detach()) if i == which else saved[i]):
+        o = s2_attn(q, k, v, 256)
+    assert [t.dtype for t in saved] == [torch.bfloat16] * 4 + [torch.float32]
+    with pytest.raises(ValueError, match="saved"):
+        torch.autograd.grad(o, (q, k, v), dO)
