@@ -217,7 +217,7 @@ int s2a_bwd_stage(const void* q, const void* k, const void* v, const void* o, co
 /*
  * Forward + backward from HOST buffers (pinned memory, or the copies are not asynchronous): q, k, v,
  * dO go to the caller's device buffers, s2a_fwd and s2a_bwd run there, and o, lse, dq, dk, dv come
- * back.  Heads and groups are independent, so the work is cut into about 16 chunks at most - equal ones,
+ * back.  Heads and groups are independent, so the work is cut into up to 17 chunks - nearly equal ones,
  * of whole KV heads and whole groups - and the copy of one chunk, the kernels of the previous
  * one and the copy back of the one before that overlap (two copy streams owned by the library,
  * created by the first call on a device, ordered

@@ -23,8 +23,11 @@ struct HostChunk {
 // the time of a chunk's copies, 40 us.  Rows stay wide: with both directions busy the copy engines moved 49.9 GB/s
 // each way with rows of 4096 bytes, 49.4 at 2048, 46.9 at 1024, 44.9 at 512 and 35.2 at 256.  Batch items are
 // cut first (rows of all heads), then the unshifted from the shifted heads and groups of tokens (rows of half
-// the heads), then heads while a row of the keys keeps kHostRowBytes.  More than 16 chunks were slower (32 heads
-// of 128, 32k tokens, groups of 8k: 28.2 ms with 32 chunks, 23.9 with 16).
+// the heads), then heads while a row of the keys keeps kHostRowBytes, each as long as that brings the number nearer to
+// the one wanted and not more than one above it.  More than 16 chunks were slower (32 heads of 128, 32k tokens, groups of
+// 8k: 28.2 ms with 32 chunks, 23.9 with 16), and most of all where the cut leaves a narrow chunk for one KV head between the
+// halves: 6 x 8192 tokens of 10 heads on 5 10.46 ms with 30 chunks, 9.88 with 18, 9.41 with 6; 13 x 8192 21.1 with 39, 19.6
+// with 13; 7 x 4096 tokens of 32 heads 22.2 with 28, 21.5 with 14 (but 12 x 2048 tokens 17.96 with 24, 18.29 with 12).
 // Against chunks of 2, 2, 4, 8, 8, 4, 2, 2 of 32 heads for all tokens: that shape 27.9 -> 24.0 ms, 8k tokens 7.20 -> 6.49
 // (link: 5.4), 64 heads on 8 at 8k 8.15 -> 7.33, 4 x 2000 tokens of 16 heads on 4 of 64 1.45 -> 1.32, 1k of 4 heads
 // of 64, one chunk, 0.207 -> 0.133.
@@ -40,14 +43,22 @@ int cut_host_job(int B, int N, int H, int Hkv, int d, int G, Emit&& emit) {
     int want = 1;
     while (want < kHostChunks && (want + 1) * (want + 1) * kHostChunkCost <= bytes_in) ++want;
     const int batches = B < want ? B : want;
-    const int per_batch = (want + batches - 1) / batches;  // more than one only where a batch item is a chunk or more
     // KV heads [0, half) have unshifted query heads only, [Hkv - half, Hkv) shifted ones only; one between has both
     const int half = H / 2 / rep;
-    const bool cut = per_batch > 1 && half > 0;
-    int by_groups = (per_batch + 1) / 2, by_heads = 1;
-    if (by_groups > groups) by_groups = groups;
+    const int between = Hkv > 2 * half ? 1 : 0;
+    // whether either half of the heads of a batch item is rather cut into `parts` parts than into `than` (0: the item stays whole)
+    auto nearer = [&](int parts, int than) {
+        auto off = [&](int n) {
+            const int chunks = batches * (n == 0 ? 1 : 2 * n + between);
+            return chunks > want ? chunks - want : want - chunks;
+        };
+        return off(parts) < off(than) && batches * (2 * parts + between) <= want + 1;
+    };
+    int by_groups = 0, by_heads = 1;
+    while (half > 0 && by_groups < groups && nearer(by_groups + 1, by_groups)) ++by_groups;
+    const bool cut = by_groups > 0;
     while (by_groups > 1 && static_cast<long long>(groups / by_groups) * G < 128) --by_groups;  // the least N of a job
-    while (3 * by_groups * by_heads <= per_batch && 2 * by_heads <= half &&  // nearer to per_batch with twice as many
+    while (cut && nearer(2 * by_groups * by_heads, by_groups * by_heads) && 2 * by_heads <= half &&
            static_cast<long long>(half / (2 * by_heads)) * d * 2 >= kHostRowBytes)
         by_heads *= 2;
     for (int b = 0; b < batches; ++b) {

@@ -51,7 +51,20 @@ int main() {
                         });
                         for (char s : seen)
                             if (rc || !s) return std::printf("FAIL rc %d B %d G %d groups %d H %d Hkv %d d %d\n", rc, B, G, groups, H, Hkv, d), 1;
-                        if (chunks > 2 * kHostChunks + 1) return std::printf("FAIL %d chunks\n", chunks), 1;
+                        if (chunks > kHostChunks + 1) return std::printf("FAIL %d chunks\n", chunks), 1;
+                        if (chunks > most) most = chunks;
+                    }
+    // the number of chunks, for sizes that call for all of them too
+    for (const auto& hh : heads)
+        for (int d : {64, 128})
+            for (int B = 1; B <= 33; ++B)
+                for (int N : {1024, 8192, 32768, 131072})
+                    for (int groups : {1, 4, 5, 16}) {
+                        if (N % (8 * groups) != 0) continue;
+                        int chunks = 0;
+                        cut_host_job(B, N, hh[0], hh[1], d, N / groups, [&](const HostChunk&) { return ++chunks, 0; });
+                        if (chunks > kHostChunks + 1)
+                            return std::printf("FAIL %d chunks: B %d N %d groups %d H %d Hkv %d d %d\n", chunks, B, N, groups, hh[0], hh[1], d), 1;
                         if (chunks > most) most = chunks;
                     }
     if (most < kHostChunks) return std::printf("FAIL at most %d chunks\n", most), 1;
