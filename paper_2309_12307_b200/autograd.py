@@ -21,8 +21,8 @@ def s2_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, G: int, *, scale:
     (default H/2), shift in tokens (default G/2), and variants 2 (`leak_free`) and 3 (`swap_wrapped`)
     of the paper's Appendix B.  With n_unshifted = H, shift = 0 and G = N it is ordinary causal attention.
     `fast_backward` chooses the backward's scratch: True allocates room for the spilled dS (2 bytes per
-    attended pair of a tile, within half of the free device memory) so that dq is a plain product, False
-    the minimum (4 bytes per query row; dq then recomputes the scores).
+    attended pair of a tile, from what torch's caching allocator holds unused or within half of the free device
+    memory) so that dq is a plain product, False the minimum (4 bytes per query row; dq then recomputes the scores).
     """
     hot = binding._hot or binding._hot_for(_check, q, k, v)
     o = hot.s2_attn(q, k, v, G, scale, n_unshifted, shift, binding._flags(leak_free, swap_wrapped), fast_backward)

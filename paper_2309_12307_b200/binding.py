@@ -232,8 +232,8 @@ def s2a_fwd(q, k, v, G, o=None, lse=None, stream=None):
 
 def s2a_bwd(q, k, v, o, lse, dO, G, dq=None, dk=None, dv=None, workspace=None, stream=None, fast=True):
     """dq, dk, dv (bf16) of sum(o * dO).  Without a workspace one is allocated: large enough for the
-    spilling backward within half of the free device memory (fast=True) or the minimum (fast=False: dq
-    recomputes the scores)."""
+    spilling backward (fast=True), taken from what torch's caching allocator holds unused or within half of
+    the free device memory, or the minimum (fast=False: dq recomputes the scores)."""
     hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
     r = hot.bwd(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, fast, _given_stream(stream))
     return r if r.__class__ is tuple else _result(r, "s2a_bwd", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)

@@ -10,6 +10,8 @@
 #include <torch/extension.h>
 
 #include <ATen/cuda/CUDAContext.h>
+#include <c10/cuda/CUDACachingAllocator.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <cuda_runtime_api.h>
@@ -25,11 +27,6 @@ namespace {
 using at::Tensor;
 using torch::autograd::AutogradContext;
 using torch::autograd::variable_list;
-
-// Part of the device memory below which a fast workspace is taken without asking how much is free: the
-// driver's answer takes 70 to 220 us and more while the GPU is busy, longer than the whole backward of a
-// small problem.  1/32 is 5.7 GB of 180: Llama2-7B up to 16k tokens.
-constexpr size_t kUnaskedPart = 32;
 
 struct Sizes {
     int64_t B, N, H, Hkv, d;
@@ -90,9 +87,20 @@ private:
     c10::cuda::OptionalCUDAStreamGuard guard_;
 };
 
-// Workspace for a call that was given none: the fast size within half of the free device memory, or the
-// minimum.  How much is free is asked only for a workspace that is a large part of the device's memory, or
-// when a smaller one cannot be had.
+// Bytes that the caching allocator has from the device, and how many of them are not in use.
+struct Held {
+    int64_t all, unused;
+    explicit Held(const Tensor& like) {
+        const auto stats = c10::cuda::CUDACachingAllocator::getDeviceStats(like.device().index());
+        const auto total = static_cast<size_t>(c10::CachingDeviceAllocator::StatType::AGGREGATE);
+        all = stats.reserved_bytes[total].current, unused = all - stats.allocated_bytes[total].current;
+    }
+};
+
+// Workspace for a call that was given none: the fast size, of which no more than half of the free device memory comes
+// from the device, or the minimum.  The driver takes 70 to 220 us and more to say how much is free while the GPU is busy,
+// longer than the whole backward of a small problem, so it is asked only where the caching allocator has to go to the
+// device: not where it finds the workspace in what it holds, as from the second backward of a program on.
 Tensor new_workspace(const Sizes& s, int G, const Tensor& like, bool fast) {
     const auto options = like.options().dtype(at::kByte);
     const int B = s.B, N = s.N, H = s.H, Hkv = s.Hkv, d = s.d;
@@ -100,13 +108,20 @@ Tensor new_workspace(const Sizes& s, int G, const Tensor& like, bool fast) {
     auto make = [&](size_t bytes) { return at::empty({static_cast<int64_t>(std::max(bytes, least))}, options); };
     if (!fast) return make(least);
     const size_t need = s2a_bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, size_t(1) << 62);
-    if (need <= at::cuda::getDeviceProperties(like.device().index())->totalGlobalMem / kUnaskedPart) {
+    size_t free_bytes = 0, total = 0;
+    const Held before(like);
+    if (static_cast<int64_t>(need) <= before.unused && c10::cuda::currentStreamCaptureStatusMayInitCtx() == c10::cuda::CaptureStatus::None) {
         try {
-            return make(need);
+            Tensor t = make(need);
+            const int64_t taken = Held(like).all - before.all;
+            if (taken <= 0) return t;
+            // the unused bytes were in pieces, or another stream's
+            if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) free_bytes = 0;
+            if (need <= (free_bytes + taken) / 2) return t;
         } catch (const c10::OutOfMemoryError&) {
         }
+        c10::cuda::CUDACachingAllocator::emptyCache();  // what was taken goes back
     }
-    size_t free_bytes = 0, total = 0;
     if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) free_bytes = 0;
     return make(s2a_bwd_workspace_bytes_fast(B, N, H, Hkv, d, G, free_bytes / 2));
 }
