@@ -98,6 +98,9 @@ def load_hot():
         spec = importlib.util.spec_from_file_location("_s2a_torch", TORCH_LIB_PATH)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)
+        if module.torch_version != torch.__version__:
+            raise ImportError(f"{TORCH_LIB_PATH} was built for torch {module.torch_version}, not {torch.__version__}: "
+                              "build it again with `python -m paper_2309_12307_b200.build`")
         _hot = module
     return _hot
 

@@ -39,21 +39,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
     return LIB
 
 
+def _built_for(path: str) -> str | None:
+    try:
+        with open(path) as f:
+            return f.read()
+    except OSError:
+        return None
+
+
 def build_torch(force: bool = False) -> str:
-    deps = [TORCH_SOURCE, os.path.join(PKG, "..", "include", "s2a.h")]
-    if not force and os.path.exists(TORCH_LIB) and os.path.getmtime(TORCH_LIB) >= _newest(deps):
-        return TORCH_LIB
     import torch
 
+    # a module that was built for another torch or Python would be loaded all the same and misread this one's objects
+    stamp, wanted = TORCH_LIB + ".built_for", f"torch {torch.__version__}, python {sys.version}"
+    deps = [TORCH_SOURCE, os.path.join(PKG, "..", "include", "s2a.h")]
+    if not force and _built_for(stamp) == wanted and os.path.exists(TORCH_LIB) and os.path.getmtime(TORCH_LIB) >= _newest(deps):
+        return TORCH_LIB
     root = os.path.join(os.path.dirname(os.path.abspath(torch.__file__)))
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     include = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
                os.path.join(cuda, "include"), sysconfig.get_paths()["include"]]
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-DTORCH_EXTENSION_NAME=_s2a_torch",
-           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(f"-I{d}" for d in include), TORCH_SOURCE,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", f'-DS2A_TORCH_VERSION="{torch.__version__}"', *(f"-I{d}" for d in include), TORCH_SOURCE,
            "-o", TORCH_LIB, f"-L{os.path.join(root, 'lib')}", f"-L{os.path.join(cuda, 'lib64')}", f"-L{PKG}", "-l:libs2a.so",
            "-lc10", "-lc10_cuda", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-lcudart", "-Wl,-rpath,$ORIGIN"]
     subprocess.run(cmd, check=True)
+    with open(stamp, "w") as f:
+        f.write(wanted)
     return TORCH_LIB
 
 

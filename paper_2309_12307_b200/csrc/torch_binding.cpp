@@ -387,6 +387,7 @@ py::object s2_attn(py::handle q_, py::handle k_, py::handle v_, int G, std::opti
 
 PYBIND11_MODULE(_s2a_torch, m) {
     m.doc() = "Hot path of the Python binding of libs2a.so; called by binding.py and autograd.py.";
+    m.attr("torch_version") = S2A_TORCH_VERSION;
     m.def("fwd", &fwd);
     m.def("fwd_ex", &fwd_ex);
     m.def("fwd_packed", &fwd_packed);
