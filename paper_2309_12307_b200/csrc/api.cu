@@ -524,9 +524,15 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
     if (const int bad = check_default_shape(N, H, d, G)) return bad;
     int rc = check_shape(B, N, H, Hkv, d, G, 1.0f, H / 2, G / 2);
     if (rc != S2A_OK) return rc;
-    if (!workspace || workspace_bytes < s2a_bwd_workspace_bytes(B, N, H, Hkv, d, G)) return S2A_ERR_INVALID_ARG;
+    // a refusal comes before the first copy is enqueued, so what the kernels' launchers ask is asked here as well
+    const void* const buffers[] = {d_q, d_k, d_v, d_dO, d_o, d_lse, d_dq, d_dk, d_dv};
+    for (const void* p : buffers)
+        if (!aligned16(p)) return S2A_ERR_INVALID_ARG;
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return S2A_ERR_INVALID_ARG;
+    if (workspace_bytes < s2a_bwd_workspace_bytes(B, N, H, Hkv, d, G)) return S2A_ERR_INVALID_ARG;
     DeviceState* ds = nullptr;
     if ((rc = prepare_device(&ds)) != S2A_OK) return rc;
+    if (*ds->host_word != 0) return S2A_ERR_TIMEOUT;  // an earlier launch gave up: see s2a_device_status()
     cudaError_t e;
     std::unique_lock<std::mutex> lock(g_dev_mutex);
     if (!ds->host_path_ready) {

@@ -92,6 +92,22 @@ def test_bad_arguments_are_rejected_without_a_device(lib):
     assert lib.s2a_bwd(a, a, a, a, a, a, a, a, a, 1, 1024, 4, 4, 64, 256, None, 1 << 20, None) == -1
 
 
+def test_host_entry_point_refuses_before_it_copies(lib):
+    P = ctypes.c_void_p
+    lib.s2a_fwd_bwd_host.argtypes = [P] * 18 + [ctypes.c_int] * 6 + [P, ctypes.c_size_t, P]
+    buf = (ctypes.c_char * 4096)()
+    a = (ctypes.addressof(buf) + 255) & ~255  # never dereferenced on these paths
+
+    def call(device=(a,) * 9, workspace=a, size=1 << 20):
+        return lib.s2a_fwd_bwd_host(*(a + 1,) * 9, *device, 1, 1024, 4, 4, 64, 256, workspace, size, None)
+
+    for i in range(9):  # device buffers and the workspace are read by the kernels; host pointers may lie anywhere
+        assert call(device=tuple(a + 8 if j == i else a for j in range(9))) == -1
+    assert call(workspace=a + 16) == -1
+    assert call(size=16384) == -1
+    assert call(workspace=None) == -1
+
+
 def test_fast_workspace_bytes(lib):
     lib.s2a_bwd_workspace_bytes.restype = ctypes.c_size_t
     lib.s2a_bwd_workspace_bytes_fast.restype = ctypes.c_size_t

@@ -63,3 +63,27 @@ def test_selftest_rejects_limits_outside_its_range():
     assert lib.s2a_selftest_wait_expiry(3_000_000_000, None) == s2a.S2A_ERR_INVALID_ARG
     torch.cuda.synchronize()
     assert s2a.device_status() == (0, 0)
+
+
+def test_host_entry_point_copies_nothing_while_the_status_is_set():
+    from paper_2309_12307_b200 import binding as s2a
+
+    B, N, G, H, d = 1, 1024, 256, 4, 64
+    q, k, v, dO = make_inputs(B, N, H, H, d, seed=32)
+    host_in = [t.pin_memory() for t in (q, k, v, dO)]
+    shapes = [(q.shape, torch.bfloat16), ((B, H, N), torch.float32)] + [(q.shape, torch.bfloat16)] * 3
+    host_out = [torch.full(s, 7.0, dtype=t).pin_memory() for s, t in shapes]
+    dev = [torch.full(t.shape, 5.0, dtype=t.dtype, device="cuda") for t in host_in + host_out]
+    ws = torch.empty(s2a.bwd_workspace_bytes(B, N, H, H, d, G), dtype=torch.uint8, device="cuda")
+    s2a.selftest_wait_expiry(1_000_000)
+    torch.cuda.synchronize()
+    with pytest.raises(s2a.S2AError) as e:
+        s2a.s2a_fwd_bwd_host(host_in, host_out, dev, G, ws)
+    assert e.value.status == s2a.S2A_ERR_TIMEOUT
+    torch.cuda.synchronize()
+    assert all(bool((t == 5).all()) for t in dev) and all(bool((t == 7).all()) for t in host_out)
+    assert s2a.device_status()[0] == s2a.S2A_ERR_TIMEOUT
+    s2a.s2a_fwd_bwd_host(host_in, host_out, dev, G, ws)
+    torch.cuda.synchronize()
+    o, lse = s2a.s2a_fwd(*(t.cuda() for t in (q, k, v)), G)
+    assert torch.equal(host_out[0], o.cpu()) and torch.equal(host_out[1], lse.cpu()) and s2a.device_status() == (0, 0)
