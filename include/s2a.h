@@ -41,8 +41,8 @@
  *     128, a NaN or infinity in one token's q, k, v or dO can reach o, dq, dk or dv of the adjacent
  *     group's tokens.
  *   - Host threads: entry points may be called from several host threads (the one-time set-up of a
- *     device is serialised); s2a_fwd_bwd_host and s2a_bwd_noalloc keep per-device state (copy streams,
- *     built-in scratch), so calls of either on one device must not overlap.
+ *     device is serialised, and so are calls of s2a_fwd_bwd_host on one device while they enqueue their
+ *     work).  s2a_bwd_noalloc keeps D in per-device scratch: its calls on one device must not overlap.
  *   - Device-side waits are bounded (about a second of SM clock cycles, so heavy time-slicing of the
  *     GPU can in principle trip one).  If a wait expires the kernel records where, in a status word on
  *     the device and in a host-visible copy of it, and stops cleanly; the outputs of that launch are

@@ -43,6 +43,7 @@ struct DeviceState {
     cudaStream_t copy_in = nullptr, copy_out = nullptr;
     cudaEvent_t ev_start = nullptr, ev_done = nullptr, ev_in_done = nullptr;
     cudaEvent_t ev_qkv = nullptr, ev_do = nullptr, ev_fwd = nullptr, ev_bwd = nullptr;  // recorded again for every chunk
+    std::mutex host_path;  // held by the call that enqueues: its events must not be recorded by another one in between
 };
 DeviceState g_dev[kMaxDevices];
 static_assert(kMaxDevices == kMaxDevicesMirror, "one mirror word per device");
@@ -534,7 +535,7 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
     if ((rc = prepare_device(&ds)) != S2A_OK) return rc;
     if (*ds->host_word != 0) return S2A_ERR_TIMEOUT;  // an earlier launch gave up: see s2a_device_status()
     cudaError_t e;
-    std::unique_lock<std::mutex> lock(g_dev_mutex);
+    std::lock_guard<std::mutex> lock(ds->host_path);
     if (!ds->host_path_ready) {
         if ((e = cudaStreamCreateWithFlags(&ds->copy_in, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(e);
         if ((e = cudaStreamCreateWithFlags(&ds->copy_out, cudaStreamNonBlocking)) != cudaSuccess) return cuda_fail(e);
@@ -542,7 +543,6 @@ int s2a_fwd_bwd_host(const void* h_q, const void* h_k, const void* h_v, const vo
             if ((e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) return cuda_fail(e);
         ds->host_path_ready = true;
     }
-    lock.unlock();
     // Heads and groups are independent, so the job is cut into chunks (host_plan.h): while chunk c is
     // computed, chunk c + 1 travels to the device and the results of chunk c - 1 travel back.  The forward
     // pass of a chunk runs while its dO is on its way, and o goes back while its backward pass runs.

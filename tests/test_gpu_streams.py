@@ -1,5 +1,7 @@
 """Calls on a stream that is not torch's current one: what the binding allocates for them must not be shared with
 work of the current stream that is still queued, neither before the call nor after it."""
+import threading
+
 import pytest
 import torch
 
@@ -54,3 +56,37 @@ def test_memory_of_a_call_on_another_stream_is_its_own(call):
     for t, w in zip(got, want):
         assert torch.equal(t, w)
     assert s2a.device_status() == (0, 0)
+
+
+def test_host_entry_point_from_several_threads():
+    """Calls from several threads on streams of their own share the library's copy streams and events."""
+    B, N, G, H, Hkv, d = 1, 4096, 1024, 16, 16, 128
+    jobs = []
+    for seed in range(4):
+        host_in = [t.pin_memory() for t in make_inputs(B, N, H, Hkv, d, seed=seed)]
+        q, k, v, dO = (t.cuda() for t in host_in)
+        ws = torch.empty(s2a.bwd_workspace_bytes(B, N, H, Hkv, d, G), dtype=torch.uint8, device="cuda")
+        o, lse = s2a.s2a_fwd(q, k, v, G)
+        want = (o, lse, *s2a.s2a_bwd(q, k, v, o, lse, dO, G, workspace=ws))
+        host_out = [torch.zeros(t.shape, dtype=t.dtype).pin_memory() for t in want]
+        jobs.append((host_in, host_out, [torch.zeros_like(t) for t in (q, k, v, dO, *want)], ws, torch.cuda.Stream(), [t.cpu() for t in want]))
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(host_in, host_out, dev, ws, stream, want):
+        try:
+            for _ in range(5):
+                for t in host_out:
+                    t.zero_()
+                s2a.s2a_fwd_bwd_host(host_in, host_out, dev, G, ws, stream=stream)
+                stream.synchronize()
+                failed.extend(i for i, (a, b) in enumerate(zip(host_out, want)) if not torch.equal(a, b))
+        except Exception as e:  # noqa: BLE001 - reported below
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=job) for job in jobs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not failed and s2a.device_status() == (0, 0)
