@@ -69,7 +69,8 @@ typedef enum s2a_status {
     S2A_OK = 0,
     S2A_ERR_INVALID_ARG = -1, /* null pointer, non-positive size, N % G, odd G or H, H % Hkv, misaligned pointer, small workspace */
     S2A_ERR_UNSUPPORTED = -2, /* d not in {64,128}, G or shift not a multiple of 4 tokens (G/2 for the default shift), N < 128,
-                                 ragged tiles with mixed shifts on one KV head, device is not sm_100 */
+                                 ragged tiles with mixed shifts on one KV head, more than 2^31 - 1 (token, head)
+                                 rows in a backward, device is not sm_100 */
     S2A_ERR_CUDA = -3,        /* a CUDA call failed while enqueuing; see s2a_last_cuda_error() */
     S2A_ERR_TIMEOUT = -4,     /* reported by s2a_device_status(): a bounded device-side wait expired */
     S2A_ERR_TOO_LARGE = -5    /* s2a_bwd_noalloc only: B*H*N is more than its built-in scratch holds */

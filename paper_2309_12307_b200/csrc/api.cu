@@ -376,6 +376,7 @@ int bwd_impl(const void* q, const void* k, const void* v, const void* o, const f
     if ((reinterpret_cast<uintptr_t>(workspace) & 255u) != 0) return S2A_ERR_INVALID_ARG;
     int rc = check_shape(B, N, H, Hkv, d, G, scale, n_unshifted, shift);
     if (rc != S2A_OK) return rc;
+    if (static_cast<long long>(B) * N * H > 0x7fffffffLL) return S2A_ERR_UNSUPPORTED;  // PreParams::rows
     if (workspace_bytes < s2a_bwd_workspace_bytes(B, N, H, Hkv, d, G)) return S2A_ERR_INVALID_ARG;
     DeviceState* ds = nullptr;
     rc = prepare_device(&ds);

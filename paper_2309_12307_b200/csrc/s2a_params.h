@@ -226,7 +226,7 @@ struct PreParams {
     const __nv_bfloat16* o;
     const __nv_bfloat16* dO;
     float* Dsum;  // [B, H, N]
-    int rows;     // B N H: o and dO of 2^31 rows would be 550 GB
+    int rows;     // B N H; the entry points refuse 2^31 and more (q alone would be 275 GB)
     int N, H;
     FastDiv by_heads, by_tokens;
 };

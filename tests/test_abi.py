@@ -92,6 +92,15 @@ def test_bad_arguments_are_rejected_without_a_device(lib):
     assert lib.s2a_bwd(a, a, a, a, a, a, a, a, a, 1, 1024, 4, 4, 64, 256, None, 1 << 20, None) == -1
 
 
+def test_backward_refuses_more_rows_than_it_counts(lib):
+    P = ctypes.c_void_p
+    lib.s2a_bwd.argtypes = [P] * 9 + [ctypes.c_int] * 6 + [P, ctypes.c_size_t, P]
+    buf = (ctypes.c_char * 4096)()
+    a = (ctypes.addressof(buf) + 255) & ~255  # never dereferenced on these paths
+    for B, N, H in ((1, 1 << 26, 32), (2, 1 << 25, 32), (1 << 20, 1024, 2)):  # 2^31 rows each
+        assert lib.s2a_bwd(*(a,) * 9, B, N, H, H, 64, 1024, a, 1 << 62, None) == -2
+
+
 def test_host_entry_point_refuses_before_it_copies(lib):
     P = ctypes.c_void_p
     lib.s2a_fwd_bwd_host.argtypes = [P] * 18 + [ctypes.c_int] * 6 + [P, ctypes.c_size_t, P]
