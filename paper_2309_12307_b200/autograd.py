@@ -30,4 +30,7 @@ def s2_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, G: int, *, scale:
 
 
 def _check(q, k, v) -> None:
+    for t, name in ((q, "q"), (k, "k"), (v, "v")):
+        if not isinstance(t, torch.Tensor):
+            raise ValueError(f"{name} must be a torch.Tensor")
     binding._dims(*(t.contiguous() for t in (q, k, v)))

@@ -8,11 +8,32 @@ from paper_2309_12307_b200.autograd import s2_attn
 from paper_2309_12307_b200.inputs import make_inputs
 
 
-@pytest.mark.parametrize("bad", ["cpu", "dtype", "none"])
-def test_s2_attn_names_a_bad_argument(bad):
-    q = torch.zeros((1, 256, 2, 64), dtype=torch.float32 if bad == "dtype" else torch.bfloat16)
-    with pytest.raises((ValueError, AttributeError)):
-        s2_attn(None if bad == "none" else q, q, q, 128)
+@pytest.mark.parametrize("which", range(3))
+@pytest.mark.parametrize("bad", [None, 3.0])
+def test_s2_attn_names_an_argument_that_is_no_tensor(bad, which):
+    args = [torch.zeros((1, 256, 2, 64), dtype=torch.bfloat16)] * 3
+    args[which] = bad
+    with pytest.raises(ValueError, match=f"{'qkv'[which]} must be a torch.Tensor"):
+        s2_attn(*args, 128)
+
+
+def test_s2_attn_names_a_tensor_on_the_cpu():
+    q = torch.zeros((1, 256, 2, 64), dtype=torch.bfloat16)
+    with pytest.raises(ValueError, match="q must be a CUDA tensor"):
+        s2_attn(q, q, q, 128)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("which", range(3))
+@pytest.mark.parametrize("change,message", [(lambda t: t.float(), "must have dtype"), (lambda t: t.cpu(), "must be a CUDA tensor"),
+                                            (lambda t: t[0], "must be|must have shape"), (lambda t: t[..., :32], "must be|must have shape")])
+def test_s2_attn_names_a_tensor_the_kernels_would_misread(change, message, which):
+    args = [torch.zeros((1, 256, 2, 64), dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    args[which] = change(args[which])
+    # q sets the sizes: a head of 32 in q alone is told of k
+    name = "k" if which == 0 and args[0].dim() == 4 and args[0].shape[-1] == 32 else "qkv"[which]
+    with pytest.raises(ValueError, match=f"^{name} ({message})"):
+        s2_attn(*args, 128)
 
 
 @pytest.mark.gpu
