@@ -25,8 +25,10 @@ def s2_attn(q: torch.Tensor, k: torch.Tensor, v: torch.Tensor, G: int, *, scale:
     memory) so that dq is a plain product, False the minimum (4 bytes per query row; dq then recomputes the scores).
     """
     hot = binding._hot or binding._hot_for(_check, q, k, v)
-    o = hot.s2_attn(q, k, v, G, scale, n_unshifted, shift, binding._flags(leak_free, swap_wrapped), fast_backward)
-    return binding._result(o, "s2_attn", _check, q, k, v) if o is None else o
+    o = hot.s2_attn(q, k, v, G, scale, n_unshifted, shift, binding._flags(leak_free, swap_wrapped), bool(fast_backward))
+    if o is None:
+        binding._result(o, "s2_attn", _check, q, k, v)
+    return o if q.__class__ in binding._PLAIN else binding._typed((o,), (q,))[0]
 
 
 def _check(q, k, v) -> None:

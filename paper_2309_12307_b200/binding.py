@@ -148,6 +148,15 @@ def _result(r, what: str, check, *args, **kw):
     return r
 
 
+_PLAIN = (torch.Tensor, torch.nn.Parameter)
+
+
+def _typed(r, made_like):
+    """Results as the operators of torch make them: one that was made (its entry in `made_like` is the argument
+    that it is like, not None) has the class of that argument, if that is a subclass of Tensor."""
+    return tuple(t if a is None or a.__class__ in _PLAIN else t.as_subclass(a.__class__) for t, a in zip(r, made_like))
+
+
 def _check(rc: int, what: str) -> None:
     if rc != S2A_OK:
         raise S2AError(rc, what)
@@ -230,7 +239,9 @@ def s2a_fwd(q, k, v, G, o=None, lse=None, stream=None):
     """o [B,N,H,d] bf16 and lse [B,H,N] fp32 of S2-Attn (second half of the heads shifted by G/2)."""
     hot = _hot or _hot_for(_check_fwd, q, k, v, o, lse)
     r = hot.fwd(q, k, v, G, o, lse, _given_stream(stream))
-    return r if r.__class__ is tuple else _result(r, "s2a_fwd", _check_fwd, q, k, v, o, lse)
+    if r.__class__ is not tuple:
+        _result(r, "s2a_fwd", _check_fwd, q, k, v, o, lse)
+    return r if q.__class__ in _PLAIN else _typed(r, (None if o is not None else q, None))
 
 
 def s2a_bwd(q, k, v, o, lse, dO, G, dq=None, dk=None, dv=None, workspace=None, stream=None, fast=True):
@@ -238,8 +249,12 @@ def s2a_bwd(q, k, v, o, lse, dO, G, dq=None, dk=None, dv=None, workspace=None, s
     spilling backward (fast=True), taken from what torch's caching allocator holds unused or within half of
     the free device memory, or the minimum (fast=False: dq recomputes the scores)."""
     hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
-    r = hot.bwd(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, fast, _given_stream(stream))
-    return r if r.__class__ is tuple else _result(r, "s2a_bwd", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    r = hot.bwd(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, bool(fast), _given_stream(stream))
+    if r.__class__ is not tuple:
+        _result(r, "s2a_bwd", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    if q.__class__ in _PLAIN and k.__class__ in _PLAIN:
+        return r
+    return _typed(r, tuple(None if out is not None else like for out, like in ((dq, q), (dk, k), (dv, k))))
 
 
 def bwd_noalloc_max_rows() -> int:
@@ -283,8 +298,9 @@ def s2a_fwd_packed(qkv, G, o=None, lse=None, stream=None):
 def s2a_bwd_packed(qkv, o, lse, dO, G, dqkv=None, workspace=None, stream=None, fast=True):
     """Backward on a packed qkv tensor; returns dqkv [B, N, 3, H, d]."""
     hot = _hot or _hot_for(_check_packed, qkv, o, lse, dO, dqkv, workspace, backward=True)
-    r = hot.bwd_packed(qkv, o, lse, dO, G, dqkv, workspace, fast, _given_stream(stream))
-    return _result(r, "s2a_bwd_packed", _check_packed, qkv, o, lse, dO, dqkv, workspace, backward=True)
+    r = hot.bwd_packed(qkv, o, lse, dO, G, dqkv, workspace, bool(fast), _given_stream(stream))
+    r = _result(r, "s2a_bwd_packed", _check_packed, qkv, o, lse, dO, dqkv, workspace, backward=True)
+    return r if qkv.__class__ in _PLAIN else _typed((r,), (None if dqkv is not None else qkv,))[0]
 
 
 def s2a_bwd_stage(q, k, v, o, lse, dO, G, dq, dk, dv, workspace, stage, stream=None):
@@ -312,15 +328,21 @@ def s2a_fwd_ex(q, k, v, G, scale=None, n_unshifted=None, shift=None, leak_free=F
     swap_wrapped=True makes its two parts change places (variant 3)."""
     hot = _hot or _hot_for(_check_fwd, q, k, v, o, lse)
     r = hot.fwd_ex(q, k, v, G, scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), o, lse, _given_stream(stream))
-    return r if r.__class__ is tuple else _result(r, "s2a_fwd_ex", _check_fwd, q, k, v, o, lse)
+    if r.__class__ is not tuple:
+        _result(r, "s2a_fwd_ex", _check_fwd, q, k, v, o, lse)
+    return r if q.__class__ in _PLAIN else _typed(r, (None if o is not None else q, None))
 
 
 def s2a_bwd_ex(q, k, v, o, lse, dO, G, scale=None, n_unshifted=None, shift=None, leak_free=False, workspace=None,
                stream=None, dq=None, dk=None, dv=None, swap_wrapped=False, fast=True):
     hot = _hot or _hot_for(_check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
-    r = hot.bwd_ex(q, k, v, o, lse, dO, G, scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), dq, dk, dv, workspace, fast,
+    r = hot.bwd_ex(q, k, v, o, lse, dO, G, scale, n_unshifted, shift, _flags(leak_free, swap_wrapped), dq, dk, dv, workspace, bool(fast),
                    _given_stream(stream))
-    return r if r.__class__ is tuple else _result(r, "s2a_bwd_ex", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    if r.__class__ is not tuple:
+        _result(r, "s2a_bwd_ex", _check_bwd, q, k, v, o, lse, dO, dq, dk, dv, workspace)
+    if q.__class__ in _PLAIN and k.__class__ in _PLAIN:
+        return r
+    return _typed(r, tuple(None if out is not None else like for out, like in ((dq, q), (dk, k), (dv, k))))
 
 
 def s2a_fwd_bwd_host(host_in, host_out, dev, G, workspace, stream=None):

@@ -84,3 +84,30 @@ def test_backward_refuses_saved_tensors_that_come_back_changed(change, which):
     assert [t.dtype for t in saved] == [torch.bfloat16] * 4 + [torch.float32]
     with pytest.raises(ValueError, match="saved"):
         torch.autograd.grad(o, (q, k, v), dO)
+
+
+class Marked(torch.Tensor):
+    """What a user's program may mark its tensors with."""
+
+
+@pytest.mark.gpu
+def test_results_have_the_class_of_their_arguments():
+    q, k, v, dO = (x.cuda() for x in make_inputs(1, 512, 4, 2, 64, seed=8))
+    o, lse = s2a.s2a_fwd(q, k, v, 256)
+    want = s2a.s2a_bwd(q, k, v, o, lse, dO, 256, fast=1)
+    mq, mk = q.as_subclass(Marked), k.as_subclass(Marked)
+    mo, mlse = s2a.s2a_fwd(mq, mk, v, 256)
+    assert type(mo) is Marked and type(mlse) is torch.Tensor and torch.equal(mo.as_subclass(torch.Tensor), o)
+    assert type(s2a.s2a_fwd_ex(q, mk, v, 256)[0]) is torch.Tensor
+    given = torch.empty_like(k)
+    got = s2a.s2a_bwd(mq, mk, v, mo, lse, dO, 256, dk=given, fast="yes")
+    assert [type(t) for t in got] == [Marked, torch.Tensor, Marked] and got[1] is given
+    assert all(torch.equal(a.as_subclass(torch.Tensor), b) for a, b in zip(got, want))
+    leaf = mq.detach().requires_grad_()
+    out = s2_attn(leaf, k, v, 256, fast_backward="yes")
+    assert type(out) is Marked and torch.equal(torch.autograd.grad(out, leaf, dO)[0].as_subclass(torch.Tensor), want[0])
+    p = torch.nn.Parameter(q)
+    assert type(s2_attn(p, k, v, 256)) is torch.Tensor and type(s2a.s2a_fwd(p.detach(), k, v, 256)[0]) is torch.Tensor
+    qkv = torch.stack((q, q, q), 2).as_subclass(Marked)
+    po, plse = s2a.s2a_fwd_packed(qkv, 256)
+    assert type(po) is torch.Tensor and type(s2a.s2a_bwd_packed(qkv, po, plse, dO, 256)) is Marked
