@@ -32,8 +32,8 @@
 // on a grouped-query shape (2 x 4096, groups of 1024, head size 64), 2 % on Llama2-7B 32k.
 //
 // What bounds it: the softmax (a step of both tiles keeps the special-function unit busy for 2048 clocks and the
-// tensor pipe for 2048) and, sustained, the power limit: 1244 TFLOP/s on Llama2-7B 32k, 0.92 of what the cuBLAS
-// loop sustains.  Microseconds a call in a loop: first form (one query tile per block, two blocks per SM, two threads
+// tensor pipe for 2048) and, sustained, the power limit: a loop of forward calls on Llama2-7B 32k runs at 1244 TFLOP/s,
+// 0.92 of what the cuBLAS loop sustains, the forward within a training step at 1142, 0.84.  Microseconds a call in a loop: first form (one query tile per block, two blocks per SM, two threads
 // per row, scores read twice), two tiles with P over S, this form:
 //   Llama2-7B 32k 2383, 1982, 1768; 8k 211, 162, 145; causal 8k 610, 497, 449;
 //   groups of 512 99, 73, 70; groups of 200 (head size 64) 40, 32, 29; head size 64 at 32k 1800, 1514, 1374
