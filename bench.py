@@ -37,12 +37,12 @@ FALLBACK_PEAKS = {"bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0, "hbm_g
 # the number of blocks.  An entry is None where the kernel has changed since its capture.
 #   name: (bytes that scale with the tensors, bytes that scale with the spill) at 8k
 NCU_TRAFFIC_8K = {
-    "fwd": (247.3e6, 0.0),
-    "bwd_preprocess": (138.2e6, 0.0),
-    "bwd_dkdv": (374.0e6, 0.0),                     # 270.6 MB read + 103.4 MB written
-    "bwd_dq": (320.5e6, 0.0),
-    "bwd_dkdv_spill": (917.0e6 - 570.4e6, 570.4e6),  # 270.9 MB read + 646.1 MB written, 570.4 MB of it the spill
-    "bwd_dq_spill": (694.7e6 - 570.4e6, 570.4e6),    # 637.6 MB read + 57.2 MB written
+    "fwd": (247.7e6, 0.0),
+    "bwd_preprocess": (138.4e6, 0.0),
+    "bwd_dkdv": (374.4e6, 0.0),                     # 270.8 MB read + 103.6 MB written
+    "bwd_dq": (320.4e6, 0.0),
+    "bwd_dkdv_spill": (917.6e6 - 570.4e6, 570.4e6),  # 270.9 MB read + 646.7 MB written, 570.4 MB of it the spill
+    "bwd_dq_spill": (694.5e6 - 570.4e6, 570.4e6),    # 637.6 MB read + 56.8 MB written
 }
 NCU_TRAFFIC_8K_SIZE = 1 * 8192 * (32 + 32) * 128
 NCU_SPILL_8K_BLOCKS = 32 * 4 * 16 * 17             # units x T (T + 1) blocks of 16 KiB, T = 2048 / 128
