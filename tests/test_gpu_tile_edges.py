@@ -56,6 +56,27 @@ def test_tile_edges_match_oracle(B, N, G, H, Hkv, d, kw):
     assert s2a.device_status() == (0, 0)
 
 
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("rows", [4, 12, 16, 20, 28, 32, 36, 48, 60, 64, 68, 124])
+def test_masked_blocks_of_the_backward(rows, d):
+    """dK/dV take the diagonal and the end of a ragged tile in blocks of 32 keys by 16 queries that are visible as a whole, in
+    part or not at all.  Two tiles per group, the second of `rows` rows; tolerance as above."""
+    from paper_2309_12307_b200 import binding as s2a
+
+    G, H = 128 + rows, 2
+    q, k, v, dO = make_inputs(1, 2 * G, H, H, d, seed=41)
+    kw = {"n_unshifted": H, "shift": 0}
+    grads_ref = orc.bwd(q, k, v, dO, G, **kw)
+    qd, kd, vd, dOd = (x.cuda() for x in (q, k, v, dO))
+    o, lse = s2a.s2a_fwd_ex(qd, kd, vd, G, **kw)
+    for fast in (False, True):
+        grads = s2a.s2a_bwd_ex(qd, kd, vd, o, lse, dOd, G, fast=fast, **kw)
+        for got, want, name in zip(grads, grads_ref, ("dq", "dk", "dv")):
+            err = rel_l2(got.double().cpu().numpy(), want)
+            assert math.isfinite(err) and err <= 1e-2, (name, fast, err)
+    assert s2a.device_status() == (0, 0)
+
+
 @pytest.mark.parametrize("B,N,G,H,Hkv,d", [(1, 8192, 2048, 32, 32, 64),   # groups and heads cut
                                            (1, 6000, 600, 16, 8, 128),    # ragged tiles; two groups in the chunk that wraps
                                            (2, 4096, 4096, 16, 4, 128),   # one group: heads cut only
