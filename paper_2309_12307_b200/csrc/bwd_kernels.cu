@@ -583,7 +583,10 @@ __global__ void __launch_bounds__(DqCfg<HD>::kThreads, 1) s2a_bwd_dq_kernel(cons
 // 3. dK, dV
 // ------------------------------------------------------------------------------------------------
 // Tensor memory columns: dV, dK (HD each), S^T, dP^T (64 each), P^T and dS^T (bf16, 64 together; two buffers where
-//                        HD = 64 leaves room), K (bf16, HD/2: the A operand of S^T = K Q^T)
+//                        HD = 64 leaves room), K (bf16, HD/2: the A operand of S^T = K Q^T), where HD = 64 V likewise
+//                        (the A operand of dP^T = V dO^T: the products read less shared memory, and V of the next item
+//                        comes as early as its K; 2 x 4096 tokens grouped query 166,000 -> 161,000 clocks a launch,
+//                        32k 3,838,000 -> 3,657,000)
 // One buffer of S^T and dP^T is enough: the elementwise warps copy them into registers at the start of a step
 // and release them at once, so the score products of the next step run while they work.  P^T and dS^T are
 // written when the gradient MMAs are done with what the buffer held.  With P^T and dS^T over S^T, in two
@@ -689,6 +692,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     using C = BwdCfg<HD>;
     using Bars = DkDvBars<C::kStages>;
     constexpr int kPBufs = HD == 64 ? 2 : 1;  // buffers of P^T and dS^T
+    constexpr bool kVInTmem = HD == 64;       // V is a tensor-memory operand like K
     constexpr int kCols = 32;  // query columns per elementwise thread and step: two threads share a key row
     constexpr int kChunks = kCols / 16;
     constexpr int kSched = 8;  // item ids in flight: the TMA warp is at most five items ahead of the read-out
@@ -756,8 +760,9 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
     tc_fence_after();
     const uint32_t tmem_base = bars->tmem_slot;
     const WaitCtx ctx{&bars->abort_flag, p.status, p.host_status};
-    constexpr uint32_t kColDV = 0, kColDK = HD, kColS = 2 * HD, kColP = kColS + 64, kColPdS = kColP + 64, kColKt = kColPdS + 64 * kPBufs;
-    static_assert(kColKt + HD / 2 <= C::kTmemCols, "tensor memory");
+    constexpr uint32_t kColDV = 0, kColDK = HD, kColS = 2 * HD, kColP = kColS + 64, kColPdS = kColP + 64, kColKt = kColPdS + 64 * kPBufs,
+                       kColVt = kColKt + HD / 2;
+    static_assert(kColVt + (kVInTmem ? HD / 2 : 0) <= C::kTmemCols, "tensor memory");
 
     // Every consumer warp walks the same sequence of items, as the scheduling thread has decoded them (the
     // divisions cost a warp more than a step): the k-th one, false = the end (or aborting).
@@ -826,7 +831,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             // of the step before in registers (warp-uniform loop, one elected lane issues; see the dQ kernel)
             constexpr uint32_t idesc_sc = idesc_bf16(128, kSubTile, 0, 0);
             const uint32_t dV = desc_lo_k_major(smem_u32(sV));
-            const uint32_t tP = tmem_base + kColP, tKt = tmem_base + kColKt;
+            const uint32_t tP = tmem_base + kColP, tKt = tmem_base + kColKt, tVt = tmem_base + kColVt;
             int it = 0;
             bool ok = true;
             for (int k = 0; ok; ++k) {
@@ -841,7 +846,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     const uint32_t aQ = smem_u32(sStage + st * C::kStageBytes);
                     const uint32_t dQ = desc_lo_k_major(aQ), dDO = desc_lo_k_major(aQ + C::kSubTileBytes);
                     const uint32_t tS = tmem_base + kColS;
-                    if (x == 0 && !mbar_wait_uniform(&bars->v_full, k & 1, ctx, kWaitBwdDkDv + 3)) { ok = false; break; }
+                    if (!kVInTmem && x == 0 && !mbar_wait_uniform(&bars->v_full, k & 1, ctx, kWaitBwdDkDv + 3)) { ok = false; break; }
                     if (it >= 1 && !mbar_wait_uniform(&bars->s_free, (it - 1) & 1, ctx, kWaitBwdDkDv + 9)) { ok = false; break; }
                     if (kPBufs > 1 && it >= kPBufs && !mbar_wait_uniform(&bars->p_free[it % kPBufs], ((it / kPBufs) & 1) ^ 1, ctx, kWaitBwdDkDv + 8)) { ok = false; break; }
                     tc_fence_after();
@@ -849,9 +854,9 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                         mbar_arrive(&bars->s_full);  // (the phase of the step before was over when s_free was)
 #pragma unroll
                         for (int kk = 0; kk < HD / 16; ++kk)
-                            mma_ss(tP, dV + desc_step_k_major(kk, C::kBigBoxBytes), dDO + desc_step_k_major(kk, C::kSubBoxBytes),
-                                   idesc_sc, kk > 0);
-                        if (last) mma_commit(&bars->v_empty);
+                            if constexpr (kVInTmem) mma_ts(tP, tVt + 8 * kk, dDO + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
+                            else mma_ss(tP, dV + desc_step_k_major(kk, C::kBigBoxBytes), dDO + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
+                        if (!kVInTmem && last) mma_commit(&bars->v_empty);
 #pragma unroll
                         for (int kk = 0; kk < HD / 16; ++kk)
                             mma_ts(tS, tKt + 8 * kk, dQ + desc_step_k_major(kk, C::kSubBoxBytes), idesc_sc, kk > 0);
@@ -923,7 +928,8 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
                     for (int bx = 0; bx < C::kBoxes; ++bx)
                         tma_load_4d(sK + bx * C::kBigBoxBytes, &p.tm_k, &bars->k_full, bx * 64, t.hk, t.tk0, t.b);
                     ++n_k;
-                    if (k > 0 && !mbar_wait(&bars->v_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 20)) break;
+                    // (where V is copied as well, the wait for kt_full stands for both)
+                    if (!kVInTmem && k > 0 && !mbar_wait(&bars->v_empty, (k - 1) & 1, ctx, kWaitBwdDkDv + 20)) break;
                     mbar_expect_tx(&bars->v_full, C::kBigTileBytes);
                     for (int bx = 0; bx < C::kBoxes; ++bx)
                         tma_load_4d(sV + bx * C::kBigBoxBytes, &p.tm_v, &bars->v_full, bx * 64, t.hk, t.tk0, t.b);
@@ -1105,17 +1111,24 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             if (!mbar_wait_uniform(&bars->k_full, k & 1, ctx, kWaitBwdDkDv + 17)) return false;
             if (k > 0 && !mbar_wait_uniform(&bars->s_done, (k - 1) & 1, ctx, kWaitBwdDkDv + 21)) return false;
             tc_fence_after();
+            auto copy_row = [&](const uint8_t* tile, uint32_t t_addr) {
 #pragma unroll
-            for (int bx = 0; bx < C::kBoxes; ++bx) {
-                const uint32_t src = smem_u32(sK) + bx * C::kBigBoxBytes + row * 128;
-                uint32_t kr[32];
+                for (int bx = 0; bx < C::kBoxes; ++bx) {
+                    const uint32_t src = smem_u32(tile) + bx * C::kBigBoxBytes + row * 128;
+                    uint32_t kr[32];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
-                                 : "=r"(kr[4 * c]), "=r"(kr[4 * c + 1]), "=r"(kr[4 * c + 2]), "=r"(kr[4 * c + 3])
-                                 : "r"(src + ((c ^ (row & 7)) << 4)));
+                    for (int c = 0; c < 8; ++c) {
+                        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                                     : "=r"(kr[4 * c]), "=r"(kr[4 * c + 1]), "=r"(kr[4 * c + 2]), "=r"(kr[4 * c + 3])
+                                     : "r"(src + ((c ^ (row & 7)) << 4)));
+                    }
+                    tmem_st_32x32(t_addr + bx * 32, kr);
                 }
-                tmem_st_32x32(t_row + kColKt + bx * 32, kr);
+            };
+            copy_row(sK, t_row + kColKt);
+            if constexpr (kVInTmem) {
+                if (!mbar_wait_uniform(&bars->v_full, k & 1, ctx, kWaitBwdDkDv + 3)) return false;
+                copy_row(sV, t_row + kColVt);
             }
             tmem_wait_st();
             tc_fence_before();
