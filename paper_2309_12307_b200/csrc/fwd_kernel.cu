@@ -67,16 +67,21 @@ struct FwdCfg {
 };
 
 // Items in flight.  A warp that has a part in an item holds the next loads back, so the producer is at most six items
-// ahead of it.  The softmax warps of tile 0 have no part in an item without that tile (the last pair of an odd number of
-// tiles, single tiles), so they walk a list of their own, of the items that have it.
+// ahead of it.  A group of softmax warps has no part in an item whose only tile (the last pair of an odd number of
+// tiles, single tiles) is the other group's, so each group walks a list of its own, of the items it has a tile of.
 constexpr int kSched = 8;
 
 struct FwdItem {
-    int b, h, hk;
+    int b, h;
     GroupLayout L;
     TilePair t;
 };
+// The later tile of a pair attends one key tile more than the other one, and it is the only tile where an item has one.
+// The two groups of softmax warps take it in turn: if one always had it, the other would wait for it in every item.
+__device__ __forceinline__ int group_of_tile(int item, int t) { return (item & 1) ^ t ^ 1; }
+__device__ __forceinline__ int tile_of_group(int item, int group) { return (item & 1) ^ group ^ 1; }
 struct FwdBars {
+    // by group of softmax warps
     uint64_t q_full[2], q_empty[2];
     uint64_t s_full[2];              // S of a tile's step is in tensor memory
     uint64_t s_empty[2];             // a score buffer has been read into registers
@@ -87,14 +92,15 @@ struct FwdBars {
     uint64_t stat_full[2], stat_empty[2];
     uint64_t kv_full[8], kv_empty[8];
     uint64_t sched_full[kSched];
-    uint64_t pair_full[kSched];      // the same for the softmax warps of tile 0: items with two tiles only
+    uint64_t list_full[2][kSched];   // the same for either group of softmax warps: items that it has a tile of
     uint64_t clc, drain[2];
     alignas(16) uint8_t clc_resp[16];
     FwdItem item[kSched];  // b = -1: no more items
-    int pair_slot[kSched];  // where the items counted on pair_full are
+    uint8_t list_slot[2][kSched];  // where the items counted on list_full are
     uint32_t tmem_slot;
     int abort_flag;
 };
+static_assert(kSched % 2 == 0, "a slot's parity is its item's");
 static_assert(sizeof(FwdBars) <= 1024, "barrier block");
 
 // Threshold (in log2 units) below which a larger running maximum is ignored: P then grows by at
@@ -115,7 +121,6 @@ __device__ __forceinline__ bool fwd_item(const FwdParams& p, int id, FwdItem* w)
     int unit, rank, g;
     p.order.decode(id, &unit, &rank);
     w->b = p.by_heads(p.geo.by_groups(unit, &g), &w->h);
-    w->hk = p.geo.by_rep(w->h);
     w->L = group_layout(p.geo, (w->h < p.geo.n_unshifted) ? 0 : p.geo.shift, g);
     if (rank >= pairs_of_group(w->L, p.single)) return false;
     w->t = tile_pair(w->L, rank, p.single);
@@ -158,7 +163,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
         }
         for (int x = 0; x < kSched; ++x) {
             mbar_init(&bars->sched_full[x], 1);
-            mbar_init(&bars->pair_full[x], 1);
+            mbar_init(&bars->list_full[0][x], 1);
+            mbar_init(&bars->list_full[1][x], 1);
         }
         mbar_init(&bars->clc, 1);
         fence_barrier_init();
@@ -208,49 +214,57 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             // ======================= work items, TMA loads ===========================================
             if (lane == 0) {
                 uint32_t kv = 0;              // K and V tiles requested so far
-                uint32_t n_q[2] = {0, 0};     // query tiles requested so far
+                uint32_t n_q[2] = {0, 0};     // query tiles requested so far for either group
                 bool ok = true;
                 ItemSource items{&bars->clc, bars->clc_resp};
                 int id = static_cast<int>(blockIdx.x);
-                uint32_t n_pairs = 0;  // items with two tiles so far
-                auto load_q = [&](const FwdItem& w, int t) {
-                    if (!mbar_wait(&bars->q_empty[t], (n_q[t] & 1) ^ 1, ctx, kWaitFwd + 2)) { ok = false; return; }
-                    mbar_expect_tx(&bars->q_full[t], C::kTileBytes);
-                    const int tok0 = tile_ref(w.L, w.t.i[t]).tok0;
+                uint32_t n_list[2] = {0, 0};  // items in the list of either group
+                auto load_q = [&](const FwdItem& w, int t, int g) {
+                    const uint32_t n = g ? n_q[1]++ : n_q[0]++;
+                    if (!mbar_wait(&bars->q_empty[g], (n & 1) ^ 1, ctx, kWaitFwd + 2)) {
+                        --(g ? n_q[1] : n_q[0]);
+                        ok = false;
+                        return;
+                    }
+                    mbar_expect_tx(&bars->q_full[g], C::kTileBytes);
+                    const int tok0 = tile_ref(w.L, t ? w.t.i[1] : w.t.i[0]).tok0;
                     for (int bx = 0; bx < C::kBoxes; ++bx)
-                        tma_load_4d(sQ + t * C::kTileBytes + bx * C::kBoxBytes, &p.tm_q, &bars->q_full[t], bx * 64, w.h, tok0, w.b);
-                    ++n_q[t];
+                        tma_load_4d(sQ + g * C::kTileBytes + bx * C::kBoxBytes, &p.tm_q, &bars->q_full[g], bx * 64, w.h, tok0, w.b);
                 };
-                auto load_kv = [&](const FwdItem& w, bool k_tile, int tok0) {
+                auto enlist = [&](int k, int g) {
+                    const uint32_t n = g ? n_list[1]++ : n_list[0]++;
+                    bars->list_slot[g][n % kSched] = static_cast<uint8_t>(k % kSched);
+                    mbar_arrive(&bars->list_full[g][n % kSched]);
+                };
+                auto load_kv = [&](const FwdItem& w, int hk, bool k_tile, int tok0) {
                     const int st = kv % C::kRing;
                     if (!mbar_wait(&bars->kv_empty[st], ((kv / C::kRing) & 1) ^ 1, ctx, kWaitFwd + 3)) { ok = false; return; }
                     mbar_expect_tx(&bars->kv_full[st], C::kTileBytes);
                     for (int bx = 0; bx < C::kBoxes; ++bx) {
                         uint8_t* dst = sKV + st * C::kTileBytes + bx * C::kBoxBytes;
-                        if (k_tile) tma_load_5d(dst, &p.tm_k, &bars->kv_full[st], w.hk * HD + bx * 64, 0, 0, tok0 / 4, w.b);
-                        else tma_load_4d(dst, &p.tm_v, &bars->kv_full[st], bx * 64, w.hk, tok0, w.b);
+                        if (k_tile) tma_load_5d(dst, &p.tm_k, &bars->kv_full[st], hk * HD + bx * 64, 0, 0, tok0 / 4, w.b);
+                        else tma_load_4d(dst, &p.tm_v, &bars->kv_full[st], bx * 64, hk, tok0, w.b);
                     }
                     ++kv;
                 };
                 for (int k = 0; ok; ++k) {
-                    FwdItem w;
+                    FwdItem& w = bars->item[k % kSched];  // kept there: the registers of these warps are few
                     while (id >= 0 && !fwd_item(p, id, &w)) {  // skip the empty slots of smaller groups
                         id = items.next(ctx, kWaitFwd + 1, &ok);
                     }
                     if (id < 0) w.b = -1;
-                    bars->item[k % kSched] = w;
                     mbar_arrive(&bars->sched_full[k % kSched]);  // release: the item is visible to whoever sees the phase
-                    if (id < 0 || w.t.n[0] > 0) {
-                        bars->pair_slot[n_pairs % kSched] = k % kSched;
-                        mbar_arrive(&bars->pair_full[n_pairs++ % kSched]);
-                    }
+                    const int g1 = group_of_tile(k, 1), g0 = group_of_tile(k, 0);
+                    enlist(k, g1);
+                    if (id < 0 || w.t.n[0] > 0) enlist(k, g0);
                     if (id < 0) break;
+                    const int hk = p.geo.by_rep(w.h);
                     for (int j = 0; ok && j < w.t.n[1]; ++j) {
                         const int tok0 = tile_ref(w.L, w.t.j_begin + j).tok0;
-                        if (j == 0 && w.t.n[0] > 0) load_q(w, 0);
-                        if (ok) load_kv(w, true, tok0);
-                        if (j == 0 && ok) load_q(w, 1);
-                        if (ok) load_kv(w, false, tok0);
+                        if (j == 0) load_q(w, 1, g1);
+                        if (ok) load_kv(w, hk, true, tok0);
+                        if (j == 0 && ok && w.t.n[0] > 0) load_q(w, 0, g0);
+                        if (ok) load_kv(w, hk, false, tok0);
                     }
                     if (ok) id = items.next(ctx, kWaitFwd + 1, &ok);
                 }
@@ -267,15 +281,16 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             // ======================= MMA issuers: warp 13 for S = Q K^T, warp 14 for O += P V ============
             // The whole warp walks the loop so that addresses and descriptors stay warp-uniform values;
             // only the MMA and commit instructions themselves are issued by one elected lane.  Both take the
-            // tiles in turn: tile 0, tile 1 of key tile j, then of j + 1 (tile 0 has no products with the
-            // last key tile).  K tiles are in the even slots of the ring, V tiles in the odd ones.
+            // tiles in turn: tile 1, tile 0 of key tile j, then of j + 1 (tile 0 has no products with the
+            // last key tile), so that the groups of softmax warps are served in turn across items as well.
+            // K tiles are in the even slots of the ring, V tiles in the odd ones.
             constexpr uint32_t idesc_s = idesc_bf16(128, kTile, 0, 0);  // S = Q K^T   (both K-major)
             constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);     // O += P V    (V is MN-major)
             const bool is_s = warp == 13;
             const uint32_t aKV = smem_u32(sKV), dQ0 = desc_lo_k_major(smem_u32(sQ));
             uint32_t kv = 0;                    // ring position of the item's K_0
-            uint32_t n_it[2] = {0, 0};          // items of either tile so far
-            uint32_t n_st[2] = {0, 0}, n_s = 0; // steps of either tile, score products
+            // parities: bit g of the steps of group g so far, bit 2 + g of its items, bit 4 of all steps
+            uint32_t parity = 0;
             bool ok = true;
             for (int k = 0; ok; ++k) {
                 FwdItem w;
@@ -283,55 +298,54 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 const int n1 = w.t.n[1], n0 = w.t.n[0];
 #pragma unroll 1
                 for (int h = 0; ok && h < 2 * n1; ++h) {
-                    const int t = h & 1, j = h >> 1, n = t ? n1 : n0;
+                    const int t = (h & 1) ^ 1, j = h >> 1, n = t ? n1 : n0, g = group_of_tile(k, t);
                     if (j >= n) continue;
                     const uint32_t x = kv + 2 * j + (is_s ? 0 : 1);
-                    // what tile 0 has used, tile 1 need not wait for again
-                    if ((t == 0 || j >= n0) && !mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, kWaitFwd + 5)) { ok = false; break; }
-                    const uint32_t it = t ? n_it[1] : n_it[0], st = t ? n_st[1] : n_st[0];
+                    const bool last_use = t == 0 || j >= n0;  // of this K or V tile
+                    const uint32_t st = (parity >> g) & 1, it = (parity >> (2 + g)) & 1;
+                    // Where the operands are, before the waits: what is left to do when a score buffer or P is handed over is
+                    // in the way of the next step.
+                    uint32_t at_g = is_s ? dQ0 + g * (C::kTileBytes >> 4) : tmem_base + C::kColP + g * 64;
+                    uint32_t at_x = is_s ? desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes) : desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
+                    uint32_t acc = tmem_base + (is_s ? C::kColS + (C::kScoreBufs == 1 ? 0 : g) * kTile : C::kColO + g * HD);
+                    // what tile 1 has used, tile 0 need not wait for again
+                    if (t == 1 && !mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, kWaitFwd + 5)) { ok = false; break; }
                     if (is_s) {
-                        if (j == 0 && !mbar_wait_uniform(&bars->q_full[t], it & 1, ctx, kWaitFwd + 4)) { ok = false; break; }
-                        const int buf = C::kScoreBufs == 1 ? 0 : t;
-                        const uint32_t use = C::kScoreBufs == 1 ? n_s : st;
-                        if (!mbar_wait_uniform(&bars->s_empty[buf], (use & 1) ^ 1, ctx, kWaitFwd + 6)) { ok = false; break; }
+                        if (j == 0 && !mbar_wait_uniform(&bars->q_full[g], it, ctx, kWaitFwd + 4)) { ok = false; break; }
+                        const int buf = C::kScoreBufs == 1 ? 0 : g;
+                        const uint32_t use = C::kScoreBufs == 1 ? parity >> 4 : st;
+                        if (!mbar_wait_uniform(&bars->s_empty[buf], use ^ 1, ctx, kWaitFwd + 6)) { ok = false; break; }
                         tc_fence_after();
-                        const uint32_t dQ = dQ0 + t * (C::kTileBytes >> 4);
-                        const uint32_t dK = desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes);
-                        const uint32_t tS = tmem_base + C::kColS + buf * kTile;
                         if (elect_one()) {
 #pragma unroll
                             for (int kk = 0; kk < HD / 16; ++kk)
-                                mma_ss(tS, dQ + desc_step_k_major(kk, C::kBoxBytes), dK + desc_step_k_major(kk, C::kBoxBytes), idesc_s, kk > 0);
-                            mma_commit(&bars->s_full[t]);
-                            if (t == 1) mma_commit(&bars->kv_empty[x % C::kRing]);  // tile 1 uses every K and V tile, and uses it last
-                            if (j == n - 1) mma_commit(&bars->q_empty[t]);
+                                mma_ss(acc, at_g + desc_step_k_major(kk, C::kBoxBytes), at_x + desc_step_k_major(kk, C::kBoxBytes), idesc_s, kk > 0);
+                            mma_commit(&bars->s_full[g]);
+                            if (last_use) mma_commit(&bars->kv_empty[x % C::kRing]);
+                            if (j == n - 1) mma_commit(&bars->q_empty[g]);
                         }
                         __syncwarp();
-                        ++n_s;
                     } else {
-                        if (j == 0 && !mbar_wait_uniform(&bars->o_empty[t], (it & 1) ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
-                        const uint32_t dV = desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
-                        const uint32_t tP = tmem_base + C::kColP + t * 64, tO = tmem_base + C::kColO + t * HD;
-                        if (!mbar_wait_uniform(&bars->p_full[t], st & 1, ctx, kWaitFwd + 8)) { ok = false; break; }
+                        if (j == 0 && !mbar_wait_uniform(&bars->o_empty[g], it ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
+                        if (!mbar_wait_uniform(&bars->p_full[g], st, ctx, kWaitFwd + 8)) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
 #pragma unroll
-                            for (int kk = 0; kk < 6; ++kk) mma_ts(tO, tP + kk * 8, dV + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
+                            for (int kk = 0; kk < 6; ++kk) mma_ts(acc, at_g + kk * 8, at_x + kk * kDescStepMn, idesc_o, (j > 0) || (kk > 0));
                         }
                         __syncwarp();
-                        if (!mbar_wait_uniform(&bars->p_rest[t], st & 1, ctx, kWaitFwd + 9)) { ok = false; break; }
+                        if (!mbar_wait_uniform(&bars->p_rest[g], st, ctx, kWaitFwd + 9)) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
 #pragma unroll
-                            for (int kk = 6; kk < 8; ++kk) mma_ts(tO, tP + kk * 8, dV + kk * kDescStepMn, idesc_o, 1);
-                            mma_commit(&bars->p_empty[t]);
-                            if (t == 1) mma_commit(&bars->kv_empty[x % C::kRing]);
-                            if (j == n - 1) mma_commit(&bars->o_full[t]);
+                            for (int kk = 6; kk < 8; ++kk) mma_ts(acc, at_g + kk * 8, at_x + kk * kDescStepMn, idesc_o, 1);
+                            mma_commit(&bars->p_empty[g]);
+                            if (last_use) mma_commit(&bars->kv_empty[x % C::kRing]);
+                            if (j == n - 1) mma_commit(&bars->o_full[g]);
                         }
                         __syncwarp();
                     }
-                    if (t) ++n_st[1], n_it[1] += j == n - 1;
-                    else ++n_st[0], n_it[0] += j == n - 1;
+                    parity ^= (1u << g) | (j == n - 1 ? 4u << g : 0u) | 16u;
                 }
                 kv += 2 * n1;
             }
@@ -356,21 +370,24 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             FwdItem w;
             // the four warps leave together, or the ones that stay would wait for the others below
             if (!named_barrier_and(1, 128, next_item(k, kWaitFwd + 11, &w))) break;
-#pragma unroll
+            // As one loop body the kernel is 5 % faster at head size 64 (groups of 200 28.4 -> 26.5 us, 2 x 4096 tokens grouped
+            // query 67.5 -> 64.7), at 128 written out twice (32k 2,527,000 -> 2,506,000 clocks, causal 8k 679,000 -> 660,000).
+#pragma unroll(HD == 128 ? 2 : 1)
             for (int t = 0; t < 2; ++t) {
-                if (w.t.n[t] == 0) continue;
-                const TileRef tq = tile_ref(w.L, w.t.i[t]);
+                if ((t ? w.t.n[1] : w.t.n[0]) == 0) continue;
+                const int g = group_of_tile(k, t);
+                const TileRef tq = tile_ref(w.L, t ? w.t.i[1] : w.t.i[0]);
+                const uint32_t n_done = g ? n_o[1]++ : n_o[0]++;
                 const bool whole = tq.valid == kTile;
                 // the tile stored last must have left the staging buffer (thread 0 of the four warps stores)
                 if (threadIdx.x == 256) bulk_wait_read<0>();
-                ok = mbar_wait_uniform(&bars->stat_full[t], n_o[t] & 1, ctx, kWaitFwd + 12) &&
-                     mbar_wait_uniform(&bars->o_full[t], n_o[t] & 1, ctx, kWaitFwd + 13);
+                ok = mbar_wait_uniform(&bars->stat_full[g], n_done & 1, ctx, kWaitFwd + 12) &&
+                     mbar_wait_uniform(&bars->o_full[g], n_done & 1, ctx, kWaitFwd + 13);
                 ok = named_barrier_and(1, 128, ok);
                 if (!ok) break;
                 tc_fence_after();
-                ++n_o[t];
-                const float m = sStat[t * 256 + row], l = sStat[t * 256 + 128 + row];
-                mbar_arrive_warp(&bars->stat_empty[t]);
+                const float m = sStat[g * 256 + row], l = sStat[g * 256 + 128 + row];
+                mbar_arrive_warp(&bars->stat_empty[g]);
                 const float inv_l = 1.0f / l;
                 const int tok = tq.tok0 + row;
                 const bool row_valid = row < tq.valid;  // rows past the end of a ragged tile are not part of the group
@@ -378,7 +395,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
 #pragma unroll
                 for (int c = 0; c < HD / 32; ++c) {
                     uint32_t r[32];
-                    tmem_ld_32x32(t_row + C::kColO + t * HD + c * 32, r);
+                    tmem_ld_32x32(t_row + C::kColO + g * HD + c * 32, r);
                     tmem_wait_ld();
                     const uint32_t dst_s = smem_u32(sO) + (c >> 1) * C::kBoxBytes + row * 128;
                     uint4* dst_g = reinterpret_cast<uint4*>(orow + c * 32);
@@ -400,7 +417,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     }
                 }
                 tc_fence_before();
-                mbar_arrive_warp(&bars->o_empty[t]);
+                mbar_arrive_warp(&bars->o_empty[g]);
                 if (whole) {
                     fence_proxy_async();
                     named_barrier(1, 128);
@@ -418,27 +435,27 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
     } else {
         // =========================== softmax =========================================================
         setmaxnreg_inc<C::kRegsSoftmax>();
-        const int t = warp >> 2;               // query tile
+        const int group = warp >> 2;           // takes a tile of every item, or of every other one
         const int quad = warp & 3;             // tensor-memory lane quadrant this warp may access
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-        const uint32_t tS = t_row + C::kColS + (C::kScoreBufs == 1 ? 0 : t * kTile), tP = t_row + C::kColP + t * 64;
+        const uint32_t tS = t_row + C::kColS + (C::kScoreBufs == 1 ? 0 : group * kTile), tP = t_row + C::kColP + group * 64;
         const float c2 = p.scale_log2;
         const uint64_t c2x2 = f2_pack(c2, c2);
         uint32_t n_s = 0, n_it = 0;
         bool ok = true;
-        uint64_t* full = t ? bars->sched_full : bars->pair_full;
         for (int k = 0; ok; ++k) {
-            if (!mbar_wait_uniform(&full[k % kSched], (k / kSched) & 1, ctx, kWaitFwd + 14)) break;
-            const FwdItem w = bars->item[t ? k % kSched : bars->pair_slot[k % kSched]];
+            if (!mbar_wait_uniform(&bars->list_full[group][k % kSched], (k / kSched) & 1, ctx, kWaitFwd + 14)) break;
+            const int slot = bars->list_slot[group][k % kSched];
+            const FwdItem w = bars->item[slot];
             if (w.b < 0) break;
-            const int n = t ? w.t.n[1] : w.t.n[0];
+            const int n = tile_of_group(slot, group) ? w.t.n[1] : w.t.n[0];
             float m_used = 0.f;   // running maximum in use, scaled to log2 units
             // running sum of exp2(s*c2 - m_used) over the keys [0, 64) and [64, 128) of the tiles
             float l[2] = {0.f, 0.f};
             for (int j = 0; j < n; ++j, ++n_s) {
                 const int k_valid = tile_ref(w.L, w.t.j_begin + j).valid;
-                if (!mbar_wait_uniform(&bars->s_full[t], n_s & 1, ctx, kWaitFwd + 15)) { ok = false; break; }
+                if (!mbar_wait_uniform(&bars->s_full[group], n_s & 1, ctx, kWaitFwd + 15)) { ok = false; break; }
                 tc_fence_after();
                 uint32_t s[4][32];
                 tmem_ld_32x32(tS, s[0]);
@@ -447,7 +464,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 tmem_ld_32x32(tS + 96, s[3]);
                 tmem_wait_ld();
                 tc_fence_before();
-                mbar_arrive_warp(&bars->s_empty[C::kScoreBufs == 1 ? 0 : t]);
+                mbar_arrive_warp(&bars->s_empty[C::kScoreBufs == 1 ? 0 : group]);
                 // Key x of the tile is visible to query row r iff it is one of the tile's valid rows and,
                 // on the diagonal tile, x <= r.  Off the diagonal a full tile needs no mask at all.
                 const bool last = (j == n - 1);
@@ -468,7 +485,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 }
                 const float m_new = fmaxf(fmaxf(mx4[0], mx4[1]), fmaxf(mx4[2], mx4[3])) * c2;
                 // the P.V product of this tile's step before is done: P and O may be written
-                if (n_s > 0 && !mbar_wait_uniform(&bars->p_empty[t], (n_s - 1) & 1, ctx, kWaitFwd + 17)) { ok = false; break; }
+                if (n_s > 0 && !mbar_wait_uniform(&bars->p_empty[group], (n_s - 1) & 1, ctx, kWaitFwd + 17)) { ok = false; break; }
                 tc_fence_after();
                 if (j == 0) {
                     m_used = m_new;
@@ -480,7 +497,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
 #pragma unroll 1
                         for (int c = 0; c < HD / 16; ++c) {
                             uint32_t o[16];
-                            const uint32_t t_o = t_row + C::kColO + t * HD + c * 16;
+                            const uint32_t t_o = t_row + C::kColO + group * HD + c * 16;
                             tmem_ld_32x16(t_o, o);
                             tmem_wait_ld();
 #pragma unroll
@@ -523,18 +540,18 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     if (c >= 2) {
                         tmem_wait_st();
                         tc_fence_before();
-                        mbar_arrive_warp(c == 2 ? &bars->p_full[t] : &bars->p_rest[t]);
+                        mbar_arrive_warp(c == 2 ? &bars->p_full[group] : &bars->p_rest[group]);
                     }
                     // the sum of a chunk beside the exponentials of the next: all sums at the end cost 2 % (head size 64, 16k)
                     if (c > 0) add_chunk(c - 1);
                     if (c == 3) add_chunk(3);
                 }
             }
-            if (!ok || !mbar_wait_uniform(&bars->stat_empty[t], (n_it & 1) ^ 1, ctx, kWaitFwd + 16)) break;
+            if (!ok || !mbar_wait_uniform(&bars->stat_empty[group], (n_it & 1) ^ 1, ctx, kWaitFwd + 16)) break;
             ++n_it;
-            sStat[t * 256 + row] = m_used;
-            sStat[t * 256 + 128 + row] = l[0] + l[1];
-            mbar_arrive_warp(&bars->stat_full[t]);
+            sStat[group * 256 + row] = m_used;
+            sStat[group * 256 + 128 + row] = l[0] + l[1];
+            mbar_arrive_warp(&bars->stat_full[group]);
         }
     }
 

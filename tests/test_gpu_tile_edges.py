@@ -57,6 +57,24 @@ def test_tile_edges_match_oracle(B, N, G, H, Hkv, d, kw):
 
 
 @pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("N,G,kw", [(6144, 384, {}),                          # a pair and a single tile to each group
+                                    (6144, 128, {"n_unshifted": 16}),         # single tiles only
+                                    (4800, 480, {"leak_free": True})])        # ragged, two to four tiles
+def test_forward_items_of_either_parity(N, G, kw, d):
+    """The two groups of softmax warps take the later tile of a block's items in turn: several items to a block, with one tile and
+    with two in every order.  Tolerance as above."""
+    from paper_2309_12307_b200 import binding as s2a
+
+    H = 16
+    q, k, v, _ = make_inputs(1, N, H, H, d, seed=43)
+    o_ref, lse_ref = orc.fwd(q, k, v, G, **kw)
+    o, lse = s2a.s2a_fwd_ex(q.cuda(), k.cuda(), v.cuda(), G, **kw)
+    assert np.abs(o.double().cpu().numpy() - o_ref).max() <= 2e-2
+    assert np.abs(lse.double().cpu().numpy() - lse_ref).max() <= 2e-3
+    assert s2a.device_status() == (0, 0)
+
+
+@pytest.mark.parametrize("d", [64, 128])
 @pytest.mark.parametrize("rows", [4, 12, 16, 20, 28, 32, 36, 48, 60, 64, 68, 124])
 def test_masked_blocks_of_the_backward(rows, d):
     """dK/dV take the diagonal and the end of a ragged tile in blocks of 32 keys by 16 queries that are visible as a whole, in
