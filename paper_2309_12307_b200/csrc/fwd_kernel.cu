@@ -374,9 +374,12 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             FwdItem w;
             // the four warps leave together, or the ones that stay would wait for the others below
             if (!named_barrier_and(1, 128, next_item(k, kWaitFwd + 11, &w))) break;
-            // As one loop body the kernel is 5 % faster at head size 64 (groups of 200 28.4 -> 26.5 us, 2 x 4096 tokens grouped
-            // query 67.5 -> 64.7), at 128 written out twice (32k 2,527,000 -> 2,506,000 clocks, causal 8k 679,000 -> 660,000).
-#pragma unroll(HD == 128 ? 2 : 1)
+            // One loop body for both tiles and all columns: what the read-out adds to the code that the softmax warps run beside
+            // costs more than its branches.  Clocks a launch with the tiles written out twice at head size 128 and all columns
+            // written out, and like this: groups of 200 114,800 and 100,000, of 384 211,900 and 180,200, of 600 398,400 and
+            // 351,400, Llama2-7B 8k 208,400 and 204,300, 32k 2,508,000 and 2,502,000; head size 64, groups of 384 161,800 and
+            // 154,300, 32k 2,440,000 and 2,420,000.
+#pragma unroll 1
             for (int t = 0; t < 2; ++t) {
                 if ((t ? w.t.n[1] : w.t.n[0]) == 0) continue;
                 const int g = group_of_tile(k, t);
@@ -396,7 +399,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                 const int tok = tq.tok0 + row;
                 const bool row_valid = row < tq.valid;  // rows past the end of a ragged tile are not part of the group
                 __nv_bfloat16* orow = p.o + ((static_cast<size_t>(w.b) * p.geo.N + tok) * p.geo.H + w.h) * HD;
-#pragma unroll
+#pragma unroll 1
                 for (int c = 0; c < HD / 32; ++c) {
                     uint32_t r[32];
                     tmem_ld_32x32(t_row + C::kColO + g * HD + c * 32, r);
