@@ -654,9 +654,9 @@ __device__ __forceinline__ DkDvItem dkdv_item(const BwdDkDvParams& p, long long 
 template <int kStages>
 struct DkDvBars {
     uint64_t k_full, v_full;      // K / V of an item landed (one phase per item)
-    uint64_t kt_full;             // K of an item has been copied into tensor memory
-    uint64_t v_empty;             // the dP^T products of an item are done: V may be overwritten
-    uint64_t s_done;              // all score products of an item are done: the copy of K may be overwritten
+    uint64_t kt_full;             // K (HD = 64: and V) of an item has been copied into tensor memory
+    uint64_t v_empty;             // HD = 128: the dP^T products of an item are done, V may be overwritten
+    uint64_t s_done;              // all score products of an item are done: the copies may be overwritten
     uint64_t acc_full;            // all gradient MMAs of an item are done
     uint64_t acc_empty;           // the accumulators of an item have been read out
     uint64_t drain;               // abort path only (gradient MMA warp)
@@ -680,8 +680,8 @@ struct DkDvBars {
 // Persistent: one CTA per SM takes over key tiles, heaviest first, by cluster launch control.  Everything
 // that belongs to the change from one item to the next runs beside the steps: the ids and the streamed
 // tiles are requested ahead (warp 0); K of the next item is loaded as soon as the current one has been
-// copied to tensor memory, V as soon as the last dP^T product is done (warp 3); the copy of K and the
-// read-out of the accumulators have four warps of their own, so that the elementwise warps go straight on
+// copied to tensor memory, V likewise where it is copied as well (HD = 64), else as soon as the last dP^T
+// product is done (warp 3); the copies and the read-out of the accumulators have four warps of their own, so that the elementwise warps go straight on
 // with the next item's first steps.  With the elementwise warps doing it and every warp decoding the item
 // for itself (64-bit divisions, one after the other), the change of item cost 10,000 to 17,000 clocks, as
 // much as ten steps.  Before and after, spilling form, us a launch in a loop: Llama2-7B 8k 354 and 325, 4 x 2048
@@ -1096,7 +1096,7 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             }
         }
     } else {
-        // ---- epilogue: the copy of K into tensor memory and the read-out of the accumulators
+        // ---- epilogue: the copies of K and V into tensor memory and the read-out of the accumulators
         setmaxnreg_dec<C::kRegsOther>();
         const int quad = warp & 3;
         const int row = quad * 32 + lane;
@@ -1104,10 +1104,10 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
         uint8_t* stage = sOut + quad * 8192;
         uint32_t used = 0;
         // K of item k goes from its shared-memory tile into tensor memory, where it is the A operand of
-        // S^T = K Q^T: an A operand in shared memory would be read again by every step (4 KB per MMA
+        // S^T = K Q^T, and where HD = 64 leaves room V, the A operand of dP^T = V dO^T: an A operand in shared memory would be read again by every step (4 KB per MMA
         // against 2 KB of B), and shared-memory bandwidth is what bounds this kernel.  One key row per thread:
         // the 16-byte chunks of the 128-byte-swizzled rows, 32 packed columns for each 64 values.
-        auto copy_k = [&](int k) -> bool {
+        auto copy_operands = [&](int k) -> bool {
             if (!mbar_wait_uniform(&bars->k_full, k & 1, ctx, kWaitBwdDkDv + 17)) return false;
             if (k > 0 && !mbar_wait_uniform(&bars->s_done, (k - 1) & 1, ctx, kWaitBwdDkDv + 21)) return false;
             tc_fence_after();
@@ -1138,12 +1138,12 @@ __global__ void __launch_bounds__(BwdCfg<HD>::kThreads, 1) s2a_bwd_dkdv_kernel(c
             return true;
         };
         DkDvItem next;
-        bool more = next_item(0, kWaitBwdDkDv + 18, &next) && copy_k(0);
+        bool more = next_item(0, kWaitBwdDkDv + 18, &next) && copy_operands(0);
         for (int k = 0; more; ++k) {
             const DkDvItem t = next;
-            // K of the next item, if there is one, as soon as this item's score products are done
+            // the operands of the next item, if there is one, as soon as this item's score products are done
             more = next_item(k + 1, kWaitBwdDkDv + 18, &next);
-            if (more && !copy_k(k + 1)) break;
+            if (more && !copy_operands(k + 1)) break;
             if (!mbar_wait_uniform(&bars->acc_full, k & 1, ctx, kWaitBwdDkDv + 7)) break;
             tc_fence_after();
             const size_t out_row = (static_cast<size_t>(t.b) * geo.N + t.tk0 + row) * p.dkv_tok_stride + static_cast<size_t>(t.hk) * HD;

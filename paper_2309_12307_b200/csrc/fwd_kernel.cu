@@ -12,12 +12,14 @@
 // original token rows, which is the roll back.
 //
 // One persistent block per SM, 512 threads:
-//   warps 0-3, 4-7   softmax of query tile 0 / 1: one thread per score row, the row's 128 scores in
-//                    registers (one trip to tensor memory per key tile, no exchange between threads)
+//   warps 0-3, 4-7   softmax, two groups that take the tiles of an item in turn (group_of_tile): one thread per
+//                    score row, the row's 128 scores in registers (one trip to tensor memory per key tile, no
+//                    exchange between threads)
 //   warps 8-11       epilogue: O / l -> bf16 -> shared memory -> TMA store (or row stores, ragged tiles)
 //   warp 12          work items (cluster launch control: a block takes over blocks that were not launched
 //                    yet, heaviest first) and TMA loads, running ahead across items
 //   warps 13, 14     tcgen05 MMAs: the score products S = Q K_j^T of both tiles in turn / the products O += P V_j
+// (what belongs to a tile's softmax - Q, P, O, statistics, barriers - is kept by group of warps, not by tile)
 // While one tile's scores are in the softmax, the tensor cores work for the other tile; K and V tiles
 // are fetched once for the 256 query rows, which halves their L2 and shared-memory traffic.
 // The scores of a step are in registers 150 clocks after they are complete, and P has tensor memory columns of
@@ -34,9 +36,13 @@
 // What bounds it: the softmax (a step of both tiles keeps the special-function unit busy for 2048 clocks and the
 // tensor pipe for 2048) and, sustained, the power limit: a loop of forward calls on Llama2-7B 32k runs at 1244 TFLOP/s,
 // 0.92 of what the cuBLAS loop sustains, the forward within a training step at 1142, 0.84.  Microseconds a call in a loop: first form (one query tile per block, two blocks per SM, two threads
-// per row, scores read twice), two tiles with P over S, this form:
+// per row, scores read twice), two tiles with P over S, P in columns of its own:
 //   Llama2-7B 32k 2383, 1982, 1768; 8k 211, 162, 145; causal 8k 610, 497, 449;
 //   groups of 512 99, 73, 70; groups of 200 (head size 64) 40, 32, 29; head size 64 at 32k 1800, 1514, 1374
+// Since then the groups of softmax warps take the tiles in turn and the read-out is one loop body; thousands of clocks a
+// launch (microseconds follow the clock of the day), before and now:
+//   32k 2500, 2502; 8k 213, 204; causal 8k 654, 656; groups of 512 112, 98; groups of 200 (head size 64) 50.7, 47.6;
+//   2 x 4096 grouped query 124, 117.6; head size 64 at 32k 2424, 2421
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
@@ -66,9 +72,11 @@ struct FwdCfg {
     static_assert(2 * kRegsSoftmax + kRegsEpilogue + kRegsIssue <= 4 * kRegsLaunch, "register split");
 };
 
-// Items in flight.  A warp that has a part in an item holds the next loads back, so the producer is at most six items
-// ahead of it.  A group of softmax warps has no part in an item whose only tile (the last pair of an odd number of
-// tiles, single tiles) is the other group's, so each group walks a list of its own, of the items it has a tile of.
+// Items in flight.  When the producer writes item k, V of item k - 1 has been requested, so the P.V products of the item
+// kRing / 2 before that one are done (single tiles, the shortest items, take two slots of the ring each), so the read-out of the
+// item that the same group of softmax warps had before, at most two earlier, is done.  Every other warp is further on than the
+// read-out.  A group of softmax warps has no part in an item whose only tile (the last pair of an odd number of tiles, single
+// tiles) is the other group's, but never misses two in a row; each group walks a list of its own, of the items it has a tile of.
 constexpr int kSched = 8;
 
 struct FwdItem {
@@ -77,7 +85,12 @@ struct FwdItem {
     TilePair t;
 };
 // The later tile of a pair attends one key tile more than the other one, and it is the only tile where an item has one.
-// The two groups of softmax warps take it in turn: if one always had it, the other would wait for it in every item.
+// The two groups of softmax warps take it in turn, from one item of the block to the next: bound to the tiles, one group has
+// nothing to do where items are single tiles.  Thousands of clocks a launch, bound and in turn: groups of 128 192 and 175, at
+// head size 64 176 and 152; groups of 384 at head size 64 168 and 155; pairs of tiles alone the same to 1 % (8k 204 and 204,
+// 32k 2491 and 2506, 2 x 4096 grouped query 118 and 118).  Ragged pairs and a single tile at head size 128 are faster bound
+// (groups of 384 173 and 181, of 600 336 and 353), but only where the binding is known when the kernel is compiled: a flag in
+// the item that has the groups change places behind single tiles alone is slower than either (186, 365; 8k 208).
 __device__ __forceinline__ int group_of_tile(int item, int t) { return (item & 1) ^ t ^ 1; }
 __device__ __forceinline__ int tile_of_group(int item, int group) { return (item & 1) ^ group ^ 1; }
 struct FwdBars {
@@ -101,6 +114,7 @@ struct FwdBars {
     int abort_flag;
 };
 static_assert(kSched % 2 == 0, "a slot's parity is its item's");
+static_assert(kSched >= FwdCfg<64>::kRing / 2 + 3 && kSched >= FwdCfg<128>::kRing / 2 + 3, "an item's slot is free when it is written again");
 static_assert(sizeof(FwdBars) <= 1024, "barrier block");
 
 // Threshold (in log2 units) below which a larger running maximum is ignored: P then grows by at
@@ -135,7 +149,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
     uint8_t* sKV = sQ + 2 * C::kTileBytes;             // ring of K and V tiles
     uint8_t* sO = sKV + C::kRing * C::kTileBytes;      // one output tile on its way out
     FwdBars* bars = reinterpret_cast<FwdBars*>(sO + C::kTileBytes);
-    float* sStat = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);  // [tile][m, l][128 rows]
+    float* sStat = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + 1024);  // [group][m, l][128 rows]
 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
@@ -286,7 +300,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             // The whole warp walks the loop so that addresses and descriptors stay warp-uniform values;
             // only the MMA and commit instructions themselves are issued by one elected lane.  Both take the
             // tiles in turn: tile 1, tile 0 of key tile j, then of j + 1 (tile 0 has no products with the
-            // last key tile), so that the groups of softmax warps are served in turn across items as well.
+            // last key tile), so that the groups of softmax warps are served in turn across items as well (tile 0 first:
+            // 8k 204,000 -> 211,000 clocks a launch, 2 x 4096 grouped query 118,000 -> 129,500).
             // K tiles are in the even slots of the ring, V tiles in the odd ones.
             constexpr uint32_t idesc_s = idesc_bf16(128, kTile, 0, 0);  // S = Q K^T   (both K-major)
             constexpr uint32_t idesc_o = idesc_bf16(128, HD, 0, 1);     // O += P V    (V is MN-major)
@@ -307,8 +322,7 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     const uint32_t x = kv + 2 * j + (is_s ? 0 : 1);
                     const bool last_use = t == 0 || j >= n0;  // of this K or V tile
                     const uint32_t st = (parity >> g) & 1, it = (parity >> (2 + g)) & 1;
-                    // Where the operands are, before the waits: what is left to do when a score buffer or P is handed over is
-                    // in the way of the next step.
+                    // where the operands are, before the waits (computed behind them the kernel takes the same time)
                     uint32_t at_g = is_s ? dQ0 + g * (C::kTileBytes >> 4) : tmem_base + C::kColP + g * 64;
                     uint32_t at_x = is_s ? desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes) : desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
                     uint32_t acc = tmem_base + (is_s ? C::kColS + (C::kScoreBufs == 1 ? 0 : g) * kTile : C::kColO + g * HD);
