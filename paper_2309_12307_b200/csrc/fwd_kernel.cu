@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     const int hk = p.geo.by_rep(w.h);
                     for (int j = 0; ok && j < w.t.n[1]; ++j) {
                         const int tok0 = tile_ref(w.L, w.t.j_begin + j).tok0;
-                        if (j == 0) load_q(w, 1, g1);
-                        if (ok) load_kv(w, hk, true, tok0);
+                        load_kv(w, hk, true, tok0);
+                        if (j == 0 && ok) load_q(w, 1, g1);
                         if (j == 0 && ok && w.t.n[0] > 0) load_q(w, 0, g0);
                         if (ok) load_kv(w, hk, false, tok0);
                     }
@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
             const bool is_s = warp == 13;
             const uint32_t aKV = smem_u32(sKV), dQ0 = desc_lo_k_major(smem_u32(sQ));
             uint32_t kv = 0;                    // ring position of the item's K_0
-            // parities: bit g of the steps of group g so far, bit 2 + g of its items, bit 4 of all steps
-            uint32_t parity = 0;
+            uint32_t n_it[2] = {0, 0};          // items of either group so far
+            uint32_t n_st[2] = {0, 0}, n_s = 0; // steps of either group, score products
             bool ok = true;
             for (int k = 0; ok; ++k) {
                 FwdItem w;
@@ -321,19 +321,18 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                     if (j >= n) continue;
                     const uint32_t x = kv + 2 * j + (is_s ? 0 : 1);
                     const bool last_use = t == 0 || j >= n0;  // of this K or V tile
-                    const uint32_t st = (parity >> g) & 1, it = (parity >> (2 + g)) & 1;
-                    // where the operands are, before the waits (computed behind them the kernel takes the same time)
-                    uint32_t at_g = is_s ? dQ0 + g * (C::kTileBytes >> 4) : tmem_base + C::kColP + g * 64;
-                    uint32_t at_x = is_s ? desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes) : desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
-                    uint32_t acc = tmem_base + (is_s ? C::kColS + (C::kScoreBufs == 1 ? 0 : g) * kTile : C::kColO + g * HD);
+                    const uint32_t st = (g ? n_st[1] : n_st[0]) & 1, it = (g ? n_it[1] : n_it[0]) & 1;
                     // what tile 1 has used, tile 0 need not wait for again
                     if (t == 1 && !mbar_wait_uniform(&bars->kv_full[x % C::kRing], (x / C::kRing) & 1, ctx, kWaitFwd + 5)) { ok = false; break; }
                     if (is_s) {
                         if (j == 0 && !mbar_wait_uniform(&bars->q_full[g], it, ctx, kWaitFwd + 4)) { ok = false; break; }
                         const int buf = C::kScoreBufs == 1 ? 0 : g;
-                        const uint32_t use = C::kScoreBufs == 1 ? parity >> 4 : st;
+                        const uint32_t use = C::kScoreBufs == 1 ? n_s & 1 : st;
                         if (!mbar_wait_uniform(&bars->s_empty[buf], use ^ 1, ctx, kWaitFwd + 6)) { ok = false; break; }
                         tc_fence_after();
+                        const uint32_t at_g = dQ0 + g * (C::kTileBytes >> 4);
+                        const uint32_t at_x = desc_lo_k_major(aKV + (x % C::kRing) * C::kTileBytes);
+                        const uint32_t acc = tmem_base + C::kColS + buf * kTile;
                         if (elect_one()) {
 #pragma unroll
                             for (int kk = 0; kk < HD / 16; ++kk)
@@ -343,8 +342,11 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                             if (j == n - 1) mma_commit(&bars->q_empty[g]);
                         }
                         __syncwarp();
+                        ++n_s;
                     } else {
                         if (j == 0 && !mbar_wait_uniform(&bars->o_empty[g], it ^ 1, ctx, kWaitFwd + 7)) { ok = false; break; }
+                        const uint32_t at_x = desc_lo_mn_major(aKV + (x % C::kRing) * C::kTileBytes, C::kBoxBytes);
+                        const uint32_t at_g = tmem_base + C::kColP + g * 64, acc = tmem_base + C::kColO + g * HD;
                         if (!mbar_wait_uniform(&bars->p_full[g], st, ctx, kWaitFwd + 8)) { ok = false; break; }
                         tc_fence_after();
                         if (elect_one()) {
@@ -363,7 +365,8 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
                         }
                         __syncwarp();
                     }
-                    parity ^= (1u << g) | (j == n - 1 ? 4u << g : 0u) | 16u;
+                    if (g) ++n_st[1], n_it[1] += j == n - 1;
+                    else ++n_st[0], n_it[0] += j == n - 1;
                 }
                 kv += 2 * n1;
             }
