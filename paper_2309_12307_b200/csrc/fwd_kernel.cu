@@ -35,14 +35,15 @@
 //
 // What bounds it: the softmax (a step of both tiles keeps the special-function unit busy for 2048 clocks and the
 // tensor pipe for 2048) and, sustained, the power limit: a loop of forward calls on Llama2-7B 32k runs at 1244 TFLOP/s,
-// 0.92 of what the cuBLAS loop sustains, the forward within a training step at 1142, 0.84.  Microseconds a call in a loop: first form (one query tile per block, two blocks per SM, two threads
-// per row, scores read twice), two tiles with P over S, P in columns of its own:
+// 0.92 of what the cuBLAS loop sustains, the forward within a training step at 1176, 0.84.  Microseconds a call in a
+// loop: first form (one query tile per block, two blocks per SM, two threads per row, scores read twice), two tiles with
+// P over S, P in columns of its own:
 //   Llama2-7B 32k 2383, 1982, 1768; 8k 211, 162, 145; causal 8k 610, 497, 449;
 //   groups of 512 99, 73, 70; groups of 200 (head size 64) 40, 32, 29; head size 64 at 32k 1800, 1514, 1374
 // Since then the groups of softmax warps take the tiles in turn and the read-out is one loop body; thousands of clocks a
 // launch (microseconds follow the clock of the day), before and now:
-//   32k 2500, 2502; 8k 213, 204; causal 8k 654, 656; groups of 512 112, 98; groups of 200 (head size 64) 50.7, 47.6;
-//   2 x 4096 grouped query 124, 117.6; head size 64 at 32k 2424, 2421
+//   32k 2503, 2506; 8k 213, 203; causal 8k 654, 657; groups of 512 112, 99; groups of 200 (head size 64) 50.5, 47.3;
+//   2 x 4096 grouped query 124, 117.5; head size 64 at 32k 2425, 2418
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
 
