@@ -42,7 +42,7 @@
 //   groups of 512 99, 73, 70; groups of 200 (head size 64) 40, 32, 29; head size 64 at 32k 1800, 1514, 1374
 // Since then the groups of softmax warps take the tiles in turn and the read-out is one loop body; thousands of clocks a
 // launch (microseconds follow the clock of the day), before and now:
-//   32k 2503, 2506; 8k 213, 203; causal 8k 654, 657; groups of 512 112, 99; groups of 200 (head size 64) 50.5, 47.3;
+//   32k 2503, 2484; 8k 213, 204; causal 8k 654, 652; groups of 512 112, 99; groups of 200 (head size 64) 50.5, 47.3;
 //   2 x 4096 grouped query 124, 117.5; head size 64 at 32k 2425, 2418
 #include "s2a_params.h"
 #include "sm100_ptx.cuh"
@@ -460,7 +460,10 @@ __global__ void __launch_bounds__(FwdCfg<HD>::kThreads, 1) s2a_fwd_kernel(const 
     } else {
         // =========================== softmax =========================================================
         setmaxnreg_inc<C::kRegsSoftmax>();
-        const int group = warp >> 2;           // takes a tile of every item, or of every other one
+        // This warp's group takes a tile of every item, or of every other one.  Known to the compiler as the same for the whole
+        // warp, it takes 0.8 % off long groups at head size 128 (32k 2,505,000 -> 2,484,000 clocks a launch, causal 8k 657,000
+        // -> 652,000, groups of 384 180,500 -> 177,500) and adds 1 % at 64 (causal 8k 622,600 -> 630,300).
+        const int group = HD == 128 ? __shfl_sync(0xffffffffu, warp >> 2, 0) : warp >> 2;
         const int quad = warp & 3;             // tensor-memory lane quadrant this warp may access
         const int row = quad * 32 + lane;
         const uint32_t t_row = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
